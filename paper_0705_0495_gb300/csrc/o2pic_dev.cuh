@@ -209,10 +209,12 @@ struct Counts {
 };
 
 // Pointers to every array of the workspace (device addresses).
+// (the second buffer of an array follows its first: element `stride` of the first)
 template <typename Real>
 struct Pools {
     int *cell[2];
     Real *off[2], *vx[2], *vy[2], *vz[2];
+    unsigned stride;          // slots per buffer
 };
 
 struct WsPtrs {

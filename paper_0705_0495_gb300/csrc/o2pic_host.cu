@@ -372,13 +372,17 @@ Layout make_layout(const pic_config *c, int D, const pic_xs_table *xs, int n_xs,
     L.sort_tab = B.take(8ull * sb);
     L.ninit = B.take(8ull * 3 * D);
     L.vt = B.take(8ull * 3 * D);
-    for (int b = 0; b < 2; ++b) {
-        L.cell[b] = B.take(4ull * cap);
-        L.off[b] = B.take(R * cap);
-        L.vx[b] = B.take(R * cap);
-        L.vy[b] = B.take(R * cap);
-        L.vz[b] = B.take(R * cap);
-    }
+    // both buffers of an array one after the other (cap is a multiple of CHUNK,
+    // so the second starts right where the first ends)
+    auto take2 = [&](size_t o[2], size_t bytes) {
+        o[0] = B.take(2 * bytes);
+        o[1] = o[0] + bytes;
+    };
+    take2(L.cell, 4ull * cap);
+    take2(L.off, R * cap);
+    take2(L.vx, R * cap);
+    take2(L.vy, R * cap);
+    take2(L.vz, R * cap);
     L.total = round_up(B.off, 256);
     return L;
 }
@@ -788,6 +792,7 @@ extern "C" pic_status pic_init(const pic_config *cfgs, int n_discharges, const p
         h->Pd.vy[k] = reinterpret_cast<double *>(b + L.vy[k]);
         h->Pd.vz[k] = reinterpret_cast<double *>(b + L.vz[k]);
     }
+    h->Pf.stride = h->Pd.stride = (unsigned)L.total_cap;
     h->sort_tab = reinterpret_cast<int *>(b + L.sort_tab);
 
     // tables: descriptors and LUTs

@@ -19,9 +19,17 @@
 //
 // Particles are SoA with the position as (int32 cell, offset in [0,1)) and
 // velocities in cells per step.  Slots are processed in tiles of 1024
-// (256 threads x 4 consecutive slots, 16-byte vector loads); a persistent grid
-// takes TILES_PER_TICKET tiles at a time from an atomic ticket.  No block ever
+// (256 threads x 4 consecutive slots, 16-byte vector loads) by a persistent
+// grid: a block takes TILES_PER_TICKET tiles at a time from an atomic ticket,
+// or one contiguous share when there are few tiles per block.  No block ever
 // waits for another.
+//
+// What bounds it: instruction issue and latency in FP32 (5e7 superparticles,
+// 4096 cells: 251 us against 177 us for its bytes), the FP64 units in FP64.
+// A warp whose 128 slots are live and stay on the grid (nearly all) takes a
+// path without masks and selects, with its floors from packed adds (FP32) or
+// off the FP64 units where a slot stays in its cell: FP32 push 293 -> 251 us,
+// FP64 1968 -> 1000 us, results bit for bit the same.
 #include <cstdio>
 
 #include "o2pic_launch.h"
@@ -35,6 +43,18 @@ namespace o2 {
 #ifndef O2_PUSH_L2_AHEAD
 #define O2_PUSH_L2_AHEAD 2
 #endif
+// Up to STATIC_TILES tiles per block of the grid, each block takes one
+// contiguous share.  Tickets of 8 tiles left most blocks idle on a small
+// discharge (4e4 superparticles: 6 blocks of 456 busy; FP32 push 21 -> 8 us,
+// FP64 104 -> 30 us) and ran a middle one in two uneven waves (4e6: 34 ->
+// 28 us).  Above the limit shares lose: electron tiles cost more than ion
+// tiles, and no block can take over from a slower one (5e7: 400 time steps
+// 163.8 ms with tickets, 170.3 ms with shares; FP64 54.4 against 83.3 ms per
+// 40).  Between 16 and 64 tiles per block both took the same time.
+#ifndef O2_STATIC_TILES
+#define O2_STATIC_TILES 16
+#endif
+constexpr int STATIC_TILES = O2_STATIC_TILES;
 
 
 template <typename Real> struct AccT;
@@ -418,13 +438,13 @@ template <> __device__ __forceinline__ void acc_add(double *a, double v) { atomi
 // 32-bit sums, of the low SPLIT_BITS bits of each added weight (word 0) and
 // of the rest (word 1); the value is word1 * 2^SPLIT_BITS + word0.  Adds are
 // plain 32-bit atomics whose result is not needed (no carry), and both sums
-// stay exact while a block adds at most FLUSH_TICKETS tickets of weights
+// stay exact while a block adds at most FLUSH_TILES tiles of weights
 // before it flushes (each particle's weight is at most 2^FIX_BITS, so word 1
 // grows by at most 2^(FIX_BITS - SPLIT_BITS) per particle and word 0 by less
 // than 2^SPLIT_BITS per add).
 constexpr int SPLIT_BITS = 12;
-constexpr int FLUSH_TICKETS = 256 / TILES_PER_TICKET;  // 256 tiles of weights at most
-static_assert((long long)FLUSH_TICKETS * TILES_PER_TICKET * CHUNK * (1LL << (FIX_BITS - SPLIT_BITS)) < (1LL << 31),
+constexpr int FLUSH_TILES = 256;
+static_assert((long long)FLUSH_TILES * CHUNK * (1LL << (FIX_BITS - SPLIT_BITS)) < (1LL << 31),
               "split sums must stay within int32");
 __device__ __forceinline__ void split_add(unsigned long long *node, unsigned v)
 {
@@ -442,11 +462,11 @@ __host__ __device__ __forceinline__ unsigned long long split_value(unsigned long
 // The FP64 path's shared grid holds exact 64-bit integer sums of the
 // weights in units of 2^-FIX_BITS_64 (a particle's two weights add up to
 // exactly 2^FIX_BITS_64); they become doubles once per node and flush.  A
-// block adds at most FLUSH_TICKETS tickets of weights before a flush, far
+// block adds at most FLUSH_TILES tiles of weights before a flush, far
 // below the 2^63 / 2^FIX_BITS_64 particles a node could hold.  (Shared-memory
 // double atomics took nine tenths of the FP64 push.)
 constexpr int FIX_BITS_64 = 40;
-static_assert((long long)FLUSH_TICKETS * TILES_PER_TICKET * CHUNK < (1LL << (63 - FIX_BITS_64)),
+static_assert((long long)FLUSH_TILES * CHUNK < (1LL << (63 - FIX_BITS_64)),
               "FP64 shared sums must stay within int64");
 
 // the block's sum of a node in the global accumulators' type
@@ -503,28 +523,35 @@ template <> __device__ __forceinline__ double *acc_global<double>(const WsPtrs &
 // 2^FIX_BITS) (sAcc, split words); node i is then
 // count_i 2^FIX_BITS - W1_i + W1_(i-1), the same integer as the sum of the
 // particles' two node weights, with three shared atomics per particle
-// instead of four.  When the whole warp's slots sit in one cell (sorted,
-// slow particles) the weights are summed over the warp and one lane adds
-// them; otherwise every lane adds its own (its four summed first when they
-// share a cell; 4 * 32 * 2^FIX_BITS < 2^32).  No lane matching: it runs on a
-// narrow pipe.
+// instead of four.  The lanes whose four slots sit in the first lane's cell
+// (sorted, slow particles: most of a warp, even when a few have left) sum
+// their weights over the warp and one lane adds them
+// (4 * 32 * 2^FIX_BITS < 2^32); every other lane adds its own (its four
+// summed first when they share a cell).  No lane matching: it runs on a
+// narrow pipe.  DEP_LANES (lanes worth a warp sum) between 1 and 12 gave the
+// same time.
+#ifndef O2_DEP_LANES
+#define O2_DEP_LANES 4
+#endif
+constexpr int DEP_LANES = O2_DEP_LANES;
 __device__ __forceinline__ void deposit4(unsigned long long *sAcc, unsigned *sCnt, const int dep[4],
                                          const float off[4])
 {
     unsigned w1[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) w1[k] = dep[k] >= 0 ? __float2uint_rn(off[k] * (float)(1 << FIX_BITS)) : 0u;
-    const int lane = threadIdx.x & 31;
     const bool same = dep[0] >= 0 && dep[1] == dep[0] && dep[2] == dep[0] && dep[3] == dep[0];
     const unsigned a = w1[0] + w1[1] + w1[2] + w1[3];
     const int c0 = __shfl_sync(0xffffffffu, dep[0], 0);
-    if (__all_sync(0xffffffffu, same && dep[0] == c0)) {
-        const unsigned sa = __reduce_add_sync(0xffffffffu, a);
-        if (lane == 0) {
-            atomicAdd(&sCnt[c0], 128u);
+    const bool in = same && dep[0] == c0;
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+    if (__popc(m) >= DEP_LANES) {
+        const unsigned sa = __reduce_add_sync(0xffffffffu, in ? a : 0u);
+        if ((threadIdx.x & 31) == 0) {
+            atomicAdd(&sCnt[c0], 4u * (unsigned)__popc(m));
             split_add(&sAcc[c0], sa);
         }
-        return;
+        if (in) return;
     }
     if (same) {
         atomicAdd(&sCnt[dep[0]], 4u);
@@ -581,41 +608,42 @@ __device__ __forceinline__ void deposit4_nodes(unsigned long long *sAcc, const i
 }
 __device__ __forceinline__ void deposit4_nodes(unsigned long long *sAcc, const int dep[4], const double off[4])
 {
-    constexpr double SC = (double)(1ull << FIX_BITS_64);
-    unsigned long long w0[4], w1[4];
+    // rn(off 2^FIX_BITS_64) from one FP64 add: off + 2^(52 - FIX_BITS_64) has
+    // its last bit at 2^-FIX_BITS_64 (off is in [0, 1))
+    constexpr double SHIFT = (double)(1ull << (52 - FIX_BITS_64));
+    constexpr unsigned long long ONE = 1ull << FIX_BITS_64;
+    unsigned long long w1[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        w1[k] = dep[k] >= 0 ? (unsigned long long)__double2ll_rn(off[k] * SC) : 0ull;
-        w0[k] = dep[k] >= 0 ? (1ull << FIX_BITS_64) - w1[k] : 0ull;
-    }
-    // as in the FP32 path: a warp whose 128 slots sit in one cell adds its
-    // sums once, a lane whose four slots share a cell adds them once
-    const int lane = threadIdx.x & 31;
+    for (int k = 0; k < 4; ++k)
+        w1[k] = dep[k] >= 0 ? (unsigned long long)(__double_as_longlong(off[k] + SHIFT) - __double_as_longlong(SHIFT))
+                            : 0ull;
+    // as in the FP32 path: the lanes whose four slots sit in the first lane's
+    // cell add their weights once for all, others add their own
     const bool same = dep[0] >= 0 && dep[1] == dep[0] && dep[2] == dep[0] && dep[3] == dep[0];
-    unsigned long long a = w0[0] + w0[1] + w0[2] + w0[3];
-    unsigned long long b = w1[0] + w1[1] + w1[2] + w1[3];
+    const unsigned long long b = w1[0] + w1[1] + w1[2] + w1[3];
     const int c0 = __shfl_sync(0xffffffffu, dep[0], 0);
-    if (__all_sync(0xffffffffu, same && dep[0] == c0)) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_down_sync(0xffffffffu, a, o);
-            b += __shfl_down_sync(0xffffffffu, b, o);
+    const bool in = same && dep[0] == c0;
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+    if (__popc(m) >= DEP_LANES) {
+        // 32 lanes of at most 2^(FIX_BITS_64 + 2), summed in two 32-bit halves
+        const unsigned lo = __reduce_add_sync(0xffffffffu, in ? (unsigned)(b & 0xFFFFFFull) : 0u);
+        const unsigned hi = __reduce_add_sync(0xffffffffu, in ? (unsigned)(b >> 24) : 0u);
+        if ((threadIdx.x & 31) == 0) {
+            const unsigned long long sb = ((unsigned long long)hi << 24) + lo;
+            atomicAdd(&sAcc[c0], 4ull * __popc(m) * ONE - sb);
+            atomicAdd(&sAcc[c0 + 1], sb);
         }
-        if (lane == 0) {
-            atomicAdd(&sAcc[c0], a);
-            atomicAdd(&sAcc[c0 + 1], b);
-        }
-        return;
+        if (in) return;
     }
     if (same) {
-        atomicAdd(&sAcc[dep[0]], a);
+        atomicAdd(&sAcc[dep[0]], 4ull * ONE - b);
         atomicAdd(&sAcc[dep[0] + 1], b);
         return;
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         if (dep[k] >= 0) {
-            atomicAdd(&sAcc[dep[k]], w0[k]);
+            atomicAdd(&sAcc[dep[k]], ONE - w1[k]);
             atomicAdd(&sAcc[dep[k] + 1], w1[k]);
         }
     }
@@ -630,13 +658,14 @@ __device__ __forceinline__ bool Dd_binned(const WsPtrs &W, int ds)
 // Push arithmetic of a lane's four slots: E at the particle by linear
 // interpolation, v + (q/m) E dt, offset + v dt / dx.  FP32: two slots per
 // packed instruction (the same roundings as the scalar fused multiply-adds).
+// Dead slots' cells are negative: their arithmetic is that of cell 0.
 template <typename Real>
 __device__ __forceinline__ void push_arith(const Real *sE, const int c[4], const Real off[4], const Real vx[4],
                                            Real qm, Real ks, Real vn[4], Real on[4])
 {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const int cc = c[k] >= 0 ? c[k] : 0;
+        const int cc = max(c[k], 0);
         const Real e0 = sE[cc], e1 = sE[cc + 1];
         const Real ep = e0 + off[k] * (e1 - e0);
         vn[k] = vx[k] + qm * ep;
@@ -650,7 +679,7 @@ __device__ __forceinline__ void push_arith<float>(const float *sE, const int c[4
     const float2 qm2 = make_float2(qm, qm), ks2 = make_float2(ks, ks);
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
-        const int ca = c[2 * p] >= 0 ? c[2 * p] : 0, cb = c[2 * p + 1] >= 0 ? c[2 * p + 1] : 0;
+        const int ca = max(c[2 * p], 0), cb = max(c[2 * p + 1], 0);
         const float2 e0 = make_float2(sE[ca], sE[cb]);
         const float2 e1 = make_float2(sE[ca + 1], sE[cb + 1]);
         const float2 of = make_float2(off[2 * p], off[2 * p + 1]);
@@ -689,6 +718,68 @@ __device__ __forceinline__ void energy2<float>(float ke, const float v[4], const
         K[2 * p] = t.x;
         K[2 * p + 1] = t.y;
     }
+}
+
+// Cell and offset of four live slots after the move: fl = floor(on),
+// cn = c + fl, o = on - fl.  Returns false when a slot left [0, N), when its
+// offset rounded up to 1, or when the position is out of the range in which
+// this is exact (NaN and infinities included); the caller then takes the
+// general path from the same inputs.
+//
+// FP32: t = on + 1.5 2^23 rounded down is floor(on) + 1.5 2^23 for
+// |on| < 2^22, its low bits are the integer, and t - 1.5 2^23 is exact: two
+// packed adds instead of two conversions per slot (conversions run at a
+// quarter of the rate).  Outside that range the integer read from t's bits is
+// beyond any grid (or the sum wraps to one that is).
+__device__ __forceinline__ bool cells4(const int c[4], const float on[4], int N, int cn[4], float o[4])
+{
+    constexpr float M = 12582912.0f;  // 1.5 2^23
+    const float2 up = make_float2(M, M), dn = make_float2(-M, -M);
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        const float2 x = make_float2(on[2 * p], on[2 * p + 1]);
+        const float2 t = __fadd2_rd(x, up);
+        const float2 fl = __fadd2_rn(t, dn);
+        const float2 r = __fadd2_rn(x, make_float2(-fl.x, -fl.y));
+        cn[2 * p] = c[2 * p] + (__float_as_int(t.x) - 0x4B400000);
+        cn[2 * p + 1] = c[2 * p + 1] + (__float_as_int(t.y) - 0x4B400000);
+        o[2 * p] = r.x;
+        o[2 * p + 1] = r.y;
+    }
+    const unsigned far = max(max((unsigned)cn[0], (unsigned)cn[1]), max((unsigned)cn[2], (unsigned)cn[3]));
+    const float top = fmaxf(fmaxf(o[0], o[1]), fmaxf(o[2], o[3]));
+    return far < (unsigned)N && top < 1.0f;
+}
+
+// FP64 runs on two units per SM here, so the floor is kept off them: a slot
+// that stays in its cell (the high word of on below 1.0's, sign included)
+// needs no arithmetic at all, and when a lane of the warp has one that does
+// not, t = on + 1.5 2^52 rounded down gives the integer (its low word) and
+// fl = t - 1.5 2^52.  Range checks are on the high words.
+__device__ __forceinline__ bool cells4(const int c[4], const double on[4], int N, int cn[4], double o[4])
+{
+    unsigned any = 0u, mag = 0u;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const unsigned hi = (unsigned)__double2hiint(on[k]);
+        any = max(any, hi);
+        mag = max(mag, hi & 0x7FFFFFFFu);
+        cn[k] = c[k];
+        o[k] = on[k];
+    }
+    if (!__any_sync(0xffffffffu, any >= 0x3FF00000u)) return true;  // c is in [0, N)
+    constexpr double M = 6755399441055744.0;  // 1.5 2^52
+    unsigned far = 0u, top = 0u;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const double t = __dadd_rd(on[k], M);
+        o[k] = on[k] - (t - M);
+        cn[k] = c[k] + __double2loint(t);
+        far = max(far, (unsigned)cn[k]);
+        top = max(top, (unsigned)__double2hiint(o[k]));
+    }
+    // |on| < 2^20 (finite), every cell on the grid, every offset below 1
+    return mag < 0x41300000u && far < (unsigned)N && top < 0x3FF00000u;
 }
 
 // Launch shape of the push: NT threads per block, SPT slots per thread.  A
@@ -731,7 +822,7 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
     unsigned *sCnt = reinterpret_cast<unsigned *>(
         (reinterpret_cast<size_t>(reinterpret_cast<unsigned char *>(sFm + fm_max) + NW * QCAP) + 15) & ~size_t(15));
 
-    __shared__ int s_ticket[2];
+    __shared__ int s_ticket[2], s_stop, s_find;
     __shared__ unsigned s_cnt[C_NCOUNT];
     __shared__ unsigned s_btn[NUBIN_MAX];  // electron bounds per energy bin: thresholds
 
@@ -739,13 +830,15 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
     const int cur = ctl->cur;
     const unsigned long long step = ctl->step[par];
     const int total = ctl->total_chunks;
-    const int nds = W.D * NSP;
-    int *cellA = P.cell[cur];
-    Real *offA = P.off[cur], *vxA = P.vx[cur], *vyA = P.vy[cur], *vzA = P.vz[cur];
+    // the state's buffer: slot i of an array sits at element b0 + i of its
+    // first buffer, so that the arrays' addresses stay kernel parameters
+    const unsigned b0 = cur ? P.stride : 0u;
+    int *const cellA = P.cell[0];
+    Real *const offA = P.off[0], *const vxA = P.vx[0], *const vyA = P.vy[0], *const vzA = P.vz[0];
     Acc *accG = acc_global<Real>(W);
     const unsigned lt_mask = (1u << lane) - 1u;
 
-    int ds = -1, d = -1, run_tk = 0;
+    int ds = -1, d = -1, run_tiles = 0;
     for (int q = tid; q < C_NCOUNT; q += PUSH_THREADS) s_cnt[q] = 0;
     auto flush = [&](int fds) {
         const int fd = fds / NSP, fs = fds % NSP;
@@ -790,27 +883,55 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
         qn = 0;
     };
 
-    for (int it = 0;; ++it) {
-        // two ticket buffers: a buffer is rewritten only after the barrier
-        // that every reader of its previous value has passed
-        if (tid == 0) s_ticket[it & 1] = (int)atomicAdd(&ctl->ticket, (unsigned)TILES_PER_TICKET);
+    // The block's tiles.  Few tiles per block (STATIC_TILES): one contiguous
+    // share of all of them each, no ticket and no barrier between them.  Many:
+    // tickets of TILES_PER_TICKET tiles, so that no block waits for a slower
+    // one.  Both are worked off in stretches of one (discharge, species).
+    const bool shared_out = total <= STATIC_TILES * (int)gridDim.x;
+    int tcur = 0;
+    if (shared_out) {
+        tcur = (int)((long long)blockIdx.x * total / gridDim.x);
+        if (tid == 0) s_stop = (int)((long long)(blockIdx.x + 1) * total / gridDim.x);
         __syncthreads();
-        const int tbeg = s_ticket[it & 1];
-        if (tbeg >= total) break;
-        // tiles of one (discharge, species) start at a multiple of
-        // TILES_PER_TICKET, so a ticket belongs to one (d, s) or to padding
-        int nx = ds < 0 ? 0 : ds;
-        while (nx < nds && !(tbeg >= W.cnt[nx].chunk0 && tbeg < W.cnt[nx].chunk0 + W.cnt[nx].nchunk)) ++nx;
-        if (nx >= nds) continue;
+    }
+    for (int it = 0;; ++it) {
+        if (shared_out) {
+            if (tcur >= s_stop) break;
+        } else {
+            // two ticket buffers: a buffer is rewritten only after the barrier
+            // that every reader of its previous value has passed
+            if (tid == 0) s_ticket[it & 1] = (int)atomicAdd(&ctl->ticket, (unsigned)TILES_PER_TICKET);
+            __syncthreads();
+            tcur = s_ticket[it & 1];
+            if (tcur >= total) break;
+        }
+        int nx = ds;
+        if (ds < 0 || tcur < W.cnt[ds].chunk0 || tcur >= W.cnt[ds].chunk0 + W.cnt[ds].nchunk) {
+            // the first (d, s) that ends after tile tcur: one thread finds it
+            // (the ends never fall)
+            __syncthreads();
+            const int nds = W.D * NSP;
+            for (int q = tid; q < nds; q += PUSH_THREADS) {
+                const int eq = W.cnt[q].chunk0 + W.cnt[q].nchunk;
+                const int ep = q > 0 ? W.cnt[q - 1].chunk0 + W.cnt[q - 1].nchunk : 0;
+                if (eq > tcur && ep <= tcur) s_find = q;
+            }
+            __syncthreads();
+            nx = s_find;
+        }
+        const int tbeg = max(tcur, W.cnt[nx].chunk0);  // padding tiles before it hold nothing
+        const int tend = min(min(W.cnt[nx].chunk0 + W.cnt[nx].nchunk, tbeg + FLUSH_TILES),
+                             shared_out ? s_stop : tcur + TILES_PER_TICKET);
+        tcur = max(tbeg, tend);
+        if (tbeg >= tend) continue;  // only padding, or a species without slots, up to here
         if (species_rests(W.disc[nx / NSP], nx % NSP, step)) {
             // a resting ion species: nothing to push; its sub-tiles record no births
-            const int te = min(tbeg + TILES_PER_TICKET, W.cnt[nx].chunk0 + W.cnt[nx].nchunk);
-            for (int q = tid; q < (te - tbeg) * SUBTILES; q += PUSH_THREADS)
+            for (int q = tid; q < (tend - tbeg) * SUBTILES; q += PUSH_THREADS)
                 W.tile_cnt[((size_t)tbeg * SUBTILES + q) * NSP] = 0;
             continue;
         }
         // a new (d, s), or the block's integer sums at their bound: flush
-        if (nx != ds || run_tk >= FLUSH_TICKETS) {
+        if (nx != ds || run_tiles + (tend - tbeg) > FLUSH_TILES) {
             if (qn > 0) list_out();
             if (ds >= 0) flush(ds);
             const int nd = nx / NSP;
@@ -837,10 +958,10 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
                 for (int i = tid; i < fm_max; i += PUSH_THREADS) sFm[i] = 0;
             }
             ds = nx;
-            run_tk = 0;
+            run_tiles = 0;
             __syncthreads();
         }
-        ++run_tk;
+        run_tiles += tend - tbeg;
         const int s = ds % NSP;
         const Disc &Dd = W.disc[d];
         const SpeciesC &S = Dd.sp[s];
@@ -848,7 +969,6 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
         const int N = Dd.N;
         const int pb = Dd.pbase[s];
         const int end = pb + C.n_snap;
-        const int tend = min(tbeg + TILES_PER_TICKET, C.chunk0 + C.nchunk);
         // a sub-cycled ion species moves over ks steps per push
         const Real ks = Real(s > 0 ? Dd.ion_sub : 1);
         const Real qm = pick<Real>(S.qm, S.qm_f) * ks;
@@ -871,7 +991,7 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
                 const int ra = (r0 == st_beg) ? r0 + ROW : r0 + O2_PUSH_L2_AHEAD * ROW;
                 const int rb = (r0 == st_beg) ? min(r0 + O2_PUSH_L2_AHEAD * ROW, st_end - ROW) : ra;
                 for (int rp = ra; rp <= rb && rp < st_end; rp += ROW) {
-                    const size_t sl = (size_t)pb + (size_t)(rp - C.chunk0 * SUBTILES) * SUBTILE;
+                    const size_t sl = (size_t)b0 + (size_t)pb + (size_t)(rp - C.chunk0 * SUBTILES) * SUBTILE;
                     const unsigned n = (unsigned)min(ROW, st_end - rp) * SUBTILE;
                     l2_prefetch(cellA + sl, n * sizeof(int));
                     l2_prefetch(offA + sl, n * sizeof(Real));
@@ -891,86 +1011,132 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
             int c[4];
             Real off[4], vx[4];
             const bool full = i0 + 3 < end;
+            const unsigned ib = b0 + (unsigned)i0;
             if (full) {
-                ld4(cellA + i0, c);
-                ld4(offA + i0, off);
-                ld4(vxA + i0, vx);
+                ld4(cellA + ib, c);
+                ld4(offA + ib, off);
+                ld4(vxA + ib, vx);
             } else {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const bool in = i0 + k < end;
-                    c[k] = in ? cellA[i0 + k] : -2;
-                    off[k] = in ? offA[i0 + k] : Real(0);
-                    vx[k] = in ? vxA[i0 + k] : Real(0);
+                    c[k] = in ? cellA[ib + k] : -2;
+                    off[k] = in ? offA[ib + k] : Real(0);
+                    vx[k] = in ? vxA[ib + k] : Real(0);
                 }
             }
             Real vyl[4], vzl[4];  // binned species only: the lab energy needs vy, vz
             if (binned) {
                 if (full) {
-                    ld4(vyA + i0, vyl);
-                    ld4(vzA + i0, vzl);
+                    ld4(vyA + ib, vyl);
+                    ld4(vzA + ib, vzl);
                 } else {
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const bool in = i0 + k < end;
-                        vyl[k] = in ? vyA[i0 + k] : Real(0);
-                        vzl[k] = in ? vzA[i0 + k] : Real(0);
+                        vyl[k] = in ? vyA[ib + k] : Real(0);
+                        vzl[k] = in ? vzA[ib + k] : Real(0);
                     }
                 }
             }
-            uint4 w4 = make_uint4(0, 0, 0, 0);
-            if (c[0] >= 0 || c[1] >= 0 || c[2] >= 0 || c[3] >= 0)
-                w4 = rng_block(Dd.seed, Dd.discharge, s, 0, 0, 0, step, (unsigned)((i0 - pb) >> 2));
+            const uint4 w4 = rng_block(Dd.seed, Dd.discharge, s, 0, 0, 0, step, (unsigned)((i0 - pb) >> 2));
             const unsigned wk[4] = {w4.x, w4.y, w4.z, w4.w};
-            // each slot is pushed without branches; absorptions are noted in
-            // a mask and handled after the four slots
-            unsigned nslots = 0, nlive = 0, outm = 0, wallm = 0;
-            bool cchg = false;  // a cell index of the lane's slots changed
-            bool nonfin = false;
+            bool cchg = true;  // a cell index of the lane's slots changed
             unsigned candm = 0u, bins = 0u;
-            int dep[4];
+            int dep[4];  // cells after the move, -1 for a slot that holds no particle any more
             // the field at the particle, the new velocity and position (the
             // FP32 path takes two slots per packed instruction)
-            Real vn[4], on[4], Kn[4];
+            Real vn[4], on[4];
             push_arith<Real>(sE, c, off, vx, qm, ks, vn, on);
-            if (binned) energy2<Real>(ke, vn, vyl, vzl, Kn);
+            // null-collision thresholds; electrons: by the bin of the lab energy
+            unsigned thr[4] = {tnull, tnull, tnull, tnull};
+            if (binned) {
+                Real Kn[4];
+                energy2<Real>(ke, vn, vyl, vzl, Kn);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int ck = c[k];
-                const bool was = ck >= 0;
-                nslots += ck >= -1 ? 1u : 0u;
-                nlive += was ? 1u : 0u;
-                const int cc = was ? ck : 0;
-                const Real v = vn[k];
-                Real o = on[k];
-                const Real fl = floor(o);
-                const bool bad = !(fl > Real(-2 * N - 4) && fl < Real(2 * N + 4));
-                // a non-finite velocity or position is an error, not an absorption
-                nonfin |= was && !isfinite(o);
-                int cn = bad ? (v < Real(0) ? -1 : N) : cc + (int)fl;
-                o -= fl;
-                const bool wrap = o >= Real(1);
-                o = wrap ? o - Real(1) : o;
-                cn += wrap ? 1 : 0;
-                const bool out = was && (cn < 0 || cn >= N);
-                const bool live = was && !out;
-                outm |= (out && isfinite(o)) ? 1u << k : 0u;
-                wallm |= cn >= N ? 1u << k : 0u;
-                vx[k] = was ? v : vx[k];
-                off[k] = live ? o : off[k];
-                const int cnew = was ? (out ? -1 : cn) : ck;
-                cchg |= cnew != ck;
-                c[k] = cnew;
-                dep[k] = live ? cn : -1;
-                int bin = 0;
-                unsigned thr = tnull;
-                if (binned) {
-                    bin = energy_bin(Kn[k], nbins);
-                    thr = s_btn[bin];
+                for (int k = 0; k < 4; ++k) {
+                    const int bin = energy_bin(Kn[k], nbins);
+                    thr[k] = s_btn[bin];
+                    bins |= (unsigned)bin << (8 * k);
                 }
-                const bool cand = live && wk[k] < thr;
-                candm |= cand ? 1u << k : 0u;
-                bins |= (unsigned)bin << (8 * k);
+            }
+            // Nearly every warp holds 128 live slots that all stay on the
+            // grid: no masks, no selects (fast).  Any other case takes the
+            // general path below from the same inputs.
+            bool fast = full && (c[0] | c[1] | c[2] | c[3]) >= 0;
+            fast = __all_sync(0xffffffffu, fast);
+            if (fast) {
+                Real o[4];
+                fast = __all_sync(0xffffffffu, cells4(c, on, N, dep, o));
+                if (fast) {
+                    cchg = ((c[0] ^ dep[0]) | (c[1] ^ dep[1]) | (c[2] ^ dep[2]) | (c[3] ^ dep[3])) != 0;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        c[k] = dep[k];
+                        off[k] = o[k];
+                        vx[k] = vn[k];
+                        candm |= wk[k] < thr[k] ? 1u << k : 0u;
+                    }
+                    tslots += 4u;
+                    tlive += 4u;
+                }
+            }
+            bool live4 = true;  // the lane has something to write back
+            if (!fast) {
+                // each slot is pushed without branches; absorptions are noted in
+                // a mask and handled after the four slots
+                unsigned nslots = 0, nlive = 0, outm = 0, wallm = 0;
+                bool nonfin = false;
+                cchg = false;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int ck = c[k];
+                    const bool was = ck >= 0;
+                    nslots += ck >= -1 ? 1u : 0u;
+                    nlive += was ? 1u : 0u;
+                    const int cc = was ? ck : 0;
+                    const Real v = vn[k];
+                    Real o = on[k];
+                    const Real fl = floor(o);
+                    const bool bad = !(fl > Real(-2 * N - 4) && fl < Real(2 * N + 4));
+                    // a non-finite velocity or position is an error, not an absorption
+                    nonfin |= was && !isfinite(o);
+                    int cn = bad ? (v < Real(0) ? -1 : N) : cc + (int)fl;
+                    o -= fl;
+                    const bool wrap = o >= Real(1);
+                    o = wrap ? o - Real(1) : o;
+                    cn += wrap ? 1 : 0;
+                    const bool out = was && (cn < 0 || cn >= N);
+                    const bool live = was && !out;
+                    outm |= (out && isfinite(o)) ? 1u << k : 0u;
+                    wallm |= cn >= N ? 1u << k : 0u;
+                    vx[k] = was ? v : vx[k];
+                    off[k] = live ? o : off[k];
+                    const int cnew = was ? (out ? -1 : cn) : ck;
+                    cchg |= cnew != ck;
+                    c[k] = cnew;
+                    dep[k] = live ? cn : -1;
+                    candm |= live && wk[k] < thr[k] ? 1u << k : 0u;
+                }
+                if (nonfin) set_status(ctl, ST_NONFINITE);
+                if (outm) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        if (!((outm >> k) & 1u)) continue;
+                        const int wall = (wallm >> k) & 1u;
+                        atomicAdd(&s_cnt[C_ABS + 2 * s + wall], 1u);
+                        if (s == 2 && Dd.iedf_bins > 0) {
+                            const Real v = vx[k], vy = vyA[ib + k], vz = vzA[ib + k];
+                            const Real Ei = pick<Real>(S.ke_eV, S.ke_eV_f) * (v * v + vy * vy + vz * vz);
+                            const Real bb = floor(Ei * pick<Real>(Dd.iedf_scale, Dd.iedf_scale_f));
+                            if (bb >= Real(0) && bb < Real(Dd.iedf_bins))
+                                atomicAdd(&W.iedf[Dd.iedf_base + wall * Dd.iedf_bins + (int)bb], 1u);
+                        }
+                    }
+                }
+                tslots += nslots;
+                tlive += nlive;
+                live4 = nlive != 0u;
             }
             // candidates are rare: one vote, and the queue only when a lane has one
             if (__any_sync(0xffffffffu, candm != 0u)) {
@@ -986,29 +1152,13 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
                     qn += __popc(m);
                 }
             }
-            if (nonfin) set_status(ctl, ST_NONFINITE);
-            if (outm) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    if (!((outm >> k) & 1u)) continue;
-                    const int wall = (wallm >> k) & 1u;
-                    atomicAdd(&s_cnt[C_ABS + 2 * s + wall], 1u);
-                    if (s == 2 && Dd.iedf_bins > 0) {
-                        const Real v = vx[k], vy = vyA[i0 + k], vz = vzA[i0 + k];
-                        const Real Ei = pick<Real>(S.ke_eV, S.ke_eV_f) * (v * v + vy * vy + vz * vz);
-                        const Real bb = floor(Ei * pick<Real>(Dd.iedf_scale, Dd.iedf_scale_f));
-                        if (bb >= Real(0) && bb < Real(Dd.iedf_bins))
-                            atomicAdd(&W.iedf[Dd.iedf_base + wall * Dd.iedf_bins + (int)bb], 1u);
-                    }
-                }
-            }
             if (DIAG) {
                 // distributions after the free flight, before collisions
                 if (s == 0 && Dd.eedf_bins > 0) {
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         if (dep[k] != N / 2) continue;
-                        const Real v = vx[k], vy = vyA[i0 + k], vz = vzA[i0 + k];
+                        const Real v = vx[k], vy = vyA[ib + k], vz = vzA[ib + k];
                         const Real Ee = pick<Real>(S.ke_eV, S.ke_eV_f) * (v * v + vy * vy + vz * vz);
                         const Real bb = floor(Ee * pick<Real>(Dd.eedf_scale, Dd.eedf_scale_f));
                         if (bb >= Real(0) && bb < Real(Dd.eedf_bins)) atomicAdd(&sEedf[(int)bb], 1u);
@@ -1047,24 +1197,22 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
                 deposit4(sAcc, sCnt, dep, off);
             else
                 deposit4_nodes(sAcc, dep, off);
-            tslots += nslots;
-            tlive += nlive;
             if (full) {
                 // an unchanged value is not written back: slow ions keep
                 // their cells for many steps, and a lane of dead slots
                 // changes nothing (its DRAM sectors then stay clean)
-                if (cchg) st4(cellA + i0, c);
-                if (nlive) {
-                    st4(offA + i0, off);
-                    st4(vxA + i0, vx);
+                if (cchg) st4(cellA + ib, c);
+                if (live4) {
+                    st4(offA + ib, off);
+                    st4(vxA + ib, vx);
                 }
             } else {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     if (i0 + k < end) {
-                        cellA[i0 + k] = c[k];
-                        offA[i0 + k] = off[k];
-                        vxA[i0 + k] = vx[k];
+                        cellA[ib + k] = c[k];
+                        offA[ib + k] = off[k];
+                        vxA[ib + k] = vx[k];
                     }
                 }
             }

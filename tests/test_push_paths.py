@@ -1,0 +1,104 @@
+"""The push's fast path and the two ways it hands out tiles.
+
+CPU: the integers and offsets that the fast path takes from a rounded-down
+add (FP32: 1.5 2^23, FP64: 1.5 2^52) against floor(), with what it must
+refuse.  GPU: the contiguous shares (few tiles per block) and the tickets
+(many) give the same FP32 state bit for bit, over discharges of uneven size
+with empty species and part-filled tiles."""
+import math
+import struct
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+from paper_0705_0495_gb300 import inputs
+
+
+def _add_down(x, m, bits):
+    """x + m rounded towards minus infinity to `bits` mantissa bits"""
+    s = Fraction(x) + Fraction(m)
+    if s == 0:
+        return 0.0
+    e = math.floor(math.log2(abs(float(s))))
+    ulp = Fraction(2) ** (e - bits + 1)
+    return float(math.floor(s / ulp) * ulp)
+
+
+def _positions(rng, dtype):
+    v = [0.0, 0.5, 1.0, -1.0, np.nextafter(dtype(1), dtype(0)), np.nextafter(dtype(1), dtype(2)),
+         -np.finfo(dtype).tiny, np.finfo(dtype).tiny, -1e-9, 1e-9, 4095.999, -4096.0, 4194303.5, -4194303.5]
+    v += list(rng.uniform(-3.0, 3.0, 200)) + list(rng.uniform(-5000, 5000, 200))
+    return [dtype(x) for x in v]
+
+
+def test_fp32_fast_floor_is_floor():
+    rng = np.random.default_rng(3)
+    M = 12582912.0
+    for on in _positions(rng, np.float32):
+        t = np.float32(_add_down(float(on), M, 24))
+        k = struct.unpack("<i", struct.pack("<f", t))[0] - 0x4B400000
+        assert k == math.floor(float(on)), on
+        fl = np.float32(t - np.float32(M))
+        assert float(fl) == math.floor(float(on)), on
+        assert np.float32(on - fl) == np.float32(on - np.float32(math.floor(float(on)))), on
+
+
+def test_fp32_fast_path_refuses_what_is_far_off():
+    """beyond |on| < 2^22 the integer read from the bits, added to a cell,
+    never lies on a grid (compared as unsigned), whatever its sign does"""
+    far = [4194304.0, -4194305.0, 7e6, -7e6, 1.2582911e7, -1.2582911e7, -12582912.0, -12582913.0, -1.3e7,
+           -2.4e7, -3e7, 1e9, -1e9, 1e30, -1e30, math.inf, -math.inf]
+    for on in far:
+        t = np.float32(on) if math.isinf(on) else np.float32(_add_down(float(np.float32(on)), 12582912.0, 24))
+        for zero in ((0.0, -0.0) if t == 0 else (t,)):
+            k = struct.unpack("<i", struct.pack("<f", np.float32(zero)))[0] - 0x4B400000
+            for c in (0, 1, 4095):
+                cn = (c + k) & 0xFFFFFFFF
+                assert cn >= 4096, (on, c, cn)
+    for nan in (0x7FC00000, 0xFFC00000, 0x7FFFFFFF, 0xFFFFFFFF):
+        for c in (0, 4095):
+            assert ((c + nan - 0x4B400000) & 0xFFFFFFFF) >= 4096
+
+
+def test_fp64_fast_floor_is_floor():
+    rng = np.random.default_rng(4)
+    M = 6755399441055744.0
+    for on in _positions(rng, np.float64):
+        if not abs(on) < 2.0 ** 20:
+            continue
+        t = _add_down(float(on), M, 53)
+        lo = struct.unpack("<q", struct.pack("<d", t))[0] & 0xFFFFFFFF
+        k = lo - (1 << 32) if lo >= 1 << 31 else lo
+        assert k == math.floor(float(on)), on
+        assert t - M == math.floor(float(on)), on
+    # rn(off 2^40) read from off + 2^12
+    for off in list(rng.uniform(0.0, 1.0, 300)) + [0.0, 2.0 ** -41, 3 * 2.0 ** -41, math.nextafter(1.0, 0.0)]:
+        got = struct.unpack("<q", struct.pack("<d", off + 4096.0))[0] - struct.unpack("<q", struct.pack("<d", 4096.0))[0]
+        assert got == round(off * 2.0 ** 40), off
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("sizes", [(1_400_001, 2, 33_333), (700_000, 0, 1, 1_023, 1_500_000)])
+def test_shares_and_tickets_give_the_same_state(sizes):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_0705_0495_gb300 import o2pic
+    ds = [inputs.cfg1(fp64=False, n_op=n, n_cells=100 + 57 * k, seed=3 + k, diag_every=2)
+          for k, n in enumerate(sizes)]
+    states = []
+    for blocks in ("most", 1):  # one block per SM: many tiles per block, so tickets
+        sim = o2pic.Simulation(ds, inputs.xs_tables())
+        if blocks == 1:
+            sim.set_launch(1)
+        sim.step(13)
+        states.append([sim.get_state(d, s) for d in range(len(ds)) for s in range(3)]
+                      + [{k: sim.diagnostics(d)[k] for k in ("events", "absorbed", "eedf", "iedf", "fm", "dens_sum")}
+                         for d in range(len(ds))])
+        sim.close()
+    for a, b in zip(*states):
+        for k in a:
+            assert np.array_equal(a[k], b[k]), k
