@@ -250,6 +250,9 @@ Layout make_layout(const pic_config *c, int D, const pic_xs_table *xs, int n_xs,
     const size_t R = fp64 ? 8 : 4;
     int tn = 0, tc = 0, mc = 0, cap = 0, sb = 0, maxN = 0, em = 0, fmm = 0;
     long long sortc = 0, csb = 0, eb = 0, ib = 0, fb = 0;
+    long long cap_all = 0;
+    for (int d = 0; d < D; ++d)
+        for (int s = 0; s < 3; ++s) cap_all += (long long)round_up((size_t)std::max(1LL, c[d].capacity[s]), CHUNK);
     L.pbase.resize(3 * D);
     L.capr.resize(3 * D);
     L.sort_cbase.resize(3 * D);
@@ -279,7 +282,11 @@ Layout make_layout(const pic_config *c, int D, const pic_xs_table *xs, int n_xs,
             cap += cr;
             mc = (mc + TILES_PER_TICKET - 1) / TILES_PER_TICKET * TILES_PER_TICKET;
             mc += cr / CHUNK;
-            const int g = (cr + SORT_CHUNK - 1) / SORT_CHUNK;
+            // sort rows: enough for the largest chunks, and for smaller ones a
+            // share of SORT_ROWS by capacity
+            const int fine = SORT_WARPS * sort_min_slots(N);
+            const int g = std::max((cr + SORT_CHUNK - 1) / SORT_CHUNK,
+                                   (int)std::min<long long>((cr + fine - 1) / fine, SORT_ROWS * (long long)cr / cap_all));
             L.sort_gmax[3 * d + s] = g;
             L.colscan_units += (long long)((N + 1 + 31) / 32) * ((g + COLSCAN_SEG - 1) / COLSCAN_SEG);
             L.sort_cbase[3 * d + s] = (int)sortc;

@@ -433,6 +433,7 @@ k_sort_count(WsPtrs W, Pools<Real> P, const int *tab)
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         // the column scan that follows: its warp order and the tag of its words
         W.ctl->colscan_ticket = 0u;
+        W.ctl->scatter_done = 0u;
         W.ctl->sort_epoch += 1u;
     }
     int ds, bi;
@@ -440,7 +441,8 @@ k_sort_count(WsPtrs W, Pools<Real> P, const int *tab)
     const int d = ds / NSP, s = ds % NSP;
     const Disc &Dd = W.disc[d];
     const int N = Dd.N, n = W.cnt[ds].n;
-    const int G = (n + SORT_CHUNK - 1) / SORT_CHUNK;
+    const int ws = sort_warp_slots(n, Dd.sort_gmax[s], N);
+    const int G = (n + SORT_WARPS * ws - 1) / (SORT_WARPS * ws);
     if (bi == 0 && threadIdx.x == 0) W.vmax2[ds] = 0ull;  // raised by the scatter
     if (bi >= G) return;
     const int stride = (N + 2) & ~1;
@@ -449,8 +451,8 @@ k_sort_count(WsPtrs W, Pools<Real> P, const int *tab)
     const int *cell = P.cell[W.ctl->cur] + Dd.pbase[s];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     unsigned short *hw = wsm + (size_t)w * stride;
-    const int lo = bi * SORT_CHUNK + w * SORT_WARP_SLOTS;
-    const int hi = min(n, lo + SORT_WARP_SLOTS);
+    const int lo = (bi * SORT_WARPS + w) * ws;
+    const int hi = min(n, lo + ws);
     for (int i0 = lo; i0 < hi; i0 += 32 * SORT_ILP) {
         int b[SORT_ILP];
 #pragma unroll
@@ -528,7 +530,8 @@ k_sort_colscan(WsPtrs W, const int *unit_base)
     const Disc &Dd = W.disc[d];
     const int N = Dd.N;
     const int n = W.cnt[ds].n;
-    const int G = (n + SORT_CHUNK - 1) / SORT_CHUNK;
+    const int chunk = SORT_WARPS * sort_warp_slots(n, Dd.sort_gmax[s], N);
+    const int G = (n + chunk - 1) / chunk;
     const int nseg = (Dd.sort_gmax[s] + COLSCAN_SEG - 1) / COLSCAN_SEG;
     const int local = u - unit_base[ds];
     const int grp = local / nseg, sg = local % nseg;
@@ -607,7 +610,21 @@ k_sort_cellscan(WsPtrs W)
     }
 }
 
-// Stable scatter: warp w of block bi owns slots [lo + w*SORT_WARP_SLOTS, ...);
+// The scatter block that comes last makes the sorted buffer and its slot
+// counts the current ones (every block has read the old ones by then; the
+// count kernel has reset the counter).
+__device__ __forceinline__ void sort_finish(const WsPtrs &W)
+{
+    __shared__ bool s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&W.ctl->scatter_done, 1u) == gridDim.x - 1u;
+    __syncthreads();
+    if (!s_last) return;
+    for (int ds = threadIdx.x; ds < W.D * NSP; ds += blockDim.x) W.cnt[ds].n = W.sort_live[ds];
+    if (threadIdx.x == 0) W.ctl->cur ^= 1;
+}
+
+// Stable scatter: warp w of block bi owns the slots from (bi SORT_WARPS + w) ws;
 // the per-warp bucket counts (16-bit) that the count kernel kept give each
 // warp its first slot per bucket relative to the block's, then each warp
 // walks its slots in order, ranking equal buckets inside a 32-slot row by
@@ -624,16 +641,20 @@ k_sort_scatter(WsPtrs W, Pools<Real> P, const int *tab)
     const int d = ds / NSP, s = ds % NSP;
     const Disc &Dd = W.disc[d];
     const int N = Dd.N, n = W.cnt[ds].n;
-    const int G = (n + SORT_CHUNK - 1) / SORT_CHUNK;
-    if (bi >= G) return;
+    const int ws = sort_warp_slots(n, Dd.sort_gmax[s], N);
+    const int G = (n + SORT_WARPS * ws - 1) / (SORT_WARPS * ws);
+    if (bi >= G) {
+        sort_finish(W);
+        return;
+    }
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int stride = (N + 2) & ~1;
     unsigned short *hw = hsm + (size_t)w * stride;
     const int cur = W.ctl->cur, nxt = cur ^ 1;
     const int pb = Dd.pbase[s];
     const int *cell = P.cell[cur] + pb;
-    const int lo = bi * SORT_CHUNK + w * SORT_WARP_SLOTS;
-    const int hi = min(n, lo + SORT_WARP_SLOTS);
+    const int lo = (bi * SORT_WARPS + w) * ws;
+    const int hi = min(n, lo + ws);
     // per bucket: warp offsets relative to the block's first slot in it, from
     // the warps' counts that the count kernel kept
     const unsigned short *wrow = W.sort_whist + ((size_t)Dd.sort_cbase[s] + (size_t)bi * (N + 1)) * SORT_WARPS;
@@ -721,14 +742,7 @@ k_sort_scatter(WsPtrs W, Pools<Real> P, const int *tab)
     }
     // speed bound of the species for the particle-target pass
     vmax_raise(W.vmax2, ds, (double)vm2);
-}
-
-__global__ void k_sort_finish(WsPtrs W)
-{
-    pdl_wait();
-    for (int ds = threadIdx.x; ds < W.D * NSP; ds += blockDim.x) W.cnt[ds].n = W.sort_live[ds];
-    __syncthreads();
-    if (threadIdx.x == 0) W.ctl->cur ^= 1;
+    sort_finish(W);
 }
 
 // ------------------------------------------------------------ pair pass
@@ -1642,7 +1656,7 @@ cudaError_t launch_field(bool fp64, bool diag, int mode, const WsPtrs &W, int pa
     return cudaGetLastError();
 }
 
-int kernels_per_sort() { return 5; }
+int kernels_per_sort() { return 4; }
 int kernels_per_pair() { return 7; }
 
 cudaError_t launch_sort(bool fp64, const WsPtrs &W, const void *pools, const int *tab, const LaunchCfg &L,
@@ -1663,7 +1677,6 @@ cudaError_t launch_sort(bool fp64, const WsPtrs &W, const void *pools, const int
         launch_k(k_sort_cellscan, W.D * NSP, 512, scan_smem, st, W);
         launch_k(k_sort_scatter<float>, L.sort_blocks, SORT_WARPS * 32, L.scatter_smem, st, W, P, tab);
     }
-    launch_k(k_sort_finish, 1, 256, 0, st, W);
     return cudaGetLastError();
 }
 
