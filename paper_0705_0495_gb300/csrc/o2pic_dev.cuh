@@ -66,11 +66,6 @@ __host__ __device__ __forceinline__ int sort_warp_slots(int n, int gmax, int N)
 constexpr int COLSCAN_SEG = 32;  // rows of the sort's count matrix per column-scan warp
 constexpr int PAIR_BIRTH_CAP = 16;     // births of (19) per cell per pass
 constexpr int MAX_GAS_CH = 16;
-#ifndef O2_FIELD_THREADS
-#define O2_FIELD_THREADS 1024
-#endif
-constexpr int FIELD_THREADS = O2_FIELD_THREADS;
-constexpr int FIELD_ILP = 4;  // nodes per thread whose accumulators the field kernel loads at once
 constexpr int FIX_BITS = 24;           // fixed-point deposit: weight * 2^24
 constexpr int MAX_DISCHARGES = 1024;
 constexpr long long SPIN_LIMIT = 1LL << 22;  // polls of a bounded wait

@@ -1,5 +1,7 @@
 // o2pic_kernels.cu -- field solve, cell sort, particle-target pass, load and
 // deposit kernels of libo2pic (GB300, sm_103a).
+#include <cooperative_groups.h>
+
 #include "o2pic_launch.h"
 
 namespace o2 {
@@ -32,48 +34,6 @@ __device__ __forceinline__ void dep_global(double *acc, int c, double off, int s
 {
     atomicAdd(&acc[c], sign * (1.0 - off));
     atomicAdd(&acc[c + 1], sign * off);
-}
-
-__device__ __forceinline__ double acc_to_weight(unsigned long long a)
-{
-    return (double)(long long)a * (1.0 / (double)(1 << FIX_BITS));
-}
-__device__ __forceinline__ double acc_to_weight(double a) { return a; }
-
-// inclusive scan of x[0..M) in shared memory by one block (deterministic order)
-template <int NT>
-__device__ void block_scan_inclusive(double *x, int M, double *warp_tot)
-{
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int per = (M + NT - 1) / NT;
-    const int lo = tid * per, hi = min(M, lo + per);
-    double run = 0.0;
-    for (int i = lo; i < hi; ++i) {
-        run += x[i];
-        x[i] = run;
-    }
-    // exclusive scan of the thread totals
-    double v = run;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        double t = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += t;
-    }
-    if (lane == 31) warp_tot[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        double w = lane < NT / 32 ? warp_tot[lane] : 0.0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            double t = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += t;
-        }
-        if (lane < NT / 32) warp_tot[lane] = w;
-    }
-    __syncthreads();
-    double excl = v - run + (warp > 0 ? warp_tot[warp - 1] : 0.0);
-    for (int i = lo; i < hi; ++i) x[i] += excl;
-    __syncthreads();
 }
 
 // exclusive scan of a[0..M) in shared memory by one block; returns the total
@@ -115,246 +75,302 @@ __device__ int block_scan_exclusive_int(int *a, int M, int *wsum)
 
 // ------------------------------------------------------------ field
 
-// Per discharge (one block): densities from the accumulators, Poisson with
+// Per discharge: densities from the accumulators, Poisson with
 // phi_0 = U_rf sin(2 pi f t + phase), phi_N = 0, and the node field.
-// The tridiagonal system (phi_{i-1} - 2 phi_i + phi_{i+1}) = -rho_i dx^2/eps0
-// is solved exactly by two prefix sums: with s_i = rho_i dx^2/eps0,
-// S1_i = sum_{k<=i} s_k and S2_i = sum_{m<=i} S1_m (i >= 1),
-// phi_i = phi_0 + i D0 - S2_{i-1}, D0 fixed by phi_N = 0.
+// The tridiagonal system (phi_{i-1} - 2 phi_i + phi_{i+1}) = -s_i,
+// s_i = rho_i dx^2/eps0, is solved exactly by prefix sums.  With the net
+// charge q_i of node i (interior nodes only), S1_i = sum_{k<=i} q_k and
+// S2_i = sum_{m<=i} S1_m (i >= 1):
+//   s_i = K dx q_i,  phi_i = phi_0 + i D0 - K dx S2_{i-1},
+//   D0 = (K dx S2_{N-1} - phi_0)/N  (phi_N = 0),  S2_{N-1} = sum (N - i) q_i,
+//   E_i = (K/2) T_i - D0/dx,  T_i = S1_i + S1_{i-1} inside,
+//   T_0 = -2 q_0, T_N = 2 (S1_{N-1} + q_N)  (Gauss's law on the half cells),
+// with K = e w / eps0 per unit of q.
+//
+// What bounds it: latency (a chain of a few loads, two scans and thread 0's
+// FP64 divisions), and in FP64 the few FP64 units of the one SM that solved a
+// discharge.  So a discharge of
+// more than FIELD_ONE cells is solved by a cluster of FIELD_CLUSTER blocks,
+// which exchange their two sums through distributed shared memory once; the
+// weighted sum S2_{N-1} needs no prefix, so D0 is ready together with the
+// prefixes; E comes from T_i alone, and densities, potential and FP64 field
+// are formed only when they are asked for (diagnostics, pic_fields).  The tile
+// table of the push (below) is built by one more block at the same time.
+// Kernel time with one block and full sums always -> this: 4096 cells FP32
+// 18.3 -> 8.3 us, FP64 62 -> 10.4 us; 128 cells FP64 13.5 -> 6.6 us; seven
+// discharges FP32 12.6 -> 5.6 us, 64 discharges 55 -> 7.3 us.
+constexpr int FIELD_THREADS = 256;
+constexpr int FIELD_CLUSTER = 8;
+constexpr int FIELD_ONE = 1024;  // nodes up to which one block per discharge is used
+constexpr int FIELD_PER = 5;     // most nodes per thread
+static_assert(FIELD_PER * FIELD_THREADS >= FIELD_ONE + 1 && FIELD_PER * FIELD_THREADS * FIELD_CLUSTER >= 4097, "");
+
 __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bool advance);
+
+// The sums of a block's nodes, in the units of the accumulators: exact
+// integers (2^-FIX_BITS of a particle) in the FP32 path, doubles in the FP64
+// path.  Sum1 holds S1 and q, Sum2 holds S2.
+template <typename Real> struct FieldSum;
+template <> struct FieldSum<float> {
+    using S1 = long long;
+    using S2 = __int128;
+    static __device__ __forceinline__ S1 load(unsigned long long v) { return (long long)v; }
+    static __device__ __forceinline__ S2 weigh(int w, S1 q) { return (S2)w * (S2)q; }
+    static __device__ __forceinline__ S2 up(S2 v, int o)
+    {
+        const unsigned long long lo = __shfl_up_sync(0xffffffffu, (unsigned long long)v, o);
+        const long long hi = __shfl_up_sync(0xffffffffu, (long long)(v >> 64), o);
+        return ((S2)hi << 64) | (S2)lo;
+    }
+};
+template <> struct FieldSum<double> {
+    using S1 = double;
+    using S2 = double;
+    static __device__ __forceinline__ S1 load(double v) { return v; }
+    static __device__ __forceinline__ S2 weigh(int w, S1 q) { return (double)w * q; }
+    static __device__ __forceinline__ S2 up(S2 v, int o) { return __shfl_up_sync(0xffffffffu, v, o); }
+};
 
 template <typename Real>
 __global__ void __launch_bounds__(FIELD_THREADS)
-k_field(WsPtrs W, int par, int diag, int mode)
+k_field(WsPtrs W, int par, int diag, int mode, int csize)
 {
     pdl_wait();
-    extern __shared__ __align__(16) double fsm[];
-    __shared__ double warp_tot[FIELD_THREADS / 32];
-    __shared__ double s_rho0, s_rhoN, s_D0;
+    namespace cg = cooperative_groups;
     using Acc = typename AccK<Real>::T;
-    const int d = blockIdx.x;
-    const Disc &Dd = W.disc[d];
-    const int N = Dd.N, g = Dd.gbase, tid = threadIdx.x;
+    using F = FieldSum<Real>;
+    using S1t = typename F::S1;
+    using S2t = typename F::S2;
+    constexpr int NW = FIELD_THREADS / 32;
+    constexpr bool EXACT = sizeof(Real) == 4;
+    __shared__ S1t w1[NW];                     // warp totals
+    __shared__ S2t w2[NW], w3[NW];
+    __shared__ S1t c1[FIELD_CLUSTER];          // block totals of the cluster
+    __shared__ S2t c2[FIELD_CLUSTER], c3[FIELD_CLUSTER];
+    __shared__ double s_phi0, s_D0, s_e0;
+    __shared__ long long s_T0i;
+    __shared__ float s_hKf, s_frf;
+    __shared__ int s_intE;
+    const int d = blockIdx.x / csize, rank = blockIdx.x % csize;
     Ctl *ctl = W.ctl;
     const unsigned long long step = ctl->step[par];
+    if (d == W.D) {  // the extra cluster (mode 0): this step's tile table and the step counter
+        if (rank == 0) tile_table(W, par, step, true);
+        return;
+    }
+    // every block of the cluster has started before another writes to its
+    // shared memory (waited for there)
+    if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    const Disc &Dd = W.disc[d];
+    const int N = Dd.N, g = Dd.gbase, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tn = W.total_nodes;
     const double dx = Dd.dx;
-    // the drive's potential, once per block by one thread: GB300 runs FP64 on
-    // few units, and 1024 threads each evaluating sin() would cost more than
-    // the whole solve
-    __shared__ double s_phi0;
-    auto drive = [&]() { return Dd.U_rf * sin(Dd.omega * ((double)step * Dd.dt) + Dd.phase); };
-    double phi0;
-    Real *Er = reinterpret_cast<Real *>(W.Ereal) + g;
-    Acc *acc = AccK<Real>::ptr(W);
-    if constexpr (sizeof(Real) == 4) {
-        // FP32 path: the accumulators are exact fixed-point sums (weight *
-        // 2^FIX_BITS).  With q_i the net charge in these units and
-        // K = e w 2^-FIX_BITS / eps0: interior s_i = K dx q_i, S1 = prefix
-        // sums of q (exact int64), S2 = prefix sums of S1 (exact int128), and
-        //   phi_i = phi_0 + i D0 - K dx S2_{i-1},  D0 = (K dx S2_{N-1} - phi_0)/N
-        //   E_i = (K/2) (T_i - T0),  T0 = 2 D0 / (K dx), with the integers
-        //   T_i = S1_i + S1_{i-1} inside, T_0 = -2 q_0, T_N = 2 (S1_{N-1} + q_N)
-        // (the wall values are Gauss's law on the half cells).  T_i - round(T0)
-        // is exact, so E leaves FP64 only through O(1) constants.
-        long long *S1 = reinterpret_cast<long long *>(fsm);  // N+1 entries
-        __shared__ long long wl[FIELD_THREADS / 32];
-        __shared__ __int128 w128[FIELD_THREADS / 32];
-        __shared__ long long s_q0, s_qN, s_T0i;
-        __shared__ float s_hKf, s_frf;
-        __shared__ int s_intE;
-        const double K = Dd.Kfix;  // e w 2^-FIX_BITS / eps0
-        const bool full = diag || mode != 0;
-        // the accumulators of FIELD_ILP nodes per thread are all loaded before
-        // any is cleared, so that their loads are in flight together (a store
-        // to one could otherwise alias the next load, one latency each)
-        bool clear[NSP];
+    const bool full = diag || mode != 0;
+    // nodes lo .. hi-1 of this thread: blocked, so that its prefix is local
+    const int NC = (N + 1 + csize - 1) / csize;
+    const int per = (NC + FIELD_THREADS - 1) / FIELD_THREADS;
+    const int lo = min(rank * NC + tid * per, N + 1);
+    const int hi = min(min(lo + per, (rank + 1) * NC), N + 1);
+    Acc *acc = AccK<Real>::ptr(W) + g;
+    Acc raw[NSP][FIELD_PER];
 #pragma unroll
-        for (int s = 0; s < NSP; ++s) clear[s] = mode == 0 && !species_rests(Dd, s, step);
-        for (int i0 = tid; i0 <= N; i0 += FIELD_THREADS * FIELD_ILP) {
-            long long aa[FIELD_ILP][NSP];
+    for (int k = 0; k < FIELD_PER; ++k)
 #pragma unroll
-            for (int j = 0; j < FIELD_ILP; ++j) {
-                const int i = i0 + j * FIELD_THREADS;
+        for (int s = 0; s < NSP; ++s) raw[s][k] = lo + k < hi ? acc[(size_t)s * tn + lo + k] : Acc(0);
+    // the drive's potential by one thread, of the warp with the fewest nodes,
+    // while the loads are in flight (the FP64 sine takes about 1.5 us)
+    if (tid == FIELD_THREADS - 1) s_phi0 = Dd.U_rf * sin(Dd.omega * ((double)step * Dd.dt) + Dd.phase);
+    bool clear[NSP];
 #pragma unroll
-                for (int s = 0; s < NSP; ++s) aa[j][s] = i <= N ? (long long)acc[(size_t)s * tn + g + i] : 0;
-            }
-            // thread 0 evaluates the drive while its loads are in flight
-            if (tid == 0 && i0 == 0) s_phi0 = drive();
+    for (int s = 0; s < NSP; ++s) clear[s] = mode == 0 && !species_rests(Dd, s, step);
+    S1t q[FIELD_PER];     // net charge of the node
+    S1t run = S1t(0);     // the thread's interior charge
+    S2t part = S2t(0);    // sum of (N - i) q_i over the thread's interior nodes
 #pragma unroll
-            for (int j = 0; j < FIELD_ILP; ++j) {
-                const int i = i0 + j * FIELD_THREADS;
-                if (i > N) break;
-                const long long *a = aa[j];
+    for (int k = 0; k < FIELD_PER; ++k) {
+        const int i = lo + k;
+        q[k] = S1t(0);
+        if (i >= hi) continue;
+        S1t a[NSP];
+#pragma unroll
+        for (int s = 0; s < NSP; ++s) {
+            a[s] = F::load(raw[s][k]);
+            if (clear[s]) acc[(size_t)s * tn + i] = Acc(0);
+        }
+        q[k] = a[2] - a[0] - a[1];
+        if (i > 0 && i < N) {
+            run += q[k];
+            part += F::weigh(N - i, q[k]);
+        }
+        if (full) {
+            if constexpr (EXACT) {
+                const double sc = (i == 0 || i == N) ? Dd.dens_fix_wall : Dd.dens_fix;
 #pragma unroll
                 for (int s = 0; s < NSP; ++s) {
-                    const size_t k = (size_t)s * tn + g + i;
-                    if (clear[s]) acc[k] = Acc(0);
-                    if (diag) W.dens_sum_fix[k] += a[s];  // exact sums; scaled at read-out
+                    const size_t j = (size_t)s * tn + g + i;
+                    if (diag) W.dens_sum_fix[j] += a[s];  // exact sums; scaled at read-out
+                    W.dens[j] = (double)a[s] * sc;
                 }
-                const long long q = a[2] - a[0] - a[1];
-                S1[i] = (i == 0 || i == N) ? 0 : q;
-                if (i == 0) s_q0 = q;
-                if (i == N) s_qN = q;
-                if (full) {
-                    const double sc = (i == 0 || i == N) ? Dd.dens_fix_wall : Dd.dens_fix;
+                W.rho[g + i] = QE_ * (double)q[k] * sc;
+            } else {
+                const double sc = Dd.weight / ((i == 0 || i == N) ? 0.5 * dx : dx);
+                double dn[NSP];
 #pragma unroll
-                    for (int s = 0; s < NSP; ++s) W.dens[(size_t)s * tn + g + i] = (double)a[s] * sc;
-                    W.rho[g + i] = QE_ * (double)q * sc;
+                for (int s = 0; s < NSP; ++s) {
+                    const size_t j = (size_t)s * tn + g + i;
+                    dn[s] = a[s] * sc;
+                    W.dens[j] = dn[s];
+                    if (diag) W.dens_sum[j] += dn[s];
                 }
+                W.rho[g + i] = QE_ * (dn[2] - dn[0] - dn[1]);
             }
         }
-        __syncthreads();
-        phi0 = s_phi0;
-        // inclusive int64 scan of S1[1..N-1] and the int128 sum of the result
-        const int M = N - 1, lane = tid & 31, warp = tid >> 5;
-        const int per = (M + FIELD_THREADS - 1) / FIELD_THREADS;
-        const int lo = 1 + tid * per, hi = min(N, lo + per);
-        long long run = 0;
-        for (int i = lo; i < hi; ++i) {
-            run += S1[i];
-            S1[i] = run;
-        }
-        long long v = run;
+    }
+    // inclusive scan of the threads' charge, sum of their weighted charge
+    S1t v = run;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long x = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += x;
-        }
-        if (lane == 31) wl[warp] = v;
-        __syncthreads();
-        if (warp == 0) {
-            long long w = lane < FIELD_THREADS / 32 ? wl[lane] : 0;
+    for (int o = 1; o < 32; o <<= 1) {
+        const S1t x = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += x;
+    }
+    S2t r = part;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const long long x = __shfl_up_sync(0xffffffffu, w, o);
-                if (lane >= o) w += x;
+    for (int o = 1; o < 32; o <<= 1) {
+        const S2t x = F::up(r, o);
+        if (lane >= o) r += x;
+    }
+    if (lane == 31) {
+        w1[warp] = v;
+        w2[warp] = r;
+    }
+    __syncthreads();
+    S1t excl = v - run;  // charge of the nodes before this thread's
+    for (int w = 0; w < warp; ++w) excl += w1[w];
+    if (csize > 1) {
+        cg::cluster_group cl = cg::this_cluster();
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (tid < csize) {
+            S1t t1 = w1[0];
+            S2t t2 = w2[0];
+            for (int w = 1; w < NW; ++w) {
+                t1 += w1[w];
+                t2 += w2[w];
             }
-            if (lane < FIELD_THREADS / 32) wl[lane] = w;
+            *cl.map_shared_rank(&c1[rank], tid) = t1;
+            *cl.map_shared_rank(&c2[rank], tid) = t2;
         }
-        __syncthreads();
-        const long long excl = v - run + (warp > 0 ? wl[warp - 1] : 0);
-        __int128 part = 0;
-        for (int i = lo; i < hi; ++i) {
-            S1[i] += excl;
-            part += (__int128)S1[i];
-        }
-        // inclusive int128 scan of the thread parts (the total is S2_{N-1})
-        __int128 pv = part;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long lo_ = __shfl_up_sync(0xffffffffu, (unsigned long long)pv, o);
-            const long long hi_ = __shfl_up_sync(0xffffffffu, (long long)(pv >> 64), o);
-            if (lane >= o) pv += ((__int128)hi_ << 64) | (__int128)lo_;
-        }
-        if (lane == 31) w128[warp] = pv;
-        __syncthreads();
-        if (tid == 0) {
-            __int128 r = 0;
-            for (int w = 0; w < FIELD_THREADS / 32; ++w) {
-                r += w128[w];
-                w128[w] = r;
-            }
-            const double D0 = (K * dx * (double)r - phi0) / (double)N;
-            s_D0 = D0;
+        cl.sync();
+        for (int c = 0; c < rank; ++c) excl += c1[c];
+    }
+    // K dx and D0, in the order of the formulas above
+    const double K = EXACT ? Dd.Kfix : QE_ * Dd.weight / EPS0_;
+    if (tid == 0) {
+        S2t tot = S2t(0);
+        if (csize > 1)
+            for (int c = 0; c < csize; ++c) tot += c2[c];
+        else
+            for (int w = 0; w < NW; ++w) tot += w2[w];
+        const double phi0 = s_phi0;
+        const double D0 = (K * dx * (double)tot - phi0) / (double)N;
+        s_D0 = D0;
+        if constexpr (EXACT) {
+            // E_i = (K/2) (T_i - T0) with T0 = 2 D0 / (K dx): T_i - round(T0) is
+            // exact, so E leaves FP64 only through O(1) constants
             const double T0 = 2.0 * D0 / (K * dx);
             s_intE = (K > 0.0 && fabs(T0) < 4.0e18) ? 1 : 0;
             const long long T0i = s_intE ? llround(T0) : 0;
             s_T0i = T0i;
             s_hKf = (float)(0.5 * K);
             s_frf = (float)(T0 - (double)T0i);
-            if (diag) {
+        } else {
+            s_e0 = D0 / dx;
+        }
+        if (diag && rank == 0) {
+            if constexpr (EXACT) {
                 W.phi0_sum[d] += phi0;
                 W.D0_sum[d] += D0;
             }
+            W.nsamp[d] += 1ull;
         }
-        __syncthreads();
-        const long long T0i = s_T0i;
-        const float hKf = s_hKf, frf = s_frf;
-        const bool intE = s_intE != 0;
-        for (int i = tid; i <= N; i += FIELD_THREADS) {
-            const long long Ti = (i == 0) ? -2 * s_q0 : (i == N ? 2 * (S1[N - 1] + s_qN) : S1[i] + S1[i - 1]);
-            if (intE) {
-                Er[i] = hKf * (__ll2float_rn(Ti - T0i) - frf);
-                if (full) W.Efield[g + i] = 0.5 * K * ((double)(Ti - T0i) - (double)frf);
+    }
+    __syncthreads();
+    const double D0 = s_D0;
+    Real *Er = reinterpret_cast<Real *>(W.Ereal) + g;
+    S1t s1 = excl;
+    S2t sum = S2t(0);  // the thread's share of S2
+#pragma unroll
+    for (int k = 0; k < FIELD_PER; ++k) {
+        const int i = lo + k;
+        if (i >= hi) break;
+        S1t T;
+        if (i == 0) T = -(q[k] + q[k]);
+        else if (i == N) T = (s1 + q[k]) + (s1 + q[k]);
+        else {
+            T = s1 + s1 + q[k];
+            s1 += q[k];
+            sum += (S2t)s1;
+        }
+        if constexpr (EXACT) {
+            if (s_intE) {
+                const long long dT = T - s_T0i;
+                Er[i] = s_hKf * (__ll2float_rn(dT) - s_frf);
+                if (full) W.Efield[g + i] = 0.5 * K * ((double)dT - (double)s_frf);
             } else {  // no charge or an extreme field: evaluate in FP64
-                const double E = -s_D0 / dx + 0.5 * K * (double)Ti;
+                const double E = -D0 / dx + 0.5 * K * (double)T;
                 Er[i] = (Real)E;
                 if (full) W.Efield[g + i] = E;
             }
-        }
-        const double D0 = s_D0;
-        if (full) {
-            // potential and the exact running sums of S2 for its average
-            const __int128 before = (warp > 0 ? w128[warp - 1] : (__int128)0) + pv - part;
-            __int128 r = before;
-            for (int i = lo; i < hi; ++i) {
-                // r = S2_{i-1} when node i is reached
-                double p = phi0 + (double)i * D0 - K * dx * (double)r;
-                if (diag) W.phi_s2_sum[g + i] += r;
-                W.phi[g + i] = p;
-                r += (__int128)S1[i];
-            }
-            if (tid == 0) W.phi[g] = phi0;
-            if (tid == 0) W.phi[g + N] = 0.0;
-        }
-    } else {
-        if (tid == 0) s_phi0 = drive();
-        __syncthreads();
-        phi0 = s_phi0;
-        double *x = fsm;  // N+1 entries
-        for (int i = tid; i <= N; i += FIELD_THREADS) {
-            const double vol = (i == 0 || i == N) ? 0.5 * dx : dx;
-            const double scale = Dd.weight / vol;
-            double dn[NSP];
-#pragma unroll
-            for (int s = 0; s < NSP; ++s) {
-                const size_t k = (size_t)s * tn + g + i;
-                dn[s] = acc_to_weight(acc[k]) * scale;
-                if (mode == 0 && !species_rests(Dd, s, step)) acc[k] = Acc(0);
-                W.dens[k] = dn[s];
-                if (diag) W.dens_sum[k] += dn[s];
-            }
-            const double rho = QE_ * (dn[2] - dn[0] - dn[1]);
-            W.rho[g + i] = rho;
-            if (i == 0) s_rho0 = rho;
-            if (i == N) s_rhoN = rho;
-            x[i] = rho * dx * dx / EPS0_;
-        }
-        __syncthreads();
-        // scans over interior nodes 1..N-1, stored at x[1..N-1]
-        const int M = N - 1;
-        if (M > 0) {
-            block_scan_inclusive<FIELD_THREADS>(x + 1, M, warp_tot);  // S1
-            block_scan_inclusive<FIELD_THREADS>(x + 1, M, warp_tot);  // S2
-        }
-        if (tid == 0) s_D0 = M > 0 ? (-phi0 + x[M]) / (double)N : -phi0 / (double)N;
-        __syncthreads();
-        const double D0 = s_D0;
-        double *phi = W.phi + g;
-        for (int i = tid; i <= N; i += FIELD_THREADS) {
-            double p;
-            if (i == 0) p = phi0;
-            else if (i == N) p = 0.0;
-            else p = phi0 + (double)i * D0 - (i >= 2 ? x[i - 1] : 0.0);
-            phi[i] = p;
-        }
-        __syncthreads();
-        for (int i = tid; i <= N; i += FIELD_THREADS) {
-            double E;
-            if (i == 0) E = -(phi[1] - phi[0]) / dx - s_rho0 * dx / (2.0 * EPS0_);
-            else if (i == N) E = -(phi[N] - phi[N - 1]) / dx + s_rhoN * dx / (2.0 * EPS0_);
-            else E = -(phi[i + 1] - phi[i - 1]) / (2.0 * dx);
-            W.Efield[g + i] = E;
-            Er[i] = (Real)E;
-            if (diag) W.phi_sum[g + i] += phi[i];
+        } else {
+            const double E = (0.5 * K) * T - s_e0;
+            Er[i] = E;
+            if (full) W.Efield[g + i] = E;
         }
     }
-    if (diag && tid == 0) W.nsamp[d] += 1ull;
-    if (mode != 0 || blockIdx.x != 0) return;
-    // block 0: tile table of this step's push and the step counter
+    if (!full) return;
+    // potential: the prefix of S2 over threads, warps and blocks, and its sums
+    S2t pv = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const S2t x = F::up(pv, o);
+        if (lane >= o) pv += x;
+    }
+    if (lane == 31) w3[warp] = pv;
     __syncthreads();
-    tile_table(W, par, step, true);
+    S2t before = pv - sum;
+    for (int w = 0; w < warp; ++w) before += w3[w];
+    if (csize > 1) {
+        cg::cluster_group cl = cg::this_cluster();
+        if (tid < csize) {
+            S2t t = w3[0];
+            for (int w = 1; w < NW; ++w) t += w3[w];
+            *cl.map_shared_rank(&c3[rank], tid) = t;
+        }
+        cl.sync();
+        for (int c = 0; c < rank; ++c) before += c3[c];
+    }
+    const double phi0 = s_phi0;
+    s1 = excl;
+#pragma unroll
+    for (int k = 0; k < FIELD_PER; ++k) {
+        const int i = lo + k;
+        if (i >= hi) break;
+        double p;
+        if (i == 0) p = phi0;
+        else if (i == N) p = 0.0;
+        else {
+            // before = S2_{i-1}
+            p = phi0 + (double)i * D0 - K * dx * (double)before;
+            if constexpr (EXACT) {
+                if (diag) W.phi_s2_sum[g + i] += before;
+            }
+            s1 += q[k];
+            before += (S2t)s1;
+        }
+        W.phi[g + i] = p;
+        if constexpr (!EXACT) {
+            if (diag) W.phi_sum[g + i] += p;
+        }
+    }
 }
 
 // Tile table of the current counts: tiles of each discharge start at a
@@ -363,44 +379,68 @@ k_field(WsPtrs W, int par, int diag, int mode)
 // TILES_PER_TICKET, so that a push ticket never spans two; the birth counts
 // of the padding tiles after each species (never pushed) are cleared.  With
 // `advance` the next step's counter is set and the candidate list emptied.
+// One thread per discharge and a block scan over them (one thread walking the
+// list took 0.25 us per entry: 50 us of every step of 64 discharges).
 __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bool advance)
 {
+    __shared__ int s_warp[32];
     Ctl *ctl = W.ctl;
-    const int tid = threadIdx.x;
-    if (tid == 0) {
-        // tiles of each discharge start at a multiple of TILE_ALIGN, so that the
-        // birth-append blocks (BIRTHS_THREADS sub-tiles) never span two, and
-        // those of each species at a multiple of TILES_PER_TICKET, so that a
-        // push ticket never spans two
-        int chunk = 0;
-        for (int ds = 0; ds < W.D * NSP; ++ds) {
-            Counts &C = W.cnt[ds];
-            if (ds % NSP == 0) chunk = (chunk + TILE_ALIGN - 1) / TILE_ALIGN * TILE_ALIGN;
-            else chunk = (chunk + TILES_PER_TICKET - 1) / TILES_PER_TICKET * TILES_PER_TICKET;
-            C.n_snap = C.n;
-            C.chunk0 = chunk;
-            C.nchunk = (C.n + CHUNK - 1) / CHUNK;
-            chunk += C.nchunk;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NT = blockDim.x;
+    constexpr int A = TILE_ALIGN, B = TILES_PER_TICKET;
+    int first = 0;  // tiles of the discharges before this pass
+    for (int d0 = 0; d0 < W.D; d0 += NT) {
+        const int d = d0 + tid;
+        int n[NSP] = {0, 0, 0}, at[NSP], end = 0;
+        if (d < W.D) {
+#pragma unroll
+            for (int s = 0; s < NSP; ++s) n[s] = W.cnt[d * NSP + s].n;
         }
-        if (chunk > W.max_chunks) {
-            set_status(ctl, ST_CAPACITY);
-            chunk = 0;
+#pragma unroll
+        for (int s = 0; s < NSP; ++s) {
+            at[s] = (end + B - 1) / B * B;
+            end = at[s] + (n[s] + CHUNK - 1) / CHUNK;
         }
-        ctl->total_chunks = chunk;
-        ctl->ticket = 0u;
-        ctl->births_ticket = 0u;
-        if (advance) {
-            ctl->cand_n = 0u;
-            ctl->step[par ^ 1] = step + 1ull;
+        const int size = d < W.D ? (end + A - 1) / A * A : 0;
+        int v = size;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += x;
+        }
+        __syncthreads();  // s_warp of the pass before has been read
+        if (lane == 31) s_warp[warp] = v;
+        __syncthreads();
+        int start = first + v - size;
+        for (int w = 0; w < warp; ++w) start += s_warp[w];
+        for (int w = 0; w < NT / 32; ++w) first += s_warp[w];
+        if (d < W.D) {
+#pragma unroll
+            for (int s = 0; s < NSP; ++s) {
+                const Counts c{n[s], n[s], start + at[s], (n[s] + CHUNK - 1) / CHUNK};
+                W.cnt[d * NSP + s] = c;
+            }
+            if (d == W.D - 1) {
+                int chunk = start + end;
+                if (chunk > W.max_chunks) {
+                    set_status(ctl, ST_CAPACITY);
+                    chunk = 0;
+                }
+                ctl->total_chunks = chunk;
+                ctl->ticket = 0u;
+                ctl->births_ticket = 0u;
+                if (advance) {
+                    ctl->cand_n = 0u;
+                    ctl->step[par ^ 1] = step + 1ull;
+                }
+            }
         }
     }
     __syncthreads();
-    for (int ds = 0; ds < W.D * NSP; ++ds) {
-        const Counts &C = W.cnt[ds];
-        const int t0 = C.chunk0 + C.nchunk;
-        const int t1 = (t0 + TILES_PER_TICKET - 1) / TILES_PER_TICKET * TILES_PER_TICKET;
-        const int n = (t1 - t0) * SUBTILES * NSP;
-        for (int k = tid; k < n; k += blockDim.x) W.tile_cnt[(size_t)t0 * SUBTILES * NSP + k] = 0;
+    constexpr int PAD = B * SUBTILES;  // sub-tiles of a ticket: more than any padding
+    for (int k = tid; k < W.D * NSP * PAD; k += NT) {
+        const Counts &C = W.cnt[k / PAD];
+        const int t0 = C.chunk0 + C.nchunk, t1 = (t0 + B - 1) / B * B;
+        if (k % PAD < (t1 - t0) * SUBTILES) W.tile_cnt[((size_t)t0 * SUBTILES + k % PAD) * NSP] = 0;
     }
 }
 
@@ -1612,12 +1652,9 @@ __global__ void k_deposit_all(WsPtrs W, Pools<Real> P, int only_disc)
 cudaError_t configure_kernels(bool fp64, LaunchCfg &L)
 {
     cudaError_t e;
-    L.field_smem = sizeof(double) * (L.maxN + 2) + 16 * (L.maxN + 2) + 16;
     L.sort_smem = sizeof(unsigned short) * SORT_WARPS * ((L.maxN + 2) & ~1);
     L.scatter_smem = sizeof(unsigned short) * SORT_WARPS * ((L.maxN + 2) & ~1);
     if (fp64) {
-        e = cudaFuncSetAttribute(k_field<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.field_smem);
-        if (e) return e;
         e = cudaFuncSetAttribute(k_sort_count<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.sort_smem);
         if (e) return e;
         e = cudaFuncSetAttribute(k_sort_scatter<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.scatter_smem);
@@ -1629,8 +1666,6 @@ cudaError_t configure_kernels(bool fp64, LaunchCfg &L)
                                  (int)coulomb_smem_bytes(true));
         if (e) return e;
     } else {
-        e = cudaFuncSetAttribute(k_field<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.field_smem);
-        if (e) return e;
         e = cudaFuncSetAttribute(k_sort_count<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.sort_smem);
         if (e) return e;
         e = cudaFuncSetAttribute(k_sort_scatter<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.scatter_smem);
@@ -1649,10 +1684,12 @@ cudaError_t configure_kernels(bool fp64, LaunchCfg &L)
 cudaError_t launch_field(bool fp64, bool diag, int mode, const WsPtrs &W, int par, const LaunchCfg &L,
                          cudaStream_t st)
 {
+    const int csize = L.maxN + 1 > FIELD_ONE + 1 ? FIELD_CLUSTER : 1;
+    const int grid = (W.D + (mode == 0 ? 1 : 0)) * csize;
     if (fp64)
-        launch_k(k_field<double>, W.D, FIELD_THREADS, L.field_smem, st, W, par, diag ? 1 : 0, mode);
+        launch_cluster(k_field<double>, grid, FIELD_THREADS, csize, st, W, par, diag ? 1 : 0, mode, csize);
     else
-        launch_k(k_field<float>, W.D, FIELD_THREADS, L.field_smem, st, W, par, diag ? 1 : 0, mode);
+        launch_cluster(k_field<float>, grid, FIELD_THREADS, csize, st, W, par, diag ? 1 : 0, mode, csize);
     return cudaGetLastError();
 }
 

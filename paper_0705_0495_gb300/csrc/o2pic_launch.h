@@ -28,6 +28,27 @@ inline cudaError_t launch_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
+// The same as a grid of clusters of `csize` blocks (1: no clusters).
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, int csize, cudaStream_t st,
+                                  Args &&...args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = O2_PDL;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)csize;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = csize > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+
 constexpr int MAX_PUSH_SHAPES = 8;
 
 struct LaunchCfg {
@@ -49,7 +70,6 @@ struct LaunchCfg {
     const int *sort_warp_base;  // device [D*3+1]: first column-scan warp per (d, s)
     int pair_blocks_sp[NSP];          // evaluation blocks per projectile species
     const int *pair_tab_sp[NSP];      // device [(d, tile)] tables per species
-    size_t field_smem;
     int maxN;             // largest cell count over discharges
     int eedf_max, fm_max; // largest histogram sizes (shared-memory copies in the push)
 };
