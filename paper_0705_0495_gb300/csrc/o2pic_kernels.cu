@@ -1687,9 +1687,9 @@ cudaError_t launch_field(bool fp64, bool diag, int mode, const WsPtrs &W, int pa
     const int csize = L.maxN + 1 > FIELD_ONE + 1 ? FIELD_CLUSTER : 1;
     const int grid = (W.D + (mode == 0 ? 1 : 0)) * csize;
     if (fp64)
-        launch_cluster(k_field<double>, grid, FIELD_THREADS, csize, st, W, par, diag ? 1 : 0, mode, csize);
+        launch_cluster(k_field<double>, grid, FIELD_THREADS, csize, st, 0, W, par, diag ? 1 : 0, mode, csize);
     else
-        launch_cluster(k_field<float>, grid, FIELD_THREADS, csize, st, W, par, diag ? 1 : 0, mode, csize);
+        launch_cluster(k_field<float>, grid, FIELD_THREADS, csize, st, 0, W, par, diag ? 1 : 0, mode, csize);
     return cudaGetLastError();
 }
 

@@ -31,11 +31,12 @@ inline cudaError_t launch_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_
 // The same as a grid of clusters of `csize` blocks (1: no clusters).
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, int csize, cudaStream_t st,
-                                  Args &&...args)
+                                  size_t smem, Args &&...args)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -10,6 +10,9 @@
 // library reserves until the process exits.  The caller passes the particle
 // arrays and the output arrays; this file never calls cudaMalloc, cudaFree
 // or an allocating library routine.
+#include <cooperative_groups.h>
+
+#include <algorithm>
 #include <mutex>
 #include <string>
 
@@ -19,9 +22,11 @@
 
 namespace {
 
+namespace cg = cooperative_groups;
+using i128 = __int128;
+
 constexpr int STATIC_MAX_CELLS = 4096;
 constexpr int STATIC_NODES = STATIC_MAX_CELLS + 1;
-constexpr int STATIC_FIELD_THREADS = 1024;
 constexpr double QE_S = 1.602176634e-19;
 constexpr double EPS0_S = 8.8541878128e-12;
 constexpr int MAX_DEVICES = 64;
@@ -34,85 +39,529 @@ static __device__ __align__(256) unsigned long long g_static_acc[3 * STATIC_NODE
 std::mutex g_mu;
 void *g_acc_ptr[MAX_DEVICES] = {};
 
-__global__ void k_static_deposit_f32(unsigned long long *acc, const int *cell, const float *off, long long n,
-                                     int N)
-{
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int c = cell[i];
-        if (c < 0 || c >= N) continue;
+// The three particle arrays of a call.
+template <typename Real>
+struct Particles {
+    const int *cell[3];
+    const Real *off[3];
+    long long n[3];
+    bool vec[3];  // both arrays start on a 16-byte (offsets: 4 elements) boundary
+};
+
+// Sums of a block, per CELL and in 32-bit words of shared memory: the number
+// of particles in the cell and the sum of their upper weights w1 = offset in
+// fixed point, cut into words small enough that every sum is exact.  Node i is
+// then count_i - W_i + W_(i-1): the integer that adding both weights of every
+// particle gives.  (64-bit shared atomics are several times slower than
+// 32-bit ones on this part, and double ones slower still.)
+//   FP32: w1 = rn(offset 2^24), words of 12 and 13 bits, 2^19 particles.
+//   FP64: w1 = rn(offset 2^52), words of 18, 17 and 18 bits, 2^14 particles;
+//         the weights are rounded at 2^-53 of a particle, finer than the
+//         rounding of one addition to a double sum above 1.
+template <typename Real> struct Sums;
+template <> struct Sums<float> {
+    static constexpr int WORDS = 2, BITS = o2::FIX_BITS, SPLIT = 12;
+    static constexpr long long MOST = 1ll << 19;  // slots between two flushes
+    static __device__ constexpr int width(int) { return SPLIT; }  // bits of a word
+    using Acc = unsigned long long;
+    static __device__ __forceinline__ void weigh(float off, unsigned w[WORDS])
+    {
         // an offset outside [0, 1] (or NaN) is clamped into it, so that the
         // two weights stay within [0, 2^FIX_BITS] and add up to one particle
-        const float o = fminf(fmaxf(off[i], 0.0f), 1.0f);
-        const unsigned w1 = __float2uint_rn(o * (float)(1 << o2::FIX_BITS));
-        const unsigned w0 = (1u << o2::FIX_BITS) - w1;
-        atomicAdd(&acc[c], (unsigned long long)w0);
-        atomicAdd(&acc[c + 1], (unsigned long long)w1);
+        const unsigned v = __float2uint_rn(fminf(fmaxf(off, 0.0f), 1.0f) * (float)(1 << BITS));
+        w[0] = v & ((1u << SPLIT) - 1u);
+        w[1] = v >> SPLIT;
     }
-}
-
-__global__ void k_static_deposit_f64(double *acc, const int *cell, const double *off, long long n, int N)
-{
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int c = cell[i];
-        if (c < 0 || c >= N) continue;
-        const double o = fmin(fmax(off[i], 0.0), 1.0);  // clamped as in the FP32 path
-        atomicAdd(&acc[c], 1.0 - o);
-        atomicAdd(&acc[c + 1], o);
+    static __device__ __forceinline__ long long value(const unsigned w[WORDS])
+    {
+        return ((long long)w[1] << SPLIT) + w[0];
     }
-}
+    // a node's sum, from the words of its cell and of the cell before it
+    static __device__ __forceinline__ i128 node(unsigned cnt, const unsigned w[WORDS], const unsigned p[WORDS])
+    {
+        return ((i128)cnt << BITS) - value(w) + value(p);
+    }
+    static __device__ __forceinline__ void flush(Acc *a, i128 v) { atomicAdd(a, (Acc)(long long)v); }
+    static __device__ __forceinline__ i128 read(Acc v) { return (i128)(long long)v; }
+};
+template <> struct Sums<double> {
+    static constexpr int WORDS = 3, BITS = 52;
+    static constexpr long long MOST = 1ll << 14;
+    static __device__ constexpr int width(int j) { return j == 0 ? 18 : 17; }
+    using Acc = double;
+    static __device__ __forceinline__ void weigh(double off, unsigned w[WORDS])
+    {
+        // outside [0, 1): clamped as in the FP32 path (on the integer units:
+        // FP64 has two units per SM here)
+        if ((unsigned)__double2hiint(off) >= 0x3FF00000u) off = fmin(fmax(off, 0.0), 1.0);
+        // offset + 1 has its last bit at 2^-52
+        const unsigned long long v =
+            (unsigned long long)(__double_as_longlong(off + 1.0) - __double_as_longlong(1.0));
+        w[0] = (unsigned)(v & 0x3FFFFull);
+        w[1] = (unsigned)((v >> 18) & 0x1FFFFull);
+        w[2] = (unsigned)(v >> 35);
+    }
+    static __device__ __forceinline__ i128 value(const unsigned w[WORDS])
+    {
+        return ((i128)w[2] << 35) + ((i128)w[1] << 18) + (i128)w[0];
+    }
+    static __device__ __forceinline__ i128 node(unsigned cnt, const unsigned w[WORDS], const unsigned p[WORDS])
+    {
+        return ((i128)cnt << BITS) - value(w) + value(p);
+    }
+    static __device__ __forceinline__ void flush(Acc *a, i128 v)
+    {
+        atomicAdd(a, (double)v * (1.0 / 4503599627370496.0));
+    }
+    // a sum of multiples of 2^-52 (any rounding of the atomics is coarser)
+    static __device__ __forceinline__ i128 read(Acc v)
+    {
+        const double hi = floor(v);
+        return ((i128)(long long)hi << BITS) + (i128)(long long)((v - hi) * 4503599627370496.0);
+    }
+};
 
-// One block: rho from the accumulators, then the Dirichlet problem
-// (phi_{i-1} - 2 phi_i + phi_{i+1}) = -rho_i dx^2 / eps0, phi_0 = U(t),
-// phi_N = 0, solved exactly by two prefix sums (phi_i = phi_0 + i D0 -
-// S2_{i-1}), and E from centred differences with Gauss's law on the half
-// cells at the walls.  Sums run sequentially in one thread: N <= 4096.
-__global__ void __launch_bounds__(STATIC_FIELD_THREADS)
-k_static_field(const unsigned long long *acc, int fp64, int N, double dx, double weight, double phi0,
-               double *rho, double *phi, double *E)
+constexpr int UNIT_THREADS = 512;         // threads of a deposit block
+constexpr int UNIT = 4 * UNIT_THREADS;    // slots a block takes at a time, four consecutive ones per thread
+constexpr int STATIC_CLUSTER = 8;
+
+// Four consecutive slots of one species into the block's sums (cnt and the
+// words, each an array of `stride` cells).  As in the push: lanes whose four
+// slots sit in the first lane's cell (ordered particles) sum over the warp and
+// one lane adds for all; a lane whose four share a cell adds them once.
+// Every lane of the warp calls it; cells are -1 for nothing.
+template <typename Real>
+__device__ __forceinline__ void add4(unsigned *cnt, int stride, const int c[4], const Real off[4])
 {
-    extern __shared__ __align__(16) double sx[];  // rho, then S2
-    const int tid = threadIdx.x;
-    for (int i = tid; i <= N; i += blockDim.x) {
-        const double vol = (i == 0 || i == N) ? 0.5 * dx : dx;
-        double a[3];
-        for (int s = 0; s < 3; ++s) {
-            const unsigned long long v = acc[s * STATIC_NODES + i];
-            a[s] = fp64 ? __longlong_as_double((long long)v)
-                        : (double)(long long)v / (double)(1 << o2::FIX_BITS);
+    using S = Sums<Real>;
+    unsigned w[4][S::WORDS], sum[S::WORDS];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) S::weigh(off[k], w[k]);
+    const bool same = c[0] >= 0 && c[1] == c[0] && c[2] == c[0] && c[3] == c[0];
+    const int c0 = __shfl_sync(0xffffffffu, c[0], 0);
+    const bool in = same && c[0] == c0;
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+#pragma unroll
+    for (int j = 0; j < S::WORDS; ++j) sum[j] = w[0][j] + w[1][j] + w[2][j] + w[3][j];
+    if (__popc(m) >= 4) {
+        unsigned all[S::WORDS];
+#pragma unroll
+        for (int j = 0; j < S::WORDS; ++j) all[j] = __reduce_add_sync(0xffffffffu, in ? sum[j] : 0u);
+        if ((threadIdx.x & 31) == 0) {
+            atomicAdd(&cnt[c0], 4u * (unsigned)__popc(m));
+#pragma unroll
+            for (int j = 0; j < S::WORDS; ++j) atomicAdd(&cnt[(j + 1) * stride + c0], all[j]);
         }
-        const double r = QE_S * weight * (a[2] - a[0] - a[1]) / vol;
-        rho[i] = r;
-        sx[i] = r * dx * dx / EPS0_S;
+        if (in) return;
     }
-    __syncthreads();
+    if (same) {
+        atomicAdd(&cnt[c[0]], 4u);
+#pragma unroll
+        for (int j = 0; j < S::WORDS; ++j) atomicAdd(&cnt[(j + 1) * stride + c[0]], sum[j]);
+        return;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (c[k] < 0) continue;
+        atomicAdd(&cnt[c[k]], 1u);
+#pragma unroll
+        for (int j = 0; j < S::WORDS; ++j) atomicAdd(&cnt[(j + 1) * stride + c[k]], w[k][j]);
+    }
+}
+
+__device__ __forceinline__ void load4(const int *p, int v[4])
+{
+    const int4 t = __ldcs(reinterpret_cast<const int4 *>(p));
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+__device__ __forceinline__ void load4(const float *p, float v[4])
+{
+    const float4 t = __ldcs(reinterpret_cast<const float4 *>(p));
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+__device__ __forceinline__ void load4(const double *p, double v[4])
+{
+    const double2 a = __ldcs(reinterpret_cast<const double2 *>(p));
+    const double2 b = __ldcs(reinterpret_cast<const double2 *>(p) + 1);
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+}
+
+// slots i .. i+3 of species s; a cell outside the grid counts as empty
+template <typename Real>
+__device__ __forceinline__ void fetch4(const Particles<Real> &P, int s, long long i, int N, int c[4], Real off[4])
+{
+    if (P.vec[s] && i + 4 <= P.n[s]) {
+        load4(P.cell[s] + i, c);
+        load4(P.off[s] + i, off);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const bool in = i + k < P.n[s];
+            c[k] = in ? P.cell[s][i + k] : -1;
+            off[k] = in ? P.off[s][i + k] : Real(0);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) c[k] = (unsigned)c[k] < (unsigned)N ? c[k] : -1;
+}
+
+template <typename Real>
+__device__ __forceinline__ i128 node_of(const unsigned *cnt, int stride, int i)
+{
+    using S = Sums<Real>;
+    unsigned w[S::WORDS], p[S::WORDS];
+#pragma unroll
+    for (int j = 0; j < S::WORDS; ++j) {
+        w[j] = cnt[(j + 1) * stride + i];
+        p[j] = i > 0 ? cnt[(j + 1) * stride + i - 1] : 0u;
+    }
+    return S::node(cnt[i], w, p);
+}
+
+// Charge deposit of many particles.  What bounds it: the particles' bytes
+// (5e7 FP32 particles: 400 MB, 59 us at the copy rate) and the shared
+// atomics.  Each block takes one contiguous share of the three species'
+// units, sums it per cell in shared memory (one species at a time) and adds
+// the cells it touched to the global accumulators.
+template <typename Real>
+__global__ void __launch_bounds__(UNIT_THREADS, 3)
+k_static_deposit(typename Sums<Real>::Acc *acc, Particles<Real> P, int N)
+{
+    using S = Sums<Real>;
+    extern __shared__ __align__(16) unsigned ssum[];
+    __shared__ int s_lo, s_hi;
+    o2::pdl_wait();
+    const int tid = threadIdx.x, stride = N + 1;
+    long long units = 0;
+#pragma unroll
+    for (int s = 0; s < 3; ++s) units += (P.n[s] + UNIT - 1) / UNIT;
+    // the block's share of the units, numbered through the three species
+    const long long ub = units / gridDim.x * blockIdx.x + units % gridDim.x * blockIdx.x / gridDim.x;
+    const long long ue = units / gridDim.x * (blockIdx.x + 1) + units % gridDim.x * (blockIdx.x + 1) / gridDim.x;
+    for (int k = tid; k < (S::WORDS + 1) * stride; k += UNIT_THREADS) ssum[k] = 0u;
     if (tid == 0) {
-        double s1 = 0.0, s2 = 0.0;
-        for (int i = 1; i < N; ++i) {
-            s1 += sx[i];
-            s2 += s1;
-            sx[i] = s2;  // S2_i
-        }
-        const double D0 = (s2 - phi0) / (double)N;
-        phi[0] = phi0;
-        for (int i = 1; i < N; ++i) phi[i] = phi0 + (double)i * D0 - (i >= 2 ? sx[i - 1] : 0.0);
-        phi[N] = 0.0;
+        s_lo = N;
+        s_hi = -1;
     }
     __syncthreads();
-    for (int i = tid; i <= N; i += blockDim.x) {
-        double e;
-        if (i == 0) e = -(phi[1] - phi[0]) / dx - rho[0] * dx / (2.0 * EPS0_S);
-        else if (i == N) e = -(phi[N] - phi[N - 1]) / dx + rho[N] * dx / (2.0 * EPS0_S);
-        else e = -(phi[i + 1] - phi[i - 1]) / (2.0 * dx);
-        E[i] = e;
+    long long u0 = 0;  // first unit of species s
+#pragma unroll 1
+    for (int s = 0; s < 3; ++s) {
+        const long long u1 = u0 + (P.n[s] + UNIT - 1) / UNIT;
+        long long a = max(ub, u0);
+        const long long e = min(ue, u1);
+        while (a < e) {
+            const long long b = min(e, a + S::MOST / UNIT);
+            int lo = N, hi = -1;
+            for (long long q = a; q < b; ++q) {
+                int c[4];
+                Real off[4];
+                fetch4<Real>(P, s, (q - u0) * UNIT + 4 * tid, N, c, off);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    hi = max(hi, c[k]);
+                    lo = min(lo, c[k] >= 0 ? c[k] : N);
+                }
+                add4<Real>(ssum, stride, c, off);
+            }
+            lo = __reduce_min_sync(0xffffffffu, lo);
+            hi = __reduce_max_sync(0xffffffffu, hi);
+            if ((tid & 31) == 0 && hi >= 0) {
+                atomicMin(&s_lo, lo);
+                atomicMax(&s_hi, hi);
+            }
+            __syncthreads();
+            lo = s_lo;
+            hi = s_hi;
+            for (int i = lo + tid; i <= hi + 1; i += UNIT_THREADS) {
+                const i128 v = node_of<Real>(ssum, stride, i);
+                if (v != 0) S::flush(&acc[(size_t)s * STATIC_NODES + i], v);
+            }
+            __syncthreads();
+            for (int i = lo + tid; i <= hi; i += UNIT_THREADS)
+#pragma unroll
+                for (int j = 0; j <= S::WORDS; ++j) ssum[j * stride + i] = 0u;
+            if (tid == 0) {
+                s_lo = N;
+                s_hi = -1;
+            }
+            __syncthreads();
+            a = b;
+        }
+        u0 = u1;
     }
+}
+
+// What the solve needs of the discharge: K dx per unit of charge, and so on.
+struct SolveC {
+    int N;
+    double dx, phi0, unit, qw;  // qw: elementary charge x weight
+    double *rho, *phi, *E;
+};
+
+__device__ __forceinline__ i128 shfl_up128(i128 v, int o)
+{
+    const unsigned long long lo = __shfl_up_sync(0xffffffffu, (unsigned long long)v, o);
+    const long long hi = __shfl_up_sync(0xffffffffu, (long long)(v >> 64), o);
+    return ((i128)hi << 64) | (i128)lo;
+}
+
+// The Dirichlet problem (phi_{i-1} - 2 phi_i + phi_{i+1}) = -rho_i dx^2 / eps0,
+// phi_0 = U(t), phi_N = 0, by two prefix sums over the nodes' net charge q_i,
+// both exact (integers): S1_i = sum q, S2_i = sum S1 over the interior,
+// phi_i = phi_0 + i D0 - c S2_{i-1}, E_i = (c / 2dx) (S1_i + S1_{i-1}) - D0/dx,
+// with Gauss's law on the half cells at the walls.  Thread t of block `rank`
+// of a cluster of `csize` holds nodes lo .. hi-1.
+template <int NT, int PER>
+__device__ void static_solve(const SolveC &C, int csize, int rank, int lo, int hi, const i128 q[PER])
+{
+    constexpr int NW = NT / 32;
+    __shared__ i128 w1[NW], w2[NW], c1[STATIC_CLUSTER], c2[STATIC_CLUSTER];
+    const int N = C.N, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const double c = C.qw * C.unit * C.dx / EPS0_S;  // K dx
+    // S2_i = (S1 of the threads before) x (nodes so far) + the thread's own,
+    // so both prefixes come from one exchange of (charge, own S2, nodes)
+    i128 run = 0, own = 0;
+    int m = 0;  // the thread's interior nodes
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int i = lo + k;
+        if (i < hi && i > 0 && i < N) {
+            run += q[k];
+            own += run;
+            ++m;
+        }
+    }
+    // fold a later stretch (r, o, m') into an earlier one (R, O): charge R + r,
+    // S2 of both O + o + m' R
+    i128 R = run, O = own;
+    int M = m;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const i128 r = shfl_up128(R, o), p = shfl_up128(O, o);
+        const int mm = __shfl_up_sync(0xffffffffu, M, o);
+        if (lane >= o) {
+            O += p + (i128)M * r;
+            R += r;
+            M += mm;
+        }
+    }
+    __shared__ int wm[NW], cm[STATIC_CLUSTER];
+    if (lane == 31) {
+        w1[warp] = R;
+        w2[warp] = O;
+        wm[warp] = M;
+    }
+    // the prefix before this thread within its warp
+    i128 pr = shfl_up128(R, 1), po = shfl_up128(O, 1);
+    int pm = __shfl_up_sync(0xffffffffu, M, 1);
+    if (lane == 0) {
+        pr = 0;
+        po = 0;
+        pm = 0;
+    }
+    __syncthreads();
+    auto fold = [](i128 &r, i128 &o, i128 r2, i128 o2, int m2) {  // (r, o) then (r2, o2, m2)
+        o += o2 + (i128)m2 * r;
+        r += r2;
+    };
+    i128 br = 0, bo = 0;  // everything before this thread
+    i128 tr, to;          // everything
+    if (csize > 1) {
+        cg::cluster_group cl = cg::this_cluster();
+        if (tid < csize) {
+            i128 r = 0, o = 0;
+            int mm = 0;
+            for (int w = 0; w < NW; ++w) {
+                fold(r, o, w1[w], w2[w], wm[w]);
+                mm += wm[w];
+            }
+            *cl.map_shared_rank(&c1[rank], tid) = r;
+            *cl.map_shared_rank(&c2[rank], tid) = o;
+            *cl.map_shared_rank(&cm[rank], tid) = mm;
+        }
+        cl.sync();
+        for (int b = 0; b < rank; ++b) fold(br, bo, c1[b], c2[b], cm[b]);
+        tr = br;
+        to = bo;
+        for (int b = rank; b < csize; ++b) fold(tr, to, c1[b], c2[b], cm[b]);
+    } else {
+        tr = 0;
+        to = 0;
+        for (int w = 0; w < NW; ++w) fold(tr, to, w1[w], w2[w], wm[w]);
+    }
+    for (int w = 0; w < warp; ++w) fold(br, bo, w1[w], w2[w], wm[w]);
+    fold(br, bo, pr, po, pm);
+    __shared__ double s_D0, s_e0, s_h;
+    if (tid == 0) {
+        s_D0 = (c * (double)to - C.phi0) / (double)N;
+        s_e0 = s_D0 / C.dx;
+        s_h = c / (2.0 * C.dx);
+    }
+    __syncthreads();
+    const double D0 = s_D0, e0 = s_e0, h = s_h, rs = C.qw * C.unit / C.dx;
+    i128 s1 = br, s2 = bo;  // S1_{i-1}, S2_{i-1}
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int i = lo + k;
+        if (i >= hi) break;
+        i128 T;
+        double p;
+        if (i == 0) {
+            T = -2 * q[k];
+            p = C.phi0;
+        } else if (i == N) {
+            T = 2 * (s1 + q[k]);
+            p = 0.0;
+        } else {
+            T = 2 * s1 + q[k];
+            p = C.phi0 + (double)i * D0 - c * (double)s2;
+            s1 += q[k];
+            s2 += s1;
+        }
+        C.rho[i] = (double)q[k] * ((i == 0 || i == N) ? 2.0 * rs : rs);
+        C.phi[i] = p;
+        C.E[i] = h * (double)T - e0;
+    }
+}
+
+// The solve from the global accumulators: one block up to 1024 cells, a
+// cluster of 8 beyond.
+constexpr int SOLVE_THREADS = 256, SOLVE_PER = 5, SOLVE_ONE = 1024;
+template <typename Real>
+__global__ void __launch_bounds__(SOLVE_THREADS)
+k_static_solve(const typename Sums<Real>::Acc *acc, SolveC C, int csize)
+{
+    using S = Sums<Real>;
+    o2::pdl_wait();
+    if (csize > 1) cg::this_cluster().sync();  // every block has started
+    const int rank = blockIdx.x, tid = threadIdx.x, NC = (C.N + csize) / csize;
+    const int per = (NC + SOLVE_THREADS - 1) / SOLVE_THREADS;
+    const int lo = min(rank * NC + tid * per, C.N + 1);
+    const int hi = min(min(lo + per, (rank + 1) * NC), C.N + 1);
+    i128 q[SOLVE_PER];
+#pragma unroll
+    for (int k = 0; k < SOLVE_PER; ++k) {
+        q[k] = 0;
+        if (lo + k < hi)
+            q[k] = S::read(acc[2 * STATIC_NODES + lo + k]) - S::read(acc[lo + k]) - S::read(acc[STATIC_NODES + lo + k]);
+    }
+    static_solve<SOLVE_THREADS, SOLVE_PER>(C, csize, rank, lo, hi, q);
+}
+
+// Deposit and solve of few particles in one launch: a cluster of 8 blocks,
+// each with the sums of all three species of its share of the particles in
+// its own shared memory; block r then collects its nodes from all eight and
+// solves them.  The separate kernels need the accumulators cleared, and three
+// launches took 53 us for 4e4 particles, most of it in one thread's sums.
+constexpr int SMALL_PER = 2;  // nodes per thread: (4097 / 8) / 512
+constexpr long long SMALL_MOST = 1ll << 17;  // slots: 2^14 per block (the FP64 sums' limit) and species units
+static_assert(SMALL_MOST / STATIC_CLUSTER <= Sums<double>::MOST && SMALL_MOST / STATIC_CLUSTER <= Sums<float>::MOST, "");
+template <typename Real>
+__global__ void __launch_bounds__(UNIT_THREADS)
+k_static_small(Particles<Real> P, SolveC C)
+{
+    using S = Sums<Real>;
+    extern __shared__ __align__(16) unsigned ssum[];
+    o2::pdl_wait();
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = blockIdx.x, tid = threadIdx.x, N = C.N, stride = N + 1;
+    const int per_species = (S::WORDS + 1) * stride;
+    for (int k = tid; k < 3 * per_species; k += UNIT_THREADS) ssum[k] = 0u;
+    __syncthreads();
+    // warps of 128 slots, dealt out block by block, so that the blocks' shares differ by one at most
+    int u[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int s = 0; s < 3; ++s) u[s + 1] = u[s] + (int)((P.n[s] + 127) / 128);
+    for (int q = rank + STATIC_CLUSTER * (tid >> 5); q < u[3]; q += STATIC_CLUSTER * (UNIT_THREADS / 32)) {
+        const int s = q < u[1] ? 0 : (q < u[2] ? 1 : 2);
+        int c[4];
+        Real off[4];
+        fetch4<Real>(P, s, (long long)(q - (s == 0 ? 0 : (s == 1 ? u[1] : u[2]))) * 128 + 4 * (tid & 31), N, c, off);
+        add4<Real>(ssum + s * per_species, stride, c, off);
+    }
+    cl.sync();
+    const int NC = (N + STATIC_CLUSTER) / STATIC_CLUSTER;
+    const int per = (NC + UNIT_THREADS - 1) / UNIT_THREADS;
+    const int lo = min(rank * NC + tid * per, N + 1);
+    const int hi = min(min(lo + per, (rank + 1) * NC), N + 1);
+    i128 q[SMALL_PER];
+#pragma unroll
+    for (int k = 0; k < SMALL_PER; ++k) {
+        q[k] = 0;
+        if (lo + k >= hi) continue;
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+            // the species' words of the node's cell and of the one before, summed over the blocks
+            unsigned long long cnt = 0, w[S::WORDS] = {}, p[S::WORDS] = {};
+            for (int b = 0; b < STATIC_CLUSTER; ++b) {
+                const unsigned *o = cl.map_shared_rank(ssum, b) + s * per_species;
+                cnt += o[lo + k];
+#pragma unroll
+                for (int j = 0; j < S::WORDS; ++j) {
+                    w[j] += o[(j + 1) * stride + lo + k];
+                    if (lo + k > 0) p[j] += o[(j + 1) * stride + lo + k - 1];
+                }
+            }
+            i128 v = (i128)cnt << S::BITS;
+            int sh = 0;
+#pragma unroll
+            for (int j = 0; j < S::WORDS; ++j) {
+                v += ((i128)p[j] - (i128)w[j]) << sh;
+                sh += S::width(j);
+            }
+            q[k] += s == 2 ? v : -v;
+        }
+    }
+    // the solve's exchange synchronises the cluster after these reads, before any block can end
+    static_solve<UNIT_THREADS, SMALL_PER>(C, STATIC_CLUSTER, rank, lo, hi, q);
 }
 
 pic_status static_fail(pic_status s, const std::string &m)
 {
     o2::set_last_error(m.c_str());
     return s;
+}
+
+template <typename Real>
+cudaError_t static_setup()
+{
+    constexpr int most = (int)sizeof(unsigned) * (Sums<Real>::WORDS + 1) * STATIC_NODES;
+    cudaError_t e = cudaFuncSetAttribute(k_static_deposit<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_static_small<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * most);
+    return e;
+}
+
+template <typename Real>
+cudaError_t static_run(void *acc, const int *const *cell, const void *const *off, const long long *n, const SolveC &C,
+                       int num_sms, cudaStream_t st)
+{
+    using S = Sums<Real>;
+    Particles<Real> P{};
+    long long all = 0;
+    for (int s = 0; s < 3; ++s) {
+        P.cell[s] = cell[s];
+        P.off[s] = static_cast<const Real *>(off[s]);
+        P.n[s] = n[s];
+        P.vec[s] = (reinterpret_cast<size_t>(cell[s]) & 15) == 0 && (reinterpret_cast<size_t>(off[s]) & 15) == 0;
+        all += n[s];
+    }
+    const size_t sm = sizeof(unsigned) * (S::WORDS + 1) * (C.N + 1);
+    if (all <= SMALL_MOST - 3 * 128 * STATIC_CLUSTER)  // a block's 128-slot shares stay within SMALL_MOST / 8
+        return o2::launch_cluster(k_static_small<Real>, STATIC_CLUSTER, UNIT_THREADS, STATIC_CLUSTER, st, 3 * sm, P, C);
+    // the array keeps the previous call's sums: clear it first
+    cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * 3 * STATIC_NODES, st);
+    if (e != cudaSuccess) return e;
+    typename S::Acc *a = static_cast<typename S::Acc *>(acc);
+    // what fits on an SM by threads and shared memory; not more blocks than units
+    const long long units = all / UNIT + 3;
+    const int per_sm = (int)std::min<size_t>(3, (224u << 10) / (sm + 1024));
+    const int grid = (int)std::min<long long>(units, (long long)num_sms * per_sm);
+    e = o2::launch_k(k_static_deposit<Real>, grid, UNIT_THREADS, sm, st, a, P, C.N);
+    if (e != cudaSuccess) return e;
+    const int csize = C.N > SOLVE_ONE ? STATIC_CLUSTER : 1;
+    return o2::launch_cluster(k_static_solve<Real>, csize, SOLVE_THREADS, csize, st, 0, a, C, csize);
 }
 
 } // namespace
@@ -139,9 +588,12 @@ extern "C" pic_status pic_field_solve_static(const pic_config *cfg, long long st
     if (e != cudaSuccess || dev < 0 || dev >= MAX_DEVICES)
         return static_fail(PIC_ECUDA, std::string("pic_field_solve_static: cudaGetDevice: ") + cudaGetErrorString(e));
     void *acc = nullptr;
+    static int num_sms[MAX_DEVICES];  // guarded by g_mu
+    int sms = 0;
     {
         // set-up, once per device, with that device current: the device
         // address of the scratch array (its host-side name is only a handle)
+        // and the kernels' shared-memory limits
         std::lock_guard<std::mutex> lock(g_mu);
         if (!g_acc_ptr[dev]) {
             void *p = nullptr;
@@ -149,35 +601,31 @@ extern "C" pic_status pic_field_solve_static(const pic_config *cfg, long long st
             if (e != cudaSuccess || !p)
                 return static_fail(PIC_ECUDA, std::string("pic_field_solve_static: cudaGetSymbolAddress: ") +
                                                   cudaGetErrorString(e));
+            e = cudaDeviceGetAttribute(&num_sms[dev], cudaDevAttrMultiProcessorCount, dev);
+            if (e == cudaSuccess) e = static_setup<float>();
+            if (e == cudaSuccess) e = static_setup<double>();
+            if (e != cudaSuccess)
+                return static_fail(PIC_ECUDA, std::string("pic_field_solve_static: ") + cudaGetErrorString(e));
             g_acc_ptr[dev] = p;
         }
         acc = g_acc_ptr[dev];
+        sms = num_sms[dev];
     }
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    // the array keeps the previous call's sums: clear it first
-    e = cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * 3 * STATIC_NODES, st);
-    if (e != cudaSuccess)
-        return static_fail(PIC_ECUDA, std::string("pic_field_solve_static: ") + cudaGetErrorString(e));
     const bool fp64 = cfg->precision == PIC_FP64;
-    for (int s = 0; s < 3; ++s) {
-        if (n[s] == 0) continue;
-        const long long blocks = (n[s] + 255) / 256;
-        const int grid = (int)(blocks < 4096 ? blocks : 4096);
-        unsigned long long *a = static_cast<unsigned long long *>(acc) + (size_t)s * STATIC_NODES;
-        if (fp64)
-            k_static_deposit_f64<<<grid, 256, 0, st>>>(reinterpret_cast<double *>(a), d_cell[s],
-                                                       static_cast<const double *>(d_off[s]), n[s], N);
-        else
-            k_static_deposit_f32<<<grid, 256, 0, st>>>(a, d_cell[s], static_cast<const float *>(d_off[s]),
-                                                       n[s], N);
-    }
     const double PI_S = 3.14159265358979323846;
     const double t = (double)step * cfg->dt_s;
-    const double phi0 = cfg->U_rf_V * sin(2.0 * PI_S * cfg->f_rf_Hz * t + cfg->rf_phase);
-    k_static_field<<<1, STATIC_FIELD_THREADS, sizeof(double) * (N + 1), st>>>(
-        static_cast<const unsigned long long *>(acc), fp64 ? 1 : 0, N, cfg->L_m / N, cfg->weight_m2, phi0, d_rho,
-        d_phi, d_E);
-    e = cudaGetLastError();
+    SolveC C{};
+    C.N = N;
+    C.dx = cfg->L_m / N;
+    C.phi0 = cfg->U_rf_V * sin(2.0 * PI_S * cfg->f_rf_Hz * t + cfg->rf_phase);
+    C.unit = fp64 ? 1.0 / 4503599627370496.0 : 1.0 / (double)(1 << o2::FIX_BITS);
+    C.qw = QE_S * cfg->weight_m2;
+    C.rho = d_rho;
+    C.phi = d_phi;
+    C.E = d_E;
+    e = fp64 ? static_run<double>(acc, d_cell, d_off, n, C, sms, st) : static_run<float>(acc, d_cell, d_off, n, C, sms, st);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess)
         return static_fail(PIC_ECUDA, std::string("pic_field_solve_static: launch: ") + cudaGetErrorString(e));
     return PIC_OK;
