@@ -186,6 +186,7 @@ struct Disc {
     double vol_fix;          // density per accumulated unit (interior node)
     double dens_fix, dens_fix_wall;  // weight / (node volume * 2^FIX_BITS), inside / at walls
     double Kfix;             // e weight 2^-FIX_BITS / eps0
+    double Kone;             // e weight / eps0
     double kE;               // dt^2/dx
     double f15, mu2_15;      // reaction (15) product speed factor
     double f16;              // (16): v_e = |v_Om| * f16

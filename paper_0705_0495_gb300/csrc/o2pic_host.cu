@@ -500,6 +500,7 @@ static void build_disc(pic_handle *h, int d, const std::vector<int> &gas_tabs_by
     D.dens_fix = q.weight_m2 / (D.dx * (double)(1 << FIX_BITS));
     D.dens_fix_wall = q.weight_m2 / (0.5 * D.dx * (double)(1 << FIX_BITS));
     D.Kfix = QE * q.weight_m2 / (double)(1 << FIX_BITS) / 8.8541878128e-12;
+    D.Kone = QE * q.weight_m2 / EPS0;
     const double mu2 = M_O * MASS[1] / (M_O + MASS[1]);
     D.mu2_15 = mu2;
     D.f15 = 2.0 * QE * mu2 / (MASS[1] * MASS[1]) * tdx * tdx;

@@ -263,7 +263,7 @@ k_field(WsPtrs W, int par, int diag, int mode, int csize)
         for (int c = 0; c < rank; ++c) excl += c1[c];
     }
     // K dx and D0, in the order of the formulas above
-    const double K = EXACT ? Dd.Kfix : QE_ * Dd.weight / EPS0_;
+    const double K = EXACT ? Dd.Kfix : Dd.Kone;
     if (tid == 0) {
         S2t tot = S2t(0);
         if (csize > 1)

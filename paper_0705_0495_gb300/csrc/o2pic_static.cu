@@ -62,7 +62,7 @@ template <typename Real> struct Sums;
 template <> struct Sums<float> {
     static constexpr int WORDS = 2, BITS = o2::FIX_BITS, SPLIT = 12;
     static constexpr long long MOST = 1ll << 19;  // slots between two flushes
-    static __device__ constexpr int width(int) { return SPLIT; }  // bits of a word
+    static constexpr bool RANGE = false;          // a flush is rare: it looks at every cell
     using Acc = unsigned long long;
     static __device__ __forceinline__ void weigh(float off, unsigned w[WORDS])
     {
@@ -87,7 +87,7 @@ template <> struct Sums<float> {
 template <> struct Sums<double> {
     static constexpr int WORDS = 3, BITS = 52;
     static constexpr long long MOST = 1ll << 14;
-    static __device__ constexpr int width(int j) { return j == 0 ? 18 : 17; }
+    static constexpr bool RANGE = true;  // a flush is frequent: it looks at the cells between the lowest and highest
     using Acc = double;
     static __device__ __forceinline__ void weigh(double off, unsigned w[WORDS])
     {
@@ -219,12 +219,14 @@ __device__ __forceinline__ i128 node_of(const unsigned *cnt, int stride, int i)
 }
 
 // Charge deposit of many particles.  What bounds it: the particles' bytes
-// (5e7 FP32 particles: 400 MB, 59 us at the copy rate) and the shared
-// atomics.  Each block takes one contiguous share of the three species'
-// units, sums it per cell in shared memory (one species at a time) and adds
-// the cells it touched to the global accumulators.
+// (5e7 FP32 particles in 4096 cells: 400 MB, 59 us at the copy rate; 94 us
+// here, 65 us without the additions) and the shared atomics.  Each block takes
+// one contiguous share of the three species' units, sums it per cell in shared
+// memory (one species at a time) and adds the cells it touched to the global
+// accumulators.  Global atomics for every particle took 3900 us.
+// Two blocks per SM with the next slots in flight: 94 us; three without: 103.
 template <typename Real>
-__global__ void __launch_bounds__(UNIT_THREADS, 3)
+__global__ void __launch_bounds__(UNIT_THREADS, 2)
 k_static_deposit(typename Sums<Real>::Acc *acc, Particles<Real> P, int N)
 {
     using S = Sums<Real>;
@@ -253,26 +255,34 @@ k_static_deposit(typename Sums<Real>::Acc *acc, Particles<Real> P, int N)
         while (a < e) {
             const long long b = min(e, a + S::MOST / UNIT);
             int lo = N, hi = -1;
+            // the next four slots are loaded before these are added up
+            int c[4], cx[4];
+            Real off[4], ox[4];
+            fetch4<Real>(P, s, (a - u0) * UNIT + 4 * tid, N, c, off);
             for (long long q = a; q < b; ++q) {
-                int c[4];
-                Real off[4];
-                fetch4<Real>(P, s, (q - u0) * UNIT + 4 * tid, N, c, off);
+                if (q + 1 < b) fetch4<Real>(P, s, (q + 1 - u0) * UNIT + 4 * tid, N, cx, ox);
+                add4<Real>(ssum, stride, c, off);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    hi = max(hi, c[k]);
-                    lo = min(lo, c[k] >= 0 ? c[k] : N);
+                    if (S::RANGE) {
+                        hi = max(hi, c[k]);
+                        lo = min(lo, c[k] >= 0 ? c[k] : N);
+                    }
+                    c[k] = cx[k];
+                    off[k] = ox[k];
                 }
-                add4<Real>(ssum, stride, c, off);
             }
-            lo = __reduce_min_sync(0xffffffffu, lo);
-            hi = __reduce_max_sync(0xffffffffu, hi);
-            if ((tid & 31) == 0 && hi >= 0) {
-                atomicMin(&s_lo, lo);
-                atomicMax(&s_hi, hi);
+            if (S::RANGE) {
+                lo = __reduce_min_sync(0xffffffffu, lo);
+                hi = __reduce_max_sync(0xffffffffu, hi);
+                if ((tid & 31) == 0 && hi >= 0) {
+                    atomicMin(&s_lo, lo);
+                    atomicMax(&s_hi, hi);
+                }
             }
             __syncthreads();
-            lo = s_lo;
-            hi = s_hi;
+            lo = S::RANGE ? s_lo : 0;
+            hi = S::RANGE ? s_hi : N - 1;
             for (int i = lo + tid; i <= hi + 1; i += UNIT_THREADS) {
                 const i128 v = node_of<Real>(ssum, stride, i);
                 if (v != 0) S::flush(&acc[(size_t)s * STATIC_NODES + i], v);
@@ -292,10 +302,14 @@ k_static_deposit(typename Sums<Real>::Acc *acc, Particles<Real> P, int N)
     }
 }
 
-// What the solve needs of the discharge: K dx per unit of charge, and so on.
+// What the solve needs of the discharge.  The constants are formed on the
+// host: an FP64 division by every thread costs more here than the whole solve.
 struct SolveC {
     int N;
-    double dx, phi0, unit, qw;  // qw: elementary charge x weight
+    double dx, phi0;
+    double c;   // e weight dx / eps0 per unit of charge (K dx)
+    double h;   // c / (2 dx)
+    double rs;  // e weight / dx per unit of charge
     double *rho, *phi, *E;
 };
 
@@ -317,8 +331,9 @@ __device__ void static_solve(const SolveC &C, int csize, int rank, int lo, int h
 {
     constexpr int NW = NT / 32;
     __shared__ i128 w1[NW], w2[NW], c1[STATIC_CLUSTER], c2[STATIC_CLUSTER];
+    // warps that can hold nodes
+    const int NC = (C.N + csize) / csize, per = (NC + NT - 1) / NT, nw = ((NC + per - 1) / per + 31) / 32;
     const int N = C.N, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const double c = C.qw * C.unit * C.dx / EPS0_S;  // K dx
     // S2_i = (S1 of the threads before) x (nodes so far) + the thread's own,
     // so both prefixes come from one exchange of (charge, own S2, nodes)
     i128 run = 0, own = 0;
@@ -336,6 +351,7 @@ __device__ void static_solve(const SolveC &C, int csize, int rank, int lo, int h
     // S2 of both O + o + m' R
     i128 R = run, O = own;
     int M = m;
+    if (warp < nw)  // (the other warps hold no nodes)
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const i128 r = shfl_up128(R, o), p = shfl_up128(O, o);
@@ -366,13 +382,13 @@ __device__ void static_solve(const SolveC &C, int csize, int rank, int lo, int h
         r += r2;
     };
     i128 br = 0, bo = 0;  // everything before this thread
-    i128 tr, to;          // everything
+    i128 tr = 0, to = 0;  // everything (the first warp)
     if (csize > 1) {
         cg::cluster_group cl = cg::this_cluster();
         if (tid < csize) {
             i128 r = 0, o = 0;
             int mm = 0;
-            for (int w = 0; w < NW; ++w) {
+            for (int w = 0; w < nw; ++w) {
                 fold(r, o, w1[w], w2[w], wm[w]);
                 mm += wm[w];
             }
@@ -381,25 +397,28 @@ __device__ void static_solve(const SolveC &C, int csize, int rank, int lo, int h
             *cl.map_shared_rank(&cm[rank], tid) = mm;
         }
         cl.sync();
-        for (int b = 0; b < rank; ++b) fold(br, bo, c1[b], c2[b], cm[b]);
-        tr = br;
-        to = bo;
-        for (int b = rank; b < csize; ++b) fold(tr, to, c1[b], c2[b], cm[b]);
-    } else {
-        tr = 0;
-        to = 0;
-        for (int w = 0; w < NW; ++w) fold(tr, to, w1[w], w2[w], wm[w]);
+        if (warp < nw) {
+            for (int b = 0; b < rank; ++b) fold(br, bo, c1[b], c2[b], cm[b]);
+            if (warp == 0) {
+                tr = br;
+                to = bo;
+                for (int b = rank; b < csize; ++b) fold(tr, to, c1[b], c2[b], cm[b]);
+            }
+        }
+    } else if (warp == 0) {
+        for (int w = 0; w < nw; ++w) fold(tr, to, w1[w], w2[w], wm[w]);
     }
-    for (int w = 0; w < warp; ++w) fold(br, bo, w1[w], w2[w], wm[w]);
-    fold(br, bo, pr, po, pm);
-    __shared__ double s_D0, s_e0, s_h;
+    if (warp < nw) {
+        for (int w = 0; w < warp; ++w) fold(br, bo, w1[w], w2[w], wm[w]);
+        fold(br, bo, pr, po, pm);
+    }
+    __shared__ double s_D0, s_e0;
     if (tid == 0) {
-        s_D0 = (c * (double)to - C.phi0) / (double)N;
+        s_D0 = (C.c * (double)to - C.phi0) / (double)N;
         s_e0 = s_D0 / C.dx;
-        s_h = c / (2.0 * C.dx);
     }
     __syncthreads();
-    const double D0 = s_D0, e0 = s_e0, h = s_h, rs = C.qw * C.unit / C.dx;
+    const double D0 = s_D0, e0 = s_e0;
     i128 s1 = br, s2 = bo;  // S1_{i-1}, S2_{i-1}
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
@@ -415,13 +434,13 @@ __device__ void static_solve(const SolveC &C, int csize, int rank, int lo, int h
             p = 0.0;
         } else {
             T = 2 * s1 + q[k];
-            p = C.phi0 + (double)i * D0 - c * (double)s2;
+            p = C.phi0 + (double)i * D0 - C.c * (double)s2;
             s1 += q[k];
             s2 += s1;
         }
-        C.rho[i] = (double)q[k] * ((i == 0 || i == N) ? 2.0 * rs : rs);
+        C.rho[i] = (double)q[k] * ((i == 0 || i == N) ? 2.0 * C.rs : C.rs);
         C.phi[i] = p;
-        C.E[i] = h * (double)T - e0;
+        C.E[i] = C.h * (double)T - e0;
     }
 }
 
@@ -452,8 +471,9 @@ k_static_solve(const typename Sums<Real>::Acc *acc, SolveC C, int csize)
 // Deposit and solve of few particles in one launch: a cluster of 8 blocks,
 // each with the sums of all three species of its share of the particles in
 // its own shared memory; block r then collects its nodes from all eight and
-// solves them.  The separate kernels need the accumulators cleared, and three
-// launches took 53 us for 4e4 particles, most of it in one thread's sums.
+// solves them.  What bounds it: the latency of its stages (4e4 FP64 particles
+// in 128 cells: 12.7 us; the five launches it replaces with one thread's sums
+// 53 us).  Divisions stay off the threads: FP64 runs on few units here.
 constexpr int SMALL_PER = 2;  // nodes per thread: (4097 / 8) / 512
 constexpr long long SMALL_MOST = 1ll << 17;  // slots: 2^14 per block (the FP64 sums' limit) and species units
 static_assert(SMALL_MOST / STATIC_CLUSTER <= Sums<double>::MOST && SMALL_MOST / STATIC_CLUSTER <= Sums<float>::MOST, "");
@@ -485,34 +505,34 @@ k_static_small(Particles<Real> P, SolveC C)
     const int per = (NC + UNIT_THREADS - 1) / UNIT_THREADS;
     const int lo = min(rank * NC + tid * per, N + 1);
     const int hi = min(min(lo + per, (rank + 1) * NC), N + 1);
+    // the block's nodes from the words of all eight blocks: eight lanes per
+    // node, one block each (all their loads in flight at once), then summed
+    __shared__ i128 s_q[STATIC_NODES / STATIC_CLUSTER + 2];
+    {
+        const int first = rank * NC, count = min(NC, N + 1 - first);
+        const unsigned *o = cl.map_shared_rank(ssum, tid % STATIC_CLUSTER);
+        for (int j0 = 0; j0 < count; j0 += UNIT_THREADS / STATIC_CLUSTER) {
+            const int j = j0 + tid / STATIC_CLUSTER, i = first + j;
+            i128 v = 0;
+            if (j < count) {
+                i128 n[3];
+#pragma unroll
+                for (int s = 0; s < 3; ++s) n[s] = node_of<Real>(o + s * per_species, stride, i);
+                v = n[2] - n[0] - n[1];
+            }
+#pragma unroll
+            for (int b = 1; b < STATIC_CLUSTER; b <<= 1) {
+                const unsigned long long lo64 = __shfl_xor_sync(0xffffffffu, (unsigned long long)v, b);
+                const long long hi64 = __shfl_xor_sync(0xffffffffu, (long long)(v >> 64), b);
+                v += ((i128)hi64 << 64) | (i128)lo64;
+            }
+            if (j < count && tid % STATIC_CLUSTER == 0) s_q[j] = v;
+        }
+        __syncthreads();
+    }
     i128 q[SMALL_PER];
 #pragma unroll
-    for (int k = 0; k < SMALL_PER; ++k) {
-        q[k] = 0;
-        if (lo + k >= hi) continue;
-#pragma unroll
-        for (int s = 0; s < 3; ++s) {
-            // the species' words of the node's cell and of the one before, summed over the blocks
-            unsigned long long cnt = 0, w[S::WORDS] = {}, p[S::WORDS] = {};
-            for (int b = 0; b < STATIC_CLUSTER; ++b) {
-                const unsigned *o = cl.map_shared_rank(ssum, b) + s * per_species;
-                cnt += o[lo + k];
-#pragma unroll
-                for (int j = 0; j < S::WORDS; ++j) {
-                    w[j] += o[(j + 1) * stride + lo + k];
-                    if (lo + k > 0) p[j] += o[(j + 1) * stride + lo + k - 1];
-                }
-            }
-            i128 v = (i128)cnt << S::BITS;
-            int sh = 0;
-#pragma unroll
-            for (int j = 0; j < S::WORDS; ++j) {
-                v += ((i128)p[j] - (i128)w[j]) << sh;
-                sh += S::width(j);
-            }
-            q[k] += s == 2 ? v : -v;
-        }
-    }
+    for (int k = 0; k < SMALL_PER; ++k) q[k] = lo + k < hi ? s_q[lo + k - rank * NC] : (i128)0;
     // the solve's exchange synchronises the cluster after these reads, before any block can end
     static_solve<UNIT_THREADS, SMALL_PER>(C, STATIC_CLUSTER, rank, lo, hi, q);
 }
@@ -556,7 +576,7 @@ cudaError_t static_run(void *acc, const int *const *cell, const void *const *off
     typename S::Acc *a = static_cast<typename S::Acc *>(acc);
     // what fits on an SM by threads and shared memory; not more blocks than units
     const long long units = all / UNIT + 3;
-    const int per_sm = (int)std::min<size_t>(3, (224u << 10) / (sm + 1024));
+    const int per_sm = (int)std::min<size_t>(2, (224u << 10) / (sm + 1024));
     const int grid = (int)std::min<long long>(units, (long long)num_sms * per_sm);
     e = o2::launch_k(k_static_deposit<Real>, grid, UNIT_THREADS, sm, st, a, P, C.N);
     if (e != cudaSuccess) return e;
@@ -619,8 +639,10 @@ extern "C" pic_status pic_field_solve_static(const pic_config *cfg, long long st
     C.N = N;
     C.dx = cfg->L_m / N;
     C.phi0 = cfg->U_rf_V * sin(2.0 * PI_S * cfg->f_rf_Hz * t + cfg->rf_phase);
-    C.unit = fp64 ? 1.0 / 4503599627370496.0 : 1.0 / (double)(1 << o2::FIX_BITS);
-    C.qw = QE_S * cfg->weight_m2;
+    const double unit = fp64 ? 1.0 / 4503599627370496.0 : 1.0 / (double)(1 << o2::FIX_BITS);
+    C.c = QE_S * cfg->weight_m2 * unit * C.dx / EPS0_S;
+    C.h = C.c / (2.0 * C.dx);
+    C.rs = QE_S * cfg->weight_m2 * unit / C.dx;
     C.rho = d_rho;
     C.phi = d_phi;
     C.E = d_E;
