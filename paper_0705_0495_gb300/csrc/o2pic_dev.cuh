@@ -13,7 +13,14 @@ constexpr int SUBTILE = 128;           // slots of one warp in a tile (32 lanes 
 constexpr int SUBTILES = 1024 / SUBTILE;
 constexpr int BIRTH_CAP_W = 32;        // births staged per sub-tile (null-collision scheme)
 constexpr int BIRTH_CAP_SEQ = 128;     // the same with the sequential gas scheme (n1 steps of collisions at once)
-constexpr int COLLIDE_THREADS = 256;   // threads per block of the collision kernel
+#ifndef O2_COLLIDE_THREADS
+#define O2_COLLIDE_THREADS 64
+#endif
+#ifndef O2_COLLIDE_PER_SM
+#define O2_COLLIDE_PER_SM 10
+#endif
+constexpr int COLLIDE_THREADS = O2_COLLIDE_THREADS;  // threads per block of the collision kernel
+constexpr int COLLIDE_PER_SM = O2_COLLIDE_PER_SM;    // its blocks per SM
 #ifndef O2_TILES_PER_TICKET
 #define O2_TILES_PER_TICKET 8
 #endif
@@ -138,13 +145,17 @@ struct SpeciesC {
     double coul_k;      // Coulomb: <tan^2(chi/2)> u_n^3 per particle of the cell (Eq. 2)
     unsigned int tnull; // null-collision threshold on a 32-bit word
     int nch;
-    int table_lo;       // first table of the shared grid (for the index)
+    int grid_off, grid_n;  // the channels' shared energy grid: its place in the LUT arrays, its nodes
+    double grid_lo, grid_hi;  // its ends [eV]
+    float grid_lo_f, grid_hi_f, grid_lnlo_f, grid_inv_f;  // log of the first node, (n-1) / log(hi/lo)
     int gtab_ld;        // row length of the node-major gas table (multiple of 4)
     int gtab_off;       // first element of this (discharge, species) gas table
     int nbins;          // energy bins of the collision-frequency bound (0: one bound)
     int bin_off;        // first entry of this species' bins in WsPtrs::nubin
     // FP32 copies (the FP32 path never converts from FP64 on the device)
     float qm_f, numax_n_f, vgas_n_f, Ek_f, mfrac_f, Mfrac_f, ke_eV_f, coul_k_f;
+    double thv[MAX_GAS_CH];   // the channels' thresholds again, side by side
+    float thv_f[MAX_GAS_CH];
     GasChan ch[MAX_GAS_CH];
 };
 
@@ -350,7 +361,9 @@ __device__ __forceinline__ uint4 rng_block(unsigned long long seed, int disc, in
 template <typename Real> __device__ __forceinline__ Real unif(unsigned w);
 template <> __device__ __forceinline__ double unif<double>(unsigned w)
 {
-    return ((double)w + 0.5) * (1.0 / 4294967296.0);
+    // (w + 1/2) 2^-32, from the bits of 1 + that value: one FP64 instruction
+    // instead of a conversion and two (exact both ways)
+    return __hiloint2double((int)(0x3FF00000u | (w >> 12)), (int)((w << 20) | 0x80000u)) - 1.0;
 }
 // FP32: (2k+1) 2^-24 with k = w >> 9, exactly representable, inside (0, 1);
 // within 2^-24 of the FP64 value.

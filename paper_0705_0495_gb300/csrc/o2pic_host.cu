@@ -570,7 +570,18 @@ static void build_disc(pic_handle *h, int d, const std::vector<int> &gas_tabs_by
                                   (8.0 * PI * EPS0 * EPS0 * mc * mc * D.dx) / (xdt * xdt * xdt)
                             : 0.0;
         S.nch = gas_count[s];
-        S.table_lo = S.nch > 0 ? gas_tabs_by_sp_flat[s * MAX_GAS_CH] : 0;
+        if (S.nch > 0) {
+            const int t0 = gas_tabs_by_sp_flat[s * MAX_GAS_CH];
+            const HostTable &t = h->tabs[t0];
+            for (int i = 0; i < t0; ++i) S.grid_off += h->tabs[i].n;
+            S.grid_n = t.n;
+            S.grid_lo = t.E[0];
+            S.grid_hi = t.E[t.n - 1];
+            S.grid_lo_f = (float)S.grid_lo;
+            S.grid_hi_f = (float)S.grid_hi;
+            S.grid_lnlo_f = (float)std::log(t.E[0]);
+            S.grid_inv_f = (float)((t.n - 1) / std::log(t.E[t.n - 1] / t.E[0]));
+        }
         for (int j = 0; j < S.nch; ++j) {
             const int ti = gas_tabs_by_sp_flat[s * MAX_GAS_CH + j];
             const HostTable &t = h->tabs[ti];
@@ -583,6 +594,8 @@ static void build_disc(pic_handle *h, int d, const std::vector<int> &gas_tabs_by
             S.ch[j].dloss_f = (float)S.ch[j].dloss;
             S.ch[j].th = t.th;
             S.ch[j].th_f = (float)t.th;
+            S.thv[j] = t.th;
+            S.thv_f[j] = (float)t.th;
         }
         // nu_max up to a centre-of-mass energy capE: [0, capE] is cut at every
         // node and threshold of the species' channels; between neighbouring

@@ -29,7 +29,8 @@
 // A warp whose 128 slots are live and stay on the grid (nearly all) takes a
 // path without masks and selects, with its floors from packed adds (FP32) or
 // off the FP64 units where a slot stays in its cell: FP32 push 293 -> 251 us,
-// FP64 1968 -> 1000 us, results bit for bit the same.
+// FP64 1968 -> 1000 us, results bit for bit the same.  The FP64 sums in 32-bit
+// words per cell took it to 733 us (4e4 superparticles: 17 -> 10.6 us).
 #include <cstdio>
 
 #include "o2pic_launch.h"
@@ -128,6 +129,14 @@ template <typename Real> __device__ __forceinline__ Real below_one();
 template <> __device__ __forceinline__ float below_one<float>() { return 0x1.fffffep-1f; }
 template <> __device__ __forceinline__ double below_one<double>() { return 0x1.fffffffffffffp-1; }
 
+// a < b for values that are not negative: FP64 compares as integers (their
+// bit patterns have the same order), off the few FP64 units
+__device__ __forceinline__ bool less_pos(float a, float b) { return a < b; }
+__device__ __forceinline__ bool less_pos(double a, double b)
+{
+    return __double_as_longlong(a) < __double_as_longlong(b);
+}
+
 // Interpolation of the gas-channel cross sections of one projectile at the
 // centre-of-mass energy E [eV]: piecewise linear in E on the shared geometric
 // grid, end values held outside it, zero below each channel's threshold.
@@ -139,41 +148,40 @@ struct XsPoint {
 };
 
 template <typename Real>
-__device__ __forceinline__ XsPoint<Real> xs_locate(const TableDesc &T, const Real *lutE, Real E)
+__device__ __forceinline__ XsPoint<Real> xs_locate(const SpeciesC &S, const Real *lutE, Real E)
 {
     XsPoint<Real> p;
-    const Real *nodes = lutE + T.off;
-    const int n = T.n;
-    if (!(E > nodes[0])) {
+    const Real *nodes = lutE + S.grid_off;
+    const int n = S.grid_n;
+    if (!less_pos(pick<Real>(S.grid_lo, S.grid_lo_f), E)) {
         p.region = 0; p.k = 0; p.f = Real(0);
         return p;
     }
-    if (E >= nodes[n - 1]) {
+    if (!less_pos(E, pick<Real>(S.grid_hi, S.grid_hi_f))) {
         p.region = 2; p.k = n - 2; p.f = Real(1);
         return p;
     }
-    Real t = (log(E) - pick<Real>(T.lnE0, T.lnE0_f)) * pick<Real>(T.inv_dlog, T.inv_dlog_f);
+    // the logarithm only guesses the segment, so a fast FP32 one will do in
+    // both precisions; the node comparison decides.  Both ends of the guess
+    // are loaded at once.
+    const float t = (__logf((float)E) - S.grid_lnlo_f) * S.grid_inv_f;
     int k = (int)t;
     k = k < 0 ? 0 : (k > n - 2 ? n - 2 : k);
-    // the logarithm only guesses the segment; the node comparison decides
-    while (k > 0 && E < nodes[k]) --k;
-    while (k < n - 2 && E >= nodes[k + 1]) ++k;
+    Real a = nodes[k], b = nodes[k + 1];
+    while (k > 0 && less_pos(E, a)) {
+        --k;
+        b = a;
+        a = nodes[k];
+    }
+    while (k < n - 2 && !less_pos(E, b)) {
+        ++k;
+        a = b;
+        b = nodes[k + 1];
+    }
     p.region = 1;
     p.k = k;
-    p.f = (E - nodes[k]) / (nodes[k + 1] - nodes[k]);
+    p.f = (E - a) / (b - a);
     return p;
-}
-
-template <typename Real>
-__device__ __forceinline__ Real xs_value(const TableDesc &T, const Real *lutS,
-                                         const XsPoint<Real> &p, Real E)
-{
-    if (E < pick<Real>(T.th, T.th_f)) return Real(0);
-    const Real *s = lutS + T.off;
-    if (p.region == 0) return s[0];
-    if (p.region == 2) return s[T.n - 1];
-    Real a = s[p.k], b = s[p.k + 1];
-    return a + p.f * (b - a);
 }
 
 // centre-of-mass binary collision in normalised units: relative speed
@@ -362,7 +370,6 @@ __device__ __forceinline__ Outcome gas_collide(const WsPtrs &W, const Disc &Dd, 
 {
     const SpeciesC &S = Dd.sp[s];
     const Real *lutE = Lut<Real>::E(W);
-    const Real *lutS = Lut<Real>::S(W);
     uint4 a = rng_block(Dd.seed, Dd.discharge, s, 1, 0, 0, step, idx);
     uint4 b = rng_block(Dd.seed, Dd.discharge, s, 1, 0, 1, step, idx);
     Real n0, n1, n2, n3;
@@ -376,8 +383,7 @@ __device__ __forceinline__ Outcome gas_collide(const WsPtrs &W, const Disc &Dd, 
     Real u = sqrt(u2);
     Real E = pick<Real>(S.Ek, S.Ek_f) * u2;
     Real target = unif<Real>(b.x) * numax_n;
-    const TableDesc &T0 = W.tables[S.table_lo];
-    XsPoint<Real> pt = xs_locate<Real>(T0, lutE, E);
+    XsPoint<Real> pt = xs_locate<Real>(S, lutE, E);
     // node-major table of n_j dx sigma_j(E_k): the rows k and k+1 of every
     // channel come in a few 16-byte loads
     const Real *row = GasTab<Real>::ptr(W) + S.gtab_off;
@@ -386,20 +392,32 @@ __device__ __forceinline__ Outcome gas_collide(const WsPtrs &W, const Disc &Dd, 
     const Real *rb = ra + ld;
     Real cum = Real(0);
     int chosen = -1;
-    // channel walk with selects only: the lanes of a warp stay together
-    for (int j0 = 0; j0 < S.nch; j0 += GasTab<Real>::VEC) {
-        Real a[GasTab<Real>::VEC], b[GasTab<Real>::VEC];
-        GasTab<Real>::load(ra + j0, a);
-        GasTab<Real>::load(rb + j0, b);
+    // channel walk with selects only: the lanes of a warp stay together; the
+    // next channels' rows are loaded before the present ones are walked
+    constexpr int VEC = GasTab<Real>::VEC;
+    Real xa[VEC], xb[VEC];
+    GasTab<Real>::load(ra, xa);
+    GasTab<Real>::load(rb, xb);
+    for (int j0 = 0; j0 < S.nch; j0 += VEC) {
+        Real a[VEC], b[VEC];
 #pragma unroll
-        for (int q = 0; q < GasTab<Real>::VEC; ++q) {
+        for (int q = 0; q < VEC; ++q) {
+            a[q] = xa[q];
+            b[q] = xb[q];
+        }
+        if (j0 + VEC < ld) {
+            GasTab<Real>::load(ra + j0 + VEC, xa);
+            GasTab<Real>::load(rb + j0 + VEC, xb);
+        }
+#pragma unroll
+        for (int q = 0; q < VEC; ++q) {
             const int j = j0 + q;
             if (j >= S.nch) break;  // uniform: one species per warp
             // below the grid f = 0 gives a exactly; above it, the last node
             Real v = pt.region == 2 ? b[q] : a[q] + pt.f * (b[q] - a[q]);
-            v = E < pick<Real>(S.ch[j].th, S.ch[j].th_f) ? Real(0) : v;
+            v = less_pos(E, pick<Real>(S.thv[j], S.thv_f[j])) ? Real(0) : v;
             cum += v * u;
-            chosen = (chosen < 0 && target < cum) ? j : chosen;
+            chosen = (chosen < 0 && less_pos(target, cum)) ? j : chosen;
         }
     }
     const bool viol = cum > numax_n;
@@ -469,31 +487,41 @@ constexpr int FIX_BITS_64 = 40;
 static_assert((long long)FLUSH_TILES * CHUNK < (1LL << (63 - FIX_BITS_64)),
               "FP64 shared sums must stay within int64");
 
-// the block's sum of a node in the global accumulators' type
+// A node's integer sum as the global accumulators' type.
 template <typename Real> __device__ __forceinline__ typename AccT<Real>::T sacc_value(unsigned long long node);
-template <> __device__ __forceinline__ unsigned long long sacc_value<float>(unsigned long long node)
-{
-    return split_value(node);
-}
+template <> __device__ __forceinline__ unsigned long long sacc_value<float>(unsigned long long node) { return node; }
 template <> __device__ __forceinline__ double sacc_value<double>(unsigned long long node)
 {
     return (double)(long long)node * (1.0 / (double)(1ull << FIX_BITS_64));
 }
 
-// a node's sum in the global accumulators' type from the block's shared sums
+// A node's integer sum (units of 2^-FIX_BITS or 2^-FIX_BITS_64 of a
+// particle) from the block's sums per cell: count_i - W_i + W_(i-1).
+// FP32: sCnt[i], and the split words of sAcc[i].  FP64: sCnt[i], and W in
+// three words of SPLIT64 bits, two of them the halves of sAcc[i] and the
+// third sCnt[stride + i] (FLUSH_TILES tiles of particles stay below 2^32 in
+// each).
+constexpr int SPLIT64_0 = 14, SPLIT64_1 = 27;  // first bits of the second and third words
+static_assert((long long)FLUSH_TILES * CHUNK <= (1LL << 18) && FIX_BITS_64 - SPLIT64_1 == 13, "words must fit 32 bits");
 template <typename Real>
-__device__ __forceinline__ typename AccT<Real>::T sacc_node(const unsigned long long *sAcc, const unsigned *sCnt, int i);
+__device__ __forceinline__ unsigned long long sacc_cells(const unsigned long long *sAcc, const unsigned *sCnt, int stride,
+                                                         int i);
 template <>
-__device__ __forceinline__ unsigned long long sacc_node<float>(const unsigned long long *sAcc, const unsigned *sCnt,
-                                                               int i)
+__device__ __forceinline__ unsigned long long sacc_cells<float>(const unsigned long long *sAcc, const unsigned *sCnt, int,
+                                                                int i)
 {
     const unsigned long long lw = i > 0 ? split_value(sAcc[i - 1]) : 0ull;
     return ((unsigned long long)sCnt[i] << FIX_BITS) - split_value(sAcc[i]) + lw;
 }
 template <>
-__device__ __forceinline__ double sacc_node<double>(const unsigned long long *sAcc, const unsigned *, int i)
+__device__ __forceinline__ unsigned long long sacc_cells<double>(const unsigned long long *sAcc, const unsigned *sCnt,
+                                                                 int stride, int i)
 {
-    return sacc_value<double>(sAcc[i]);
+    auto w = [&](int j) {
+        const unsigned long long a = sAcc[j];
+        return (a & 0xFFFFFFFFull) + ((a >> 32) << SPLIT64_0) + ((unsigned long long)sCnt[stride + j] << SPLIT64_1);
+    };
+    return ((unsigned long long)sCnt[i] << FIX_BITS_64) - w(i) + (i > 0 ? w(i - 1) : 0ull);
 }
 
 // charge of one particle added to (sign > 0) or removed from the global
@@ -534,7 +562,7 @@ template <> __device__ __forceinline__ double *acc_global<double>(const WsPtrs &
 #define O2_DEP_LANES 4
 #endif
 constexpr int DEP_LANES = O2_DEP_LANES;
-__device__ __forceinline__ void deposit4(unsigned long long *sAcc, unsigned *sCnt, const int dep[4],
+__device__ __forceinline__ void deposit4(unsigned long long *sAcc, unsigned *sCnt, int, const int dep[4],
                                          const float off[4])
 {
     unsigned w1[4];
@@ -565,6 +593,54 @@ __device__ __forceinline__ void deposit4(unsigned long long *sAcc, unsigned *sCn
         atomicAdd(&sCnt[ck], dep[k] >= 0 ? 1u : 0u);
         split_add(&sAcc[ck], w1[k]);
     }
+}
+
+// The same for the FP64 sums: four 32-bit shared atomics where two 64-bit
+// ones per particle (compare-and-swap loops here) contended for the few cells
+// of a sorted warp.
+__device__ __forceinline__ void split_add64(unsigned long long *sAcc, unsigned *sCnt, int stride, int c,
+                                            unsigned long long v, unsigned n)
+{
+    unsigned *w = reinterpret_cast<unsigned *>(&sAcc[c]);
+    atomicAdd(&sCnt[c], n);
+    atomicAdd(&w[0], (unsigned)v & ((1u << SPLIT64_0) - 1u));
+    atomicAdd(&w[1], (unsigned)(v >> SPLIT64_0) & ((1u << (SPLIT64_1 - SPLIT64_0)) - 1u));
+    atomicAdd(&sCnt[stride + c], (unsigned)(v >> SPLIT64_1));
+}
+// rn(off 2^FIX_BITS_64) from one FP64 add: off + 2^(52 - FIX_BITS_64) has its
+// last bit at 2^-FIX_BITS_64 (off is in [0, 1))
+__device__ __forceinline__ unsigned long long weight64(double off)
+{
+    constexpr double SHIFT = (double)(1ull << (52 - FIX_BITS_64));
+    return (unsigned long long)(__double_as_longlong(off + SHIFT) - __double_as_longlong(SHIFT));
+}
+__device__ __forceinline__ void deposit4(unsigned long long *sAcc, unsigned *sCnt, int stride, const int dep[4],
+                                         const double off[4])
+{
+    unsigned long long w1[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w1[k] = dep[k] >= 0 ? weight64(off[k]) : 0ull;
+    const bool same = dep[0] >= 0 && dep[1] == dep[0] && dep[2] == dep[0] && dep[3] == dep[0];
+    const unsigned long long b = w1[0] + w1[1] + w1[2] + w1[3];
+    const int c0 = __shfl_sync(0xffffffffu, dep[0], 0);
+    const bool in = same && dep[0] == c0;
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+    if (__popc(m) >= DEP_LANES) {
+        // 32 lanes of at most 2^(FIX_BITS_64 + 2), summed in two 32-bit halves;
+        // a third word of up to 20 bits is one add of 128 particles' weight
+        const unsigned lo = __reduce_add_sync(0xffffffffu, in ? (unsigned)(b & 0xFFFFFFull) : 0u);
+        const unsigned hi = __reduce_add_sync(0xffffffffu, in ? (unsigned)(b >> 24) : 0u);
+        if ((threadIdx.x & 31) == 0)
+            split_add64(sAcc, sCnt, stride, c0, ((unsigned long long)hi << 24) + lo, 4u * (unsigned)__popc(m));
+        if (in) return;
+    }
+    if (same) {
+        split_add64(sAcc, sCnt, stride, dep[0], b, 4u);
+        return;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (dep[k] >= 0) split_add64(sAcc, sCnt, stride, dep[k], w1[k], 1u);
 }
 
 // The push that also samples the diagnostics keeps its FP32 sums per NODE
@@ -608,15 +684,10 @@ __device__ __forceinline__ void deposit4_nodes(unsigned long long *sAcc, const i
 }
 __device__ __forceinline__ void deposit4_nodes(unsigned long long *sAcc, const int dep[4], const double off[4])
 {
-    // rn(off 2^FIX_BITS_64) from one FP64 add: off + 2^(52 - FIX_BITS_64) has
-    // its last bit at 2^-FIX_BITS_64 (off is in [0, 1))
-    constexpr double SHIFT = (double)(1ull << (52 - FIX_BITS_64));
     constexpr unsigned long long ONE = 1ull << FIX_BITS_64;
     unsigned long long w1[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-        w1[k] = dep[k] >= 0 ? (unsigned long long)(__double_as_longlong(off[k] + SHIFT) - __double_as_longlong(SHIFT))
-                            : 0ull;
+    for (int k = 0; k < 4; ++k) w1[k] = dep[k] >= 0 ? weight64(off[k]) : 0ull;
     // as in the FP32 path: the lanes whose four slots sit in the first lane's
     // cell add their weights once for all, others add their own
     const bool same = dep[0] >= 0 && dep[1] == dep[0] && dep[2] == dep[0] && dep[3] == dep[0];
@@ -806,8 +877,8 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
     pdl_wait();
     using Acc = typename AccT<Real>::T;
     constexpr int PUSH_THREADS = SH::threads, NW = SH::nw, G = SH::groups, QCAP = SH::qcap;
-    // FP32 without diagnostics: per-cell sums (counts + upper weights)
-    constexpr bool CELLS = sizeof(Real) == 4 && !DIAG;
+    // without diagnostics: per-cell sums (counts + upper weights)
+    constexpr bool CELLS = !DIAG;
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned long long *sAcc = reinterpret_cast<unsigned long long *>(smem);  // integer sums (both paths)
     Real *sE = reinterpret_cast<Real *>(sAcc + (Nmax + 2));
@@ -818,7 +889,7 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
     unsigned *sEedf = reinterpret_cast<unsigned *>(sE + (Nmax + 2)) + NW * QCAP;
     unsigned *sFm = sEedf + eedf_max;
     unsigned char *qBin = reinterpret_cast<unsigned char *>(sFm + fm_max) + w * QCAP;
-    // FP32: particles per cell of the block's sums, after the queues' bins
+    // particles per cell of the block's sums (FP64: and third words), after the queues' bins
     unsigned *sCnt = reinterpret_cast<unsigned *>(
         (reinterpret_cast<size_t>(reinterpret_cast<unsigned char *>(sFm + fm_max) + NW * QCAP) + 15) & ~size_t(15));
 
@@ -846,8 +917,9 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
         __syncthreads();
         Acc *g = accG + (size_t)fs * W.total_nodes + Dd.gbase;
         for (int i = tid; i <= Dd.N; i += PUSH_THREADS) {
-            const Acc v = CELLS ? sacc_node<Real>(sAcc, sCnt, i) : sacc_value<Real>(sAcc[i]);
-            if (v != Acc(0)) acc_add(&g[i], v);
+            const unsigned long long v = CELLS ? sacc_cells<Real>(sAcc, sCnt, Nmax + 2, i)
+                                               : (sizeof(Real) == 4 ? split_value(sAcc[i]) : sAcc[i]);
+            if (v != 0ull) acc_add(&g[i], sacc_value<Real>(v));
         }
         for (int q = tid; q < C_NCOUNT; q += PUSH_THREADS) {
             if (s_cnt[q]) atomicAdd(&W.counters[(size_t)fd * C_NCOUNT + q], (unsigned long long)s_cnt[q]);
@@ -944,6 +1016,7 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
             for (int i = tid; i <= Dn.N + 1; i += PUSH_THREADS) {
                 sAcc[i] = 0ull;
                 if (CELLS) sCnt[i] = 0u;
+                if (CELLS && sizeof(Real) == 8) sCnt[Nmax + 2 + i] = 0u;
             }
             {
                 const SpeciesC &Sn = Dn.sp[nx % NSP];
@@ -1194,7 +1267,7 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
                 }
             }
             if constexpr (CELLS)
-                deposit4(sAcc, sCnt, dep, off);
+                deposit4(sAcc, sCnt, Nmax + 2, dep, off);
             else
                 deposit4_nodes(sAcc, dep, off);
             if (full) {
@@ -1240,37 +1313,52 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
 // charge leaves the global grid, births go to its sub-tile's records.  A
 // candidate's cell and offset are read only when its collision has products
 // or kills it, and its velocity is written back only after an event (a
-// null event changes nothing): each field is a scattered access.  Event
-// counts are summed per block for the discharge of the block's first
-// candidate (the list holds runs of one discharge), others go straight to
-// the global counters.
-#ifndef O2_COLLIDE_MIN_BLOCKS
-#define O2_COLLIDE_MIN_BLOCKS 1
-#endif
+// null event changes nothing): each field is a scattered access.
+//
+// What bounds it: the chain of dependent loads in FP32, the FP64 units in
+// FP64 (about 500 FP64 instructions per warp of candidates, 16 cycles each on
+// an SM's two units).  So the list is dealt out in batches of 32, one warp per
+// block and SM first: a hundred FP64 candidates in one block took 28 us, on
+// four SMs 15 us (FP32 8.8 -> 5.7 us; 1.3e5 candidates FP32 30 -> 26, FP64
+// 140 -> 122 us, the latter from fewer FP64 instructions: uniforms from bits,
+// comparisons of positive values as integers).  Blocks of 32, 64 or 128
+// threads gave the same times.  The constants that a candidate needs are in its
+// species' record, its table's ends included, one load level below the list.
+// Event counts are summed per block for the discharge of the block's first
+// candidate (the list holds runs of one discharge); lanes of another add
+// theirs to the global counters, one add per warp and kind.
 template <typename Real>
-__global__ void __launch_bounds__(COLLIDE_THREADS, O2_COLLIDE_MIN_BLOCKS)
+__global__ void __launch_bounds__(COLLIDE_THREADS)
 k_collide(WsPtrs W, Pools<Real> P, int par)
 {
     pdl_wait();
     using Acc = typename AccT<Real>::T;
+    constexpr int NW = COLLIDE_THREADS / 32;
     __shared__ unsigned s_ev[C_NCOUNT];
     Ctl *ctl = W.ctl;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // the first batch's entry is loaded together with the list's length
+    int q = (blockIdx.x + gridDim.x * warp) * 32 + lane;
+    int2 e = q < W.cand_cap ? W.cand[q] : make_int2(0, 0);
+    const int yblk = W.cand[min(blockIdx.x * 32u, (unsigned)W.cand_cap - 1u)].y;
     const int n = (int)min((long long)ctl->cand_n, (long long)W.cand_cap);
     const unsigned long long step = ctl->step[par];
-    const int cur = ctl->cur;
-    int *cellA = P.cell[cur];
-    Real *offA = P.off[cur], *vxA = P.vx[cur], *vyA = P.vy[cur], *vzA = P.vz[cur];
+    const unsigned b0 = ctl->cur ? P.stride : 0u;
+    if ((int)blockIdx.x * 32 >= n) return;
+    const int dblk = (yblk >> 8) / NSP;
+    for (int k = threadIdx.x; k < C_NCOUNT; k += COLLIDE_THREADS) s_ev[k] = 0;
+    __syncthreads();
     BirthRec<Real> *stage = reinterpret_cast<BirthRec<Real> *>(W.births);
     Acc *accG = acc_global<Real>(W);
-    for (int base = blockIdx.x * COLLIDE_THREADS; base < n; base += gridDim.x * COLLIDE_THREADS) {
-        for (int q = threadIdx.x; q < C_NCOUNT; q += COLLIDE_THREADS) s_ev[q] = 0;
-        __syncthreads();
-        const int dblk = (W.cand[base].y >> 8) / NSP;
-        const int q = base + threadIdx.x;
+    for (; q - lane < n; q += gridDim.x * COLLIDE_THREADS) {
+        const int qn = q + gridDim.x * COLLIDE_THREADS;
+        const int2 en = qn < n ? W.cand[qn] : make_int2(0, 0);
+        int d = dblk, code = -1;  // what the lane counts: the reaction, its number + 32 with a violation
         if (q < n) {
-            const int2 e = W.cand[q];
             const int i = e.x, ds = e.y >> 8, bin = e.y & 0xFF;
-            const int d = ds / NSP, s = ds % NSP;
+            const unsigned ib = b0 + (unsigned)i;
+            const int s = ds % NSP;
+            d = ds / NSP;
             const Disc &Dd = W.disc[d];
             const SpeciesC &S = Dd.sp[s];
             const int rel = i - Dd.pbase[s];
@@ -1278,37 +1366,45 @@ k_collide(WsPtrs W, Pools<Real> P, int par)
             const int slot = rel % SUBTILE;
             int c = 0;
             Real off = Real(0);
-            Real vx = vxA[i], vy = vyA[i], vz = vzA[i];
-            const Real nun = S.nbins > 0 ? pick<Real>(W.nubin[S.bin_off + bin].numax_n, W.nubin[S.bin_off + bin].numax_n_f)
-                                         : pick<Real>(S.numax_n, S.numax_n_f);
+            Real vx = P.vx[0][ib], vy = P.vy[0][ib], vz = P.vz[0][ib];
+            const NuBin &nb = W.nubin[(size_t)d * NUBIN_MAX + (s == 0 ? bin : 0)];
+            const Real nbin = pick<Real>(nb.numax_n, nb.numax_n_f);
+            const Real nun = S.nbins > 0 ? nbin : pick<Real>(S.numax_n, S.numax_n_f);
             const BirthSink<Real> B{stage + (size_t)sub * W.birth_cap, W.tile_cnt + (size_t)sub * NSP, ctl, W.birth_cap};
-            const Outcome o = gas_collide<Real>(W, Dd, s, (unsigned)rel, step, nun, vx, vy, vz, cellA + i,
-                                                offA + i, c, off, slot << 1, B);
+            const Outcome o = gas_collide<Real>(W, Dd, s, (unsigned)rel, step, nun, vx, vy, vz, P.cell[0] + ib,
+                                                P.off[0] + ib, c, off, slot << 1, B);
             // a null event leaves the particle as it was: nothing to write
             if (o.alive) {
                 if (o.reaction >= 0) {
-                    vxA[i] = vx;
-                    vyA[i] = vy;
-                    vzA[i] = vz;
+                    P.vx[0][ib] = vx;
+                    P.vy[0][ib] = vy;
+                    P.vz[0][ib] = vz;
                 }
             } else {
-                cellA[i] = -1;
+                P.cell[0][ib] = -1;
                 deposit_global(accG + (size_t)s * W.total_nodes + Dd.gbase, c, off, -1);
             }
-            if (d == dblk) {
-                if (o.viol) atomicAdd(&s_ev[C_VIOL_GAS], 1u);
-                if (o.reaction >= 0) atomicAdd(&s_ev[C_EVENTS + o.reaction], 1u);
-            } else {
+            if (o.reaction >= 0 || o.viol) code = (o.reaction >= 0 ? o.reaction : 31) + (o.viol ? 32 : 0);
+        }
+        if (code >= 0 && d == dblk) {
+            if (code >= 32) atomicAdd(&s_ev[C_VIOL_GAS], 1u);
+            if ((code & 31) < 31) atomicAdd(&s_ev[C_EVENTS + (code & 31)], 1u);
+            code = -1;
+        }
+        if (__any_sync(0xffffffffu, code >= 0)) {
+            const unsigned peers = __match_any_sync(0xffffffffu, code < 0 ? -1 : d * 64 + code);
+            if (code >= 0 && lane == __ffs(peers) - 1) {
                 unsigned long long *g = W.counters + (size_t)d * C_NCOUNT;
-                if (o.viol) atomicAdd(&g[C_VIOL_GAS], 1ull);
-                if (o.reaction >= 0) atomicAdd(&g[C_EVENTS + o.reaction], 1ull);
+                const unsigned long long m = (unsigned long long)__popc(peers);
+                if (code >= 32) atomicAdd(&g[C_VIOL_GAS], m);
+                if ((code & 31) < 31) atomicAdd(&g[C_EVENTS + (code & 31)], m);
             }
         }
-        __syncthreads();
-        for (int k = threadIdx.x; k < C_NCOUNT; k += COLLIDE_THREADS)
-            if (s_ev[k]) atomicAdd(&W.counters[(size_t)dblk * C_NCOUNT + k], (unsigned long long)s_ev[k]);
-        __syncthreads();
+        e = en;
     }
+    __syncthreads();
+    for (int k = threadIdx.x; k < C_NCOUNT; k += COLLIDE_THREADS)
+        if (s_ev[k]) atomicAdd(&W.counters[(size_t)dblk * C_NCOUNT + k], (unsigned long long)s_ev[k]);
 }
 
 // Bound on P = n dx sigma u_n n1 of channel j of species S for a particle
@@ -1325,7 +1421,7 @@ __device__ __forceinline__ void dsmc_locate(const WsPtrs &W, const SpeciesC &S, 
                                             int &k, int &region)
 {
     umax = sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]) + Real(10) * pick<Real>(S.vgas_n, S.vgas_n_f);
-    const XsPoint<Real> pm = xs_locate<Real>(W.tables[S.table_lo], Lut<Real>::E(W), pick<Real>(S.Ek, S.Ek_f) * umax * umax);
+    const XsPoint<Real> pm = xs_locate<Real>(S, Lut<Real>::E(W), pick<Real>(S.Ek, S.Ek_f) * umax * umax);
     k = pm.k;
     region = pm.region;
 }
@@ -1482,7 +1578,7 @@ k_dsmc(WsPtrs W, Pools<Real> P, int par, int part)
                 const Real u = sqrt(u2);
                 const Real E = pick<Real>(S.Ek, S.Ek_f) * u2;
                 // n_j dx sigma_j(E) from the species' node-major table
-                const XsPoint<Real> pt = xs_locate<Real>(W.tables[S.table_lo], lutE, E);
+                const XsPoint<Real> pt = xs_locate<Real>(S, lutE, E);
                 const Real *ra = GasTab<Real>::ptr(W) + S.gtab_off + (size_t)pt.k * S.gtab_ld;
                 const Real xa = ra[e.j], xb = ra[S.gtab_ld + e.j];
                 Real xs = pt.region == 2 ? xb : xa + pt.f * (xb - xa);
@@ -1737,7 +1833,7 @@ static size_t push_smem_bytes(int Nmax, int eedf_max, int fm_max, int nw, int qc
     b += sizeof(unsigned) * (eedf_max + fm_max);
     b += (size_t)nw * qcap;        // candidate energy bins
     b = (b + 15) & ~size_t(15);
-    if (cells) b += sizeof(unsigned) * (Nmax + 2);  // particles per cell
+    if (cells) b += sizeof(Real) * (Nmax + 2);  // particles per cell; FP64: and the third word
     return (b + 15) & ~size_t(15);
 }
 
@@ -1755,7 +1851,7 @@ using PushD0 = PushShape<256, 4, 2>;
 template <typename Real, typename SH>
 static cudaError_t push_shape_setup(LaunchCfg &L, int k)
 {
-    const size_t sm = push_smem_bytes<Real>(L.maxN, 0, 0, SH::nw, SH::qcap, sizeof(Real) == 4);
+    const size_t sm = push_smem_bytes<Real>(L.maxN, 0, 0, SH::nw, SH::qcap, true);
     const size_t smd = push_smem_bytes<Real>(L.maxN, L.eedf_max, L.fm_max, SH::nw, SH::qcap, false);
     cudaError_t e = cudaFuncSetAttribute(k_push<Real, false, SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
@@ -1793,7 +1889,7 @@ cudaError_t push_configure(bool fp64, LaunchCfg &L, int num_sms)
     L.push_blocks = num_sms * L.push_per_sm;
     L.push_smem = L.shape_smem[0];
     L.push_smem_diag = L.shape_smem_diag[0];
-    L.collide_blocks = num_sms * 8;
+    L.collide_blocks = num_sms * COLLIDE_PER_SM;
     return cudaSuccess;
 }
 

@@ -78,6 +78,27 @@ def test_fp64_fast_floor_is_floor():
         assert got == round(off * 2.0 ** 40), off
 
 
+def test_fp64_uniform_from_bits_is_exact():
+    """1 + (w + 1/2) 2^-32 written as a bit pattern, minus 1"""
+    rng = np.random.default_rng(6)
+    for w in [0, 1, 0xFFF, 0x1000, 0x7FFFFFFF, 0x80000000, 0xFFFFFFFF] + [int(x) for x in rng.integers(0, 2 ** 32, 300)]:
+        hi, lo = 0x3FF00000 | (w >> 12), ((w << 20) & 0xFFFFFFFF) | 0x80000
+        got = struct.unpack("<d", struct.pack("<Q", (hi << 32) | lo))[0] - 1.0
+        assert got == (w + 0.5) / 4294967296.0, w
+
+
+def test_fp64_charge_words_stay_exact():
+    """a cell's sum in 14, 13 and 13-bit words of 32 bits, at the most
+    particles a block adds before it flushes, each of the largest weight"""
+    most, one = 256 * 1024, 1 << 40
+    for w1 in (one, one - 1, 0x5555555555, 1):
+        words = (w1 & 0x3FFF, (w1 >> 14) & 0x1FFF, w1 >> 27)
+        assert all(most * x < 2 ** 32 for x in words), w1
+        assert sum((most * x) << b for x, b in zip(words, (0, 14, 27))) == most * w1
+    # 128 particles at once (a warp's sum, in two halves of 24 and 18 bits)
+    assert 32 * 4 * ((one - 1) & 0xFFFFFF) < 2 ** 32 and 32 * ((4 * one) >> 24) < 2 ** 32
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("sizes", [(1_400_001, 2, 33_333), (700_000, 0, 1, 1_023, 1_500_000)])
 def test_shares_and_tickets_give_the_same_state(sizes):
