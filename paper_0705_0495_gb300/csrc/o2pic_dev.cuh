@@ -231,7 +231,6 @@ struct Ctl {
     unsigned int ticket;          // dynamic chunk counter of the push
     int total_chunks;             // chunks in the current push
     int D;                        // discharges
-    unsigned int births_ticket;   // block order of the birth-append kernel
     unsigned int cand_n;          // collision candidates listed by the push this step
     unsigned int colscan_ticket;  // warp order of the sort's column scan
     unsigned int sort_epoch;      // sorts so far (tags the column scan's words)
@@ -260,11 +259,11 @@ struct WsPtrs {
     Disc *disc;
     Counts *cnt;              // [D*3]
     int *chunk_ds;            // [D*3 + 1] first chunk per (d,s) (prefix), device copy
-    int *tile_cnt;            // [max_chunks * SUBTILES * 3] births per sub-tile and product species
+    int *tile_cnt;            // [max_chunks * SUBTILES] birth records per sub-tile (zero outside a step)
     void *births;             // [max_chunks * SUBTILES * birth_cap] staged birth records
     int birth_cap;            // records per sub-tile
     unsigned long long *colscan_agg;  // column totals of the sort's row segments, tagged with the sort
-    unsigned long long *births_lb;  // [max_chunks * SUBTILES / BIRTHS_THREADS * 3] look-back words
+    int *birth_blk;           // [max_chunks / TILE_ALIGN + 1][3] births per append block and product species
     unsigned long long *acc_fix;  // [3 * total_nodes] fixed-point density accumulators
     double *acc_dbl;          // [3 * total_nodes] FP64 accumulators
     double *Efield;           // [total_nodes] E [V/m]

@@ -81,7 +81,7 @@ struct Bump {
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 struct Layout {
-    size_t colscan_agg, sort_whist, ctl, disc, cnt, phi_s2_sum, phi0_sum, D0_sum, gtab, gtabf, gpm, gpmf, tile_cnt, births, births_lb, sort_tot, warp_base, pair_first, vmax2, nubin, cand, pair_kills, pair_tab[3], acc, Efield, Ereal, phi, rho, dens, dens_sum, phi_sum, nsamp,
+    size_t colscan_agg, sort_whist, ctl, disc, cnt, phi_s2_sum, phi0_sum, D0_sum, gtab, gtabf, gpm, gpmf, tile_cnt, births, birth_blk, sort_tot, warp_base, pair_first, vmax2, nubin, cand, pair_kills, pair_tab[3], acc, Efield, Ereal, phi, rho, dens, dens_sum, phi_sum, nsamp,
         counters, eedf, iedf, fm, tables, lutE, lutS, lutEf, lutSf, sort_counts, cell_start,
         sort_live, pair_bcount, cell_disc, pair_births, sort_tab, ninit, vt;
     size_t cell[2], off[2], vx[2], vy[2], vz[2];
@@ -324,10 +324,10 @@ Layout make_layout(const pic_config *c, int D, const pic_xs_table *xs, int n_xs,
     L.ctl = B.take(sizeof(Ctl));
     L.disc = B.take(sizeof(Disc) * D);
     L.cnt = B.take(sizeof(Counts) * 3 * D);
-    L.tile_cnt = B.take(4ull * 3 * SUBTILES * mc);
+    L.tile_cnt = B.take(4ull * SUBTILES * mc);
     L.birth_cap = c[0].gas_scheme == 1 ? BIRTH_CAP_SEQ : BIRTH_CAP_W;
     L.births = B.take((size_t)mc * SUBTILES * L.birth_cap * (fp64 ? 40 : 24));
-    L.births_lb = B.take(8ull * 3 * (mc / TILE_ALIGN + 1));
+    L.birth_blk = B.take(4ull * 3 * (mc / TILE_ALIGN + 1));
     L.acc = B.take(8ull * 3 * tn);
     L.Efield = B.take(8ull * tn);
     L.Ereal = B.take(R * tn);
@@ -755,7 +755,7 @@ extern "C" pic_status pic_init(const pic_config *cfgs, int n_discharges, const p
     W.tile_cnt = reinterpret_cast<int *>(b + L.tile_cnt);
     W.births = b + L.births;
     W.birth_cap = L.birth_cap;
-    W.births_lb = reinterpret_cast<unsigned long long *>(b + L.births_lb);
+    W.birth_blk = reinterpret_cast<int *>(b + L.birth_blk);
     W.colscan_agg = reinterpret_cast<unsigned long long *>(b + L.colscan_agg);
     W.acc_fix = reinterpret_cast<unsigned long long *>(b + L.acc);
     W.acc_dbl = reinterpret_cast<double *>(b + L.acc);
@@ -1019,7 +1019,7 @@ static cudaError_t enqueue_step(pic_handle *h, long long n, int &nk, bool timed)
     e = launch_collide(h->fp64, h->W, h->pools(), par, h->L.collide_blocks, st);
     if (e) return e;
     ++nk;
-    e = launch_births(h->fp64, h->W, h->pools(), par, h->W.max_chunks / TILE_ALIGN + 1, st);
+    e = launch_births(h->fp64, h->W, h->pools(), st);
     if (e) return e;
     ++nk;
     const long long next = n + 1;
@@ -1055,7 +1055,7 @@ static cudaError_t enqueue_step(pic_handle *h, long long n, int &nk, bool timed)
         if ((e = time_open(h, timed, st))) return e;
         if ((e = launch_dsmc(h->fp64, h->W, h->pools(), par, 1, st))) return e;
         if ((e = time_close(h, timed, st, 2))) return e;
-        if ((e = launch_births(h->fp64, h->W, h->pools(), par, h->W.max_chunks / TILE_ALIGN + 1, st, 1))) return e;
+        if ((e = launch_births(h->fp64, h->W, h->pools(), st))) return e;
         if ((e = launch_sort(h->fp64, h->W, h->pools(), h->sort_tab, h->L, st))) return e;
         // the kill counts of (13), (14) refer to the cells before the sort
         if ((e = cudaMemsetAsync(h->W.pair_kills, 0, sizeof(int) * NSP * (size_t)h->W.total_cells, st))) return e;
@@ -1226,8 +1226,6 @@ extern "C" pic_status pic_set_step(pic_handle *h, long long step)
     if (!h || step < 0) return fail(h, PIC_EINVAL, "bad handle or step");
     unsigned long long v = (unsigned long long)step;
     CK(cudaMemcpyAsync(&h->W.ctl->step[step & 1], &v, 8, cudaMemcpyHostToDevice, h->stream));
-    // look-back words are tagged with the step; a step number can now repeat
-    CK(cudaMemsetAsync(h->W.births_lb, 0, 8ull * 3 * (h->W.max_chunks / TILE_ALIGN + 1), h->stream));
     CK(cudaStreamSynchronize(h->stream));
     h->step = step;
     return PIC_OK;

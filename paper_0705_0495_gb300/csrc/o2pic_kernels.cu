@@ -376,9 +376,9 @@ k_field(WsPtrs W, int par, int diag, int mode, int csize)
 // Tile table of the current counts: tiles of each discharge start at a
 // multiple of TILE_ALIGN, so that the birth-append blocks (BIRTHS_THREADS
 // sub-tiles) never span two, and those of each species at a multiple of
-// TILES_PER_TICKET, so that a push ticket never spans two; the birth counts
-// of the padding tiles after each species (never pushed) are cleared.  With
-// `advance` the next step's counter is set and the candidate list emptied.
+// TILES_PER_TICKET, so that a push ticket never spans two; the birth-append
+// blocks' counts are cleared.  With `advance` the next step's counter is set
+// and the candidate list emptied.
 // One thread per discharge and a block scan over them (one thread walking the
 // list took 0.25 us per entry: 50 us of every step of 64 discharges).
 __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bool advance)
@@ -427,7 +427,6 @@ __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bo
                 }
                 ctl->total_chunks = chunk;
                 ctl->ticket = 0u;
-                ctl->births_ticket = 0u;
                 if (advance) {
                     ctl->cand_n = 0u;
                     ctl->step[par ^ 1] = step + 1ull;
@@ -435,13 +434,7 @@ __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bo
             }
         }
     }
-    __syncthreads();
-    constexpr int PAD = B * SUBTILES;  // sub-tiles of a ticket: more than any padding
-    for (int k = tid; k < W.D * NSP * PAD; k += NT) {
-        const Counts &C = W.cnt[k / PAD];
-        const int t0 = C.chunk0 + C.nchunk, t1 = (t0 + B - 1) / B * B;
-        if (k % PAD < (t1 - t0) * SUBTILES) W.tile_cnt[((size_t)t0 * SUBTILES + k % PAD) * NSP] = 0;
-    }
+    for (int k = tid; k < (W.max_chunks / TILE_ALIGN + 1) * NSP; k += NT) W.birth_blk[k] = 0;
 }
 
 __global__ void __launch_bounds__(256) k_retile(WsPtrs W, int par)

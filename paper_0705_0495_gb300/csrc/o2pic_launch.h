@@ -81,10 +81,7 @@ cudaError_t launch_push(bool fp64, bool diag, const WsPtrs &W, const void *pools
 cudaError_t push_configure(bool fp64, LaunchCfg &L, int num_sms);
 // births of the push appended in parent order
 cudaError_t launch_collide(bool fp64, const WsPtrs &W, const void *pools, int par, int blocks, cudaStream_t st);
-// salt: 0 for the append after the collisions, 1 for the one after the
-// sequential gas scheme in the same step
-cudaError_t launch_births(bool fp64, const WsPtrs &W, const void *pools, int par, int max_blocks,
-                          cudaStream_t s, int salt = 0);
+cudaError_t launch_births(bool fp64, const WsPtrs &W, const void *pools, cudaStream_t s);
 // the sequential gas scheme, part 0 (channels below (13)) or 1 (above (14))
 constexpr int DSMC_THREADS = 256;
 cudaError_t launch_dsmc(bool fp64, const WsPtrs &W, const void *pools, int par, int part, cudaStream_t st);
