@@ -1405,6 +1405,85 @@ __device__ __forceinline__ void coulomb_pair_ab(Real va[3], Real vb[3], Real kn,
     }
 }
 
+#ifndef O2_INTER_CHAINS
+#define O2_INTER_CHAINS 128
+#endif
+constexpr int INTER_CHAINS = O2_INTER_CHAINS;  // most chains (B particles) run on prepared random numbers
+constexpr int INTER_TILE = 1024;               // collisions prepared at a time
+
+// The same collision with its random numbers prepared (xi, and sp, cp = sin,
+// cos of the azimuth).  Chains of these are what the inter-species pass waits
+// for, so FP32 takes the hardware's reciprocal and square root directly: they
+// equal the guarded functions of CoulMath for normal inputs, and any other
+// input (checked beside the chain) goes through those.
+template <typename Real>
+__device__ __forceinline__ void coulomb_dg(const Real g0, const Real g1, const Real g2, const Real u, const Real d,
+                                           const Real up2, const Real rp, const Real up, Real sp, Real cp, Real dg[3])
+{
+    using M = CoulMath<Real>;
+    Real sn, om;
+    if (fabs(d) <= Real(1)) {
+        const Real r = M::rcp(Real(1) + d * d);
+        sn = Real(2) * d * r;
+        om = Real(2) * d * d * r;
+    } else {
+        const Real e = M::rcp(d);
+        const Real r = M::rcp(Real(1) + e * e);
+        sn = Real(2) * e * r;
+        om = Real(2) * r;
+    }
+    if (up2 > Real(0)) {
+        const Real ex = g0 * rp, ey = g1 * rp;
+        const Real a = g2 * sn * cp, b = u * sn * sp;
+        dg[0] = ex * a - ey * b - g0 * om;
+        dg[1] = ey * a + ex * b - g1 * om;
+        dg[2] = -up * sn * cp - g2 * om;
+    } else {
+        dg[0] = u * sn * cp;
+        dg[1] = u * sn * sp;
+        dg[2] = -g2 * om;
+    }
+}
+__device__ __forceinline__ float rsqrt_hw(float x)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+template <typename Real>
+__device__ __forceinline__ void coulomb_pair_chain(Real va[3], Real vb[3], Real kn, Real fa, Real fb, Real xi, Real sp,
+                                                   Real cp)
+{
+    using M = CoulMath<Real>;
+    const Real g0 = va[0] - vb[0], g1 = va[1] - vb[1], g2 = va[2] - vb[2];
+    const Real u2 = g0 * g0 + g1 * g1 + g2 * g2;
+    if (!(u2 > Real(0))) return;
+    const Real up2 = g0 * g0 + g1 * g1;
+    Real dg[3];
+    bool plain = true;
+    if constexpr (sizeof(Real) == 4) {
+        const float u = u2 * rsqrt_hw(u2);
+        const float q = rsqrt_hw(u);
+        const float x = kn * (q * q * q * q * q * q);
+        const float d = x * rsqrt_hw(x) * xi;
+        const float up = up2 * rsqrt_hw(up2);
+        constexpr float LOW = 1.1754944e-38f, HIGH = 1e37f;  // normal, and far from overflow
+        plain = !(u2 >= LOW && u2 <= HIGH && x >= LOW && x <= HIGH && fabsf(d) <= HIGH && (up2 >= LOW || up2 == 0.0f));
+        if (!plain) coulomb_dg<float>(g0, g1, g2, u, d, up2, M::rcp(up), up, sp, cp, dg);
+    }
+    if (plain) {
+        const Real u = M::sqrt_(u2);
+        const Real d = M::sqrt_(kn * M::inv_u32(Real(0), u2, u)) * xi;
+        const Real up = M::sqrt_(up2);
+        coulomb_dg<Real>(g0, g1, g2, u, d, up2, M::rcp(up), up, sp, cp, dg);
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        va[q] += fa * dg[q];
+        vb[q] -= fb * dg[q];
+    }
+}
+
 // Inter-species Coulomb collisions of species pair `pair` in one cell per
 // block (Takizuka and Abe for unlike particles), after the intra-species
 // pass: the nA particles of the more numerous species (A) each collide once,
@@ -1415,14 +1494,21 @@ __device__ __forceinline__ void coulomb_pair_ab(Real va[3], Real vb[3], Real kn,
 // A pi_A(r), pi_A(r + nB), ... in that order, its velocity in registers; the
 // A particles are disjoint across threads.  A is staged in shared memory
 // when it has at most `cap` particles.
+//
+// What bounds it: the longest chain.  In the sheaths a handful of electrons
+// meet thousands of ions one after the other, while the collisions of all
+// other cells are done.  So with at most INTER_CHAINS chains the random
+// numbers, normals and azimuths, which do not depend on the chain, are
+// prepared by all threads, the next link's inputs are loaded ahead, and the
+// cells at both walls start first.
 template <typename Real>
-__global__ void __launch_bounds__(COUL_THREADS, 2)
+__global__ void __launch_bounds__(COUL_THREADS, sizeof(Real) == 4 ? 2 : 1)
 k_coulomb_inter(WsPtrs W, Pools<Real> P, int par, int pair, int cap)
 {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char coul_smem[];
     __shared__ unsigned prm[4];  // a, b of A's permutation, a, b of B's
-    const int gw = blockIdx.x;
+    const int gw = (blockIdx.x & 1) ? W.total_cells - 1 - (int)(blockIdx.x >> 1) : (int)(blockIdx.x >> 1);
     const int d = W.cell_disc[gw];
     const Disc &Dd = W.disc[d];
     const int N = Dd.N, c = gw - Dd.ccell_base;
@@ -1499,6 +1585,63 @@ k_coulomb_inter(WsPtrs W, Pools<Real> P, int par, int pair, int cap)
     const unsigned stepA = (unsigned)(((unsigned long long)aA * COUL_THREADS) % uA);
     const unsigned chainA = (unsigned)(((unsigned long long)aA * uB) % uA);
     Real m2b = Real(0);  // largest new speed^2 of this thread's B particles
+    if (nB <= INTER_CHAINS) {
+        // few, long chains: all threads prepare the random numbers of
+        // INTER_TILE collisions, then the chains run through them
+        Real *txi = reinterpret_cast<Real *>(coul_smem) + 3 * cap, *tsp = txi + INTER_TILE, *tcp = tsp + INTER_TILE;
+        const bool mine = t0 < uB;
+        Real vb[3] = {Real(0), Real(0), Real(0)};
+        if (mine) {
+            vb[0] = gbx[j];
+            vb[1] = gby[j];
+            vb[2] = gbz[j];
+        }
+        unsigned k = t0, i = i0;
+        for (unsigned k0 = 0; k0 < uA; k0 += INTER_TILE) {
+            const unsigned ke = min(k0 + (unsigned)INTER_TILE, uA);
+            for (unsigned q = t0; 2 * q < INTER_TILE && k0 + 2 * q < ke; q += COUL_THREADS) {
+                const uint4 w = coulomb_rng(seed, disc, sfield, step, c, 1u + (k0 >> 1) + q);
+                CoulMath<Real>::normal2(w.x, w.y, txi[2 * q], txi[2 * q + 1]);
+                CoulMath<Real>::sincos2pi(unif<Real>(w.z), &tsp[2 * q], &tcp[2 * q]);
+                CoulMath<Real>::sincos2pi(unif<Real>(w.w), &tsp[2 * q + 1], &tcp[2 * q + 1]);
+            }
+            __syncthreads();
+            if (mine && k < ke) {
+                // the next collision's inputs are loaded before the present one
+                Real va[3] = {ax[i], ay[i], az[i]};
+                Real xi = txi[k - k0], sp = tsp[k - k0], cp = tcp[k - k0];
+                for (;;) {
+                    const unsigned k2 = k + uB;
+                    unsigned i2 = i + chainA;
+                    if (i2 >= uA) i2 -= uA;
+                    const bool more = k2 < ke;
+                    const unsigned in = more ? i2 : i, kn2 = more ? k2 - k0 : 0u;
+                    const Real va2[3] = {ax[in], ay[in], az[in]};
+                    const Real xi2 = txi[kn2], sp2 = tsp[kn2], cp2 = tcp[kn2];
+                    coulomb_pair_chain<Real>(va, vb, kn, fa, fb, xi, sp, cp);
+                    ax[i] = va[0];
+                    ay[i] = va[1];
+                    az[i] = va[2];
+                    k = k2;
+                    i = i2;
+                    if (!more) break;
+                    va[0] = va2[0];
+                    va[1] = va2[1];
+                    va[2] = va2[2];
+                    xi = xi2;
+                    sp = sp2;
+                    cp = cp2;
+                }
+            }
+            __syncthreads();
+        }
+        if (mine) {
+            gbx[j] = vb[0];
+            gby[j] = vb[1];
+            gbz[j] = vb[2];
+            m2b = vb[0] * vb[0] + vb[1] * vb[1] + vb[2] * vb[2];
+        }
+    } else
     for (unsigned r = t0; r < uB; r += COUL_THREADS) {
         Real vb[3] = {gbx[j], gby[j], gbz[j]};
         unsigned i = i0;
@@ -1642,6 +1785,12 @@ __global__ void k_deposit_all(WsPtrs W, Pools<Real> P, int only_disc)
 
 // ------------------------------------------------------------ launchers
 
+// the inter-species pass: A's velocities and one tile of random numbers
+static size_t inter_smem_bytes(bool fp64)
+{
+    return coulomb_smem_bytes(fp64) + (size_t)INTER_TILE * 3 * (fp64 ? 8 : 4);
+}
+
 cudaError_t configure_kernels(bool fp64, LaunchCfg &L)
 {
     cudaError_t e;
@@ -1656,7 +1805,7 @@ cudaError_t configure_kernels(bool fp64, LaunchCfg &L)
                                  (int)coulomb_smem_bytes(true));
         if (e) return e;
         e = cudaFuncSetAttribute(k_coulomb_inter<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)coulomb_smem_bytes(true));
+                                 (int)inter_smem_bytes(true));
         if (e) return e;
     } else {
         e = cudaFuncSetAttribute(k_sort_count<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.sort_smem);
@@ -1667,7 +1816,7 @@ cudaError_t configure_kernels(bool fp64, LaunchCfg &L)
                                  (int)coulomb_smem_bytes(false));
         if (e) return e;
         e = cudaFuncSetAttribute(k_coulomb_inter<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)coulomb_smem_bytes(false));
+                                 (int)inter_smem_bytes(false));
         if (e) return e;
     }
     return cudaFuncSetAttribute(k_sort_cellscan, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1728,7 +1877,7 @@ cudaError_t launch_coulomb(bool fp64, const WsPtrs &W, const void *pools, int pa
 
 cudaError_t launch_coulomb_inter(bool fp64, const WsPtrs &W, const void *pools, int par, int pair, cudaStream_t st)
 {
-    const size_t smem = coulomb_smem_bytes(fp64);
+    const size_t smem = inter_smem_bytes(fp64);
     if (fp64)
         launch_k(k_coulomb_inter<double>, W.total_cells, COUL_THREADS, smem, st, W,
                  *static_cast<const Pools<double> *>(pools), par, pair, COUL_STAGE);
