@@ -1037,9 +1037,8 @@ static cudaError_t enqueue_step(pic_handle *h, long long n, int &nk, bool timed)
         if (e) return e;
         ++nk;
         if (q.coulomb_inter) {
-            for (int pr = 0; pr < 3; ++pr)
-                if ((e = launch_coulomb_inter(h->fp64, h->W, h->pools(), par, pr, st))) return e;
-            nk += 3;
+            if ((e = launch_coulomb_inter(h->fp64, h->W, h->pools(), par, st))) return e;
+            ++nk;
         }
         if ((e = time_close(h, timed, st, 1))) return e;
     }

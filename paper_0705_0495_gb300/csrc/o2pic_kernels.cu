@@ -1186,9 +1186,8 @@ __device__ __forceinline__ uint4 coulomb_rng(unsigned long long seed, int disc, 
 // Copy n values of each component, COUL_COPY elements per thread in flight.
 constexpr int COUL_COPY = 4;
 template <typename Real>
-__device__ __forceinline__ void coulomb_copy(Real *__restrict__ dx, Real *__restrict__ dy, Real *__restrict__ dz,
-                                             const Real *__restrict__ sx, const Real *__restrict__ sy,
-                                             const Real *__restrict__ sz, int n)
+__device__ __forceinline__ void coulomb_copy(Real *dx, Real *dy, Real *dz, const Real *sx, const Real *sy,
+                                             const Real *sz, int n)
 {
     for (int k0 = threadIdx.x; k0 < n; k0 += COUL_COPY * COUL_THREADS) {
         Real ax[COUL_COPY], ay[COUL_COPY], az[COUL_COPY];
@@ -1411,16 +1410,17 @@ __device__ __forceinline__ void coulomb_pair_ab(Real va[3], Real vb[3], Real kn,
 constexpr int INTER_CHAINS = O2_INTER_CHAINS;  // most chains (B particles) run on prepared random numbers
 constexpr int INTER_TILE = 1024;               // collisions prepared at a time
 
-// The same collision with its random numbers prepared (xi, and sp, cp = sin,
-// cos of the azimuth).  Chains of these are what the inter-species pass waits
-// for, so FP32 takes the hardware's reciprocal and square root directly: they
-// equal the guarded functions of CoulMath for normal inputs, and any other
-// input (checked beside the chain) goes through those.
+// The change of g of one collision, from its random numbers (xi, and sp, cp =
+// sin, cos of the azimuth): coulomb_pair_ab's arithmetic.
 template <typename Real>
-__device__ __forceinline__ void coulomb_dg(const Real g0, const Real g1, const Real g2, const Real u, const Real d,
-                                           const Real up2, const Real rp, const Real up, Real sp, Real cp, Real dg[3])
+__device__ __forceinline__ void coulomb_change(Real g0, Real g1, Real g2, Real kn, Real xi, Real sp, Real cp, Real dg[3])
 {
     using M = CoulMath<Real>;
+    dg[0] = dg[1] = dg[2] = Real(0);
+    const Real u2 = g0 * g0 + g1 * g1 + g2 * g2;
+    if (!(u2 > Real(0))) return;
+    const Real u = M::sqrt_(u2);
+    const Real d = M::sqrt_(kn * M::inv_u32(Real(0), u2, u)) * xi;
     Real sn, om;
     if (fabs(d) <= Real(1)) {
         const Real r = M::rcp(Real(1) + d * d);
@@ -1432,7 +1432,9 @@ __device__ __forceinline__ void coulomb_dg(const Real g0, const Real g1, const R
         sn = Real(2) * e * r;
         om = Real(2) * r;
     }
+    const Real up2 = g0 * g0 + g1 * g1;
     if (up2 > Real(0)) {
+        const Real up = M::sqrt_(up2), rp = M::rcp(up);
         const Real ex = g0 * rp, ey = g1 * rp;
         const Real a = g2 * sn * cp, b = u * sn * sp;
         dg[0] = ex * a - ey * b - g0 * om;
@@ -1444,49 +1446,79 @@ __device__ __forceinline__ void coulomb_dg(const Real g0, const Real g1, const R
         dg[2] = -g2 * om;
     }
 }
+__device__ __noinline__ float3 coulomb_change_any(float g0, float g1, float g2, float kn, float xi, float sp, float cp)
+{
+    float dg[3];
+    coulomb_change<float>(g0, g1, g2, kn, xi, sp, cp, dg);
+    return make_float3(dg[0], dg[1], dg[2]);
+}
 __device__ __forceinline__ float rsqrt_hw(float x)
 {
     float r;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-template <typename Real>
-__device__ __forceinline__ void coulomb_pair_chain(Real va[3], Real vb[3], Real kn, Real fa, Real fb, Real xi, Real sp,
-                                                   Real cp)
+__device__ __forceinline__ float rcp_hw(float x)
 {
-    using M = CoulMath<Real>;
-    const Real g0 = va[0] - vb[0], g1 = va[1] - vb[1], g2 = va[2] - vb[2];
-    const Real u2 = g0 * g0 + g1 * g1 + g2 * g2;
-    if (!(u2 > Real(0))) return;
-    const Real up2 = g0 * g0 + g1 * g1;
-    Real dg[3];
-    bool plain = true;
-    if constexpr (sizeof(Real) == 4) {
-        const float u = u2 * rsqrt_hw(u2);
-        const float q = rsqrt_hw(u);
-        const float x = kn * (q * q * q * q * q * q);
-        const float d = x * rsqrt_hw(x) * xi;
-        const float up = up2 * rsqrt_hw(up2);
-        constexpr float LOW = 1.1754944e-38f, HIGH = 1e37f;  // normal, and far from overflow
-        plain = !(u2 >= LOW && u2 <= HIGH && x >= LOW && x <= HIGH && fabsf(d) <= HIGH && (up2 >= LOW || up2 == 0.0f));
-        if (!plain) coulomb_dg<float>(g0, g1, g2, u, d, up2, M::rcp(up), up, sp, cp, dg);
-    }
-    if (plain) {
-        const Real u = M::sqrt_(u2);
-        const Real d = M::sqrt_(kn * M::inv_u32(Real(0), u2, u)) * xi;
-        const Real up = M::sqrt_(up2);
-        coulomb_dg<Real>(g0, g1, g2, u, d, up2, M::rcp(up), up, sp, cp, dg);
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+// One link of a chain: what the inter-species pass waits for.  The FP32 link
+// has no branch: the hardware's reciprocal and square root (equal to the
+// guarded functions of CoulMath for the inputs accepted here, every one of
+// them checked), the common small-angle form, and one check beside the chain
+// that sends any other case through coulomb_change.  From about 470 to 320
+// cycles a link (4e6 superparticles: one electron among 3900 ions, 970 -> 660
+// us).
+__device__ __forceinline__ void coulomb_link(float va[3], float vb[3], float kn, float fa, float fb, float xi, float sp,
+                                             float cp)
+{
+    const float g0 = va[0] - vb[0], g1 = va[1] - vb[1], g2 = va[2] - vb[2];
+    const float u2 = g0 * g0 + g1 * g1 + g2 * g2;
+    const float u = u2 * rsqrt_hw(u2);
+    const float q = rsqrt_hw(u);
+    const float x = kn * (q * q * q * q * q * q);
+    const float d = x * rsqrt_hw(x) * xi;
+    const float r = rcp_hw(1.0f + d * d);
+    const float sn = 2.0f * d * r, om = 2.0f * d * d * r;
+    const float up2 = g0 * g0 + g1 * g1;
+    const float up = up2 * rsqrt_hw(up2), rp = rcp_hw(up);
+    const float ex = g0 * rp, ey = g1 * rp;
+    const float a = g2 * sn * cp, b = u * sn * sp;
+    float dg[3];
+    dg[0] = ex * a - ey * b - g0 * om;
+    dg[1] = ey * a + ex * b - g1 * om;
+    dg[2] = -up * sn * cp - g2 * om;
+    constexpr float LOW = 1.1754944e-38f, HIGH = 1e37f;  // normal, and far from overflow
+    if (!(up2 >= LOW && u2 <= HIGH && x >= LOW && x <= HIGH && fabsf(d) <= 1.0f)) {
+        const float3 t = coulomb_change_any(g0, g1, g2, kn, xi, sp, cp);
+        dg[0] = t.x;
+        dg[1] = t.y;
+        dg[2] = t.z;
     }
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        va[q] += fa * dg[q];
-        vb[q] -= fb * dg[q];
+    for (int k = 0; k < 3; ++k) {
+        va[k] += fa * dg[k];
+        vb[k] -= fb * dg[k];
+    }
+}
+__device__ __forceinline__ void coulomb_link(double va[3], double vb[3], double kn, double fa, double fb, double xi,
+                                             double sp, double cp)
+{
+    double dg[3];
+    coulomb_change<double>(va[0] - vb[0], va[1] - vb[1], va[2] - vb[2], kn, xi, sp, cp, dg);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        va[k] += fa * dg[k];
+        vb[k] -= fb * dg[k];
     }
 }
 
-// Inter-species Coulomb collisions of species pair `pair` in one cell per
-// block (Takizuka and Abe for unlike particles), after the intra-species
-// pass: the nA particles of the more numerous species (A) each collide once,
+// Inter-species Coulomb collisions of one cell per block (Takizuka and Abe for
+// unlike particles), after the intra-species pass, the species pairs e-O-,
+// e-O2+, O- - O2+ in turn (cells do not meet, so one launch does all three and
+// a cell with long chains does not hold up the others' next pair): the nA particles of the more numerous species (A) each collide once,
 // those of the other (B) in turn; collision k joins A pi_A(k) with B
 // pi_B(k mod nB) (affine permutations from draw 0 of the cell's stream 5
 // with species field 3 + pair) with the random numbers of draw 1 + k/2.
@@ -1503,7 +1535,7 @@ __device__ __forceinline__ void coulomb_pair_chain(Real va[3], Real vb[3], Real 
 // cells at both walls start first.
 template <typename Real>
 __global__ void __launch_bounds__(COUL_THREADS, sizeof(Real) == 4 ? 2 : 1)
-k_coulomb_inter(WsPtrs W, Pools<Real> P, int par, int pair, int cap)
+k_coulomb_inter(WsPtrs W, Pools<Real> P, int par, int cap)
 {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char coul_smem[];
@@ -1512,165 +1544,168 @@ k_coulomb_inter(WsPtrs W, Pools<Real> P, int par, int pair, int cap)
     const int d = W.cell_disc[gw];
     const Disc &Dd = W.disc[d];
     const int N = Dd.N, c = gw - Dd.ccell_base;
-    const int s0 = pair == 2 ? 1 : 0, s1 = pair == 0 ? 1 : 2;
-    const int *cs = W.cell_start + Dd.cs_base;
-    const int q0 = cs[s0 * (N + 2) + c], n0 = cs[s0 * (N + 2) + c + 1] - q0;
-    const int q1 = cs[s1 * (N + 2) + c], n1 = cs[s1 * (N + 2) + c + 1] - q1;
-    if (n0 <= 0 || n1 <= 0) return;
-    const bool zeroA = n0 >= n1;
-    const int sA = zeroA ? s0 : s1, sB = zeroA ? s1 : s0;
-    const int nA = zeroA ? n0 : n1, nB = zeroA ? n1 : n0;
-    const int pA = zeroA ? q0 : q1, pB = zeroA ? q1 : q0;
-    if (nA >= (1 << 29)) {
-        if (threadIdx.x == 0) set_status(W.ctl, ST_BADSTATE);
-        return;
-    }
-    if (threadIdx.x == 0) atomicAdd(&W.counters[(size_t)d * C_NCOUNT + C_COUL], (unsigned long long)(nA + nB));
-    const unsigned long long step = W.ctl->step[par];
-    const unsigned long long seed = Dd.seed;
-    const int disc = Dd.discharge;
-    const int cur = W.ctl->cur;
-    const int sfield = 3 + pair;
-    if (threadIdx.x == 0) {
-        const uint4 w0 = coulomb_rng(seed, disc, sfield, step, c, 0u);
-        const unsigned w[4] = {w0.x, w0.y, w0.z, w0.w};
-        const unsigned nn[2] = {(unsigned)nA, (unsigned)nB};
-        for (int h = 0; h < 2; ++h) {
-            const unsigned un = nn[h];
-            unsigned a = 1u, b = 0u;
-            if (un >= 2u) {
-                a = 1u + w[2 * h] % (un - 1u);
-                for (;;) {
-                    unsigned x = a, y = un;
-                    while (y) {
-                        const unsigned t = x % y;
-                        x = y;
-                        y = t;
+    for (int pair = 0; pair < 3; ++pair) {
+        __syncthreads();  // the pair before is done with the shared memory and the velocities
+        const int s0 = pair == 2 ? 1 : 0, s1 = pair == 0 ? 1 : 2;
+        const int *cs = W.cell_start + Dd.cs_base;
+        const int q0 = cs[s0 * (N + 2) + c], n0 = cs[s0 * (N + 2) + c + 1] - q0;
+        const int q1 = cs[s1 * (N + 2) + c], n1 = cs[s1 * (N + 2) + c + 1] - q1;
+        if (n0 <= 0 || n1 <= 0) continue;
+        const bool zeroA = n0 >= n1;
+        const int sA = zeroA ? s0 : s1, sB = zeroA ? s1 : s0;
+        const int nA = zeroA ? n0 : n1, nB = zeroA ? n1 : n0;
+        const int pA = zeroA ? q0 : q1, pB = zeroA ? q1 : q0;
+        if (nA >= (1 << 29)) {
+            if (threadIdx.x == 0) set_status(W.ctl, ST_BADSTATE);
+            continue;
+        }
+        if (threadIdx.x == 0) atomicAdd(&W.counters[(size_t)d * C_NCOUNT + C_COUL], (unsigned long long)(nA + nB));
+        const unsigned long long step = W.ctl->step[par];
+        const unsigned long long seed = Dd.seed;
+        const int disc = Dd.discharge;
+        const int cur = W.ctl->cur;
+        const int sfield = 3 + pair;
+        if (threadIdx.x == 0) {
+            const uint4 w0 = coulomb_rng(seed, disc, sfield, step, c, 0u);
+            const unsigned w[4] = {w0.x, w0.y, w0.z, w0.w};
+            const unsigned nn[2] = {(unsigned)nA, (unsigned)nB};
+            for (int h = 0; h < 2; ++h) {
+                const unsigned un = nn[h];
+                unsigned a = 1u, b = 0u;
+                if (un >= 2u) {
+                    a = 1u + w[2 * h] % (un - 1u);
+                    for (;;) {
+                        unsigned x = a, y = un;
+                        while (y) {
+                            const unsigned t = x % y;
+                            x = y;
+                            y = t;
+                        }
+                        if (x == 1u) break;
+                        a = a % (un - 1u) + 1u;
                     }
-                    if (x == 1u) break;
-                    a = a % (un - 1u) + 1u;
+                    b = w[2 * h + 1] % un;
                 }
-                b = w[2 * h + 1] % un;
+                prm[2 * h] = a;
+                prm[2 * h + 1] = b;
             }
-            prm[2 * h] = a;
-            prm[2 * h + 1] = b;
         }
-    }
-    Real *gax = P.vx[cur] + Dd.pbase[sA] + pA, *gay = P.vy[cur] + Dd.pbase[sA] + pA,
-         *gaz = P.vz[cur] + Dd.pbase[sA] + pA;
-    Real *gbx = P.vx[cur] + Dd.pbase[sB] + pB, *gby = P.vy[cur] + Dd.pbase[sB] + pB,
-         *gbz = P.vz[cur] + Dd.pbase[sB] + pB;
-    const bool staged = nA <= cap;
-    Real *ax = gax, *ay = gay, *az = gaz;
-    if (staged) {
-        ax = reinterpret_cast<Real *>(coul_smem);
-        ay = ax + cap;
-        az = ay + cap;
-        coulomb_copy<Real>(ax, ay, az, gax, gay, gaz, nA);
-    }
-    __syncthreads();
-    const unsigned aA = prm[0], bA = prm[1], aB = prm[2], bB = prm[3];
-    const unsigned uA = (unsigned)nA, uB = (unsigned)nB;
-    const Real kn = pick<Real>(Dd.ci_k[pair], Dd.ci_k_f[pair]) * Real(nB);
-    const int ia = zeroA ? 0 : 1;  // index of A's share
-    const Real fa = pick<Real>(Dd.ci_frac[pair][ia], Dd.ci_frac_f[pair][ia]);
-    const Real fb = pick<Real>(Dd.ci_frac[pair][1 - ia], Dd.ci_frac_f[pair][1 - ia]);
-    // indices advanced by additions mod n: j(r) = (aB r + bB) mod nB steps by
-    // aB T mod nB, i(k) = (aA k + bA) mod nA by aA T mod nA over r and by
-    // aA nB mod nA along a chain
-    const unsigned t0 = threadIdx.x;
-    unsigned j = (unsigned)(((unsigned long long)aB * t0 + bB) % uB);
-    unsigned i0 = (unsigned)(((unsigned long long)aA * t0 + bA) % uA);
-    const unsigned stepB = (unsigned)(((unsigned long long)aB * COUL_THREADS) % uB);
-    const unsigned stepA = (unsigned)(((unsigned long long)aA * COUL_THREADS) % uA);
-    const unsigned chainA = (unsigned)(((unsigned long long)aA * uB) % uA);
-    Real m2b = Real(0);  // largest new speed^2 of this thread's B particles
-    if (nB <= INTER_CHAINS) {
-        // few, long chains: all threads prepare the random numbers of
-        // INTER_TILE collisions, then the chains run through them
-        Real *txi = reinterpret_cast<Real *>(coul_smem) + 3 * cap, *tsp = txi + INTER_TILE, *tcp = tsp + INTER_TILE;
-        const bool mine = t0 < uB;
-        Real vb[3] = {Real(0), Real(0), Real(0)};
-        if (mine) {
-            vb[0] = gbx[j];
-            vb[1] = gby[j];
-            vb[2] = gbz[j];
+        Real *gax = P.vx[cur] + Dd.pbase[sA] + pA, *gay = P.vy[cur] + Dd.pbase[sA] + pA,
+             *gaz = P.vz[cur] + Dd.pbase[sA] + pA;
+        Real *gbx = P.vx[cur] + Dd.pbase[sB] + pB, *gby = P.vy[cur] + Dd.pbase[sB] + pB,
+             *gbz = P.vz[cur] + Dd.pbase[sB] + pB;
+        const bool staged = nA <= cap;
+        Real *ax = gax, *ay = gay, *az = gaz;
+        if (staged) {
+            ax = reinterpret_cast<Real *>(coul_smem);
+            ay = ax + cap;
+            az = ay + cap;
+            coulomb_copy<Real>(ax, ay, az, gax, gay, gaz, nA);
         }
-        unsigned k = t0, i = i0;
-        for (unsigned k0 = 0; k0 < uA; k0 += INTER_TILE) {
-            const unsigned ke = min(k0 + (unsigned)INTER_TILE, uA);
-            for (unsigned q = t0; 2 * q < INTER_TILE && k0 + 2 * q < ke; q += COUL_THREADS) {
-                const uint4 w = coulomb_rng(seed, disc, sfield, step, c, 1u + (k0 >> 1) + q);
-                CoulMath<Real>::normal2(w.x, w.y, txi[2 * q], txi[2 * q + 1]);
-                CoulMath<Real>::sincos2pi(unif<Real>(w.z), &tsp[2 * q], &tcp[2 * q]);
-                CoulMath<Real>::sincos2pi(unif<Real>(w.w), &tsp[2 * q + 1], &tcp[2 * q + 1]);
+        __syncthreads();
+        const unsigned aA = prm[0], bA = prm[1], aB = prm[2], bB = prm[3];
+        const unsigned uA = (unsigned)nA, uB = (unsigned)nB;
+        const Real kn = pick<Real>(Dd.ci_k[pair], Dd.ci_k_f[pair]) * Real(nB);
+        const int ia = zeroA ? 0 : 1;  // index of A's share
+        const Real fa = pick<Real>(Dd.ci_frac[pair][ia], Dd.ci_frac_f[pair][ia]);
+        const Real fb = pick<Real>(Dd.ci_frac[pair][1 - ia], Dd.ci_frac_f[pair][1 - ia]);
+        // indices advanced by additions mod n: j(r) = (aB r + bB) mod nB steps by
+        // aB T mod nB, i(k) = (aA k + bA) mod nA by aA T mod nA over r and by
+        // aA nB mod nA along a chain
+        const unsigned t0 = threadIdx.x;
+        unsigned j = (unsigned)(((unsigned long long)aB * t0 + bB) % uB);
+        unsigned i0 = (unsigned)(((unsigned long long)aA * t0 + bA) % uA);
+        const unsigned stepB = (unsigned)(((unsigned long long)aB * COUL_THREADS) % uB);
+        const unsigned stepA = (unsigned)(((unsigned long long)aA * COUL_THREADS) % uA);
+        const unsigned chainA = (unsigned)(((unsigned long long)aA * uB) % uA);
+        Real m2b = Real(0);  // largest new speed^2 of this thread's B particles
+        if (nB <= INTER_CHAINS) {
+            // few, long chains: all threads prepare the random numbers of
+            // INTER_TILE collisions, then the chains run through them
+            Real *txi = reinterpret_cast<Real *>(coul_smem) + 3 * cap, *tsp = txi + INTER_TILE, *tcp = tsp + INTER_TILE;
+            const bool mine = t0 < uB;
+            Real vb[3] = {Real(0), Real(0), Real(0)};
+            if (mine) {
+                vb[0] = gbx[j];
+                vb[1] = gby[j];
+                vb[2] = gbz[j];
             }
-            __syncthreads();
-            if (mine && k < ke) {
-                // the next collision's inputs are loaded before the present one
+            unsigned k = t0, i = i0;
+            for (unsigned k0 = 0; k0 < uA; k0 += INTER_TILE) {
+                const unsigned ke = min(k0 + (unsigned)INTER_TILE, uA);
+                for (unsigned q = t0; 2 * q < INTER_TILE && k0 + 2 * q < ke; q += COUL_THREADS) {
+                    const uint4 w = coulomb_rng(seed, disc, sfield, step, c, 1u + (k0 >> 1) + q);
+                    CoulMath<Real>::normal2(w.x, w.y, txi[2 * q], txi[2 * q + 1]);
+                    CoulMath<Real>::sincos2pi(unif<Real>(w.z), &tsp[2 * q], &tcp[2 * q]);
+                    CoulMath<Real>::sincos2pi(unif<Real>(w.w), &tsp[2 * q + 1], &tcp[2 * q + 1]);
+                }
+                __syncthreads();
+                if (mine && k < ke) {
+                    // the next collision's inputs are loaded before the present one
+                    Real va[3] = {ax[i], ay[i], az[i]};
+                    Real xi = txi[k - k0], sp = tsp[k - k0], cp = tcp[k - k0];
+                    for (;;) {
+                        const unsigned k2 = k + uB;
+                        unsigned i2 = i + chainA;
+                        if (i2 >= uA) i2 -= uA;
+                        const bool more = k2 < ke;
+                        const unsigned in = more ? i2 : i, kn2 = more ? k2 - k0 : 0u;
+                        const Real va2[3] = {ax[in], ay[in], az[in]};
+                        const Real xi2 = txi[kn2], sp2 = tsp[kn2], cp2 = tcp[kn2];
+                        coulomb_link(va, vb, kn, fa, fb, xi, sp, cp);
+                        ax[i] = va[0];
+                        ay[i] = va[1];
+                        az[i] = va[2];
+                        k = k2;
+                        i = i2;
+                        if (!more) break;
+                        va[0] = va2[0];
+                        va[1] = va2[1];
+                        va[2] = va2[2];
+                        xi = xi2;
+                        sp = sp2;
+                        cp = cp2;
+                    }
+                }
+                __syncthreads();
+            }
+            if (mine) {
+                gbx[j] = vb[0];
+                gby[j] = vb[1];
+                gbz[j] = vb[2];
+                m2b = vb[0] * vb[0] + vb[1] * vb[1] + vb[2] * vb[2];
+            }
+        } else
+        for (unsigned r = t0; r < uB; r += COUL_THREADS) {
+            Real vb[3] = {gbx[j], gby[j], gbz[j]};
+            unsigned i = i0;
+            for (unsigned k = r; k < uA; k += uB) {
+                const uint4 w = coulomb_rng(seed, disc, sfield, step, c, 1u + (k >> 1));
+                Real n0r, n1r;
+                CoulMath<Real>::normal2(w.x, w.y, n0r, n1r);
                 Real va[3] = {ax[i], ay[i], az[i]};
-                Real xi = txi[k - k0], sp = tsp[k - k0], cp = tcp[k - k0];
-                for (;;) {
-                    const unsigned k2 = k + uB;
-                    unsigned i2 = i + chainA;
-                    if (i2 >= uA) i2 -= uA;
-                    const bool more = k2 < ke;
-                    const unsigned in = more ? i2 : i, kn2 = more ? k2 - k0 : 0u;
-                    const Real va2[3] = {ax[in], ay[in], az[in]};
-                    const Real xi2 = txi[kn2], sp2 = tsp[kn2], cp2 = tcp[kn2];
-                    coulomb_pair_chain<Real>(va, vb, kn, fa, fb, xi, sp, cp);
-                    ax[i] = va[0];
-                    ay[i] = va[1];
-                    az[i] = va[2];
-                    k = k2;
-                    i = i2;
-                    if (!more) break;
-                    va[0] = va2[0];
-                    va[1] = va2[1];
-                    va[2] = va2[2];
-                    xi = xi2;
-                    sp = sp2;
-                    cp = cp2;
-                }
+                coulomb_pair_ab<Real>(va, vb, kn, fa, fb, (k & 1u) ? n1r : n0r, (k & 1u) ? w.w : w.z);
+                ax[i] = va[0];
+                ay[i] = va[1];
+                az[i] = va[2];
+                i += chainA;
+                if (i >= uA) i -= uA;
             }
-            __syncthreads();
-        }
-        if (mine) {
             gbx[j] = vb[0];
             gby[j] = vb[1];
             gbz[j] = vb[2];
-            m2b = vb[0] * vb[0] + vb[1] * vb[1] + vb[2] * vb[2];
+            m2b = fmax(m2b, Real(vb[0] * vb[0] + vb[1] * vb[1] + vb[2] * vb[2]));
+            j += stepB;
+            if (j >= uB) j -= uB;
+            i0 += stepA;
+            if (i0 >= uA) i0 -= uA;
         }
-    } else
-    for (unsigned r = t0; r < uB; r += COUL_THREADS) {
-        Real vb[3] = {gbx[j], gby[j], gbz[j]};
-        unsigned i = i0;
-        for (unsigned k = r; k < uA; k += uB) {
-            const uint4 w = coulomb_rng(seed, disc, sfield, step, c, 1u + (k >> 1));
-            Real n0r, n1r;
-            CoulMath<Real>::normal2(w.x, w.y, n0r, n1r);
-            Real va[3] = {ax[i], ay[i], az[i]};
-            coulomb_pair_ab<Real>(va, vb, kn, fa, fb, (k & 1u) ? n1r : n0r, (k & 1u) ? w.w : w.z);
-            ax[i] = va[0];
-            ay[i] = va[1];
-            az[i] = va[2];
-            i += chainA;
-            if (i >= uA) i -= uA;
-        }
-        gbx[j] = vb[0];
-        gby[j] = vb[1];
-        gbz[j] = vb[2];
-        m2b = fmax(m2b, Real(vb[0] * vb[0] + vb[1] * vb[1] + vb[2] * vb[2]));
-        j += stepB;
-        if (j >= uB) j -= uB;
-        i0 += stepA;
-        if (i0 >= uA) i0 -= uA;
+        __syncthreads();
+        if (staged) coulomb_copy<Real>(gax, gay, gaz, ax, ay, az, nA);
+        // the new speeds raise both species' recorded largest speeds
+        vmax_raise(W.vmax2, d * NSP + sA, speed2_max<Real>(ax, ay, az, nA));
+        vmax_raise(W.vmax2, d * NSP + sB, (double)m2b);
     }
-    __syncthreads();
-    if (staged) coulomb_copy<Real>(gax, gay, gaz, ax, ay, az, nA);
-    // the new speeds raise both species' recorded largest speeds
-    vmax_raise(W.vmax2, d * NSP + sA, speed2_max<Real>(ax, ay, az, nA));
-    vmax_raise(W.vmax2, d * NSP + sB, (double)m2b);
 }
 
 // Births of (19) appended to the electron array of each discharge in cell
@@ -1875,15 +1910,15 @@ cudaError_t launch_coulomb(bool fp64, const WsPtrs &W, const void *pools, int pa
 }
 
 
-cudaError_t launch_coulomb_inter(bool fp64, const WsPtrs &W, const void *pools, int par, int pair, cudaStream_t st)
+cudaError_t launch_coulomb_inter(bool fp64, const WsPtrs &W, const void *pools, int par, cudaStream_t st)
 {
     const size_t smem = inter_smem_bytes(fp64);
     if (fp64)
         launch_k(k_coulomb_inter<double>, W.total_cells, COUL_THREADS, smem, st, W,
-                 *static_cast<const Pools<double> *>(pools), par, pair, COUL_STAGE);
+                 *static_cast<const Pools<double> *>(pools), par, COUL_STAGE);
     else
         launch_k(k_coulomb_inter<float>, W.total_cells, COUL_THREADS, smem, st, W,
-                 *static_cast<const Pools<float> *>(pools), par, pair, COUL_STAGE);
+                 *static_cast<const Pools<float> *>(pools), par, COUL_STAGE);
     return cudaGetLastError();
 }
 
