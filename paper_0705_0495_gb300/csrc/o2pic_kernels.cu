@@ -1185,15 +1185,16 @@ __device__ __forceinline__ uint4 coulomb_rng(unsigned long long seed, int disc, 
 
 // Copy n values of each component, COUL_COPY elements per thread in flight.
 constexpr int COUL_COPY = 4;
-template <typename Real>
+// (T threads, this one number t)
+template <typename Real, int T>
 __device__ __forceinline__ void coulomb_copy(Real *dx, Real *dy, Real *dz, const Real *sx, const Real *sy,
-                                             const Real *sz, int n)
+                                             const Real *sz, int n, int t)
 {
-    for (int k0 = threadIdx.x; k0 < n; k0 += COUL_COPY * COUL_THREADS) {
+    for (int k0 = t; k0 < n; k0 += COUL_COPY * T) {
         Real ax[COUL_COPY], ay[COUL_COPY], az[COUL_COPY];
 #pragma unroll
         for (int q = 0; q < COUL_COPY; ++q) {
-            const int k = k0 + q * COUL_THREADS;
+            const int k = k0 + q * T;
             if (k < n) {
                 ax[q] = sx[k];
                 ay[q] = sy[k];
@@ -1202,7 +1203,7 @@ __device__ __forceinline__ void coulomb_copy(Real *dx, Real *dy, Real *dz, const
         }
 #pragma unroll
         for (int q = 0; q < COUL_COPY; ++q) {
-            const int k = k0 + q * COUL_THREADS;
+            const int k = k0 + q * T;
             if (k < n) {
                 dx[k] = ax[q];
                 dy[k] = ay[q];
@@ -1212,12 +1213,12 @@ __device__ __forceinline__ void coulomb_copy(Real *dx, Real *dy, Real *dz, const
     }
 }
 
-// largest speed^2 among n velocities (a block-strided share per thread)
-template <typename Real>
-__device__ __forceinline__ double speed2_max(const Real *x, const Real *y, const Real *z, int n)
+// largest speed^2 among n velocities (a strided share per thread)
+template <typename Real, int T>
+__device__ __forceinline__ double speed2_max(const Real *x, const Real *y, const Real *z, int n, int t)
 {
     Real m = Real(0);
-    for (int k = threadIdx.x; k < n; k += blockDim.x)
+    for (int k = t; k < n; k += T)
         m = fmax(m, Real(x[k] * x[k] + y[k] * y[k] + z[k] * z[k]));
     return (double)m;
 }
@@ -1240,19 +1241,18 @@ __device__ __forceinline__ void coulomb_one(Real *vx, Real *vy, Real *vz, int i,
 // q = t, t + T, ..., which share one draw: pi(4q) = (b + q (4a mod n)) mod n,
 // advanced by T (4a mod n) mod n per iteration; pi(4q+2) = pi(4q) + 2a mod
 // n and pi(k+1) = pi(k) + a mod n.  prm holds a, b, 2a mod n and 4a mod n.
-template <typename Real>
+template <typename Real, int T>
 __device__ __forceinline__ void coulomb_cell_pairs(Real *vx, Real *vy, Real *vz, unsigned un,
                                                    const unsigned *prm, Real kn, unsigned long long seed,
-                                                   int disc, int s, unsigned long long step, int c)
+                                                   int disc, int s, unsigned long long step, int c, unsigned t)
 {
     using M = CoulMath<Real>;
     const unsigned a = prm[0], b = prm[1], a2 = prm[2], a4 = prm[3];
     const unsigned pairs = (un & 1u) ? (un - 3u) / 2u : un / 2u;
-    const unsigned t = threadIdx.x;
     unsigned x = un <= (1u << 22) ? (b + (t * a4) % un) % un
                                   : (unsigned)(((unsigned long long)t * a4 + b) % un);
-    const unsigned stepA = (unsigned)(((unsigned long long)COUL_THREADS * a4) % un);
-    for (unsigned q = t; 2u * q < pairs; q += COUL_THREADS) {
+    const unsigned stepA = (unsigned)(((unsigned long long)T * a4) % un);
+    for (unsigned q = t; 2u * q < pairs; q += T) {
         const uint4 w = coulomb_rng(seed, disc, s, step, c, 1u + q);
         Real n0, n1;
         M::normal2(w.x, w.y, n0, n1);
@@ -1280,52 +1280,46 @@ __device__ __forceinline__ void coulomb_cell_pairs(Real *vx, Real *vy, Real *vz,
     }
 }
 
-// Coulomb pass of one species in one cell per block, right after the sort
-// (every slot of the cell is live).  Blocks run the O2+ cells first, then
-// O-, then electrons (the largest cells first).  The n particles are paired
-// by the affine permutation pi(k) = (a k + b) mod n, a coprime to n, from
-// draw 0 of the cell's stream 5; collision m is (pi(2m), pi(2m+1)) with the
-// random numbers of draw 1 + m/2 (two collisions per draw); for odd n thread
-// 0 then runs the triangle of the last three, (A, B), (B, C), (C, A), with
-// half the time each.  The pairs are disjoint, so no ordering is needed
-// between threads.  A cell of at most `cap` particles is staged in shared
-// memory (coalesced copies in and out); a larger one is worked on in place.
-template <typename Real>
-__global__ void __launch_bounds__(COUL_THREADS, 2)
-k_coulomb(WsPtrs W, Pools<Real> P, int par, int cap)
+// Coulomb collisions of one species in one cell by T threads (a block or a
+// warp).  The n particles are paired by the affine permutation pi(k) = (a k +
+// b) mod n, a coprime to n, from draw 0 of the cell's stream 5; collision m is
+// (pi(2m), pi(2m+1)) with the random numbers of draw 1 + m/2 (two collisions
+// per draw); for odd n thread 0 then runs the triangle of the last three, (A,
+// B), (B, C), (C, A), with half the time each.  The pairs are disjoint, so no
+// ordering is needed between threads.  A cell of at most `cap` particles is
+// staged in shared memory sh (coalesced copies in and out); a larger one is
+// worked on in place.  prm: four shared words of these threads.
+template <typename Real, int T>
+__device__ __forceinline__ void coulomb_cell(const WsPtrs &W, const Pools<Real> &P, int par, int gw, int s, int p0, int n,
+                                             int t, Real *sh, int cap, unsigned *prm)
 {
-    pdl_wait();
-    extern __shared__ __align__(16) unsigned char coul_smem[];
-    const int gw = blockIdx.x % W.total_cells, s = NSP - 1 - (int)(blockIdx.x / W.total_cells);
+    auto sync = []() {
+        if constexpr (T == 32) __syncwarp(); else __syncthreads();
+    };
     const int d = W.cell_disc[gw];
     const Disc &Dd = W.disc[d];
-    const int N = Dd.N, c = gw - Dd.ccell_base;
-    const int *cs = W.cell_start + Dd.cs_base;
-    const int p0 = cs[s * (N + 2) + c], p1 = cs[s * (N + 2) + c + 1];
-    const int n = p1 - p0;
-    if (n < 2) return;
+    const int c = gw - Dd.ccell_base;
     if (n >= (1 << 29)) {
-        if (threadIdx.x == 0) set_status(W.ctl, ST_BADSTATE);
+        if (t == 0) set_status(W.ctl, ST_BADSTATE);
         return;
     }
-    if (threadIdx.x == 0) atomicAdd(&W.counters[(size_t)d * C_NCOUNT + C_COUL], (unsigned long long)n);
+    if (t == 0) atomicAdd(&W.counters[(size_t)d * C_NCOUNT + C_COUL], (unsigned long long)n);
     const unsigned long long step = W.ctl->step[par];
     const unsigned long long seed = Dd.seed;
     const int disc = Dd.discharge;
-    const int cur = W.ctl->cur;
-    const int base = Dd.pbase[s] + p0;
-    Real *gx = P.vx[cur] + base, *gy = P.vy[cur] + base, *gz = P.vz[cur] + base;
+    const unsigned b0 = W.ctl->cur ? P.stride : 0u;
+    const size_t base = (size_t)b0 + Dd.pbase[s] + p0;
+    Real *gx = P.vx[0] + base, *gy = P.vy[0] + base, *gz = P.vz[0] + base;
     const unsigned un = (unsigned)n;
-    __shared__ unsigned prm[4];  // a, b, 2a mod n, 4a mod n of the cell's permutation
-    if (threadIdx.x == 0) {
+    if (t == 0) {  // a, b, 2a mod n, 4a mod n of the cell's permutation
         const uint4 w0 = coulomb_rng(seed, disc, s, step, c, 0u);
         unsigned a = 1u + w0.x % (un - 1u);
         for (;;) {  // a -> a mod (n-1) + 1 until coprime; a = 1 always is
             unsigned x = a, y = un;
             while (y) {
-                const unsigned t = x % y;
+                const unsigned r = x % y;
                 x = y;
-                y = t;
+                y = r;
             }
             if (x == 1u) break;
             a = a % (un - 1u) + 1u;
@@ -1341,20 +1335,72 @@ k_coulomb(WsPtrs W, Pools<Real> P, int par, int cap)
     // P in a particle-target pass of the same step
     double m2;
     if (n <= cap) {
-        Real *sx = reinterpret_cast<Real *>(coul_smem), *sy = sx + cap, *sz = sy + cap;
-        coulomb_copy<Real>(sx, sy, sz, gx, gy, gz, n);
-        __syncthreads();
-        coulomb_cell_pairs<Real>(sx, sy, sz, un, prm, kn, seed, disc, s, step, c);
-        __syncthreads();
-        coulomb_copy<Real>(gx, gy, gz, sx, sy, sz, n);
-        m2 = speed2_max<Real>(sx, sy, sz, n);
+        Real *sx = sh, *sy = sx + cap, *sz = sy + cap;
+        coulomb_copy<Real, T>(sx, sy, sz, gx, gy, gz, n, t);
+        sync();
+        coulomb_cell_pairs<Real, T>(sx, sy, sz, un, prm, kn, seed, disc, s, step, c, (unsigned)t);
+        sync();
+        coulomb_copy<Real, T>(gx, gy, gz, sx, sy, sz, n, t);
+        m2 = speed2_max<Real, T>(sx, sy, sz, n, t);
     } else {
-        __syncthreads();
-        coulomb_cell_pairs<Real>(gx, gy, gz, un, prm, kn, seed, disc, s, step, c);
-        __syncthreads();
-        m2 = speed2_max<Real>(gx, gy, gz, n);
+        sync();
+        coulomb_cell_pairs<Real, T>(gx, gy, gz, un, prm, kn, seed, disc, s, step, c, (unsigned)t);
+        sync();
+        m2 = speed2_max<Real, T>(gx, gy, gz, n, t);
     }
     vmax_raise(W.vmax2, d * NSP + s, m2);
+}
+
+// Coulomb pass of every (species, cell), right after the sort (every slot of a
+// cell is live), O2+ cells first, then O-, then electrons (the largest cells
+// first).  GROUP = false: a block per cell.  GROUP = true: a block takes
+// COUL_GROUP cells, a warp each those of at most COUL_WARP particles, and then
+// the larger ones with all its warps.  What bounds small cells is latency (the
+// permutation's greatest common divisor, the copies, a few collisions per
+// thread): 2688 cells of about 150 particles took 56 us with a block each, in
+// nine waves, and 11.7 us so (cells of 2000 to 4000 particles
+// took 54 us with a block each and 5% of the whole run more in groups).  Both forms handle every size; the host
+// picks the groups when the capacity is at most COUL_GROUP_CAP slots per cell
+// (larger cells fill a block's warps, and a block per cell balances better).
+constexpr int COUL_GROUP = COUL_THREADS / 32;
+constexpr int COUL_WARP = COUL_STAGE / COUL_GROUP;  // staged particles per warp
+template <typename Real, bool GROUP>
+__global__ void __launch_bounds__(COUL_THREADS, sizeof(Real) == 4 ? 2 : 1)
+k_coulomb(WsPtrs W, Pools<Real> P, int par)
+{
+    pdl_wait();
+    extern __shared__ __align__(16) unsigned char coul_smem[];
+    __shared__ unsigned prm[COUL_GROUP][4];
+    Real *sh = reinterpret_cast<Real *>(coul_smem);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto place = [&](int idx, int &gw, int &s, int &p0) {  // returns the cell's particles
+        gw = idx % W.total_cells;
+        s = NSP - 1 - idx / W.total_cells;
+        const Disc &Dd = W.disc[W.cell_disc[gw]];
+        const int *cs = W.cell_start + Dd.cs_base + s * (Dd.N + 2) + gw - Dd.ccell_base;
+        p0 = cs[0];
+        return cs[1] - cs[0];
+    };
+    int gw, s, p0;
+    if constexpr (!GROUP) {
+        const int n = place(blockIdx.x, gw, s, p0);
+        if (n >= 2) coulomb_cell<Real, COUL_THREADS>(W, P, par, gw, s, p0, n, threadIdx.x, sh, COUL_STAGE, prm[0]);
+    } else {
+        __shared__ int s_n[COUL_GROUP];
+        const int first = blockIdx.x * COUL_GROUP, end = NSP * W.total_cells;
+        int n = 0;
+        if (first + warp < end) n = place(first + warp, gw, s, p0);
+        if (lane == 0) s_n[warp] = n;
+        if (n >= 2 && n <= COUL_WARP)
+            coulomb_cell<Real, 32>(W, P, par, gw, s, p0, n, lane, sh + (size_t)warp * 3 * COUL_WARP, COUL_WARP, prm[warp]);
+        __syncthreads();
+        for (int q = 0; q < COUL_GROUP; ++q) {
+            if (s_n[q] <= COUL_WARP) continue;
+            n = place(first + q, gw, s, p0);
+            coulomb_cell<Real, COUL_THREADS>(W, P, par, gw, s, p0, n, threadIdx.x, sh, COUL_STAGE, prm[0]);
+            __syncthreads();
+        }
+    }
 }
 
 // One Coulomb collision between particles a (velocity va) and b (vb) of
@@ -1600,7 +1646,7 @@ k_coulomb_inter(WsPtrs W, Pools<Real> P, int par, int cap)
             ax = reinterpret_cast<Real *>(coul_smem);
             ay = ax + cap;
             az = ay + cap;
-            coulomb_copy<Real>(ax, ay, az, gax, gay, gaz, nA);
+            coulomb_copy<Real, COUL_THREADS>(ax, ay, az, gax, gay, gaz, nA, threadIdx.x);
         }
         __syncthreads();
         const unsigned aA = prm[0], bA = prm[1], aB = prm[2], bB = prm[3];
@@ -1701,9 +1747,9 @@ k_coulomb_inter(WsPtrs W, Pools<Real> P, int par, int cap)
             if (i0 >= uA) i0 -= uA;
         }
         __syncthreads();
-        if (staged) coulomb_copy<Real>(gax, gay, gaz, ax, ay, az, nA);
+        if (staged) coulomb_copy<Real, COUL_THREADS>(gax, gay, gaz, ax, ay, az, nA, threadIdx.x);
         // the new speeds raise both species' recorded largest speeds
-        vmax_raise(W.vmax2, d * NSP + sA, speed2_max<Real>(ax, ay, az, nA));
+        vmax_raise(W.vmax2, d * NSP + sA, speed2_max<Real, COUL_THREADS>(ax, ay, az, nA, threadIdx.x));
         vmax_raise(W.vmax2, d * NSP + sB, (double)m2b);
     }
 }
@@ -1836,7 +1882,10 @@ cudaError_t configure_kernels(bool fp64, LaunchCfg &L)
         if (e) return e;
         e = cudaFuncSetAttribute(k_sort_scatter<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.scatter_smem);
         if (e) return e;
-        e = cudaFuncSetAttribute(k_coulomb<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(k_coulomb<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)coulomb_smem_bytes(true));
+        if (e) return e;
+        e = cudaFuncSetAttribute(k_coulomb<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)coulomb_smem_bytes(true));
         if (e) return e;
         e = cudaFuncSetAttribute(k_coulomb_inter<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1847,7 +1896,10 @@ cudaError_t configure_kernels(bool fp64, LaunchCfg &L)
         if (e) return e;
         e = cudaFuncSetAttribute(k_sort_scatter<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.scatter_smem);
         if (e) return e;
-        e = cudaFuncSetAttribute(k_coulomb<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(k_coulomb<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)coulomb_smem_bytes(false));
+        if (e) return e;
+        e = cudaFuncSetAttribute(k_coulomb<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)coulomb_smem_bytes(false));
         if (e) return e;
         e = cudaFuncSetAttribute(k_coulomb_inter<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1896,19 +1948,25 @@ cudaError_t launch_sort(bool fp64, const WsPtrs &W, const void *pools, const int
 
 size_t coulomb_smem_bytes(bool fp64) { return (size_t)COUL_STAGE * 3 * (fp64 ? 8 : 4); }
 
-cudaError_t launch_coulomb(bool fp64, const WsPtrs &W, const void *pools, int par, cudaStream_t st)
+template <typename Real>
+static void launch_coulomb_real(const WsPtrs &W, const Pools<Real> &P, int par, size_t smem, cudaStream_t st)
 {
-    const int grid = W.total_cells * NSP;
-    const size_t smem = coulomb_smem_bytes(fp64);
-    if (fp64)
-        launch_k(k_coulomb<double>, grid, COUL_THREADS, smem, st, W, *static_cast<const Pools<double> *>(pools),
-                 par, COUL_STAGE);
+    const int cells = W.total_cells * NSP;
+    if ((long long)P.stride <= (long long)COUL_GROUP_CAP * cells)
+        launch_k(k_coulomb<Real, true>, (cells + COUL_GROUP - 1) / COUL_GROUP, COUL_THREADS, smem, st, W, P, par);
     else
-        launch_k(k_coulomb<float>, grid, COUL_THREADS, smem, st, W, *static_cast<const Pools<float> *>(pools),
-                 par, COUL_STAGE);
-    return cudaGetLastError();
+        launch_k(k_coulomb<Real, false>, cells, COUL_THREADS, smem, st, W, P, par);
 }
 
+cudaError_t launch_coulomb(bool fp64, const WsPtrs &W, const void *pools, int par, cudaStream_t st)
+{
+    const size_t smem = coulomb_smem_bytes(fp64);
+    if (fp64)
+        launch_coulomb_real<double>(W, *static_cast<const Pools<double> *>(pools), par, smem, st);
+    else
+        launch_coulomb_real<float>(W, *static_cast<const Pools<float> *>(pools), par, smem, st);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_coulomb_inter(bool fp64, const WsPtrs &W, const void *pools, int par, cudaStream_t st)
 {

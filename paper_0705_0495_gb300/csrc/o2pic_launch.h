@@ -96,8 +96,9 @@ cudaError_t launch_field(bool fp64, bool diag, int mode, const WsPtrs &W, int pa
 
 cudaError_t launch_sort(bool fp64, const WsPtrs &W, const void *pools,
                         const int *sort_block_ds, const LaunchCfg &L, cudaStream_t s);
-// Coulomb pass: a block per (cell, species) of COUL_THREADS threads; cells of
-// at most COUL_STAGE particles are staged in shared memory
+// Coulomb pass: blocks of COUL_THREADS threads, one per (cell, species) or, up to
+// COUL_GROUP_CAP slots per cell, one per group of cells; cells of at most
+// COUL_STAGE particles are staged in shared memory
 #ifndef O2_COUL_THREADS
 #define O2_COUL_THREADS 384
 #endif
@@ -106,6 +107,10 @@ cudaError_t launch_sort(bool fp64, const WsPtrs &W, const void *pools,
 #endif
 constexpr int COUL_THREADS = O2_COUL_THREADS;
 constexpr int COUL_STAGE = O2_COUL_STAGE;
+#ifndef O2_COUL_GROUP_CAP
+#define O2_COUL_GROUP_CAP 4096
+#endif
+constexpr int COUL_GROUP_CAP = O2_COUL_GROUP_CAP;
 size_t coulomb_smem_bytes(bool fp64);
 cudaError_t launch_coulomb(bool fp64, const WsPtrs &W, const void *pools, int par, cudaStream_t st);
 // inter-species Coulomb collisions (e-O-, e-O2+, O- - O2+ in turn)
