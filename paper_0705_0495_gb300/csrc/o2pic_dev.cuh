@@ -293,14 +293,12 @@ struct WsPtrs {
     int *sort_tot;            // [sum over d of 3*(N+2)] slots per bucket
     int *pair_bcount;         // [total cells] births of (19) per cell
     int *cell_disc;           // [total cells] discharge of each global cell
-    int *pair_first;          // [total cells] first flagged projectile of the current reaction
     unsigned long long *vmax2;// [D * 3] largest speed^2 (cells/step, double bits): at the last
                               // sort, raised by the velocity changes since (Coulomb pass, first
                               // part of the sequential gas scheme); the particle-target pass's cap
     struct NuBin *nubin;      // [D * NUBIN_MAX] electron collision-frequency bounds per energy bin
     int2 *cand;               // [cand_cap] collision candidates: (slot, ds << 8 | energy bin)
     int cand_cap;
-    int *pair_kills;          // [total cells * 3] particles killed per species in this pass
     void *pair_births;        // [total cells * PAIR_BIRTH_CAP] records
     int total_nodes;
     int total_cells;

@@ -81,7 +81,7 @@ struct Bump {
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 struct Layout {
-    size_t colscan_agg, sort_whist, ctl, disc, cnt, phi_s2_sum, phi0_sum, D0_sum, gtab, gtabf, gpm, gpmf, tile_cnt, births, birth_blk, sort_tot, warp_base, pair_first, vmax2, nubin, cand, pair_kills, pair_tab[3], acc, Efield, Ereal, phi, rho, dens, dens_sum, phi_sum, nsamp,
+    size_t colscan_agg, sort_whist, ctl, disc, cnt, phi_s2_sum, phi0_sum, D0_sum, gtab, gtabf, gpm, gpmf, tile_cnt, births, birth_blk, sort_tot, warp_base, vmax2, nubin, cand, acc, Efield, Ereal, phi, rho, dens, dens_sum, phi_sum, nsamp,
         counters, eedf, iedf, fm, tables, lutE, lutS, lutEf, lutSf, sort_counts, cell_start,
         sort_live, pair_bcount, cell_disc, pair_births, sort_tab, ninit, vt;
     size_t cell[2], off[2], vx[2], vy[2], vz[2];
@@ -362,19 +362,12 @@ Layout make_layout(const pic_config *c, int D, const pic_xs_table *xs, int n_xs,
     L.colscan_agg = B.take(8ull * 32 * (size_t)std::max(1LL, L.colscan_units));
     L.pair_bcount = B.take(4ull * tc);
     L.cell_disc = B.take(4ull * tc);
-    L.pair_first = B.take(4ull * tc);
     L.vmax2 = B.take(8ull * 3 * D);
     L.nubin = B.take(sizeof(NuBin) * NUBIN_MAX * (size_t)D);
     // collision candidates of one step: a quarter of all slots (a candidate
     // probability up to 1/4 on average); more is reported as PIC_ECAPACITY
     L.cand_cap = (int)std::min<long long>((long long)cap / 4 + 65536, (1LL << 31) - 1);
     L.cand = B.take(8ull * (size_t)L.cand_cap);
-    L.pair_kills = B.take(4ull * 3 * tc);
-    for (int s = 0; s < 3; ++s) {
-        long long tiles = 0;
-        for (int d = 0; d < D; ++d) tiles += (c[d].capacity[s] + 255) / 256;
-        L.pair_tab[s] = B.take(8ull * std::max(1LL, tiles));
-    }
     L.pair_births = B.take((size_t)tc * PAIR_BIRTH_CAP * (8 + 4 * 8));
     L.sort_tab = B.take(8ull * sb);
     L.ninit = B.take(8ull * 3 * D);
@@ -791,12 +784,10 @@ extern "C" pic_status pic_init(const pic_config *cfgs, int n_discharges, const p
     W.sort_tot = reinterpret_cast<int *>(b + L.sort_tot);
     W.pair_bcount = reinterpret_cast<int *>(b + L.pair_bcount);
     W.cell_disc = reinterpret_cast<int *>(b + L.cell_disc);
-    W.pair_first = reinterpret_cast<int *>(b + L.pair_first);
     W.vmax2 = reinterpret_cast<unsigned long long *>(b + L.vmax2);
     W.nubin = reinterpret_cast<NuBin *>(b + L.nubin);
     W.cand = reinterpret_cast<int2 *>(b + L.cand);
     W.cand_cap = L.cand_cap;
-    W.pair_kills = reinterpret_cast<int *>(b + L.pair_kills);
     W.pair_births = b + L.pair_births;
     W.total_nodes = L.total_nodes;
     W.total_cells = L.total_cells;
@@ -956,19 +947,6 @@ extern "C" pic_status pic_init(const pic_config *cfgs, int n_discharges, const p
     CK(cudaMemcpyAsync(h->sort_tab, stab.data(), 4 * stab.size(), cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(W.cell_disc, cdisc.data(), 4 * cdisc.size(), cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(b + L.warp_base, wbase.data(), 4 * wbase.size(), cudaMemcpyHostToDevice, st));
-    CK(cudaMemsetAsync(W.pair_first, 0x7F, 4ull * L.total_cells, st));
-    for (int s = 0; s < 3; ++s) {
-        std::vector<int> pt;
-        for (int d = 0; d < n_discharges; ++d)
-            for (long long t = 0; t < (h->cfg[d].capacity[s] + 255) / 256; ++t) {
-                pt.push_back(d);
-                pt.push_back((int)t);
-            }
-        h->L.pair_blocks_sp[s] = (int)(pt.size() / 2);
-        h->L.pair_tab_sp[s] = reinterpret_cast<const int *>(b + L.pair_tab[s]);
-        if (!pt.empty())
-            CK(cudaMemcpyAsync(b + L.pair_tab[s], pt.data(), 4 * pt.size(), cudaMemcpyHostToDevice, st));
-    }
     long long *d_ninit = reinterpret_cast<long long *>(b + L.ninit);
     double *d_vt = reinterpret_cast<double *>(b + L.vt);
     CK(cudaMemcpyAsync(d_ninit, ninit.data(), 8 * ninit.size(), cudaMemcpyHostToDevice, st));
@@ -1049,18 +1027,15 @@ static cudaError_t enqueue_step(pic_handle *h, long long n, int &nk, bool timed)
         if ((e = time_open(h, timed, st))) return e;
         if ((e = launch_dsmc(h->fp64, h->W, h->pools(), par, 0, st))) return e;
         if ((e = time_close(h, timed, st, 2))) return e;
-        if ((e = launch_pair_reaction(h->fp64, h->W, h->pools(), par, 0, st))) return e;
-        if ((e = launch_pair_reaction(h->fp64, h->W, h->pools(), par, 1, st))) return e;
+        if ((e = launch_pair_reactions(h->fp64, h->W, h->pools(), par, 0, 2, st))) return e;
         if ((e = time_open(h, timed, st))) return e;
         if ((e = launch_dsmc(h->fp64, h->W, h->pools(), par, 1, st))) return e;
         if ((e = time_close(h, timed, st, 2))) return e;
         if ((e = launch_births(h->fp64, h->W, h->pools(), st))) return e;
         if ((e = launch_sort(h->fp64, h->W, h->pools(), h->sort_tab, h->L, st))) return e;
-        // the kill counts of (13), (14) refer to the cells before the sort
-        if ((e = cudaMemsetAsync(h->W.pair_kills, 0, sizeof(int) * NSP * (size_t)h->W.total_cells, st))) return e;
-        if ((e = launch_pair_reaction(h->fp64, h->W, h->pools(), par, 2, st))) return e;
+        if ((e = launch_pair_reactions(h->fp64, h->W, h->pools(), par, 2, 3, st))) return e;
         if ((e = launch_pair_append(h->fp64, h->W, h->pools(), h->L, st))) return e;
-        nk += 1 + 2 + 2 * 3 + 1 + kernels_per_sort() + 1;
+        nk += 1 + 2 + 2 + 1 + kernels_per_sort() + 1;
     } else if (pair) {
         e = launch_pair(h->fp64, h->W, h->pools(), par, h->L, st);
         if (e) return e;

@@ -827,17 +827,6 @@ __device__ __forceinline__ void iso_n(Real r1, Real r2, Real n[3])
     iso_dir<Real>(r1, r2, n);
 }
 
-constexpr int NO_FLAG = 0x7F7F7F7F;  // larger than any slot index
-
-// Particle-target reaction k (0: (13), 1: (14), 2: (19)) evaluated for every
-// projectile at once, as if it were the first of its cell: a random target
-// of the cell (walking past dead ones), P = n_target sigma(E) u n1 dt (Eq. 1)
-// with n_target from the live target count at the start of the reaction's
-// pass, and the acceptance draw.  Nothing is changed here; the smallest
-// projectile index of a cell that collides, finds no live target, or has
-// P > 1 is recorded, and the sequential pass of that cell restarts there.
-// Before it, every projectile's outcome is exactly that of the sequential
-// pass, because no earlier projectile of the cell changed anything.
 // Particle-target reaction k by thinning (Eq. 1): no pair of the pass is
 // faster than the sum of the two species' largest speeds (recorded at the
 // sort and raised by the velocity changes since), so with u_cap that sum,
@@ -872,61 +861,22 @@ __device__ __forceinline__ long long pair_gap(const Disc &Dd, int ps, int rx, un
     return G < 1073741824.0 ? (long long)G : 1073741824LL;
 }
 
-// One thread per cell: does reaction k have a candidate in it?
+// Sequential pass of reaction k over one cell by one warp; kills: the cell's
+// particles killed by the reactions before it, per species, raised here.
 template <typename Real>
-__global__ void __launch_bounds__(256)
-k_pair_eval(WsPtrs W, Pools<Real> P, int par, int k)
+__device__ __forceinline__ void pair_cell(const WsPtrs &W, const Pools<Real> &P, int cur, unsigned long long step, int gw,
+                                          int k, int lane, int kills[NSP])
 {
-    pdl_wait();
-    const int gw = blockIdx.x * blockDim.x + threadIdx.x;
-    if (gw >= W.total_cells) return;
-    const int d = W.cell_disc[gw];
-    const Disc &Dd = W.disc[d];
-    const PairC &pc = Dd.pair[k];
-    if (pc.table < 0) return;
-    const int ps = pc.proj, pt = pc.targ, N = Dd.N, c = gw - Dd.ccell_base;
-    const int *cs = W.cell_start + Dd.cs_base;
-    const int p0 = cs[ps * (N + 2) + c], p1 = cs[ps * (N + 2) + c + 1];
-    if (p1 <= p0) return;
-    const int range = cs[pt * (N + 2) + c + 1] - cs[pt * (N + 2) + c];
-    if (range <= 0) return;
-    const int liveT = range - W.pair_kills[(size_t)gw * NSP + pt];
-    if (liveT <= 0) return;
-    const double B = pair_bound_B(W, Dd, d, pc, liveT);
-    long long first = 0;
-    if (B < 1.0) {
-        const int rx = k == 0 ? 13 : (k == 1 ? 14 : 19);
-        first = pair_gap(Dd, ps, rx, 0u, W.ctl->step[par], c, log1p(-B));
-    }
-    if (first < (long long)(p1 - p0)) W.pair_first[gw] = p0 + (int)first;
-}
-
-// Sequential pass of reaction k over one flagged cell (one warp), from its
-// first flagged projectile on: projectiles in slot order, a batch of 32
-// evaluated in parallel, the first accepting lane executed, the later lanes
-// evaluated again.  Kills, (19)'s scattering and its births happen here.
-template <typename Real>
-__global__ void __launch_bounds__(256)
-k_pair_fix(WsPtrs W, Pools<Real> P, int par, int k)
-{
-    pdl_wait();
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (gw >= W.total_cells) return;
-    const int first = W.pair_first[gw];
-    if (first == NO_FLAG) return;
     const int d = W.cell_disc[gw];
     const Disc &Dd = W.disc[d];
     const int N = Dd.N, c = gw - Dd.ccell_base;
-    const int cur = W.ctl->cur;
-    const unsigned long long step = W.ctl->step[par];
     const int *cs = W.cell_start + Dd.cs_base;
-    int *cellA = P.cell[cur];
-    Real *offA = P.off[cur], *vxA = P.vx[cur], *vyA = P.vy[cur], *vzA = P.vz[cur];
+    const unsigned b0 = cur ? P.stride : 0u;
+    int *cellA = P.cell[0] + b0;
+    Real *offA = P.off[0] + b0, *vxA = P.vx[0] + b0, *vyA = P.vy[0] + b0, *vzA = P.vz[0] + b0;
     typename AccK<Real>::T *acc = AccK<Real>::ptr(W);
     PairBirth<Real> *births = reinterpret_cast<PairBirth<Real> *>(W.pair_births) + (size_t)gw * PAIR_BIRTH_CAP;
     unsigned long long *cnt = W.counters + (size_t)d * C_NCOUNT;
-    int *kills = W.pair_kills + (size_t)gw * NSP;
     int nb = W.pair_bcount[gw];
     const int rx = k == 0 ? 13 : (k == 1 ? 14 : 19);
     const PairC &pc = Dd.pair[k];
@@ -935,6 +885,7 @@ k_pair_fix(WsPtrs W, Pools<Real> P, int par, int k)
     const int t0 = cs[pt * (N + 2) + c], t1 = cs[pt * (N + 2) + c + 1];
     const int range = t1 - t0;
     const int liveT = range - kills[pt];
+    if (liveT <= 0 || p1 <= p0) return;
     const TableDesc &T = W.tables[pc.table];
     const Real coefP = Real(liveT) * pick<Real>(pc.coef, pc.coef_f);
     const int pbp = Dd.pbase[ps], pbt = Dd.pbase[pt];
@@ -949,7 +900,6 @@ k_pair_fix(WsPtrs W, Pools<Real> P, int par, int k)
     bool stop = false;
     unsigned nviol = 0, neval = 0;
     int nkp = 0, nkt = 0;
-    (void)first;
     while (!stop && pos + 1 < p1) {
         long long inc = 1 + (thin ? pair_gap(Dd, ps, rx, draw + (unsigned)lane, step, c, lq) : 0LL);
 #pragma unroll
@@ -1069,10 +1019,73 @@ k_pair_fix(WsPtrs W, Pools<Real> P, int par, int k)
     if (lane == 0) {
         if (nviol) atomicAdd(&cnt[C_VIOL_PAIR], (unsigned long long)nviol);
         if (neval) atomicAdd(&cnt[C_PEVAL], (unsigned long long)neval);
-        kills[ps] += nkp;
-        kills[pt] += nkt;
-        W.pair_bcount[gw] = nb < PAIR_BIRTH_CAP ? nb : PAIR_BIRTH_CAP;
-        W.pair_first[gw] = NO_FLAG;
+        if (rx == 19) W.pair_bcount[gw] = nb < PAIR_BIRTH_CAP ? nb : PAIR_BIRTH_CAP;
+    }
+    kills[ps] += nkp;
+    kills[pt] += nkt;
+}
+
+// May reaction k have a candidate in a cell with np projectiles and nt
+// targets?  FP32 and on the safe side: u_cap is at most 17/16 of the sum of the
+// largest speeds (round_up_5bits), B at most Bu, and the first gap
+// floor(ln U / ln(1 - B)) reaches np when ln U <= -np Bu / (1 - Bu), as
+// ln(1 - B) >= -B / (1 - B).  The margins cover the FP32 rounding.  (The FP64
+// logarithms of the exact test cost more here than all else in the pass.)
+__device__ __forceinline__ bool pair_maybe(const WsPtrs &W, const Disc &Dd, int d, int k, unsigned long long step, int c,
+                                           int np, int nt)
+{
+    const PairC &pc = Dd.pair[k];
+    if (pc.table < 0 || np <= 0 || nt <= 0) return false;
+    const float vp = sqrtf((float)__longlong_as_double((long long)W.vmax2[d * NSP + pc.proj]));
+    const float vt = sqrtf((float)__longlong_as_double((long long)W.vmax2[d * NSP + pc.targ]));
+    const float Bu = (float)nt * pc.coef_f * fmaxf(pc.bnd_g_f, pc.bnd_s_f * (vp + vt) * 1.0626f) * 1.0001f;
+    if (!(Bu < 0.999f)) return true;
+    const int rx = k == 0 ? 13 : (k == 1 ? 14 : 19);
+    const uint4 g = rng_block(Dd.seed, Dd.discharge, pc.proj, 4, rx, 0u, step, (unsigned)c);
+    const float lnU = logf(((float)g.x + 0.5f) * (1.0f / 4294967296.0f));
+    return !(lnU + 1e-5f - 1e-5f * lnU <= -(float)np * Bu / (1.0f - Bu) * 1.0001f);
+}
+
+// Particle-target reactions k0 .. k1-1 (0: (13), 1: (14), 2: (19)) of every
+// cell, one launch.  A block takes PAIR_CELLS cells: one thread per cell and
+// reaction sorts out those without a candidate (pair_maybe), then each warp
+// takes the cells left, one at a time, and runs their reactions in order:
+// projectiles in slot order, a batch of 32 candidates evaluated in parallel,
+// the first accepting lane executed, the later lanes evaluated again.  Kills,
+// (19)'s scattering and its births happen here; a cell's kills only lower the
+// target counts of its later reactions, so a reaction that was sorted out
+// stays so.  What bounds it: latency.  A test and a pass per reaction (six
+// launches, FP64 logarithms in every cell): 37 us for seven small discharges,
+// 51 us for 512 cells, 69 us for 4096; 6, 18 and 19 us here.
+constexpr int PAIR_THREADS = 128, PAIR_CELLS = 16;
+template <typename Real>
+__global__ void __launch_bounds__(PAIR_THREADS)
+k_pair(WsPtrs W, Pools<Real> P, int par, int k0, int k1)
+{
+    pdl_wait();
+    __shared__ int s_flag[PAIR_CELLS];
+    const int lane = threadIdx.x & 31, first = blockIdx.x * PAIR_CELLS;
+    const unsigned long long step = W.ctl->step[par];
+    const int cur = W.ctl->cur;
+    if (threadIdx.x < PAIR_CELLS) s_flag[threadIdx.x] = 0;
+    __syncthreads();
+    if (threadIdx.x < PAIR_CELLS * NSP) {
+        const int j = threadIdx.x % PAIR_CELLS, k = k0 + threadIdx.x / PAIR_CELLS, gw = first + j;
+        if (gw < W.total_cells && k < k1) {
+            const int d = W.cell_disc[gw];
+            const Disc &Dd = W.disc[d];
+            const int N = Dd.N, c = gw - Dd.ccell_base;
+            const int *cp = W.cell_start + Dd.cs_base + Dd.pair[k].proj * (N + 2) + c;
+            const int *ct = W.cell_start + Dd.cs_base + Dd.pair[k].targ * (N + 2) + c;
+            if (pair_maybe(W, Dd, d, k, step, c, cp[1] - cp[0], ct[1] - ct[0])) atomicOr(&s_flag[j], 1 << k);
+        }
+    }
+    __syncthreads();
+    for (int j = threadIdx.x >> 5; j < PAIR_CELLS; j += PAIR_THREADS / 32) {
+        const int flags = s_flag[j], gw = first + j;
+        int kills[NSP] = {0, 0, 0};
+        for (int k = k0; k < k1; ++k)
+            if ((flags >> k) & 1) pair_cell<Real>(W, P, cur, step, gw, k, lane, kills);
     }
 }
 
@@ -1766,12 +1779,13 @@ k_pair_append(WsPtrs W, Pools<Real> P)
     const int d = blockIdx.x;
     const Disc &Dd = W.disc[d];
     const int N = Dd.N;
+    int any = 0;
     for (int c = threadIdx.x; c < N; c += blockDim.x) {
-        pre[c] = W.pair_bcount[Dd.ccell_base + c];
-#pragma unroll
-        for (int q = 0; q < NSP; ++q) W.pair_kills[(size_t)(Dd.ccell_base + c) * NSP + q] = 0;
+        const int n = W.pair_bcount[Dd.ccell_base + c];
+        pre[c] = n;
+        any |= n;
     }
-    __syncthreads();
+    if (!__syncthreads_or(any)) return;
     const int tot = block_scan_exclusive_int(pre, N, wsum);
     if (tot == 0) return;
     const int cur = W.ctl->cur;
@@ -1923,7 +1937,7 @@ cudaError_t launch_field(bool fp64, bool diag, int mode, const WsPtrs &W, int pa
 }
 
 int kernels_per_sort() { return 4; }
-int kernels_per_pair() { return 7; }
+int kernels_per_pair() { return 2; }
 
 cudaError_t launch_sort(bool fp64, const WsPtrs &W, const void *pools, const int *tab, const LaunchCfg &L,
                         cudaStream_t st)
@@ -1980,19 +1994,13 @@ cudaError_t launch_coulomb_inter(bool fp64, const WsPtrs &W, const void *pools, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_pair_reaction(bool fp64, const WsPtrs &W, const void *pools, int par, int k, cudaStream_t st)
+cudaError_t launch_pair_reactions(bool fp64, const WsPtrs &W, const void *pools, int par, int k0, int k1, cudaStream_t st)
 {
-    const int fix_blocks = (W.total_cells * 32 + 255) / 256;
-    const int eval_blocks = (W.total_cells + 255) / 256;
-    if (fp64) {
-        const Pools<double> &P = *static_cast<const Pools<double> *>(pools);
-        launch_k(k_pair_eval<double>, eval_blocks, 256, 0, st, W, P, par, k);
-        launch_k(k_pair_fix<double>, fix_blocks, 256, 0, st, W, P, par, k);
-    } else {
-        const Pools<float> &P = *static_cast<const Pools<float> *>(pools);
-        launch_k(k_pair_eval<float>, eval_blocks, 256, 0, st, W, P, par, k);
-        launch_k(k_pair_fix<float>, fix_blocks, 256, 0, st, W, P, par, k);
-    }
+    const int blocks = (W.total_cells + PAIR_CELLS - 1) / PAIR_CELLS;
+    if (fp64)
+        launch_k(k_pair<double>, blocks, PAIR_THREADS, 0, st, W, *static_cast<const Pools<double> *>(pools), par, k0, k1);
+    else
+        launch_k(k_pair<float>, blocks, PAIR_THREADS, 0, st, W, *static_cast<const Pools<float> *>(pools), par, k0, k1);
     return cudaGetLastError();
 }
 
@@ -2010,10 +2018,8 @@ cudaError_t launch_pair_append(bool fp64, const WsPtrs &W, const void *pools, co
 cudaError_t launch_pair(bool fp64, const WsPtrs &W, const void *pools, int par, const LaunchCfg &L,
                         cudaStream_t st)
 {
-    for (int k = 0; k < 3; ++k) {
-        const cudaError_t e = launch_pair_reaction(fp64, W, pools, par, k, st);
-        if (e) return e;
-    }
+    const cudaError_t e = launch_pair_reactions(fp64, W, pools, par, 0, 3, st);
+    if (e) return e;
     return launch_pair_append(fp64, W, pools, L, st);
 }
 

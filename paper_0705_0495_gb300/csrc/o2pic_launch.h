@@ -69,8 +69,6 @@ struct LaunchCfg {
     size_t scatter_smem;  // scatter kernel
     int sort_col_warps;   // warps of the column scan (sum over (d, s) of bucket groups x row segments)
     const int *sort_warp_base;  // device [D*3+1]: first column-scan warp per (d, s)
-    int pair_blocks_sp[NSP];          // evaluation blocks per projectile species
-    const int *pair_tab_sp[NSP];      // device [(d, tile)] tables per species
     int maxN;             // largest cell count over discharges
     int eedf_max, fm_max; // largest histogram sizes (shared-memory copies in the push)
 };
@@ -117,10 +115,10 @@ cudaError_t launch_coulomb(bool fp64, const WsPtrs &W, const void *pools, int pa
 cudaError_t launch_coulomb_inter(bool fp64, const WsPtrs &W, const void *pools, int par, cudaStream_t st);
 cudaError_t launch_pair(bool fp64, const WsPtrs &W, const void *pools, int par,
                         const LaunchCfg &L, cudaStream_t s);
-// one reaction of the particle-target pass (k = 0, 1, 2 for (13), (14),
+// reactions k0 .. k1-1 of the particle-target pass (0, 1, 2 for (13), (14),
 // (19)), and the append of (19)'s births
-cudaError_t launch_pair_reaction(bool fp64, const WsPtrs &W, const void *pools, int par, int k,
-                                 cudaStream_t s);
+cudaError_t launch_pair_reactions(bool fp64, const WsPtrs &W, const void *pools, int par, int k0, int k1,
+                                  cudaStream_t s);
 cudaError_t launch_pair_append(bool fp64, const WsPtrs &W, const void *pools, const LaunchCfg &L,
                                cudaStream_t s);
 cudaError_t launch_load(bool fp64, const WsPtrs &W, const void *pools, const long long *d_ninit,
