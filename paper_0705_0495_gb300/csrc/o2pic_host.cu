@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <numeric>
 #include <string>
 #include <vector>
@@ -431,6 +432,11 @@ struct pic_handle {
     std::vector<cudaEvent_t> ev;
     std::vector<int> ev_kind;          // kind of each event pair
     int ev_used = 0;
+    // page-locked host buffer that k_gather writes (mapped), large enough for
+    // the largest single read (diagnostics, fields, status and counters)
+    unsigned *pin = nullptr;
+    size_t pin_bytes = 0;
+    std::mutex pin_mu;  // one read at a time (two threads may ask one handle)
     unsigned long long slots0 = 0, cands0 = 0, bslots0 = 0, bcands0 = 0, coul0 = 0, dsmc0 = 0;
     const void *pools() const { return fp64 ? (const void *)&Pd : (const void *)&Pf; }
 };
@@ -447,6 +453,50 @@ static pic_status cuda_fail(pic_handle *h, cudaError_t e, const char *where)
     std::string m = std::string(where) + ": " + cudaGetErrorString(e);
     return fail(h, PIC_ECUDA, m);
 }
+
+// One read of small device arrays: add() what is wanted, run(), then at().
+namespace {
+struct Gather {
+    explicit Gather(pic_handle *h_) : h(h_), lock(h_->pin_mu) {}
+    pic_handle *h;
+    std::unique_lock<std::mutex> lock;  // until the caller has read the buffer
+    GatherList g{};
+    size_t used = 0;  // bytes of the host buffer
+    // bytes: a multiple of 4; returns the place in the host buffer (16-byte aligned)
+    size_t add(const void *src, size_t bytes, bool clear = false, bool copy = true)
+    {
+        if (bytes == 0) return 0;
+        const int k = g.n++;
+        g.src[k] = static_cast<unsigned *>(const_cast<void *>(src));
+        g.first[k + 1] = g.first[k] + (unsigned)(bytes / 4);
+        g.clear[k] = clear ? 1 : 0;
+        g.dst[k] = ~0u;
+        if (!copy) return 0;
+        const size_t at = used;
+        g.dst[k] = (unsigned)(at / 4);
+        used += (bytes + 15) / 16 * 16;
+        return at;
+    }
+    // the arrays as they are at this point of the handle's stream
+    cudaError_t run()
+    {
+        if (used > h->pin_bytes) return cudaErrorInvalidValue;
+        cudaError_t e = launch_gather(g, h->pin, h->stream);
+        return e != cudaSuccess ? e : cudaStreamSynchronize(h->stream);
+    }
+};
+size_t gather_bytes(const pic_config *c, int D)
+{
+    size_t most = 8ull * C_NCOUNT * D + 64;
+    for (int d = 0; d < D; ++d) {
+        const size_t nodes = c[d].n_cells + 1, fm = c[d].fm_bins > 0 ? (size_t)c[d].fm_xbins * c[d].fm_bins : 0;
+        const size_t diag = 8 * 3 * nodes + 16 * nodes + 4 * (size_t)c[d].eedf_bins + 8 * (size_t)c[d].iedf_bins + 4 * fm +
+                            8 * C_NCOUNT + sizeof(Counts) * 3 + 64;
+        most = std::max(most, diag);
+    }
+    return most + 16 * GATHER_MAX;
+}
+} // namespace
 
 #define CK(call)                                                   \
     do {                                                           \
@@ -728,6 +778,12 @@ extern "C" pic_status pic_init(const pic_config *cfgs, int n_discharges, const p
         return fail(nullptr, PIC_ENOMEM, "workspace smaller than pic_workspace_size()");
     }
     h->ws = static_cast<char *>(d_workspace);
+    struct Guard {  // a failed call leaves nothing behind
+        pic_handle *h;
+        ~Guard() { if (h) pic_destroy(h); }
+    } guard{h};
+    h->pin_bytes = gather_bytes(cfgs, n_discharges);
+    CK(cudaHostAlloc(reinterpret_cast<void **>(&h->pin), h->pin_bytes, cudaHostAllocMapped | cudaHostAllocPortable));
     for (int i = 0; i < n_xs; ++i) {
         HostTable t;
         t.reaction = xs[i].reaction;
@@ -955,6 +1011,7 @@ extern "C" pic_status pic_init(const pic_config *cfgs, int n_discharges, const p
     CK(launch_deposit_all(h->fp64, W, h->pools(), -1, max_n, st));
     CK(cudaStreamSynchronize(st));
     h->launches = 0;
+    guard.h = nullptr;
     *out = h;
     return PIC_OK;
 }
@@ -1061,12 +1118,13 @@ static pic_status harvest_events(pic_handle *h)
 
 static pic_status check_status(pic_handle *h)
 {
-    unsigned status = 0;
-    CK(cudaMemcpyAsync(&status, &h->W.ctl->status, sizeof status, cudaMemcpyDeviceToHost, h->stream));
-    std::vector<unsigned long long> c((size_t)h->D * C_NCOUNT);
-    CK(cudaMemcpyAsync(c.data(), h->W.counters, 8 * c.size(), cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-    if (status & ST_TIMEOUT) return fail(h, PIC_ETIMEOUT, "a bounded device wait (birth look-back) gave up");
+    Gather G(h);
+    const size_t o_st = G.add(&h->W.ctl->status, 4), o_c = G.add(h->W.counters, 8ull * h->D * C_NCOUNT);
+    CK(G.run());
+    const char *pin = reinterpret_cast<const char *>(h->pin);
+    const unsigned status = *reinterpret_cast<const unsigned *>(pin + o_st);
+    const unsigned long long *c = reinterpret_cast<const unsigned long long *>(pin + o_c);
+    if (status & ST_TIMEOUT) return fail(h, PIC_ETIMEOUT, "a bounded device wait (sort column scan) gave up");
     if (status & (ST_CAPACITY | ST_BIRTHBUF))
         return fail(h, PIC_ECAPACITY, (status & ST_CAPACITY) ? "particle capacity exceeded; births were dropped"
                                                              : "a per-chunk or per-cell birth buffer overflowed");
@@ -1213,51 +1271,42 @@ extern "C" pic_status pic_diagnostics(pic_handle *h, int d, double *dens_sum, do
     const pic_config &q = h->cfg[d];
     const Disc &D = h->disc[d];
     const int N = q.n_cells, tn = h->W.total_nodes;
-    cudaStream_t st = h->stream;
-    // FP32 path: exact integer sums, scaled here; FP64 path: FP64 sums
-    std::vector<long long> dfix(h->fp64 ? 0 : 3 * (size_t)(N + 1));
-    std::vector<__int128> s2(h->fp64 ? 0 : (size_t)(N + 1));
-    double p0s = 0.0, d0s = 0.0;
-    if (dens_sum) {
-        for (int s = 0; s < 3; ++s) {
-            if (h->fp64)
-                CK(cudaMemcpyAsync(dens_sum + (size_t)s * (N + 1), h->W.dens_sum + (size_t)s * tn + D.gbase,
-                                   8 * (N + 1), cudaMemcpyDeviceToHost, st));
-            else
-                CK(cudaMemcpyAsync(dfix.data() + (size_t)s * (N + 1), h->W.dens_sum_fix + (size_t)s * tn + D.gbase,
-                                   8 * (N + 1), cudaMemcpyDeviceToHost, st));
-        }
+    const bool rs = reset != 0;
+    const size_t nb = 8ull * (N + 1);
+    // FP32 path: exact integer sums, scaled here; FP64 path: FP64 sums.  What
+    // is read is cleared in the same pass when the window ends here.
+    Gather G(h);
+    size_t o_dens[3];
+    for (int s = 0; s < 3; ++s) o_dens[s] = G.add(h->W.dens_sum + (size_t)s * tn + D.gbase, nb, rs, dens_sum != nullptr);
+    const size_t o_phi = G.add(h->W.phi_sum + D.gbase, nb, rs, h->fp64 && phi_sum);
+    const size_t o_s2 = G.add(h->W.phi_s2_sum + D.gbase, 2 * nb, rs, !h->fp64 && phi_sum);
+    const size_t o_p0 = G.add(h->W.phi0_sum + d, 8, rs), o_d0 = G.add(h->W.D0_sum + d, 8, rs);
+    const size_t o_e = G.add(h->W.eedf + D.eedf_base, 4ull * q.eedf_bins, rs);
+    const size_t o_i = G.add(h->W.iedf + D.iedf_base, 8ull * q.iedf_bins, rs);
+    const size_t o_f = G.add(h->W.fm + D.fm_base, 4ull * D.fm_xbins * q.fm_bins, rs);
+    const size_t o_ns = G.add(h->W.nsamp + d, 8, rs);
+    const size_t o_c = G.add(h->W.counters + (size_t)d * C_NCOUNT, 8ull * C_NCOUNT);
+    const size_t o_cn = G.add(h->W.cnt + 3 * d, sizeof(Counts) * 3);
+    CK(G.run());
+    const char *pin = reinterpret_cast<const char *>(h->pin);
+    const long long *dfix[3];
+    for (int s = 0; s < 3; ++s) {
+        dfix[s] = reinterpret_cast<const long long *>(pin + o_dens[s]);
+        if (h->fp64 && dens_sum) memcpy(dens_sum + (size_t)s * (N + 1), pin + o_dens[s], nb);
     }
-    if (phi_sum) {
-        if (h->fp64) {
-            CK(cudaMemcpyAsync(phi_sum, h->W.phi_sum + D.gbase, 8 * (N + 1), cudaMemcpyDeviceToHost, st));
-        } else {
-            CK(cudaMemcpyAsync(s2.data(), h->W.phi_s2_sum + D.gbase, 16 * (N + 1), cudaMemcpyDeviceToHost, st));
-            CK(cudaMemcpyAsync(&p0s, h->W.phi0_sum + d, 8, cudaMemcpyDeviceToHost, st));
-            CK(cudaMemcpyAsync(&d0s, h->W.D0_sum + d, 8, cudaMemcpyDeviceToHost, st));
-        }
-    }
-    std::vector<unsigned> e(std::max(1, q.eedf_bins)), i2(std::max(1, 2 * q.iedf_bins)),
-        f(std::max(1, D.fm_xbins * q.fm_bins));
-    if (q.eedf_bins)
-        CK(cudaMemcpyAsync(e.data(), h->W.eedf + D.eedf_base, 4 * q.eedf_bins, cudaMemcpyDeviceToHost, st));
-    if (q.iedf_bins)
-        CK(cudaMemcpyAsync(i2.data(), h->W.iedf + D.iedf_base, 8 * q.iedf_bins, cudaMemcpyDeviceToHost, st));
-    if (q.fm_bins)
-        CK(cudaMemcpyAsync(f.data(), h->W.fm + D.fm_base, 4 * (size_t)D.fm_xbins * q.fm_bins,
-                           cudaMemcpyDeviceToHost, st));
-    std::vector<unsigned long long> c(C_NCOUNT);
-    CK(cudaMemcpyAsync(c.data(), h->W.counters + (size_t)d * C_NCOUNT, 8 * C_NCOUNT, cudaMemcpyDeviceToHost, st));
-    unsigned long long ns = 0;
-    CK(cudaMemcpyAsync(&ns, h->W.nsamp + d, 8, cudaMemcpyDeviceToHost, st));
-    Counts cn[3];
-    CK(cudaMemcpyAsync(cn, h->W.cnt + 3 * d, sizeof cn, cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
+    if (h->fp64 && phi_sum) memcpy(phi_sum, pin + o_phi, nb);
+    const __int128 *s2 = reinterpret_cast<const __int128 *>(pin + o_s2);
+    const double p0s = *reinterpret_cast<const double *>(pin + o_p0), d0s = *reinterpret_cast<const double *>(pin + o_d0);
+    const unsigned *e = reinterpret_cast<const unsigned *>(pin + o_e), *i2 = reinterpret_cast<const unsigned *>(pin + o_i),
+                   *f = reinterpret_cast<const unsigned *>(pin + o_f);
+    const unsigned long long *c = reinterpret_cast<const unsigned long long *>(pin + o_c);
+    const unsigned long long ns = *reinterpret_cast<const unsigned long long *>(pin + o_ns);
+    const Counts *cn = reinterpret_cast<const Counts *>(pin + o_cn);
     if (!h->fp64 && dens_sum)
         for (int s = 0; s < 3; ++s)
             for (int i = 0; i <= N; ++i)
                 dens_sum[(size_t)s * (N + 1) + i] =
-                    (double)dfix[(size_t)s * (N + 1) + i] * ((i == 0 || i == N) ? D.dens_fix_wall : D.dens_fix);
+                    (double)dfix[s][i] * ((i == 0 || i == N) ? D.dens_fix_wall : D.dens_fix);
     if (!h->fp64 && phi_sum) {
         const double Kdx = 1.602176634e-19 * q.weight_m2 / (double)(1 << FIX_BITS) / 8.8541878128e-12 * D.dx;
         phi_sum[0] = p0s;
@@ -1281,19 +1330,6 @@ extern "C" pic_status pic_diagnostics(pic_handle *h, int d, double *dens_sum, do
         counters[39] = h->graph_calls;
     }
     if (n_samples) *n_samples = (long long)ns;
-    if (reset) {
-        for (int s = 0; s < 3; ++s)
-            CK(cudaMemsetAsync(h->W.dens_sum + (size_t)s * tn + D.gbase, 0, 8 * (N + 1), st));
-        CK(cudaMemsetAsync(h->W.phi_sum + D.gbase, 0, 8 * (N + 1), st));
-        CK(cudaMemsetAsync(h->W.phi_s2_sum + D.gbase, 0, 16 * (N + 1), st));
-        CK(cudaMemsetAsync(h->W.phi0_sum + d, 0, 8, st));
-        CK(cudaMemsetAsync(h->W.D0_sum + d, 0, 8, st));
-        if (q.eedf_bins) CK(cudaMemsetAsync(h->W.eedf + D.eedf_base, 0, 4 * q.eedf_bins, st));
-        if (q.iedf_bins) CK(cudaMemsetAsync(h->W.iedf + D.iedf_base, 0, 8 * q.iedf_bins, st));
-        if (q.fm_bins) CK(cudaMemsetAsync(h->W.fm + D.fm_base, 0, 4 * (size_t)D.fm_xbins * q.fm_bins, st));
-        CK(cudaMemsetAsync(h->W.nsamp + d, 0, 8, st));
-        CK(cudaStreamSynchronize(st));
-    }
     return PIC_OK;
 }
 
@@ -1301,11 +1337,12 @@ extern "C" pic_status pic_get_state(pic_handle *h, int d, int s, double *x, doub
                                     int *alive, long long capacity_n, long long *n)
 {
     if (!h || d < 0 || d >= h->D || s < 0 || s > 2) return fail(h, PIC_EINVAL, "bad handle, discharge or species");
-    Counts cn;
-    int cur = 0;
-    CK(cudaMemcpyAsync(&cn, h->W.cnt + 3 * d + s, sizeof cn, cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemcpyAsync(&cur, &h->W.ctl->cur, sizeof cur, cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
+    Gather G(h);
+    const size_t o_cn = G.add(h->W.cnt + 3 * d + s, sizeof(Counts)), o_cur = G.add(&h->W.ctl->cur, 4);
+    CK(G.run());
+    const char *pin = reinterpret_cast<const char *>(h->pin);
+    const Counts cn = *reinterpret_cast<const Counts *>(pin + o_cn);
+    const int cur = *reinterpret_cast<const int *>(pin + o_cur);
     if (n) *n = cn.n;
     if (!x && !vx && !vy && !vz && !alive) return PIC_OK;
     if (capacity_n < cn.n) return fail(h, PIC_EINVAL, "host arrays shorter than the slot count");
@@ -1413,10 +1450,15 @@ extern "C" pic_status pic_fields(pic_handle *h, int d, double *rho, double *phi,
     CK(launch_field(h->fp64, false, 1, h->W, (int)(h->step & 1), h->L, h->stream));
     const Disc &D = h->disc[d];
     const int N = D.N;
-    if (rho) CK(cudaMemcpyAsync(rho, h->W.rho + D.gbase, 8 * (N + 1), cudaMemcpyDeviceToHost, h->stream));
-    if (phi) CK(cudaMemcpyAsync(phi, h->W.phi + D.gbase, 8 * (N + 1), cudaMemcpyDeviceToHost, h->stream));
-    if (E) CK(cudaMemcpyAsync(E, h->W.Efield + D.gbase, 8 * (N + 1), cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
+    const size_t nb = 8ull * (N + 1);
+    Gather G(h);
+    const size_t o_r = G.add(h->W.rho + D.gbase, nb, false, rho != nullptr), o_p = G.add(h->W.phi + D.gbase, nb, false, phi != nullptr),
+                 o_e = G.add(h->W.Efield + D.gbase, nb, false, E != nullptr);
+    CK(G.run());
+    const char *pin = reinterpret_cast<const char *>(h->pin);
+    if (rho) memcpy(rho, pin + o_r, nb);
+    if (phi) memcpy(phi, pin + o_p, nb);
+    if (E) memcpy(E, pin + o_e, nb);
     return PIC_OK;
 }
 
@@ -1619,6 +1661,7 @@ extern "C" void pic_destroy(pic_handle *h)
     if (h->gexec) cudaGraphExecDestroy(h->gexec);
     if (h->gexec_cycle) cudaGraphExecDestroy(h->gexec_cycle);
     for (auto &e : h->ev) cudaEventDestroy(e);
+    if (h->pin) cudaFreeHost(h->pin);
     delete h;
 }
 

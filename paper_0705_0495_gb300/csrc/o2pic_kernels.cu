@@ -1878,6 +1878,28 @@ __global__ void k_deposit_all(WsPtrs W, Pools<Real> P, int only_disc)
     }
 }
 
+// ------------------------------------------------------------ host reads
+
+__global__ void __launch_bounds__(256) k_gather(GatherList g, unsigned *host)
+{
+    pdl_wait();
+    const unsigned total = g.first[g.n];
+    for (unsigned w = blockIdx.x * 256u + threadIdx.x; w < total; w += gridDim.x * 256u) {
+        int k = 0;
+        while (w >= g.first[k + 1]) ++k;
+        const unsigned i = w - g.first[k];
+        if (g.dst[k] != ~0u) host[g.dst[k] + i] = g.src[k][i];
+        if (g.clear[k]) g.src[k][i] = 0u;
+    }
+}
+
+cudaError_t launch_gather(const GatherList &g, unsigned *host, cudaStream_t st)
+{
+    const unsigned blocks = (g.first[g.n] + 255u) / 256u;
+    launch_k(k_gather, blocks < 1u ? 1u : (blocks < 304u ? blocks : 304u), 256, 0, st, g, host);
+    return cudaGetLastError();
+}
+
 // ------------------------------------------------------------ launchers
 
 // the inter-species pass: A's velocities and one tile of random numbers

@@ -127,6 +127,19 @@ cudaError_t launch_deposit_all(bool fp64, const WsPtrs &W, const void *pools, in
                                int max_n, cudaStream_t s);
 cudaError_t configure_kernels(bool fp64, LaunchCfg &L);
 
+// Copies of a few device arrays into a page-locked host buffer (mapped) by one
+// kernel, and their clearing: what the host reads between steps.  A call reads
+// a dozen small arrays; one copy each takes about 10 us a piece.
+constexpr int GATHER_MAX = 16;
+struct GatherList {
+    unsigned *src[GATHER_MAX];   // 4-byte words
+    unsigned first[GATHER_MAX + 1];  // first word of each array in the list's numbering
+    unsigned dst[GATHER_MAX];    // first word in the host buffer, ~0u: cleared only
+    unsigned char clear[GATHER_MAX];
+    int n;
+};
+cudaError_t launch_gather(const GatherList &g, unsigned *host, cudaStream_t st);
+
 // text returned by pic_last_error(NULL) for calls without a handle
 void set_last_error(const char *msg);
 
