@@ -1008,7 +1008,10 @@ extern "C" pic_status pic_init(const pic_config *cfgs, int n_discharges, const p
     CK(cudaMemcpyAsync(d_ninit, ninit.data(), 8 * ninit.size(), cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(d_vt, vt.data(), 8 * vt.size(), cudaMemcpyHostToDevice, st));
     CK(launch_load(h->fp64, W, h->pools(), d_ninit, d_vt, max_n, st));
-    CK(launch_deposit_all(h->fp64, W, h->pools(), -1, max_n, st));
+    long long max_slots = 0;
+    for (int d = 0; d < n_discharges; ++d)
+        max_slots = std::max(max_slots, h->cfg[d].n_init[0] + h->cfg[d].n_init[1] + h->cfg[d].n_init[2]);
+    CK(launch_deposit_all(h->fp64, W, h->pools(), -1, max_slots, h->L, st));
     CK(cudaStreamSynchronize(st));
     h->launches = 0;
     guard.h = nullptr;
@@ -1333,6 +1336,9 @@ extern "C" pic_status pic_diagnostics(pic_handle *h, int d, double *dens_sum, do
     return PIC_OK;
 }
 
+// slots whose state fits into the spare particle buffer as SI doubles
+static size_t state_chunk(const pic_handle *h) { return (size_t)h->lay.total_cap / (h->fp64 ? 1 : 2); }
+
 extern "C" pic_status pic_get_state(pic_handle *h, int d, int s, double *x, double *vx, double *vy, double *vz,
                                     int *alive, long long capacity_n, long long *n)
 {
@@ -1347,32 +1353,19 @@ extern "C" pic_status pic_get_state(pic_handle *h, int d, int s, double *x, doub
     if (!x && !vx && !vy && !vz && !alive) return PIC_OK;
     if (capacity_n < cn.n) return fail(h, PIC_EINVAL, "host arrays shorter than the slot count");
     const Disc &D = h->disc[d];
-    const size_t g = D.pbase[s], m = cn.n;
-    const size_t R = h->fp64 ? 8 : 4;
-    const char *base = h->ws;
+    const size_t m = cn.n, chunk = state_chunk(h);
+    char *const spare = h->ws;
     const Layout &L = h->lay;
-    std::vector<int> cell(m);
-    std::vector<char> o(m * R), a(m * R), bb(m * R), cc(m * R);
-    if (m) {
-        CK(cudaMemcpyAsync(cell.data(), base + L.cell[cur] + 4 * g, 4 * m, cudaMemcpyDeviceToHost, h->stream));
-        CK(cudaMemcpyAsync(o.data(), base + L.off[cur] + R * g, R * m, cudaMemcpyDeviceToHost, h->stream));
-        CK(cudaMemcpyAsync(a.data(), base + L.vx[cur] + R * g, R * m, cudaMemcpyDeviceToHost, h->stream));
-        CK(cudaMemcpyAsync(bb.data(), base + L.vy[cur] + R * g, R * m, cudaMemcpyDeviceToHost, h->stream));
-        CK(cudaMemcpyAsync(cc.data(), base + L.vz[cur] + R * g, R * m, cudaMemcpyDeviceToHost, h->stream));
-        CK(cudaStreamSynchronize(h->stream));
-    }
-    const double dx = D.dx, vs = D.dx / D.dt;
-    auto rd = [&](const std::vector<char> &v, size_t i) {
-        return h->fp64 ? reinterpret_cast<const double *>(v.data())[i]
-                       : (double)reinterpret_cast<const float *>(v.data())[i];
-    };
-    for (size_t i = 0; i < m; ++i) {
-        const bool al = cell[i] >= 0;
-        if (x) x[i] = al ? ((double)cell[i] + rd(o, i)) * dx : 0.0;
-        if (vx) vx[i] = rd(a, i) * vs;
-        if (vy) vy[i] = rd(bb, i) * vs;
-        if (vz) vz[i] = rd(cc, i) * vs;
-        if (alive) alive[i] = al ? 1 : 0;
+    const int nx = cur ^ 1;
+    double *const to[4] = {x, vx, vy, vz};
+    const size_t from[4] = {L.off[nx], L.vx[nx], L.vy[nx], L.vz[nx]};
+    for (size_t i = 0; i < m; i += chunk) {
+        const size_t k = std::min(chunk, m - i);
+        CK(launch_state_out(h->fp64, h->pools(), cur, D.pbase[s] + i, (int)k, D.dx, D.dx / D.dt, h->stream));
+        for (int q = 0; q < 4; ++q)
+            if (to[q]) CK(cudaMemcpyAsync(to[q] + i, spare + from[q], 8 * k, cudaMemcpyDeviceToHost, h->stream));
+        if (alive) CK(cudaMemcpyAsync(alive + i, spare + L.cell[nx], 4 * k, cudaMemcpyDeviceToHost, h->stream));
+        CK(cudaStreamSynchronize(h->stream));  // the spare buffer is used again
     }
     return PIC_OK;
 }
@@ -1385,51 +1378,42 @@ extern "C" pic_status pic_set_state(pic_handle *h, int d, int s, long long n, co
     if (n > 0 && (!x || !vx || !vy || !vz)) return fail(h, PIC_EINVAL, "NULL state array");
     const Disc &D = h->disc[d];
     const int N = D.N;
-    const size_t R = h->fp64 ? 8 : 4;
-    std::vector<int> cell(n);
-    std::vector<char> o(n * R), a(n * R), bb(n * R), cc(n * R);
-    const double tdx = D.dt / D.dx;
-    for (long long i = 0; i < n; ++i) {
-        const bool al = alive ? alive[i] != 0 : true;
-        const double xx = x[i] / D.dx;
-        int c = al ? (int)std::floor(xx) : -1;
-        if (al && (!(x[i] >= 0.0) || !(x[i] < D.L))) return fail(h, PIC_EINVAL, "live particle outside [0, L)");
-        if (c > N - 1) c = N - 1;
-        double off = al ? xx - c : 0.0;
-        if (h->fp64) {
-            reinterpret_cast<double *>(o.data())[i] = off;
-            reinterpret_cast<double *>(a.data())[i] = vx[i] * tdx;
-            reinterpret_cast<double *>(bb.data())[i] = vy[i] * tdx;
-            reinterpret_cast<double *>(cc.data())[i] = vz[i] * tdx;
-        } else {
-            float of = (float)off;
-            if (al && of >= 1.0f) {
-                if (c + 1 < N) {
-                    ++c;
-                    of = 0.0f;
-                } else {
-                    of = std::nextafter(1.0f, 0.0f);
-                }
-            }
-            reinterpret_cast<float *>(o.data())[i] = of;
-            reinterpret_cast<float *>(a.data())[i] = (float)(vx[i] * tdx);
-            reinterpret_cast<float *>(bb.data())[i] = (float)(vy[i] * tdx);
-            reinterpret_cast<float *>(cc.data())[i] = (float)(vz[i] * tdx);
-        }
-        cell[i] = c;
-    }
     int cur = 0;
-    CK(cudaMemcpyAsync(&cur, &h->W.ctl->cur, sizeof cur, cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-    const size_t g = D.pbase[s];
-    char *base = h->ws;
-    const Layout &L = h->lay;
-    if (n) {
-        CK(cudaMemcpyAsync(base + L.cell[cur] + 4 * g, cell.data(), 4 * n, cudaMemcpyHostToDevice, h->stream));
-        CK(cudaMemcpyAsync(base + L.off[cur] + R * g, o.data(), R * n, cudaMemcpyHostToDevice, h->stream));
-        CK(cudaMemcpyAsync(base + L.vx[cur] + R * g, a.data(), R * n, cudaMemcpyHostToDevice, h->stream));
-        CK(cudaMemcpyAsync(base + L.vy[cur] + R * g, bb.data(), R * n, cudaMemcpyHostToDevice, h->stream));
-        CK(cudaMemcpyAsync(base + L.vz[cur] + R * g, cc.data(), R * n, cudaMemcpyHostToDevice, h->stream));
+    {
+        Gather G(h);
+        const size_t o_cur = G.add(&h->W.ctl->cur, 4);
+        CK(G.run());
+        cur = *reinterpret_cast<const int *>(reinterpret_cast<const char *>(h->pin) + o_cur);
+        const int nx = cur ^ 1;
+        char *const spare = h->ws;
+        const Layout &L = h->lay;
+        const size_t chunk = state_chunk(h), m = (size_t)n;
+        // the positions of every chunk are checked before anything is replaced
+        *h->pin = 0u;
+        auto upload_x = [&](size_t i, size_t k) {
+            cudaError_t e = cudaMemcpyAsync(spare + L.off[nx], x + i, 8 * k, cudaMemcpyHostToDevice, h->stream);
+            if (e == cudaSuccess && alive)
+                e = cudaMemcpyAsync(spare + L.cell[nx], alive + i, 4 * k, cudaMemcpyHostToDevice, h->stream);
+            return e;
+        };
+        for (size_t i = 0; i < m; i += chunk) {
+            const size_t k = std::min(chunk, m - i);
+            CK(upload_x(i, k));
+            CK(launch_state_check(reinterpret_cast<const double *>(spare + L.off[nx]),
+                                  alive ? reinterpret_cast<const int *>(spare + L.cell[nx]) : nullptr, (int)k, D.L, h->pin,
+                                  h->stream));
+        }
+        CK(cudaStreamSynchronize(h->stream));
+        if (*h->pin) return fail(h, PIC_EINVAL, "live particle outside [0, L)");
+        for (size_t i = 0; i < m; i += chunk) {
+            const size_t k = std::min(chunk, m - i);
+            if (m > chunk) CK(upload_x(i, k));  // (one chunk: still there)
+            CK(cudaMemcpyAsync(spare + L.vx[nx], vx + i, 8 * k, cudaMemcpyHostToDevice, h->stream));
+            CK(cudaMemcpyAsync(spare + L.vy[nx], vy + i, 8 * k, cudaMemcpyHostToDevice, h->stream));
+            CK(cudaMemcpyAsync(spare + L.vz[nx], vz + i, 8 * k, cudaMemcpyHostToDevice, h->stream));
+            CK(launch_state_in(h->fp64, h->pools(), cur, D.pbase[s] + i, (int)k, N, D.dx, D.dt / D.dx, alive != nullptr,
+                               h->stream));
+        }
     }
     Counts cn{(int)n, 0, 0, 0};
     CK(cudaMemcpyAsync(h->W.cnt + 3 * d + s, &cn, sizeof cn, cudaMemcpyHostToDevice, h->stream));
@@ -1437,9 +1421,8 @@ extern "C" pic_status pic_set_state(pic_handle *h, int d, int s, long long n, co
     for (int sp = 0; sp < 3; ++sp)
         CK(cudaMemsetAsync(reinterpret_cast<char *>(h->W.acc_dbl) + 8 * ((size_t)sp * tn + D.gbase), 0,
                            8 * (N + 1), h->stream));
-    int max_n = 1;
-    for (int sp = 0; sp < 3; ++sp) max_n = std::max(max_n, (int)h->cfg[d].capacity[sp]);
-    CK(launch_deposit_all(h->fp64, h->W, h->pools(), d, max_n, h->stream));
+    const pic_config &q = h->cfg[d];
+    CK(launch_deposit_all(h->fp64, h->W, h->pools(), d, q.capacity[0] + q.capacity[1] + q.capacity[2], h->L, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     return PIC_OK;
 }

@@ -1859,23 +1859,100 @@ __global__ void k_load(WsPtrs W, Pools<Real> P, const long long *n_init, const d
     }
 }
 
-// Deposit of every live slot (set-up and after a state change); the caller
-// has cleared the accumulators of the affected discharges.
-template <typename Real>
-__global__ void k_deposit_all(WsPtrs W, Pools<Real> P, int only_disc)
+// ------------------------------------------------------------ state copies
+
+// The caller's state arrays pass through the buffer that the next sort will
+// write (free between steps): positions in its offsets, velocities in its
+// velocities, alive flags in its cells; SI doubles there, so a chunk holds
+// half the buffer's slots in the FP32 path.  Arithmetic as on a host: one
+// division, floor, one product per value.  Converted on one host core, the
+// states of 1e6 particles in and out took 7 ms; copies and kernels take 0.6 ms.
+
+// does a live particle lie outside [0, L)?  *bad is set to 1
+__global__ void __launch_bounds__(256) k_state_check(const double *x, const int *alive, int n, double L, unsigned *bad)
 {
-    const int ds = blockIdx.y;
-    const int d = ds / NSP, s = ds % NSP;
-    if (only_disc >= 0 && d != only_disc) return;
-    const Disc &Dd = W.disc[d];
-    const int n = W.cnt[ds].n;
-    const int cur = W.ctl->cur;
-    typename AccK<Real>::T *acc = AccK<Real>::ptr(W) + (size_t)s * W.total_nodes + Dd.gbase;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int g = Dd.pbase[s] + i;
-        const int c = P.cell[cur][g];
-        if (c >= 0 && c < Dd.N) dep_global(acc, c, P.off[cur][g], 1);
+    bool out = false;
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256)
+        out |= (!alive || alive[i] != 0) && !(x[i] >= 0.0 && x[i] < L);
+    if (out) *bad = 1u;
+}
+
+// chunk of n slots from slot g on
+template <typename Real>
+__global__ void __launch_bounds__(256)
+k_state_in(Pools<Real> P, int cur, size_t g, int n, int N, double dx, double tdx, bool flags)
+{
+    const int nx = cur ^ 1;
+    const double *x = reinterpret_cast<const double *>(P.off[nx]), *vx = reinterpret_cast<const double *>(P.vx[nx]),
+                 *vy = reinterpret_cast<const double *>(P.vy[nx]), *vz = reinterpret_cast<const double *>(P.vz[nx]);
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
+        const bool al = !flags || P.cell[nx][i] != 0;
+        const double xx = x[i] / dx;
+        int c = al ? (int)floor(xx) : -1;
+        if (c > N - 1) c = N - 1;
+        const double off = al ? xx - c : 0.0;
+        Real of = (Real)off;
+        if (sizeof(Real) == 4 && al && of >= Real(1)) {
+            if (c + 1 < N) {
+                ++c;
+                of = Real(0);
+            } else {
+                of = (Real)0x1.fffffep-1f;
+            }
+        }
+        P.cell[cur][g + i] = c;
+        P.off[cur][g + i] = of;
+        P.vx[cur][g + i] = (Real)(vx[i] * tdx);
+        P.vy[cur][g + i] = (Real)(vy[i] * tdx);
+        P.vz[cur][g + i] = (Real)(vz[i] * tdx);
     }
+}
+
+template <typename Real>
+__global__ void __launch_bounds__(256)
+k_state_out(Pools<Real> P, int cur, size_t g, int n, double dx, double vs)
+{
+    const int nx = cur ^ 1;
+    double *x = reinterpret_cast<double *>(P.off[nx]), *vx = reinterpret_cast<double *>(P.vx[nx]),
+           *vy = reinterpret_cast<double *>(P.vy[nx]), *vz = reinterpret_cast<double *>(P.vz[nx]);
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
+        const int c = P.cell[cur][g + i];
+        x[i] = c >= 0 ? ((double)c + (double)P.off[cur][g + i]) * dx : 0.0;
+        vx[i] = (double)P.vx[cur][g + i] * vs;
+        vy[i] = (double)P.vy[cur][g + i] * vs;
+        vz[i] = (double)P.vz[cur][g + i] * vs;
+        P.cell[nx][i] = c >= 0 ? 1 : 0;
+    }
+}
+
+static int state_blocks(int n) { return n <= 0 ? 1 : ((n + 255) / 256 < 1216 ? (n + 255) / 256 : 1216); }
+
+cudaError_t launch_state_check(const double *x, const int *alive, int n, double L, unsigned *bad, cudaStream_t st)
+{
+    k_state_check<<<state_blocks(n), 256, 0, st>>>(x, alive, n, L, bad);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_state_in(bool fp64, const void *pools, int cur, size_t g, int n, int N, double dx, double tdx,
+                            bool flags, cudaStream_t st)
+{
+    if (fp64)
+        k_state_in<double><<<state_blocks(n), 256, 0, st>>>(*static_cast<const Pools<double> *>(pools), cur, g, n, N, dx,
+                                                            tdx, flags);
+    else
+        k_state_in<float><<<state_blocks(n), 256, 0, st>>>(*static_cast<const Pools<float> *>(pools), cur, g, n, N, dx,
+                                                           tdx, flags);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_state_out(bool fp64, const void *pools, int cur, size_t g, int n, double dx, double vs,
+                             cudaStream_t st)
+{
+    if (fp64)
+        k_state_out<double><<<state_blocks(n), 256, 0, st>>>(*static_cast<const Pools<double> *>(pools), cur, g, n, dx, vs);
+    else
+        k_state_out<float><<<state_blocks(n), 256, 0, st>>>(*static_cast<const Pools<float> *>(pools), cur, g, n, dx, vs);
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------ host reads
@@ -2060,18 +2137,6 @@ cudaError_t launch_load(bool fp64, const WsPtrs &W, const void *pools, const lon
         k_load<double><<<grid, 256, 0, st>>>(W, *static_cast<const Pools<double> *>(pools), d_ninit, d_vt);
     else
         k_load<float><<<grid, 256, 0, st>>>(W, *static_cast<const Pools<float> *>(pools), d_ninit, d_vt);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_deposit_all(bool fp64, const WsPtrs &W, const void *pools, int disc, int max_n,
-                               cudaStream_t st)
-{
-    dim3 grid((max_n + 255) / 256 > 0 ? ((max_n + 255) / 256 < 4096 ? (max_n + 255) / 256 : 4096) : 1,
-              W.D * NSP);
-    if (fp64)
-        k_deposit_all<double><<<grid, 256, 0, st>>>(W, *static_cast<const Pools<double> *>(pools), disc);
-    else
-        k_deposit_all<float><<<grid, 256, 0, st>>>(W, *static_cast<const Pools<float> *>(pools), disc);
     return cudaGetLastError();
 }
 

@@ -123,8 +123,16 @@ cudaError_t launch_pair_append(bool fp64, const WsPtrs &W, const void *pools, co
                                cudaStream_t s);
 cudaError_t launch_load(bool fp64, const WsPtrs &W, const void *pools, const long long *d_ninit,
                         const double *d_vt, int max_n, cudaStream_t s);
-cudaError_t launch_deposit_all(bool fp64, const WsPtrs &W, const void *pools, int disc,
-                               int max_n, cudaStream_t s);
+// charge of every live slot of a discharge (-1: of all), added to cleared
+// accumulators; max_slots: the most slots a discharge can hold
+cudaError_t launch_deposit_all(bool fp64, const WsPtrs &W, const void *pools, int disc, long long max_slots,
+                               const LaunchCfg &L, cudaStream_t s);
+// state arrays in SI doubles, through the spare particle buffer (see the kernels)
+cudaError_t launch_state_check(const double *x, const int *alive, int n, double L, unsigned *bad, cudaStream_t st);
+cudaError_t launch_state_in(bool fp64, const void *pools, int cur, size_t g, int n, int N, double dx, double tdx,
+                            bool flags, cudaStream_t st);
+cudaError_t launch_state_out(bool fp64, const void *pools, int cur, size_t g, int n, double dx, double vs,
+                             cudaStream_t st);
 cudaError_t configure_kernels(bool fp64, LaunchCfg &L);
 
 // Copies of a few device arrays into a page-locked host buffer (mapped) by one
