@@ -29,8 +29,11 @@
 // A warp whose 128 slots are live and stay on the grid (nearly all) takes a
 // path without masks and selects, with its floors from packed adds (FP32) or
 // off the FP64 units where a slot stays in its cell: FP32 push 293 -> 251 us,
-// FP64 1968 -> 1000 us, results bit for bit the same.  The FP64 sums in 32-bit
-// words per cell took it to 733 us (4e4 superparticles: 17 -> 10.6 us).
+// FP64 1968 -> 960 us, results bit for bit the same.  The FP64 sums in 32-bit
+// words per cell took it to 733 us (4e4 superparticles: 17 -> 10.6 us), the
+// field's steps from a table, floors and energy bins off the FP64 units and one
+// block per SM to 578 us (835 with diagnostics, 1350 before; 9.2 us): about
+// five FP64 instructions a particle, 340 us for its bytes.
 #include <cstdio>
 
 #include "o2pic_launch.h"
@@ -739,21 +742,22 @@ __device__ __forceinline__ bool Dd_binned(const WsPtrs &W, int ds)
 // interpolation, v + (q/m) E dt, offset + v dt / dx.  FP32: two slots per
 // packed instruction (the same roundings as the scalar fused multiply-adds).
 // Dead slots' cells are negative: their arithmetic is that of cell 0.
-template <typename Real>
-__device__ __forceinline__ void push_arith(const Real *sE, const int c[4], const Real off[4], const Real vx[4],
-                                           Real qm, Real ks, Real vn[4], Real on[4])
+// The block's field table: E per node in FP32; in FP64 E and its step to the
+// next node side by side, which takes the subtraction out of every particle.
+template <typename Real> struct FieldT;
+template <> struct FieldT<float> { using T = float; };
+template <> struct FieldT<double> { using T = double2; };
+__device__ __forceinline__ void push_arith(const double2 *sE, const int c[4], const double off[4], const double vx[4],
+                                           double qm, double ks, double vn[4], double on[4])
 {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const int cc = max(c[k], 0);
-        const Real e0 = sE[cc], e1 = sE[cc + 1];
-        const Real ep = e0 + off[k] * (e1 - e0);
-        vn[k] = vx[k] + qm * ep;
+        const double2 e = sE[max(c[k], 0)];
+        vn[k] = vx[k] + qm * (e.x + off[k] * e.y);
         on[k] = off[k] + vn[k] * ks;
     }
 }
-template <>
-__device__ __forceinline__ void push_arith<float>(const float *sE, const int c[4], const float off[4],
+__device__ __forceinline__ void push_arith(const float *sE, const int c[4], const float off[4],
                                                   const float vx[4], float qm, float ks, float vn[4], float on[4])
 {
     const float2 qm2 = make_float2(qm, qm), ks2 = make_float2(ks, ks);
@@ -811,7 +815,7 @@ __device__ __forceinline__ void energy2<float>(float ke, const float v[4], const
 // packed adds instead of two conversions per slot (conversions run at a
 // quarter of the rate).  Outside that range the integer read from t's bits is
 // beyond any grid (or the sum wraps to one that is).
-__device__ __forceinline__ bool cells4(const int c[4], const float on[4], int N, int cn[4], float o[4])
+__device__ __forceinline__ bool cells4(const int c[4], const float on[4], int N, const double *, int cn[4], float o[4])
 {
     constexpr float M = 12582912.0f;  // 1.5 2^23
     const float2 up = make_float2(M, M), dn = make_float2(-M, -M);
@@ -831,12 +835,14 @@ __device__ __forceinline__ bool cells4(const int c[4], const float on[4], int N,
     return far < (unsigned)N && top < 1.0f;
 }
 
-// FP64 runs on two units per SM here, so the floor is kept off them: a slot
-// that stays in its cell (the high word of on below 1.0's, sign included)
-// needs no arithmetic at all, and when a lane of the warp has one that does
-// not, t = on + 1.5 2^52 rounded down gives the integer (its low word) and
-// fl = t - 1.5 2^52.  Range checks are on the high words.
-__device__ __forceinline__ bool cells4(const int c[4], const double on[4], int N, int cn[4], double o[4])
+// FP64 runs on two units per SM here (an instruction takes a warp 64 cycles of
+// its scheduler's unit), so the floor is kept off them: a slot that stays in
+// its cell (the high word of on below 1.0's, sign included) needs no arithmetic
+// at all, and when a lane of the warp has one that does not, the integer part
+// comes from on's bits and its double from a table of -64 .. 63 (sT), for one
+// FP64 instruction per slot.  Range checks are on the high words.
+constexpr int FLOOR_MAX = 64;
+__device__ __forceinline__ bool cells4(const int c[4], const double on[4], int N, const double *sT, int cn[4], double o[4])
 {
     unsigned any = 0u, mag = 0u;
 #pragma unroll
@@ -848,18 +854,57 @@ __device__ __forceinline__ bool cells4(const int c[4], const double on[4], int N
         o[k] = on[k];
     }
     if (!__any_sync(0xffffffffu, any >= 0x3FF00000u)) return true;  // c is in [0, N)
-    constexpr double M = 6755399441055744.0;  // 1.5 2^52
     unsigned far = 0u, top = 0u;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const double t = __dadd_rd(on[k], M);
-        o[k] = on[k] - (t - M);
-        cn[k] = c[k] + __double2loint(t);
+        const int h = __double2hiint(on[k]);
+        const unsigned a = (unsigned)h & 0x7FFFFFFFu;
+        const int e = max((int)(a >> 20) - 1023, -1);  // 2^e <= |on| (e = -1: below 1)
+        const int ip = (int)(((a & 0xFFFFFu) | 0x100000u) >> ((20 - e) & 31));
+        const bool frac = e < 0 || (((a << ((12 + e) & 31)) | (unsigned)__double2loint(on[k])) != 0u);
+        // floor, in [-FLOOR_MAX, FLOOR_MAX) for |on| < FLOOR_MAX (others are sent back below)
+        const int fl = h < 0 ? -(ip + (frac ? 1 : 0)) : ip;
+        o[k] = on[k] - sT[(fl + FLOOR_MAX) & (2 * FLOOR_MAX - 1)];
+        cn[k] = c[k] + fl;
         far = max(far, (unsigned)cn[k]);
         top = max(top, (unsigned)__double2hiint(o[k]));
     }
-    // |on| < 2^20 (finite), every cell on the grid, every offset below 1
-    return mag < 0x41300000u && far < (unsigned)N && top < 0x3FF00000u;
+    // |on| < 64 (finite), every cell on the grid, every offset below 1
+    return mag < 0x40500000u && far < (unsigned)N && top < 0x3FF00000u;
+}
+
+// Bins of the lab energies ke (v^2 + vy^2 + vz^2) of four slots.  FP64: the bin
+// is the exponent and two mantissa bits, so an FP32 estimate (the values cut to
+// 24 bits by moving bits, off the FP64 units) decides it unless it lies within
+// 64 units of the last place of a bin's edge; its error is below 12 such units.
+__device__ __forceinline__ void energy_bins(float ke, const float v[4], const float vy[4], const float vz[4], int nb,
+                                            int bin[4])
+{
+    float K[4];
+    energy2<float>(ke, v, vy, vz, K);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) bin[k] = energy_bin(K[k], nb);
+}
+// |x| cut to an FP32 number (0 below FP32's normal range)
+__device__ __forceinline__ float cut32(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x) & 0x7FFFFFFFu;
+    const unsigned b = __funnelshift_l((unsigned)__double2loint(x), hi - 0x38000000u, 3);
+    return hi >= 0x38100000u && hi < 0x47E00000u ? __uint_as_float(b) : (hi < 0x38100000u ? 0.0f : 3e38f);
+}
+__device__ __forceinline__ void energy_bins(double ke, const double v[4], const double vy[4], const double vz[4], int nb,
+                                            int bin[4])
+{
+    const float kf = cut32(ke);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float a = cut32(v[k]), b = cut32(vy[k]), c = cut32(vz[k]);
+        const float K = kf * (a * a + b * b + c * c);
+        const unsigned edge = (__float_as_uint(K) + 64u) & 0x1FFFFFu;
+        bin[k] = energy_bin(K, nb);
+        if (edge < 128u || !(K > 1e-20f && K < 1e20f))
+            bin[k] = energy_bin(ke * (v[k] * v[k] + vy[k] * vy[k] + vz[k] * vz[k]), nb);
+    }
 }
 
 // Launch shape of the push: NT threads per block, SPT slots per thread.  A
@@ -886,16 +931,24 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
     pdl_wait();
     using Acc = typename AccT<Real>::T;
     constexpr int PUSH_THREADS = SH::threads, NW = SH::nw, G = SH::groups, QCAP = SH::qcap;
-    // without diagnostics: per-cell sums (counts + upper weights)
-    constexpr bool CELLS = !DIAG;
+    // per-cell sums (counts + upper weights); the FP32 diagnostics push has no room for them
+    constexpr bool FP64 = sizeof(Real) == 8;
+    constexpr bool CELLS = !DIAG || FP64;
+    using ET = typename FieldT<Real>::T;
     extern __shared__ __align__(16) unsigned char smem[];
-    unsigned long long *sAcc = reinterpret_cast<unsigned long long *>(smem);  // integer sums (both paths)
-    Real *sE = reinterpret_cast<Real *>(sAcc + (Nmax + 2));
+    // FP32: sums, field; FP64: field, sums, the floors' doubles
+    unsigned long long *sAcc = reinterpret_cast<unsigned long long *>(smem + (FP64 ? sizeof(ET) * (Nmax + 2) : 0));
+    ET *sE = reinterpret_cast<ET *>(FP64 ? smem : smem + 8 * (size_t)(Nmax + 2));
+    double *sT = reinterpret_cast<double *>(sAcc + (Nmax + 2));
+    unsigned char *rest = FP64 ? reinterpret_cast<unsigned char *>(sT + 2 * FLOOR_MAX)
+                               : reinterpret_cast<unsigned char *>(sE + (Nmax + 2));
+    if (FP64)
+        for (int i = threadIdx.x; i < 2 * FLOOR_MAX; i += SH::threads) sT[i] = (double)(i - FLOOR_MAX);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     // per-warp list of collision candidates (slot, energy bin) before it is
     // written out, and the histograms
-    int *qIdx = reinterpret_cast<int *>(sE + (Nmax + 2)) + w * QCAP;
-    unsigned *sEedf = reinterpret_cast<unsigned *>(sE + (Nmax + 2)) + NW * QCAP;
+    int *qIdx = reinterpret_cast<int *>(rest) + w * QCAP;
+    unsigned *sEedf = reinterpret_cast<unsigned *>(rest) + NW * QCAP;
     unsigned *sFm = sEedf + eedf_max;
     unsigned char *qBin = reinterpret_cast<unsigned char *>(sFm + fm_max) + w * QCAP;
     // particles per cell of the block's sums (FP64: and third words), after the queues' bins
@@ -1017,7 +1070,12 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
             const Disc &Dn = W.disc[nd];
             if (nd != d) {
                 const Real *Eg = reinterpret_cast<const Real *>(W.Ereal) + Dn.gbase;
-                for (int i = tid; i <= Dn.N; i += PUSH_THREADS) sE[i] = Eg[i];
+                for (int i = tid; i <= Dn.N; i += PUSH_THREADS) {
+                    if constexpr (FP64)
+                        sE[i] = make_double2(Eg[i], i < Dn.N ? Eg[i + 1] - Eg[i] : 0.0);
+                    else
+                        sE[i] = Eg[i];
+                }
                 d = nd;
             }
             for (int i = tid; i <= Dn.N + 1; i += PUSH_THREADS) {
@@ -1126,17 +1184,16 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
             // the field at the particle, the new velocity and position (the
             // FP32 path takes two slots per packed instruction)
             Real vn[4], on[4];
-            push_arith<Real>(sE, c, off, vx, qm, ks, vn, on);
+            push_arith(sE, c, off, vx, qm, ks, vn, on);
             // null-collision thresholds; electrons: by the bin of the lab energy
             unsigned thr[4] = {tnull, tnull, tnull, tnull};
             if (binned) {
-                Real Kn[4];
-                energy2<Real>(ke, vn, vyl, vzl, Kn);
+                int bin[4];
+                energy_bins(ke, vn, vyl, vzl, nbins, bin);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const int bin = energy_bin(Kn[k], nbins);
-                    thr[k] = s_btn[bin];
-                    bins |= (unsigned)bin << (8 * k);
+                    thr[k] = s_btn[bin[k]];
+                    bins |= (unsigned)bin[k] << (8 * k);
                 }
             }
             // Nearly every warp holds 128 live slots that all stay on the
@@ -1146,7 +1203,7 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
             fast = __all_sync(0xffffffffu, fast);
             if (fast) {
                 Real o[4];
-                fast = __all_sync(0xffffffffu, cells4(c, on, N, dep, o));
+                fast = __all_sync(0xffffffffu, cells4(c, on, N, sT, dep, o));
                 if (fast) {
                     cchg = ((c[0] ^ dep[0]) | (c[1] ^ dep[1]) | (c[2] ^ dep[2]) | (c[3] ^ dep[3])) != 0;
 #pragma unroll
@@ -1794,7 +1851,8 @@ k_births(WsPtrs W, Pools<Real> P)
 template <typename Real>
 static size_t push_smem_bytes(int Nmax, int eedf_max, int fm_max, int nw, int qcap, bool cells)
 {
-    size_t b = sizeof(unsigned long long) * (Nmax + 2) + sizeof(Real) * (Nmax + 2);
+    size_t b = sizeof(unsigned long long) * (Nmax + 2) + sizeof(typename FieldT<Real>::T) * (Nmax + 2);
+    if (sizeof(Real) == 8) b += sizeof(double) * 2 * FLOOR_MAX;
     b += sizeof(int) * nw * qcap;  // candidate slots
     b += sizeof(unsigned) * (eedf_max + fm_max);
     b += (size_t)nw * qcap;        // candidate energy bins
@@ -1812,13 +1870,15 @@ using PushF1 = PushShape<128, 4, 6>;
 using PushF2 = PushShape<512, 4, 1>;
 using PushF3 = PushShape<128, 8, 4>;
 using PushF4 = PushShape<256, 8, 2>;
-using PushD0 = PushShape<256, 4, 2>;
+// (FP64: one block of 16 warps per SM, so that its field and sums are held once:
+// 32 bytes per cell, with room for the histograms)
+using PushD0 = PushShape<512, 4, 1>;
 
 template <typename Real, typename SH>
 static cudaError_t push_shape_setup(LaunchCfg &L, int k)
 {
     const size_t sm = push_smem_bytes<Real>(L.maxN, 0, 0, SH::nw, SH::qcap, true);
-    const size_t smd = push_smem_bytes<Real>(L.maxN, L.eedf_max, L.fm_max, SH::nw, SH::qcap, false);
+    const size_t smd = push_smem_bytes<Real>(L.maxN, L.eedf_max, L.fm_max, SH::nw, SH::qcap, sizeof(Real) == 8);
     cudaError_t e = cudaFuncSetAttribute(k_push<Real, false, SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_push<Real, true, SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smd);

@@ -1,7 +1,7 @@
 """The push's fast path and the two ways it hands out tiles.
 
 CPU: the integers and offsets that the fast path takes from a rounded-down
-add (FP32: 1.5 2^23, FP64: 1.5 2^52) against floor(), with what it must
+add (FP32, 1.5 2^23) and from the bits (FP64) against floor(), with what it must
 refuse.  GPU: the contiguous shares (few tiles per block) and the tickets
 (many) give the same FP32 state bit for bit, over discharges of uneven size
 with empty species and part-filled tiles."""
@@ -61,17 +61,64 @@ def test_fp32_fast_path_refuses_what_is_far_off():
             assert ((c + nan - 0x4B400000) & 0xFFFFFFFF) >= 4096
 
 
+def _words(x):
+    u = struct.unpack("<Q", struct.pack("<d", x))[0]
+    return u >> 32, u & 0xFFFFFFFF
+
+
+def _floor_bits(on):
+    """the FP64 fast path's floor from the bits of |on| < 64"""
+    hi, lo = _words(on)
+    a = hi & 0x7FFFFFFF
+    e = max((a >> 20) - 1023, -1)
+    ip = ((a & 0xFFFFF) | 0x100000) >> (20 - e)
+    frac = e < 0 or (((a << (12 + e)) & 0xFFFFFFFF) | lo) != 0
+    return -(ip + (1 if frac else 0)) if hi >> 31 else ip
+
+
 def test_fp64_fast_floor_is_floor():
     rng = np.random.default_rng(4)
-    M = 6755399441055744.0
-    for on in _positions(rng, np.float64):
-        if not abs(on) < 2.0 ** 20:
+    v = _positions(rng, np.float64) + [np.float64(k + d) for k in range(-63, 64) for d in (0.0, 2.0 ** -46, -2.0 ** -46, 0.5)]
+    v += [np.nextafter(np.float64(k), np.float64(s)) for k in range(-63, 64) for s in (-100.0, 100.0)]
+    for on in v:
+        on = float(on)
+        if not abs(on) < 64.0:
+            assert _words(on)[0] & 0x7FFFFFFF >= 0x40500000  # sent to the general path
             continue
-        t = _add_down(float(on), M, 53)
-        lo = struct.unpack("<q", struct.pack("<d", t))[0] & 0xFFFFFFFF
-        k = lo - (1 << 32) if lo >= 1 << 31 else lo
-        assert k == math.floor(float(on)), on
-        assert t - M == math.floor(float(on)), on
+        if on == 0.0 and math.copysign(1.0, on) < 0:
+            assert _floor_bits(on) == -1  # offset 1: sent to the general path
+            continue
+        assert _floor_bits(on) == math.floor(on), on
+
+
+def test_fp64_energy_bin_from_the_fp32_estimate():
+    """the estimate, from values cut to 24 bits, decides the bin except within
+    64 units of the last place of an edge; its error stays below 12 units"""
+    rng = np.random.default_rng(9)
+
+    def cut(x):
+        hi, lo = _words(abs(x))
+        if hi < 0x38100000:
+            return np.float32(0)
+        b = (((hi - 0x38000000) << 3) | (lo >> 29)) & 0xFFFFFFFF
+        return struct.unpack("<f", struct.pack("<I", b))[0]
+
+    for _ in range(3000):
+        v = rng.normal(0, 1, 3) * 10.0 ** rng.uniform(-4, 2)
+        ke = 10.0 ** rng.uniform(-6, 2)
+        K = ke * (v[0] * v[0] + v[1] * v[1] + v[2] * v[2])
+        f = [np.float32(cut(x)) for x in v]
+        Kf = np.float32(np.float32(cut(ke)) * np.float32(f[0] * f[0] + f[1] * f[1] + f[2] * f[2]))
+        bits = struct.unpack("<I", struct.pack("<f", Kf))[0]
+        exact = struct.unpack("<I", struct.pack("<f", np.float32(K)))[0]
+        assert abs(bits - exact) < 13, (v, ke)
+        if ((bits + 64) & 0x1FFFFF) >= 128:
+            hi = _words(K)[0]
+            assert (bits >> 21) - 4 * 127 == 4 * ((hi >> 20) - 1023) + ((hi >> 18) & 3)
+
+
+def test_fp64_weight_from_one_add():
+    rng = np.random.default_rng(4)
     # rn(off 2^40) read from off + 2^12
     for off in list(rng.uniform(0.0, 1.0, 300)) + [0.0, 2.0 ** -41, 3 * 2.0 ** -41, math.nextafter(1.0, 0.0)]:
         got = struct.unpack("<q", struct.pack("<d", off + 4096.0))[0] - struct.unpack("<q", struct.pack("<d", 4096.0))[0]
