@@ -25,8 +25,8 @@ constexpr int COLLIDE_PER_SM = O2_COLLIDE_PER_SM;    // its blocks per SM
 #define O2_TILES_PER_TICKET 8
 #endif
 constexpr int TILES_PER_TICKET = O2_TILES_PER_TICKET;  // tiles taken per atomic ticket by a push block
-constexpr int BIRTHS_THREADS = 512;    // block of the birth-append kernel (sub-tiles)
-constexpr int TILE_ALIGN = BIRTHS_THREADS / (1024 / 128);  // tiles per birth-append block
+constexpr int BIRTHS_TILES = 512;      // sub-tiles of a birth-append block
+constexpr int TILE_ALIGN = BIRTHS_TILES / (1024 / 128);  // tiles per birth-append block
 #ifndef O2_SORT_WARPS
 #define O2_SORT_WARPS 4
 #endif
@@ -235,6 +235,7 @@ struct Ctl {
     unsigned int colscan_ticket;  // warp order of the sort's column scan
     unsigned int sort_epoch;      // sorts so far (tags the column scan's words)
     unsigned int scatter_done;    // scatter blocks that have finished
+    int tab_total[2];             // tiles of the tables in WsPtrs::tab
 };
 
 // Per (discharge, species) dynamic counts.
@@ -263,7 +264,8 @@ struct WsPtrs {
     void *births;             // [max_chunks * SUBTILES * birth_cap] staged birth records
     int birth_cap;            // records per sub-tile
     unsigned long long *colscan_agg;  // column totals of the sort's row segments, tagged with the sort
-    int *birth_blk;           // [max_chunks / TILE_ALIGN + 1][3] births per append block and product species
+    int *birth_blk;           // [2][max_chunks / TILE_ALIGN + 1][3] births per append block and product species, by step parity
+    Counts *tab;              // [2][D * 3] the tile table of a step by its parity, for its births
     unsigned long long *acc_fix;  // [3 * total_nodes] fixed-point density accumulators
     double *acc_dbl;          // [3 * total_nodes] FP64 accumulators
     double *Efield;           // [total_nodes] E [V/m]
@@ -304,6 +306,14 @@ struct WsPtrs {
     int total_cells;
     int max_chunks;
     int D;
+};
+
+// a staged birth
+template <typename Real>
+struct BirthRec {
+    int c;
+    int tag;    // (slot in the sub-tile << 1 | product) << 2 | species
+    Real off, vx, vy, vz;
 };
 
 // FP64 constant for the FP64 path, its FP32 copy for the FP32 path
@@ -402,6 +412,12 @@ __device__ __forceinline__ void iso_dir(Real r1, Real r2, Real n[3])
 __device__ __forceinline__ void pdl_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// the birth counts of the append blocks for steps of parity par
+__device__ __forceinline__ int *birth_words(const WsPtrs &W, int par)
+{
+    return W.birth_blk + (par ? (size_t)(W.max_chunks / TILE_ALIGN + 1) * NSP : 0);
 }
 
 // a sub-cycled ion species rests (is not pushed) at this step

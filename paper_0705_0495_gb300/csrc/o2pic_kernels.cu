@@ -105,8 +105,6 @@ constexpr int FIELD_ONE = 1024;  // nodes up to which one block per discharge is
 constexpr int FIELD_PER = 5;     // most nodes per thread
 static_assert(FIELD_PER * FIELD_THREADS >= FIELD_ONE + 1 && FIELD_PER * FIELD_THREADS * FIELD_CLUSTER >= 4097, "");
 
-__device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bool advance);
-
 // The sums of a block's nodes, in the units of the accumulators: exact
 // integers (2^-FIX_BITS of a particle) in the FP32 path, doubles in the FP64
 // path.  Sum1 holds S1 and q, Sum2 holds S2.
@@ -132,10 +130,8 @@ template <> struct FieldSum<double> {
 };
 
 template <typename Real>
-__global__ void __launch_bounds__(FIELD_THREADS)
-k_field(WsPtrs W, int par, int diag, int mode, int csize)
+__device__ __forceinline__ void field_block(const WsPtrs &W, int par, int diag, int mode, int csize, int d, int rank)
 {
-    pdl_wait();
     namespace cg = cooperative_groups;
     using Acc = typename AccK<Real>::T;
     using F = FieldSum<Real>;
@@ -151,13 +147,8 @@ k_field(WsPtrs W, int par, int diag, int mode, int csize)
     __shared__ long long s_T0i;
     __shared__ float s_hKf, s_frf;
     __shared__ int s_intE;
-    const int d = blockIdx.x / csize, rank = blockIdx.x % csize;
     Ctl *ctl = W.ctl;
     const unsigned long long step = ctl->step[par];
-    if (d == W.D) {  // the extra cluster (mode 0): this step's tile table and the step counter
-        if (rank == 0) tile_table(W, par, step, true);
-        return;
-    }
     // every block of the cluster has started before another writes to its
     // shared memory (waited for there)
     if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -373,27 +364,51 @@ k_field(WsPtrs W, int par, int diag, int mode, int csize)
     }
 }
 
-// Tile table of the current counts: tiles of each discharge start at a
-// multiple of TILE_ALIGN, so that the birth-append blocks (BIRTHS_THREADS
-// sub-tiles) never span two, and those of each species at a multiple of
-// TILES_PER_TICKET, so that a push ticket never spans two; the birth-append
-// blocks' counts are cleared.  With `advance` the next step's counter is set
-// and the candidate list emptied.
+// Tile table for the step of parity par: tiles of each discharge start at a
+// multiple of TILE_ALIGN, so that the birth-append blocks never span two, and
+// those of each species at a multiple of TILES_PER_TICKET, so that a push
+// ticket never spans two; the step's birth counts are cleared.  With `advance`
+// the next step's counter is set and the candidate list emptied.  The counts
+// are the current ones, or (after_births) those that the births of the step
+// before will leave: its table's counts plus what staging has counted.
 // One thread per discharge and a block scan over them (one thread walking the
 // list took 0.25 us per entry: 50 us of every step of 64 discharges).
-__device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bool advance)
+__device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bool advance, bool after_births)
 {
     __shared__ int s_warp[32];
+    __shared__ int s_add[MAX_DISCHARGES * NSP];
     Ctl *ctl = W.ctl;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NT = blockDim.x;
     constexpr int A = TILE_ALIGN, B = TILES_PER_TICKET;
+    const Counts *old = W.tab + (par ? 0 : W.D * NSP);  // the table of the other parity
+    Counts *keep = W.tab + (par ? W.D * NSP : 0);
+    if (after_births) {
+        for (int k = tid; k < W.D * NSP; k += NT) s_add[k] = 0;
+        __syncthreads();
+        const int *words = birth_words(W, par ^ 1);
+        const int n = (ctl->tab_total[par ^ 1] * SUBTILES + BIRTHS_TILES - 1) / BIRTHS_TILES * NSP;
+        for (int k = tid; k < n; k += NT) {
+            const int v = words[k];
+            if (v == 0) continue;
+            const int tile = k / NSP * TILE_ALIGN;
+            int lo = 0, hi = W.D;
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (old[mid * NSP].chunk0 <= tile) lo = mid; else hi = mid;
+            }
+            atomicAdd(&s_add[lo * NSP + k % NSP], v);
+        }
+        __syncthreads();
+    }
     int first = 0;  // tiles of the discharges before this pass
     for (int d0 = 0; d0 < W.D; d0 += NT) {
         const int d = d0 + tid;
         int n[NSP] = {0, 0, 0}, at[NSP], end = 0;
         if (d < W.D) {
 #pragma unroll
-            for (int s = 0; s < NSP; ++s) n[s] = W.cnt[d * NSP + s].n;
+            for (int s = 0; s < NSP; ++s)
+                n[s] = after_births ? min(old[d * NSP + s].n_snap + s_add[d * NSP + s], W.disc[d].cap[s])
+                                    : W.cnt[d * NSP + s].n;
         }
 #pragma unroll
         for (int s = 0; s < NSP; ++s) {
@@ -418,6 +433,7 @@ __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bo
             for (int s = 0; s < NSP; ++s) {
                 const Counts c{n[s], n[s], start + at[s], (n[s] + CHUNK - 1) / CHUNK};
                 W.cnt[d * NSP + s] = c;
+                keep[d * NSP + s] = c;
             }
             if (d == W.D - 1) {
                 int chunk = start + end;
@@ -426,6 +442,7 @@ __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bo
                     chunk = 0;
                 }
                 ctl->total_chunks = chunk;
+                ctl->tab_total[par] = chunk;
                 ctl->ticket = 0u;
                 if (advance) {
                     ctl->cand_n = 0u;
@@ -434,13 +451,193 @@ __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bo
             }
         }
     }
-    for (int k = tid; k < (W.max_chunks / TILE_ALIGN + 1) * NSP; k += NT) W.birth_blk[k] = 0;
+    int *mine = birth_words(W, par);
+    for (int k = tid; k < (W.max_chunks / TILE_ALIGN + 1) * NSP; k += NT) mine[k] = 0;
 }
 
 __global__ void __launch_bounds__(256) k_retile(WsPtrs W, int par)
 {
     pdl_wait();
-    tile_table(W, par, 0ull, false);
+    tile_table(W, par, 0ull, false, false);
+}
+
+// The field of every discharge, and (mode 0) by one more cluster the step's
+// tile table and the step counter.
+template <typename Real>
+__global__ void __launch_bounds__(FIELD_THREADS)
+k_field(WsPtrs W, int par, int diag, int mode, int csize)
+{
+    pdl_wait();
+    const int d = blockIdx.x / csize, rank = blockIdx.x % csize;
+    if (d < W.D)
+        field_block<Real>(W, par, diag, mode, csize, d, rank);
+    else if (rank == 0)
+        tile_table(W, par, W.ctl->step[par], true, false);
+}
+
+// Births of one step appended after the survivors, per discharge and
+// product species in tile order (tiles are numbered in (parent species,
+// slot) order), i.e. in parent order (staging has deposited their charge).  A
+// block takes BIRTHS_TILES consecutive sub-tiles, two per thread.  Staging has
+// counted the births of every block by product species (birth_blk), so a
+// block's place among the blocks of its discharge is the sum of the earlier
+// ones' counts: nothing waits, and a block without births ends at once (the
+// one with the discharge's last sub-tile sets the slot counts).  When the
+// blocks published totals and read those of their predecessors as these
+// arrived: 5e7 superparticles 20 us, 9.7 us here; 4e6 8.5 us, 5.8 us here.
+// The sub-tiles' record counts are cleared as they are read, for the next use.
+template <typename Real>
+__device__ __forceinline__ void births_block(const WsPtrs &W, const Pools<Real> &P, int par, int blk, bool set_counts)
+{
+    constexpr int NW = FIELD_THREADS / 32, TPT = BIRTHS_TILES / FIELD_THREADS;  // sub-tiles per thread
+    __shared__ int wsum[NSP][NW];
+    __shared__ int s_excl[NSP];
+    __shared__ unsigned s_part[NSP][NW];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    Ctl *ctl = W.ctl;
+    const Counts *tab = W.tab + (par ? W.D * NSP : 0);
+    const int *words = birth_words(W, par);
+    int own[NSP];  // the block's births
+#pragma unroll
+    for (int q = 0; q < NSP; ++q) own[q] = words[(size_t)blk * NSP + q];
+    const int total = ctl->tab_total[par] * SUBTILES;  // sub-tiles
+    if (blk * BIRTHS_TILES >= total) return;
+    // discharge of the block: every discharge's tiles start at a multiple of
+    // BIRTHS_TILES sub-tiles, so a block never spans two discharges
+    int d = 0;
+    {
+        int lo = 0, hi = W.D;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (tab[mid * NSP].chunk0 * SUBTILES <= blk * BIRTHS_TILES) lo = mid; else hi = mid;
+        }
+        d = lo;
+    }
+    const Counts last_sp = tab[d * NSP + 2];
+    const int T1 = (last_sp.chunk0 + last_sp.nchunk) * SUBTILES;  // end of the discharge's sub-tiles
+    const bool last = set_counts && T1 > blk * BIRTHS_TILES && T1 <= (blk + 1) * BIRTHS_TILES;
+    const int any = own[0] + own[1] + own[2];
+    if (!last && any == 0) return;
+    // births of the discharge's earlier blocks, three words each
+    {
+        const int first_blk = tab[d * NSP].chunk0 * SUBTILES / BIRTHS_TILES;
+        const int npred = (blk - first_blk) * NSP;
+        unsigned part[NSP] = {0u, 0u, 0u};
+        for (int k = tid; k < npred; k += FIELD_THREADS) {
+            const unsigned a = (unsigned)words[(size_t)first_blk * NSP + k];
+            const int q = k % NSP;
+#pragma unroll
+            for (int r = 0; r < NSP; ++r) part[r] += r == q ? a : 0u;
+        }
+#pragma unroll
+        for (int q = 0; q < NSP; ++q) {
+            const unsigned v = __reduce_add_sync(0xffffffffu, part[q]);
+            if (lane == 0) s_part[q][warp] = v;
+        }
+        __syncthreads();
+        if (tid < NSP) {
+            unsigned ex = 0;
+            for (int w = 0; w < NW; ++w) ex += s_part[tid][w];
+            s_excl[tid] = (int)ex;
+            if (last) {
+                const long long nn = (long long)tab[d * NSP + tid].n_snap + ex + words[(size_t)blk * NSP + tid];
+                W.cnt[d * NSP + tid].n = (int)(nn < W.disc[d].cap[tid] ? nn : W.disc[d].cap[tid]);
+            }
+        }
+    }
+    if (any == 0) return;
+    const BirthRec<Real> *rec0 = reinterpret_cast<const BirthRec<Real> *>(W.births);
+    const int t0 = blk * BIRTHS_TILES + tid * TPT;
+    int mine[NSP] = {0, 0, 0}, nrec[TPT];
+#pragma unroll
+    for (int j = 0; j < TPT; ++j) {
+        const int t = t0 + j;
+        nrec[j] = 0;  // records of the sub-tile (any order; the tag gives species and parent order)
+        if (t < total && t < T1) {
+            nrec[j] = min(W.tile_cnt[t], W.birth_cap);
+            if (nrec[j]) W.tile_cnt[t] = 0;
+            for (int r = 0; r < nrec[j]; ++r) ++mine[rec0[(size_t)t * W.birth_cap + r].tag & 3];
+        }
+    }
+    int excl[NSP];
+#pragma unroll
+    for (int q = 0; q < NSP; ++q) {
+        int v = mine[q];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += x;
+        }
+        if (lane == 31) wsum[q][warp] = v;
+        excl[q] = v - mine[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NSP; ++q)
+        for (int w = 0; w < warp; ++w) excl[q] += wsum[q][w];
+    const Disc &Dd = W.disc[d];
+    const unsigned b0 = ctl->cur ? P.stride : 0u;
+#pragma unroll
+    for (int j = 0; j < TPT; ++j) {
+        const BirthRec<Real> *rec = rec0 + (size_t)(t0 + j) * W.birth_cap;
+        // a record's place among its species: the number of that species'
+        // records with a smaller tag (parent slot, then product)
+        for (int r = 0; r < nrec[j]; ++r) {
+            const BirthRec<Real> &b = rec[r];
+            const int q = b.tag & 3;
+            int rank = 0;
+            for (int k = 0; k < nrec[j]; ++k) {
+                const int tk = rec[k].tag;
+                rank += (tk & 3) == q && tk < b.tag;
+            }
+            const long long dst = (long long)tab[d * NSP + q].n_snap + s_excl[q] + excl[q] + rank;
+            if (dst >= Dd.cap[q]) {
+                set_status(ctl, ST_CAPACITY);
+                continue;
+            }
+            const size_t g = (size_t)b0 + Dd.pbase[q] + (size_t)dst;
+            P.cell[0][g] = b.c;
+            P.off[0][g] = b.off;
+            P.vx[0][g] = b.vx;
+            P.vy[0][g] = b.vy;
+            P.vz[0][g] = b.vz;
+        }
+        for (int r = 0; r < nrec[j]; ++r) {
+            const int q = rec[r].tag & 3;
+#pragma unroll
+            for (int p = 0; p < NSP; ++p) excl[p] += p == q ? 1 : 0;
+        }
+    }
+}
+
+template <typename Real>
+__global__ void __launch_bounds__(FIELD_THREADS)
+k_births(WsPtrs W, Pools<Real> P, int par)
+{
+    pdl_wait();
+    births_block<Real>(W, P, par, blockIdx.x, true);
+}
+
+// The births of the step of parity par and, between two steps without a sort,
+// the next step's field and tile table in the same launch: the field needs the
+// births' charge (deposited when they were staged) and the table their numbers
+// (counted then), not the append itself.  Both are chains of latencies: 5.5 and
+// 5.6 us one after the other for seven small discharges, 6.0 us together; 9.7 and
+// 8.3 us for one of 5e7 superparticles, 10.0 together.
+template <typename Real>
+__global__ void __launch_bounds__(FIELD_THREADS)
+k_births_field(WsPtrs W, Pools<Real> P, int par, int diag, int csize)
+{
+    pdl_wait();
+    const int d = blockIdx.x / csize, rank = blockIdx.x % csize;
+    if (d < W.D) {
+        field_block<Real>(W, par ^ 1, diag, 0, csize, d, rank);
+    } else if (d == W.D) {
+        if (rank == 0) tile_table(W, par ^ 1, W.ctl->step[par ^ 1], true, true);
+    } else {
+        const int blk = blockIdx.x - (W.D + 1) * csize;
+        if (blk <= W.max_chunks / TILE_ALIGN) births_block<Real>(W, P, par, blk, false);
+    }
 }
 
 // ------------------------------------------------------------- sort
@@ -2032,6 +2229,31 @@ cudaError_t launch_field(bool fp64, bool diag, int mode, const WsPtrs &W, int pa
         launch_cluster(k_field<double>, grid, FIELD_THREADS, csize, st, 0, W, par, diag ? 1 : 0, mode, csize);
     else
         launch_cluster(k_field<float>, grid, FIELD_THREADS, csize, st, 0, W, par, diag ? 1 : 0, mode, csize);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_births(bool fp64, const WsPtrs &W, const void *pools, int par, cudaStream_t st)
+{
+    const int blocks = W.max_chunks / TILE_ALIGN + 1;
+    if (fp64)
+        launch_k(k_births<double>, blocks, FIELD_THREADS, 0, st, W, *static_cast<const Pools<double> *>(pools), par);
+    else
+        launch_k(k_births<float>, blocks, FIELD_THREADS, 0, st, W, *static_cast<const Pools<float> *>(pools), par);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_births_field(bool fp64, bool diag, const WsPtrs &W, const void *pools, int par, const LaunchCfg &L,
+                                cudaStream_t st)
+{
+    const int csize = L.maxN + 1 > FIELD_ONE + 1 ? FIELD_CLUSTER : 1;
+    const int births = W.max_chunks / TILE_ALIGN + 1;
+    const int grid = (W.D + 1) * csize + (births + csize - 1) / csize * csize;
+    if (fp64)
+        launch_cluster(k_births_field<double>, grid, FIELD_THREADS, csize, st, 0, W,
+                       *static_cast<const Pools<double> *>(pools), par, diag ? 1 : 0, csize);
+    else
+        launch_cluster(k_births_field<float>, grid, FIELD_THREADS, csize, st, 0, W,
+                       *static_cast<const Pools<float> *>(pools), par, diag ? 1 : 0, csize);
     return cudaGetLastError();
 }
 

@@ -79,7 +79,10 @@ cudaError_t launch_push(bool fp64, bool diag, const WsPtrs &W, const void *pools
 cudaError_t push_configure(bool fp64, LaunchCfg &L, int num_sms);
 // births of the push appended in parent order
 cudaError_t launch_collide(bool fp64, const WsPtrs &W, const void *pools, int par, int blocks, cudaStream_t st);
-cudaError_t launch_births(bool fp64, const WsPtrs &W, const void *pools, cudaStream_t s);
+cudaError_t launch_births(bool fp64, const WsPtrs &W, const void *pools, int par, cudaStream_t s);
+// the same together with the next step's field (and tile table); diag: that step's
+cudaError_t launch_births_field(bool fp64, bool diag, const WsPtrs &W, const void *pools, int par, const LaunchCfg &L,
+                                cudaStream_t s);
 // the sequential gas scheme, part 0 (channels below (13)) or 1 (above (14))
 constexpr int DSMC_THREADS = 256;
 cudaError_t launch_dsmc(bool fp64, const WsPtrs &W, const void *pools, int par, int part, cudaStream_t st);

@@ -218,29 +218,47 @@ __device__ __forceinline__ void ee_elastic(Real a[3], Real b[3], const Real n[3]
     }
 }
 
-template <typename Real>
-struct BirthRec {
-    int c;
-    int tag;    // (slot in the sub-tile << 1 | product) << 2 | species
-    Real off, vx, vy, vz;
-};
+// charge of one particle added to (sign > 0) or removed from the global
+// accumulator of its species (births, pair-pass kills)
+__device__ __forceinline__ void deposit_global(unsigned long long *acc, int c, float off, int sign)
+{
+    unsigned w1 = __float2uint_rn(off * (float)(1 << FIX_BITS));
+    unsigned w0 = (1u << FIX_BITS) - w1;
+    unsigned long long a = w0, b = w1;
+    if (sign < 0) { a = 0ull - a; b = 0ull - b; }
+    atomicAdd(&acc[c], a);
+    atomicAdd(&acc[c + 1], b);
+}
+__device__ __forceinline__ void deposit_global(double *acc, int c, double off, int sign)
+{
+    atomicAdd(&acc[c], sign * (1.0 - off));
+    atomicAdd(&acc[c + 1], sign * off);
+}
+
+template <typename Real> __device__ __forceinline__ typename AccT<Real>::T *acc_global(const WsPtrs &W);
+template <> __device__ __forceinline__ unsigned long long *acc_global<float>(const WsPtrs &W) { return W.acc_fix; }
+template <> __device__ __forceinline__ double *acc_global<double>(const WsPtrs &W) { return W.acc_dbl; }
 
 // Births of one candidate go straight to its sub-tile's records, in any
-// order; the tag restores parent order when they are appended.
+// order; the tag restores parent order when they are appended.  Their charge
+// is deposited here, so that the next field does not wait for the append.
 template <typename Real>
 struct BirthSink {
     BirthRec<Real> *rec;  // the sub-tile's birth_cap records
     int *n;               // the sub-tile's record count
     int *blk;             // births per product species of the sub-tile's birth-append block
+    typename AccT<Real>::T *acc;  // the discharge's charge accumulators, first species
+    int acc_ld;           // from one species' accumulators to the next
     Ctl *ctl;
     int cap;
 };
 
 template <typename Real>
-__device__ __forceinline__ BirthSink<Real> birth_sink(const WsPtrs &W, int sub)
+__device__ __forceinline__ BirthSink<Real> birth_sink(const WsPtrs &W, const Disc &Dd, int par, int sub)
 {
     return BirthSink<Real>{reinterpret_cast<BirthRec<Real> *>(W.births) + (size_t)sub * W.birth_cap, W.tile_cnt + sub,
-                           W.birth_blk + (size_t)(sub / BIRTHS_THREADS) * NSP, W.ctl, W.birth_cap};
+                           birth_words(W, par) + (size_t)(sub / BIRTHS_TILES) * NSP, acc_global<Real>(W) + Dd.gbase,
+                           W.total_nodes, W.ctl, W.birth_cap};
 }
 
 // ask the L2 cache to fetch [p, p + bytes) (16-byte aligned, a multiple of
@@ -260,6 +278,7 @@ __device__ __forceinline__ void stage_birth(const BirthSink<Real> &B, int tag, i
         return;
     }
     atomicAdd(B.blk + sp, 1);
+    deposit_global(B.acc + (size_t)sp * B.acc_ld, c, off, 1);
     BirthRec<Real> &r = B.rec[pos];
     r.c = c;
     r.tag = (tag << 2) | sp;
@@ -535,27 +554,6 @@ __device__ __forceinline__ unsigned long long sacc_cells<double>(const unsigned 
     };
     return ((unsigned long long)sCnt[i] << FIX_BITS_64) - w(i) + (i > 0 ? w(i - 1) : 0ull);
 }
-
-// charge of one particle added to (sign > 0) or removed from the global
-// accumulator of its species (births, pair-pass kills)
-__device__ __forceinline__ void deposit_global(unsigned long long *acc, int c, float off, int sign)
-{
-    unsigned w1 = __float2uint_rn(off * (float)(1 << FIX_BITS));
-    unsigned w0 = (1u << FIX_BITS) - w1;
-    unsigned long long a = w0, b = w1;
-    if (sign < 0) { a = 0ull - a; b = 0ull - b; }
-    atomicAdd(&acc[c], a);
-    atomicAdd(&acc[c + 1], b);
-}
-__device__ __forceinline__ void deposit_global(double *acc, int c, double off, int sign)
-{
-    atomicAdd(&acc[c], sign * (1.0 - off));
-    atomicAdd(&acc[c + 1], sign * off);
-}
-
-template <typename Real> __device__ __forceinline__ typename AccT<Real>::T *acc_global(const WsPtrs &W);
-template <> __device__ __forceinline__ unsigned long long *acc_global<float>(const WsPtrs &W) { return W.acc_fix; }
-template <> __device__ __forceinline__ double *acc_global<double>(const WsPtrs &W) { return W.acc_dbl; }
 
 // Charge of the four slots of a thread into the block's shared sums.  The
 // FP32 sums are kept per CELL: the particles that land in it (sCnt, one
@@ -1432,7 +1430,7 @@ k_collide(WsPtrs W, Pools<Real> P, int par)
             const NuBin &nb = W.nubin[(size_t)d * NUBIN_MAX + (s == 0 ? bin : 0)];
             const Real nbin = pick<Real>(nb.numax_n, nb.numax_n_f);
             const Real nun = S.nbins > 0 ? nbin : pick<Real>(S.numax_n, S.numax_n_f);
-            const BirthSink<Real> B = birth_sink<Real>(W, sub);
+            const BirthSink<Real> B = birth_sink<Real>(W, Dd, par, sub);
             const Outcome o = gas_collide<Real>(W, Dd, s, (unsigned)rel, step, nun, vx, vy, vz, P.cell[0] + ib,
                                                 P.off[0] + ib, c, off, slot << 1, B);
             // a null event leaves the particle as it was: nothing to write
@@ -1667,7 +1665,7 @@ k_dsmc(WsPtrs W, Pools<Real> P, int par, int part)
                     if (pr.n > 0) {
                         const int i = pb + rel;
                         const int sub = chunk * SUBTILES + local / SUBTILE;
-                        const BirthSink<Real> B = birth_sink<Real>(W, sub);
+                        const BirthSink<Real> B = birth_sink<Real>(W, Dd, par, sub);
                         for (int q = 0; q < pr.n; ++q)
                             stage_birth<Real>(B, ((local % SUBTILE) << 1) | pr.prod[q], pr.sp[q], cellA[i], offA[i],
                                               pr.v[q]);
@@ -1710,7 +1708,7 @@ k_dsmc(WsPtrs W, Pools<Real> P, int par, int part)
             cellA[i] = -1;
             deposit_global(acc_global<Real>(W) + (size_t)s * W.total_nodes + Dd.gbase, c, off, -1);
             const int sub = chunk * SUBTILES + local / SUBTILE;
-            const BirthSink<Real> B = birth_sink<Real>(W, sub);
+            const BirthSink<Real> B = birth_sink<Real>(W, Dd, par, sub);
             stage_birth<Real>(B, ((local % SUBTILE) << 1) | 1, ssp[local], c, off, v);
         }
     }
@@ -1718,134 +1716,6 @@ k_dsmc(WsPtrs W, Pools<Real> P, int par, int part)
     __syncthreads();
     for (int k = tid; k < C_NCOUNT; k += DSMC_THREADS)
         if (s_ev[k]) atomicAdd(&W.counters[(size_t)d * C_NCOUNT + k], (unsigned long long)s_ev[k]);
-}
-
-// Births of one step appended after the survivors, per discharge and
-// product species in tile order (tiles are numbered in (parent species,
-// slot) order), i.e. in parent order; their charge is deposited.  A block
-// takes BIRTHS_THREADS consecutive sub-tiles, one per thread.  Staging has
-// counted the births of every block by product species (birth_blk), so a
-// block's place among the blocks of its discharge is the sum of the earlier
-// ones' counts: nothing waits, and a block without births ends at once (the
-// one with the discharge's last sub-tile sets the slot counts).  When the
-// blocks published totals and read those of their predecessors as these
-// arrived: 5e7 superparticles 20 us, 12 us here; 4e6 8.5 us, 5.8 us here.
-// The sub-tiles' record counts are cleared as they are read, for the next use.
-template <typename Real>
-__global__ void __launch_bounds__(BIRTHS_THREADS)
-k_births(WsPtrs W, Pools<Real> P)
-{
-    pdl_wait();
-    using Acc = typename AccT<Real>::T;
-    __shared__ int wsum[NSP][BIRTHS_THREADS / 32];
-    __shared__ int s_excl[NSP];
-    __shared__ unsigned s_part[NSP][BIRTHS_THREADS / 32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    Ctl *ctl = W.ctl;
-    const int blk = blockIdx.x;
-    const int t = blk * BIRTHS_THREADS + tid;  // this thread's sub-tile
-    int own[NSP];                              // the block's births
-#pragma unroll
-    for (int q = 0; q < NSP; ++q) own[q] = W.birth_blk[(size_t)blk * NSP + q];
-    const int total = ctl->total_chunks * SUBTILES;  // sub-tiles
-    if (blk * BIRTHS_THREADS >= total) return;
-    // discharge of the block: every discharge's tiles start at a multiple of
-    // BIRTHS_THREADS sub-tiles, so a block never spans two discharges
-    int d = 0;
-    {
-        int lo = 0, hi = W.D;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (W.cnt[mid * NSP].chunk0 * SUBTILES <= blk * BIRTHS_THREADS) lo = mid; else hi = mid;
-        }
-        d = lo;
-    }
-    const Counts last_sp = W.cnt[d * NSP + 2];
-    const int T1 = (last_sp.chunk0 + last_sp.nchunk) * SUBTILES;  // end of the discharge's sub-tiles
-    const bool last = T1 > blk * BIRTHS_THREADS && T1 <= (blk + 1) * BIRTHS_THREADS;
-    const int any = own[0] + own[1] + own[2];
-    if (!last && any == 0) return;
-    // births of the discharge's earlier blocks, three words each
-    {
-        const int first_blk = W.cnt[d * NSP].chunk0 * SUBTILES / BIRTHS_THREADS;
-        const int npred = (blk - first_blk) * NSP;
-        unsigned part[NSP] = {0u, 0u, 0u};
-        for (int k = tid; k < npred; k += BIRTHS_THREADS) {
-            const unsigned a = (unsigned)W.birth_blk[(size_t)first_blk * NSP + k];
-            const int q = k % NSP;
-#pragma unroll
-            for (int r = 0; r < NSP; ++r) part[r] += r == q ? a : 0u;
-        }
-#pragma unroll
-        for (int q = 0; q < NSP; ++q) {
-            const unsigned v = __reduce_add_sync(0xffffffffu, part[q]);
-            if (lane == 0) s_part[q][warp] = v;
-        }
-        __syncthreads();
-        if (tid < NSP) {
-            unsigned ex = 0;
-            for (int w = 0; w < BIRTHS_THREADS / 32; ++w) ex += s_part[tid][w];
-            s_excl[tid] = (int)ex;
-            if (last) {
-                Counts &cs = W.cnt[d * NSP + tid];
-                const long long nn = (long long)cs.n_snap + ex + W.birth_blk[(size_t)blk * NSP + tid];
-                cs.n = (int)(nn < W.disc[d].cap[tid] ? nn : W.disc[d].cap[tid]);
-            }
-        }
-    }
-    if (any == 0) return;
-    int mine[NSP] = {0, 0, 0};
-    const bool in = t < total && t < T1;
-    const BirthRec<Real> *rec = reinterpret_cast<const BirthRec<Real> *>(W.births) + (size_t)t * W.birth_cap;
-    int nrec = 0;  // records of this sub-tile (any order; the tag gives species and parent order)
-    if (in) {
-        nrec = min(W.tile_cnt[t], W.birth_cap);
-        if (nrec) W.tile_cnt[t] = 0;
-        for (int r = 0; r < nrec; ++r) ++mine[rec[r].tag & 3];
-    }
-    int excl[NSP];
-#pragma unroll
-    for (int q = 0; q < NSP; ++q) {
-        int v = mine[q];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int x = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += x;
-        }
-        if (lane == 31) wsum[q][warp] = v;
-        excl[q] = v - mine[q];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < NSP; ++q)
-        for (int w = 0; w < warp; ++w) excl[q] += wsum[q][w];
-    if (!in || nrec == 0) return;
-    const Disc &Dd = W.disc[d];
-    const int cur = ctl->cur;
-    Acc *accG = acc_global<Real>(W);
-    // a record's place among its species: the number of that species'
-    // records with a smaller tag (parent slot, then product)
-    for (int r = 0; r < nrec; ++r) {
-        const BirthRec<Real> &b = rec[r];
-        const int q = b.tag & 3;
-        int rank = 0;
-        for (int k = 0; k < nrec; ++k) {
-            const int tk = rec[k].tag;
-            rank += (tk & 3) == q && tk < b.tag;
-        }
-        const long long dst = (long long)W.cnt[d * NSP + q].n_snap + s_excl[q] + excl[q] + rank;
-        if (dst >= Dd.cap[q]) {
-            set_status(ctl, ST_CAPACITY);
-            continue;
-        }
-        const int g = Dd.pbase[q] + (int)dst;
-        P.cell[cur][g] = b.c;
-        P.off[cur][g] = b.off;
-        P.vx[cur][g] = b.vx;
-        P.vy[cur][g] = b.vy;
-        P.vz[cur][g] = b.vz;
-        deposit_global(accG + (size_t)q * W.total_nodes + Dd.gbase, b.c, b.off, 1);
-    }
 }
 
 template <typename Real>
@@ -1955,16 +1825,6 @@ cudaError_t launch_collide(bool fp64, const WsPtrs &W, const void *pools, int pa
         launch_k(k_collide<double>, blocks, COLLIDE_THREADS, 0, st, W, *static_cast<const Pools<double> *>(pools), par);
     else
         launch_k(k_collide<float>, blocks, COLLIDE_THREADS, 0, st, W, *static_cast<const Pools<float> *>(pools), par);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_births(bool fp64, const WsPtrs &W, const void *pools, cudaStream_t st)
-{
-    const int blocks = W.max_chunks / TILE_ALIGN + 1;
-    if (fp64)
-        launch_k(k_births<double>, blocks, BIRTHS_THREADS, 0, st, W, *static_cast<const Pools<double> *>(pools));
-    else
-        launch_k(k_births<float>, blocks, BIRTHS_THREADS, 0, st, W, *static_cast<const Pools<float> *>(pools));
     return cudaGetLastError();
 }
 
