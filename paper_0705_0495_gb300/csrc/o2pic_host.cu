@@ -82,7 +82,7 @@ struct Bump {
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 struct Layout {
-    size_t colscan_agg, sort_whist, ctl, disc, cnt, phi_s2_sum, phi0_sum, D0_sum, gtab, gtabf, gpm, gpmf, tile_cnt, births, birth_blk, sort_tot, warp_base, vmax2, nubin, cand, acc, Efield, Ereal, phi, rho, dens, dens_sum, phi_sum, nsamp,
+    size_t colscan_agg, sort_whist, ctl, disc, cnt, phi_s2_sum, phi0_sum, D0_sum, gtab, gtabf, gpm, gpmf, tile_cnt, births, birth_blk, tab, sort_tot, warp_base, vmax2, nubin, cand, acc, Efield, Ereal, phi, rho, dens, dens_sum, phi_sum, nsamp,
         counters, eedf, iedf, fm, tables, lutE, lutS, lutEf, lutSf, sort_counts, cell_start,
         sort_live, pair_bcount, cell_disc, pair_births, sort_tab, ninit, vt;
     size_t cell[2], off[2], vx[2], vy[2], vz[2];
@@ -328,7 +328,8 @@ Layout make_layout(const pic_config *c, int D, const pic_xs_table *xs, int n_xs,
     L.tile_cnt = B.take(4ull * SUBTILES * mc);
     L.birth_cap = c[0].gas_scheme == 1 ? BIRTH_CAP_SEQ : BIRTH_CAP_W;
     L.births = B.take((size_t)mc * SUBTILES * L.birth_cap * (fp64 ? 40 : 24));
-    L.birth_blk = B.take(4ull * 3 * (mc / TILE_ALIGN + 1));
+    L.birth_blk = B.take(2 * 4ull * 3 * (mc / TILE_ALIGN + 1));
+    L.tab = B.take(2 * sizeof(Counts) * 3 * D);
     L.acc = B.take(8ull * 3 * tn);
     L.Efield = B.take(8ull * tn);
     L.Ereal = B.take(R * tn);
@@ -805,6 +806,7 @@ extern "C" pic_status pic_init(const pic_config *cfgs, int n_discharges, const p
     W.births = b + L.births;
     W.birth_cap = L.birth_cap;
     W.birth_blk = reinterpret_cast<int *>(b + L.birth_blk);
+    W.tab = reinterpret_cast<Counts *>(b + L.tab);
     W.colscan_agg = reinterpret_cast<unsigned long long *>(b + L.colscan_agg);
     W.acc_fix = reinterpret_cast<unsigned long long *>(b + L.acc);
     W.acc_dbl = reinterpret_cast<double *>(b + L.acc);
@@ -1021,7 +1023,6 @@ extern "C" pic_status pic_init(const pic_config *cfgs, int n_discharges, const p
 
 static long long lcm_ll(long long a, long long b) { return a / std::gcd(a, b) * b; }
 
-// Kernels of one step; returns the number launched.
 // events around one kernel launch in timing mode (kind 0 push, 1 Coulomb)
 static cudaError_t time_open(pic_handle *h, bool on, cudaStream_t st)
 {
@@ -1040,15 +1041,23 @@ static cudaError_t time_close(pic_handle *h, bool on, cudaStream_t st, int kind)
     return cudaSuccess;
 }
 
-static cudaError_t enqueue_step(pic_handle *h, long long n, int &nk, bool timed)
+// Kernels of step n; nk counts them.  follows: step n + 1 is queued right after
+// (nothing can change the state between them).  with_field tells a step that
+// the one before has queued its field (in and out).
+static cudaError_t enqueue_step(pic_handle *h, long long n, int &nk, bool timed, bool follows, bool &with_field)
 {
     const pic_config &q = h->cfg[0];
     const int par = (int)(n & 1);
-    const bool diag = q.diag_every > 0 && (n % q.diag_every) == 0;
+    auto diag_at = [&](long long m) { return q.diag_every > 0 && (m % q.diag_every) == 0; };
+    const bool diag = diag_at(n);
     cudaStream_t st = h->stream;
-    cudaError_t e = launch_field(h->fp64, diag, 0, h->W, par, h->L, st);
-    if (e) return e;
-    ++nk;
+    cudaError_t e = cudaSuccess;
+    if (!with_field) {
+        e = launch_field(h->fp64, diag, 0, h->W, par, h->L, st);
+        if (e) return e;
+        ++nk;
+    }
+    with_field = false;
     if ((e = time_open(h, timed, st))) return e;
     e = launch_push(h->fp64, diag, h->W, h->pools(), par, h->L, st);
     if (e) return e;
@@ -1057,13 +1066,17 @@ static cudaError_t enqueue_step(pic_handle *h, long long n, int &nk, bool timed)
     e = launch_collide(h->fp64, h->W, h->pools(), par, h->L.collide_blocks, st);
     if (e) return e;
     ++nk;
-    e = launch_births(h->fp64, h->W, h->pools(), st);
-    if (e) return e;
-    ++nk;
     const long long next = n + 1;
     const bool pair = q.n1 > 0 && next % q.n1 == 0;
     const bool coul = q.n2 > 0 && next % q.n2 == 0;
     const bool sort = pair || coul || (q.sort_interval > 0 && next % q.sort_interval == 0);
+    with_field = follows && !sort;
+    if (with_field)
+        e = launch_births_field(h->fp64, diag_at(next), h->W, h->pools(), par, h->L, st);
+    else
+        e = launch_births(h->fp64, h->W, h->pools(), par, st);
+    if (e) return e;
+    ++nk;
     if (sort) {
         e = launch_sort(h->fp64, h->W, h->pools(), h->sort_tab, h->L, st);
         if (e) return e;
@@ -1091,7 +1104,7 @@ static cudaError_t enqueue_step(pic_handle *h, long long n, int &nk, bool timed)
         if ((e = time_open(h, timed, st))) return e;
         if ((e = launch_dsmc(h->fp64, h->W, h->pools(), par, 1, st))) return e;
         if ((e = time_close(h, timed, st, 2))) return e;
-        if ((e = launch_births(h->fp64, h->W, h->pools(), st))) return e;
+        if ((e = launch_births(h->fp64, h->W, h->pools(), par, st))) return e;
         if ((e = launch_sort(h->fp64, h->W, h->pools(), h->sort_tab, h->L, st))) return e;
         if ((e = launch_pair_reactions(h->fp64, h->W, h->pools(), par, 2, 3, st))) return e;
         if ((e = launch_pair_append(h->fp64, h->W, h->pools(), h->L, st))) return e;
@@ -1159,7 +1172,9 @@ static bool capture_steps(pic_handle *h, long long nsteps, cudaGraphExec_t *out,
     int nk = 0;
     cudaStream_t keep = h->stream;
     h->stream = cs;
-    for (long long k = 0; ok && k < nsteps; ++k) ok = enqueue_step(h, h->step + k, nk, false) == cudaSuccess;
+    bool with_field = false;
+    for (long long k = 0; ok && k < nsteps; ++k)
+        ok = enqueue_step(h, h->step + k, nk, false, k + 1 < nsteps, with_field) == cudaSuccess;
     h->stream = keep;
     cudaError_t ee = cudaStreamEndCapture(cs, &g);
     ok = ok && ee == cudaSuccess && g;
@@ -1234,7 +1249,8 @@ extern "C" pic_status pic_step(pic_handle *h, long long n_steps)
             pic_status s = harvest_events(h);
             if (s != PIC_OK) return s;
         }
-        cudaError_t e = enqueue_step(h, h->step, nk, h->timing);
+        bool with_field = false;
+        cudaError_t e = enqueue_step(h, h->step, nk, h->timing, false, with_field);
         if (e) return cuda_fail(h, e, "kernel launch");
         h->launches += nk;
         h->step += 1;
@@ -1336,6 +1352,20 @@ extern "C" pic_status pic_diagnostics(pic_handle *h, int d, double *dens_sum, do
     return PIC_OK;
 }
 
+// The GPU copies straight from and to the caller's memory here, and a page that
+// the host has not touched yet costs far more when the copy finds it (20 ms more
+// for a first read of 1e6 particles into fresh arrays): touch each page first.
+static void touch_pages(const void *p, size_t bytes, bool write)
+{
+    volatile char *c = static_cast<volatile char *>(const_cast<void *>(p));
+    if (!c || bytes == 0) return;
+    for (size_t i = 0; i < bytes + 4095; i += 4096) {
+        const size_t k = std::min(i, bytes - 1);
+        const char v = c[k];
+        if (write) c[k] = v;
+    }
+}
+
 // slots whose state fits into the spare particle buffer as SI doubles
 static size_t state_chunk(const pic_handle *h) { return (size_t)h->lay.total_cap / (h->fp64 ? 1 : 2); }
 
@@ -1359,6 +1389,8 @@ extern "C" pic_status pic_get_state(pic_handle *h, int d, int s, double *x, doub
     const int nx = cur ^ 1;
     double *const to[4] = {x, vx, vy, vz};
     const size_t from[4] = {L.off[nx], L.vx[nx], L.vy[nx], L.vz[nx]};
+    for (double *a : to) touch_pages(a, 8 * m, true);
+    touch_pages(alive, 4 * m, true);
     for (size_t i = 0; i < m; i += chunk) {
         const size_t k = std::min(chunk, m - i);
         CK(launch_state_out(h->fp64, h->pools(), cur, D.pbase[s] + i, (int)k, D.dx, D.dx / D.dt, h->stream));
@@ -1388,6 +1420,8 @@ extern "C" pic_status pic_set_state(pic_handle *h, int d, int s, long long n, co
         char *const spare = h->ws;
         const Layout &L = h->lay;
         const size_t chunk = state_chunk(h), m = (size_t)n;
+        for (const double *a : {x, vx, vy, vz}) touch_pages(a, 8 * m, false);
+        touch_pages(alive, 4 * m, false);
         // the positions of every chunk are checked before anything is replaced
         *h->pin = 0u;
         auto upload_x = [&](size_t i, size_t k) {
