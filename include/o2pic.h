@@ -34,10 +34,10 @@
  * Memory: the caller allocates ONE device workspace of pic_workspace_size()
  * bytes (256-byte aligned) and keeps it alive until pic_destroy().  The
  * library never allocates device memory after pic_init(); host-side staging
- * uses ordinary host memory for states and, for diagnostics, fields and the
- * status check, a page-locked buffer of the largest of them, which pic_init()
- * allocates and pic_destroy() frees.  All work is issued on the CUDA stream
- * given to pic_init().
+ * uses a page-locked buffer for diagnostics, fields and the status check (of
+ * the largest of them, allocated by pic_init()) and one of 4.7 MB for states
+ * (allocated by the first pic_get_state()); pic_destroy() frees both.  All
+ * work is issued on the CUDA stream given to pic_init().
  *
  * Errors: every call returns a pic_status; nothing is thrown across the ABI.
  * After an error the handle stays valid and may be destroyed; pic_last_error()

@@ -391,6 +391,8 @@ Layout make_layout(const pic_config *c, int D, const pic_xs_table *xs, int n_xs,
 
 } // namespace
 
+constexpr size_t STATE_CHUNK = 65536;  // slots pic_get_state converts at a time
+
 struct pic_handle {
     int D = 0;
     bool fp64 = false;
@@ -437,6 +439,10 @@ struct pic_handle {
     // the largest single read (diagnostics, fields, status and counters)
     unsigned *pin = nullptr;
     size_t pin_bytes = 0;
+    // two halves of STATE_CHUNK slots' state (four doubles and an int each), page-
+    // locked, allocated by the first pic_get_state
+    char *state_pin = nullptr;
+    cudaEvent_t state_ev[2] = {nullptr, nullptr};
     std::mutex pin_mu;  // one read at a time (two threads may ask one handle)
     unsigned long long slots0 = 0, cands0 = 0, bslots0 = 0, bcands0 = 0, coul0 = 0, dsmc0 = 0;
     const void *pools() const { return fp64 ? (const void *)&Pd : (const void *)&Pf; }
@@ -1352,20 +1358,6 @@ extern "C" pic_status pic_diagnostics(pic_handle *h, int d, double *dens_sum, do
     return PIC_OK;
 }
 
-// The GPU copies straight from and to the caller's memory here, and a page that
-// the host has not touched yet costs far more when the copy finds it (20 ms more
-// for a first read of 1e6 particles into fresh arrays): touch each page first.
-static void touch_pages(const void *p, size_t bytes, bool write)
-{
-    volatile char *c = static_cast<volatile char *>(const_cast<void *>(p));
-    if (!c || bytes == 0) return;
-    for (size_t i = 0; i < bytes + 4095; i += 4096) {
-        const size_t k = std::min(i, bytes - 1);
-        const char v = c[k];
-        if (write) c[k] = v;
-    }
-}
-
 // slots whose state fits into the spare particle buffer as SI doubles
 static size_t state_chunk(const pic_handle *h) { return (size_t)h->lay.total_cap / (h->fp64 ? 1 : 2); }
 
@@ -1383,21 +1375,32 @@ extern "C" pic_status pic_get_state(pic_handle *h, int d, int s, double *x, doub
     if (!x && !vx && !vy && !vz && !alive) return PIC_OK;
     if (capacity_n < cn.n) return fail(h, PIC_EINVAL, "host arrays shorter than the slot count");
     const Disc &D = h->disc[d];
-    const size_t m = cn.n, chunk = state_chunk(h);
-    char *const spare = h->ws;
-    const Layout &L = h->lay;
-    const int nx = cur ^ 1;
+    // Converted by the GPU into one half of a page-locked buffer while the host
+    // copies the other half out.  (Copies straight into the caller's arrays are
+    // faster into memory that is in use, 0.3 ms for 1e6 particles, but take 7 ms
+    // more into fresh arrays; this takes 1.5 ms and what the pages cost.)
+    constexpr size_t CH = STATE_CHUNK;
+    if (!h->state_pin) {
+        CK(cudaHostAlloc(reinterpret_cast<void **>(&h->state_pin), 2 * CH * 36, cudaHostAllocMapped | cudaHostAllocPortable));
+        for (auto &e : h->state_ev) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    }
     double *const to[4] = {x, vx, vy, vz};
-    const size_t from[4] = {L.off[nx], L.vx[nx], L.vy[nx], L.vz[nx]};
-    for (double *a : to) touch_pages(a, 8 * m, true);
-    touch_pages(alive, 4 * m, true);
-    for (size_t i = 0; i < m; i += chunk) {
-        const size_t k = std::min(chunk, m - i);
-        CK(launch_state_out(h->fp64, h->pools(), cur, D.pbase[s] + i, (int)k, D.dx, D.dx / D.dt, h->stream));
+    const size_t m = cn.n;
+    auto convert = [&](size_t i) {
+        char *half = h->state_pin + (i / CH % 2) * CH * 36;
+        const cudaError_t e = launch_state_out(h->fp64, h->pools(), cur, D.pbase[s] + i, (int)std::min(CH, m - i),
+                                               reinterpret_cast<double *>(half), (int)CH, D.dx, D.dx / D.dt, h->stream);
+        return e != cudaSuccess ? e : cudaEventRecord(h->state_ev[i / CH % 2], h->stream);
+    };
+    if (m) CK(convert(0));
+    for (size_t i = 0; i < m; i += CH) {
+        if (i + CH < m) CK(convert(i + CH));
+        CK(cudaEventSynchronize(h->state_ev[i / CH % 2]));
+        const size_t k = std::min(CH, m - i);
+        const char *half = h->state_pin + (i / CH % 2) * CH * 36;
         for (int q = 0; q < 4; ++q)
-            if (to[q]) CK(cudaMemcpyAsync(to[q] + i, spare + from[q], 8 * k, cudaMemcpyDeviceToHost, h->stream));
-        if (alive) CK(cudaMemcpyAsync(alive + i, spare + L.cell[nx], 4 * k, cudaMemcpyDeviceToHost, h->stream));
-        CK(cudaStreamSynchronize(h->stream));  // the spare buffer is used again
+            if (to[q]) memcpy(to[q] + i, half + q * 8 * CH, 8 * k);
+        if (alive) memcpy(alive + i, half + 32 * CH, 4 * k);
     }
     return PIC_OK;
 }
@@ -1420,8 +1423,6 @@ extern "C" pic_status pic_set_state(pic_handle *h, int d, int s, long long n, co
         char *const spare = h->ws;
         const Layout &L = h->lay;
         const size_t chunk = state_chunk(h), m = (size_t)n;
-        for (const double *a : {x, vx, vy, vz}) touch_pages(a, 8 * m, false);
-        touch_pages(alive, 4 * m, false);
         // the positions of every chunk are checked before anything is replaced
         *h->pin = 0u;
         auto upload_x = [&](size_t i, size_t k) {
@@ -1679,6 +1680,9 @@ extern "C" void pic_destroy(pic_handle *h)
     if (h->gexec_cycle) cudaGraphExecDestroy(h->gexec_cycle);
     for (auto &e : h->ev) cudaEventDestroy(e);
     if (h->pin) cudaFreeHost(h->pin);
+    if (h->state_pin) cudaFreeHost(h->state_pin);
+    for (auto &e : h->state_ev)
+        if (e) cudaEventDestroy(e);
     delete h;
 }
 

@@ -130,12 +130,12 @@ cudaError_t launch_load(bool fp64, const WsPtrs &W, const void *pools, const lon
 // accumulators; max_slots: the most slots a discharge can hold
 cudaError_t launch_deposit_all(bool fp64, const WsPtrs &W, const void *pools, int disc, long long max_slots,
                                const LaunchCfg &L, cudaStream_t s);
-// state arrays in SI doubles, through the spare particle buffer (see the kernels)
+// state arrays in SI doubles (see the kernels)
 cudaError_t launch_state_check(const double *x, const int *alive, int n, double L, unsigned *bad, cudaStream_t st);
 cudaError_t launch_state_in(bool fp64, const void *pools, int cur, size_t g, int n, int N, double dx, double tdx,
                             bool flags, cudaStream_t st);
-cudaError_t launch_state_out(bool fp64, const void *pools, int cur, size_t g, int n, double dx, double vs,
-                             cudaStream_t st);
+cudaError_t launch_state_out(bool fp64, const void *pools, int cur, size_t g, int n, double *out, int ld, double dx,
+                             double vs, cudaStream_t st);
 cudaError_t configure_kernels(bool fp64, LaunchCfg &L);
 
 // Copies of a few device arrays into a page-locked host buffer (mapped) by one
