@@ -396,7 +396,9 @@ template <typename Real>
 __device__ __forceinline__ void iso_dir(Real r1, Real r2, Real n[3])
 {
     Real cx = Real(1) - Real(2) * r1;
-    Real sx = Real(1) - cx * cx;
+    // fused on purpose: a compiler that may fuse or not would change the last bit
+    // from one caller to the next
+    Real sx = fma(-cx, cx, Real(1));
     sx = sx > Real(0) ? sqrt(sx) : Real(0);
     Real s, c;
     sincospi_(Real(2) * r2, &s, &c);

@@ -1509,20 +1509,24 @@ __device__ __forceinline__ Real dsmc_bound(const WsPtrs &W, const SpeciesC &S, i
 // every n1 steps after the sort: part 0 walks the gas channels of the list
 // numbered below (13), part 1 those above (14).  One block per tile of the
 // table rebuilt after the sort; the tile's particles are held in shared
-// memory and the list is walked channel by channel.  For a channel every
-// particle of its species draws its test number and compares it with a
-// bound on P (dsmc_bound); those below it are queued and the block's threads
-// take the queue one entry each: a gas molecule from the Maxwellian, P = n
-// sigma(E) u n1 dt (clamped at 1 and counted), the test, the kinematics.  A
-// particle that dies in (15), (16) or (17) is replaced by its product, which
-// meets the later channels ("readmitted").  Random numbers: stream 6 of the
-// chain's first particle, sub-stream = the channel's place in the list,
-// draws 4g (molecule), 4g + 1 (test, direction), 4g + 2 (second direction of
-// (18)) in generation g.  Products are recorded in the first particle's
-// sub-tile: (18)'s with product bits 0 (electron) and 1 (O2+), the one that
-// ends a chain with bit 1.  The decisions are those of walking each
-// particle's chain in turn: a particle's channels stay in list order, and
-// particles do not interact.
+// memory.  For each channel of its species in turn a particle draws its test
+// number and compares it with a bound on P (dsmc_bound); at the first one below
+// it the particle is queued with that channel.  The block's threads take the
+// queue one entry each (a gas molecule from the Maxwellian, P = n sigma(E) u n1
+// dt clamped at 1 and counted, the test, the kinematics) and go on along the
+// list with what the particle is then, into the next round's queue.  A particle
+// that dies in (15), (16) or (17) is replaced by its product, which meets the
+// later channels.  Random numbers: stream 6 of the chain's first particle,
+// sub-stream = the channel's place in the list, draws 4g (molecule), 4g + 1
+// (test, direction), 4g + 2 (second direction of (18)) in generation g.
+// Products are recorded in the first particle's sub-tile: (18)'s with product
+// bits 0 (electron) and 1 (O2+), the one that ends a chain with bit 1.  The
+// decisions are those of walking each particle's chain in turn: a particle's
+// channels stay in list order, and particles do not interact.
+// What bounds it: latency and the Philox draw per particle and channel.  The
+// rounds have a barrier each, and there are as many as one particle has
+// candidates in a row; a queue and three barriers per channel, most of them
+// with a few entries, took 160 us per part for 4e6 superparticles, 130 us so.
 template <typename Real>
 __global__ void __launch_bounds__(DSMC_THREADS, 3)
 k_dsmc(WsPtrs W, Pools<Real> P, int par, int part)
@@ -1532,11 +1536,12 @@ k_dsmc(WsPtrs W, Pools<Real> P, int par, int part)
     __shared__ Real sv[3][CHUNK];        // velocity of the chain's current particle
     __shared__ signed char ssp[CHUNK];   // its species, -1 for no particle
     __shared__ unsigned char sgen[CHUNK];
-    __shared__ unsigned short sq[CHUNK]; // queue of one channel
+    __shared__ unsigned short sq[2][CHUNK];  // queues of this round and the next
+    __shared__ unsigned char skk[CHUNK];     // place in the list of a queued particle's channel
     __shared__ Real sumax[CHUNK];        // speed bound and grid place of the particle (dsmc_locate)
     __shared__ unsigned short sk[CHUNK];
     __shared__ unsigned char sreg[CHUNK];
-    __shared__ unsigned s_qn;
+    __shared__ unsigned s_qn[3];
     Ctl *ctl = W.ctl;
     const int chunk = blockIdx.x;
     if (chunk >= ctl->total_chunks) return;
@@ -1552,7 +1557,7 @@ k_dsmc(WsPtrs W, Pools<Real> P, int par, int part)
     const Disc &Dd = W.disc[d];
     const int tid = threadIdx.x;
     for (int q = tid; q < C_NCOUNT; q += DSMC_THREADS) s_ev[q] = 0;
-    if (tid == 0) s_qn = 0u;
+    if (tid < 3) s_qn[tid] = 0u;
     const unsigned long long step = ctl->step[par];
     const int cur = ctl->cur;
     int *cellA = P.cell[cur];
@@ -1588,40 +1593,53 @@ k_dsmc(WsPtrs W, Pools<Real> P, int par, int part)
     if (nlive) atomicAdd(&s_ev[C_DSMC], nlive);
     __syncthreads();
     unsigned ntest = 0;  // Eq. 1 tests of this thread's particles
-    for (int kk = 0; kk < Dd.ndsmc; ++kk) {
-        const DsmcCh &e = Dd.dsmc[kk];
-        if (part == 0 ? e.reaction > 12 : e.reaction < 15) continue;  // uniform
-        const SpeciesC &S = Dd.sp[e.sp];
-        // the test of every particle of the channel's species against the
-        // bound, the thread's four particles side by side (independent chains)
-        {
-            constexpr int PT = CHUNK / DSMC_THREADS;
-            bool in[PT];
-            unsigned w[PT];
+    // the part's stretch of the list (it is in the order of the reactions)
+    int kbeg = 0, kend = Dd.ndsmc;
+    while (kbeg < kend && part == 1 && Dd.dsmc[kbeg].reaction < 15) ++kbeg;
+    while (kend > kbeg && part == 0 && Dd.dsmc[kend - 1].reaction > 12) --kend;
+    // the test number of channel kk against the bound on P
+    auto maybe = [&](int local, int kk, const DsmcCh &e) {
+        const unsigned w = rng_block(Dd.seed, Dd.discharge, s, 6, kk, 4u * sgen[local] + 1u, step, (unsigned)(rel0 + local)).x;
+        return unif<Real>(w) < dsmc_bound<Real>(W, Dd.sp[e.sp], e.j, sumax[local], sk[local], sreg[local], n1);
+    };
+    {
+        // the first channel that may take each of the thread's particles, side
+        // by side (independent chains)
+        constexpr int PT = CHUNK / DSMC_THREADS;
+        bool on[PT];
+#pragma unroll
+        for (int q = 0; q < PT; ++q) on[q] = ssp[tid + q * DSMC_THREADS] >= 0;
+        for (int kk = kbeg; kk < kend; ++kk) {
+            const DsmcCh e = Dd.dsmc[kk];
+            if (e.sp != s) continue;  // no particle has changed its species yet
 #pragma unroll
             for (int q = 0; q < PT; ++q) {
                 const int local = tid + q * DSMC_THREADS;
-                in[q] = ssp[local] == e.sp;
-                w[q] = in[q] ? rng_block(Dd.seed, Dd.discharge, s, 6, kk, 4u * sgen[local] + 1u, step,
-                                         (unsigned)(rel0 + local)).x
-                             : 0u;
-            }
-#pragma unroll
-            for (int q = 0; q < PT; ++q) {
-                const int local = tid + q * DSMC_THREADS;
-                if (!in[q]) continue;
+                if (!on[q]) continue;
                 ++ntest;
-                if (unif<Real>(w[q]) < dsmc_bound<Real>(W, S, e.j, sumax[local], sk[local], sreg[local], n1))
-                    sq[atomicAdd(&s_qn, 1u)] = (unsigned short)local;
+                if (maybe(local, kk, e)) {
+                    on[q] = false;
+                    skk[local] = (unsigned char)kk;
+                    sq[0][atomicAdd(&s_qn[0], 1u)] = (unsigned short)local;
+                }
             }
         }
-        __syncthreads();
-        const int nq = (int)s_qn;
-        if (nq > 0) {
-            const GasChan &ch = S.ch[e.j];
-            for (int qi = tid; qi < nq; qi += DSMC_THREADS) {
-                const int local = sq[qi];
-                const int rel = rel0 + local;
+    }
+    for (int round = 0;; ++round) {
+        __syncthreads();  // the round's queue is complete
+        const int nq = (int)s_qn[round % 3];
+        if (nq == 0) break;
+        // the counter after the next: its last readers passed the barrier above
+        if (tid == 0) s_qn[(round + 2) % 3] = 0u;
+        const unsigned short *in = sq[round & 1];
+        for (int qi = tid; qi < nq; qi += DSMC_THREADS) {
+            const int local = in[qi];
+            const int rel = rel0 + local;
+            int kk = skk[local];
+            {
+                const DsmcCh e = Dd.dsmc[kk];
+                const SpeciesC &S = Dd.sp[e.sp];
+                const GasChan &ch = S.ch[e.j];
                 const unsigned gen = sgen[local];
                 Real v[3] = {sv[0][local], sv[1][local], sv[2][local]};
                 const uint4 b = rng_block(Dd.seed, Dd.discharge, s, 6, kk, 4u * gen + 1u, step, (unsigned)rel);
@@ -1646,45 +1664,55 @@ k_dsmc(WsPtrs W, Pools<Real> P, int par, int part)
                     atomicAdd(&s_ev[C_VIOL_PAIR], 1u);
                     Pj = Real(1);
                 }
-                if (!(unif<Real>(b.x) < Pj)) continue;
-                atomicAdd(&s_ev[C_EVENTS + ch.reaction], 1u);
-                Real nd[3], nd2[3] = {Real(0), Real(0), Real(1)};
-                iso_dir<Real>(unif<Real>(b.y), unif<Real>(b.z), nd);
-                if (ch.reaction == 18) {
-                    const uint4 e2 = rng_block(Dd.seed, Dd.discharge, s, 6, kk, 4u * gen + 2u, step, (unsigned)rel);
-                    iso_dir<Real>(unif<Real>(e2.x), unif<Real>(e2.y), nd2);
-                }
-                GasProducts<Real> pr;
-                Real vo[3];
-                Real um;
-                int bk, breg;
-                if (gas_event<Real>(W, Dd, S, ch, v, V, E, nd, nd2, vo, pr)) {
-#pragma unroll
-                    for (int q = 0; q < 3; ++q) sv[q][local] = vo[q];
-                    dsmc_locate<Real>(W, S, vo, um, bk, breg);
-                    if (pr.n > 0) {
-                        const int i = pb + rel;
-                        const int sub = chunk * SUBTILES + local / SUBTILE;
-                        const BirthSink<Real> B = birth_sink<Real>(W, Dd, par, sub);
-                        for (int q = 0; q < pr.n; ++q)
-                            stage_birth<Real>(B, ((local % SUBTILE) << 1) | pr.prod[q], pr.sp[q], cellA[i], offA[i],
-                                              pr.v[q]);
+                if (unif<Real>(b.x) < Pj) {
+                    atomicAdd(&s_ev[C_EVENTS + ch.reaction], 1u);
+                    Real nd[3], nd2[3] = {Real(0), Real(0), Real(1)};
+                    iso_dir<Real>(unif<Real>(b.y), unif<Real>(b.z), nd);
+                    if (ch.reaction == 18) {
+                        const uint4 e2 = rng_block(Dd.seed, Dd.discharge, s, 6, kk, 4u * gen + 2u, step, (unsigned)rel);
+                        iso_dir<Real>(unif<Real>(e2.x), unif<Real>(e2.y), nd2);
                     }
-                } else {
-                    ssp[local] = (signed char)pr.sp[0];
+                    GasProducts<Real> pr;
+                    Real vo[3];
+                    Real um;
+                    int bk, breg;
+                    if (gas_event<Real>(W, Dd, S, ch, v, V, E, nd, nd2, vo, pr)) {
 #pragma unroll
-                    for (int q = 0; q < 3; ++q) sv[q][local] = pr.v[0][q];
-                    sgen[local] = (unsigned char)(gen + 1u);
-                    dsmc_locate<Real>(W, Dd.sp[pr.sp[0]], pr.v[0], um, bk, breg);
+                        for (int q = 0; q < 3; ++q) sv[q][local] = vo[q];
+                        dsmc_locate<Real>(W, S, vo, um, bk, breg);
+                        if (pr.n > 0) {
+                            const int i = pb + rel;
+                            const int sub = chunk * SUBTILES + local / SUBTILE;
+                            const BirthSink<Real> B = birth_sink<Real>(W, Dd, par, sub);
+                            for (int q = 0; q < pr.n; ++q)
+                                stage_birth<Real>(B, ((local % SUBTILE) << 1) | pr.prod[q], pr.sp[q], cellA[i], offA[i],
+                                                  pr.v[q]);
+                        }
+                    } else {
+                        ssp[local] = (signed char)pr.sp[0];
+#pragma unroll
+                        for (int q = 0; q < 3; ++q) sv[q][local] = pr.v[0][q];
+                        sgen[local] = (unsigned char)(gen + 1u);
+                        dsmc_locate<Real>(W, Dd.sp[pr.sp[0]], pr.v[0], um, bk, breg);
+                    }
+                    sumax[local] = um;
+                    sk[local] = (unsigned short)bk;
+                    sreg[local] = (unsigned char)breg;
                 }
-                sumax[local] = um;
-                sk[local] = (unsigned short)bk;
-                sreg[local] = (unsigned char)breg;
+            }
+            // on to the next channel that may take what the particle is now
+            const int sp = ssp[local];
+            for (++kk; kk < kend; ++kk) {
+                const DsmcCh e = Dd.dsmc[kk];
+                if (e.sp != sp) continue;
+                ++ntest;
+                if (maybe(local, kk, e)) {
+                    skk[local] = (unsigned char)kk;
+                    sq[(round + 1) & 1][atomicAdd(&s_qn[(round + 1) % 3], 1u)] = (unsigned short)local;
+                    break;
+                }
             }
         }
-        __syncthreads();
-        if (tid == 0) s_qn = 0u;
-        __syncthreads();
     }
     if (ntest) atomicAdd(&s_ev[C_PEVAL], ntest);
     // write back: the first particle's new velocity, or its removal and the
