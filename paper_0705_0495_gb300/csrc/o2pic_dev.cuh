@@ -236,6 +236,7 @@ struct Ctl {
     unsigned int sort_epoch;      // sorts so far (tags the column scan's words)
     unsigned int scatter_done;    // scatter blocks that have finished
     int tab_total[2];             // tiles of the tables in WsPtrs::tab
+    int over[2];                  // by step parity: a species has more births than room
 };
 
 // Per (discharge, species) dynamic counts.
@@ -265,6 +266,7 @@ struct WsPtrs {
     int birth_cap;            // records per sub-tile
     unsigned long long *colscan_agg;  // column totals of the sort's row segments, tagged with the sort
     int *birth_blk;           // [2][max_chunks / TILE_ALIGN + 1][3] births per append block and product species, by step parity
+    int *birth_room;          // [2][D * 3] by step parity: free slots less the births staged so far
     Counts *tab;              // [2][D * 3] the tile table of a step by its parity, for its births
     unsigned long long *acc_fix;  // [3 * total_nodes] fixed-point density accumulators
     double *acc_dbl;          // [3 * total_nodes] FP64 accumulators

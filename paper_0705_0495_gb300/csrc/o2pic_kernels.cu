@@ -367,7 +367,8 @@ __device__ __forceinline__ void field_block(const WsPtrs &W, int par, int diag, 
 // Tile table for the step of parity par: tiles of each discharge start at a
 // multiple of TILE_ALIGN, so that the birth-append blocks never span two, and
 // those of each species at a multiple of TILES_PER_TICKET, so that a push
-// ticket never spans two; the step's birth counts are cleared.  With `advance`
+// ticket never spans two; the step's birth counts are cleared and its room for
+// births is set.  With `advance`
 // the next step's counter is set and the candidate list emptied.  The counts
 // are the current ones, or (after_births) those that the births of the step
 // before will leave: its table's counts plus what staging has counted.
@@ -382,6 +383,7 @@ __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bo
     constexpr int A = TILE_ALIGN, B = TILES_PER_TICKET;
     const Counts *old = W.tab + (par ? 0 : W.D * NSP);  // the table of the other parity
     Counts *keep = W.tab + (par ? W.D * NSP : 0);
+    int *room = W.birth_room + (par ? W.D * NSP : 0);
     if (after_births) {
         for (int k = tid; k < W.D * NSP; k += NT) s_add[k] = 0;
         __syncthreads();
@@ -434,6 +436,7 @@ __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bo
                 const Counts c{n[s], n[s], start + at[s], (n[s] + CHUNK - 1) / CHUNK};
                 W.cnt[d * NSP + s] = c;
                 keep[d * NSP + s] = c;
+                room[d * NSP + s] = W.disc[d].cap[s] - n[s];
             }
             if (d == W.D - 1) {
                 int chunk = start + end;
@@ -444,6 +447,7 @@ __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bo
                 ctl->total_chunks = chunk;
                 ctl->tab_total[par] = chunk;
                 ctl->ticket = 0u;
+                ctl->over[par] = 0;
                 if (advance) {
                     ctl->cand_n = 0u;
                     ctl->step[par ^ 1] = step + 1ull;
@@ -577,6 +581,7 @@ __device__ __forceinline__ void births_block(const WsPtrs &W, const Pools<Real> 
         for (int w = 0; w < warp; ++w) excl[q] += wsum[q][w];
     const Disc &Dd = W.disc[d];
     const unsigned b0 = ctl->cur ? P.stride : 0u;
+    typename AccK<Real>::T *acc = AccK<Real>::ptr(W) + Dd.gbase;
 #pragma unroll
     for (int j = 0; j < TPT; ++j) {
         const BirthRec<Real> *rec = rec0 + (size_t)(t0 + j) * W.birth_cap;
@@ -591,8 +596,9 @@ __device__ __forceinline__ void births_block(const WsPtrs &W, const Pools<Real> 
                 rank += (tk & 3) == q && tk < b.tag;
             }
             const long long dst = (long long)tab[d * NSP + q].n_snap + s_excl[q] + excl[q] + rank;
-            if (dst >= Dd.cap[q]) {
+            if (dst >= Dd.cap[q]) {  // dropped, with the charge that staging deposited
                 set_status(ctl, ST_CAPACITY);
+                dep_global(acc + (size_t)q * W.total_nodes, b.c, b.off, -1);
                 continue;
             }
             const size_t g = (size_t)b0 + Dd.pbase[q] + (size_t)dst;
@@ -624,20 +630,33 @@ k_births(WsPtrs W, Pools<Real> P, int par)
 // (counted then), not the append itself.  Both are chains of latencies: 5.5 and
 // 5.6 us one after the other for seven small discharges, 6.0 us together; 9.7 and
 // 8.3 us for one of 5e7 superparticles, 10.0 together.
+// When a species has more births than room (an error that the call reports),
+// the field has to wait for the append, which drops some and takes their charge
+// back: the first cluster then does one after the other, for all discharges.
 template <typename Real>
 __global__ void __launch_bounds__(FIELD_THREADS)
 k_births_field(WsPtrs W, Pools<Real> P, int par, int diag, int csize)
 {
     pdl_wait();
     const int d = blockIdx.x / csize, rank = blockIdx.x % csize;
-    if (d < W.D) {
-        field_block<Real>(W, par ^ 1, diag, 0, csize, d, rank);
-    } else if (d == W.D) {
-        if (rank == 0) tile_table(W, par ^ 1, W.ctl->step[par ^ 1], true, true);
-    } else {
-        const int blk = blockIdx.x - (W.D + 1) * csize;
-        if (blk <= W.max_chunks / TILE_ALIGN) births_block<Real>(W, P, par, blk, false);
+    const bool over = W.ctl->over[par] != 0;
+    if (over && d != 0) return;
+    int blk = over ? rank : (int)blockIdx.x - (W.D + 1) * csize;
+    const int bend = over ? W.max_chunks / TILE_ALIGN + 1 : min(blk + 1, W.max_chunks / TILE_ALIGN + 1);
+    if (blk >= 0)
+        for (; blk < bend; blk += csize) {
+            births_block<Real>(W, P, par, blk, over);
+            if (over) __syncthreads();
+        }
+    if (over) {
+        __threadfence();
+        cooperative_groups::this_cluster().sync();
     }
+    for (int k = over ? 0 : d; k < (over ? W.D : min(d + 1, W.D)); ++k) {
+        field_block<Real>(W, par ^ 1, diag, 0, csize, k, rank);
+        if (over) __syncthreads();
+    }
+    if ((over || d == W.D) && rank == 0) tile_table(W, par ^ 1, W.ctl->step[par ^ 1], true, !over);
 }
 
 // ------------------------------------------------------------- sort
