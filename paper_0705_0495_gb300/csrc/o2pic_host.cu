@@ -968,6 +968,7 @@ extern "C" pic_status pic_init(const pic_config *cfgs, int n_discharges, const p
     h->L.sort_col_warps = wbase[3 * n_discharges];
     CK(configure_kernels(h->fp64, h->L));
     CK(push_configure(h->fp64, h->L, nsm));
+    CK(deposit_configure(h->fp64, h->L));
 
     // host-built small tables
     std::vector<int> stab;

@@ -2,6 +2,8 @@
 // deposit kernels of libo2pic (GB300, sm_103a).
 #include <cooperative_groups.h>
 
+#include <mutex>
+
 #include "o2pic_launch.h"
 
 namespace o2 {
@@ -2201,42 +2203,45 @@ static size_t inter_smem_bytes(bool fp64)
     return coulomb_smem_bytes(fp64) + (size_t)INTER_TILE * 3 * (fp64 ? 8 : 4);
 }
 
+cudaError_t allow_smem(const void *kernel, size_t bytes)
+{
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
+    cudaFuncAttributes a{};
+    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess || (size_t)a.maxDynamicSharedSizeBytes >= bytes) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 cudaError_t configure_kernels(bool fp64, LaunchCfg &L)
 {
     cudaError_t e;
     L.sort_smem = sizeof(unsigned short) * SORT_WARPS * ((L.maxN + 2) & ~1);
     L.scatter_smem = sizeof(unsigned short) * SORT_WARPS * ((L.maxN + 2) & ~1);
     if (fp64) {
-        e = cudaFuncSetAttribute(k_sort_count<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.sort_smem);
+        e = allow_smem(k_sort_count<double>, L.sort_smem);
         if (e) return e;
-        e = cudaFuncSetAttribute(k_sort_scatter<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.scatter_smem);
+        e = allow_smem(k_sort_scatter<double>, L.scatter_smem);
         if (e) return e;
-        e = cudaFuncSetAttribute(k_coulomb<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)coulomb_smem_bytes(true));
+        e = allow_smem(k_coulomb<double, false>, coulomb_smem_bytes(true));
         if (e) return e;
-        e = cudaFuncSetAttribute(k_coulomb<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)coulomb_smem_bytes(true));
+        e = allow_smem(k_coulomb<double, true>, coulomb_smem_bytes(true));
         if (e) return e;
-        e = cudaFuncSetAttribute(k_coulomb_inter<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)inter_smem_bytes(true));
+        e = allow_smem(k_coulomb_inter<double>, inter_smem_bytes(true));
         if (e) return e;
     } else {
-        e = cudaFuncSetAttribute(k_sort_count<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.sort_smem);
+        e = allow_smem(k_sort_count<float>, L.sort_smem);
         if (e) return e;
-        e = cudaFuncSetAttribute(k_sort_scatter<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.scatter_smem);
+        e = allow_smem(k_sort_scatter<float>, L.scatter_smem);
         if (e) return e;
-        e = cudaFuncSetAttribute(k_coulomb<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)coulomb_smem_bytes(false));
+        e = allow_smem(k_coulomb<float, false>, coulomb_smem_bytes(false));
         if (e) return e;
-        e = cudaFuncSetAttribute(k_coulomb<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)coulomb_smem_bytes(false));
+        e = allow_smem(k_coulomb<float, true>, coulomb_smem_bytes(false));
         if (e) return e;
-        e = cudaFuncSetAttribute(k_coulomb_inter<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)inter_smem_bytes(false));
+        e = allow_smem(k_coulomb_inter<float>, inter_smem_bytes(false));
         if (e) return e;
     }
-    return cudaFuncSetAttribute(k_sort_cellscan, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(sizeof(int) * (L.maxN + 2)));
+    return allow_smem(k_sort_cellscan, sizeof(int) * (L.maxN + 2));
 }
 
 cudaError_t launch_field(bool fp64, bool diag, int mode, const WsPtrs &W, int par, const LaunchCfg &L,

@@ -50,6 +50,16 @@ inline cudaError_t launch_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block,
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
+// The dynamic shared memory that a kernel may be launched with is one number
+// per kernel and device for the whole process: raised to what a handle asks
+// for and never lowered, so that handles of any size work side by side.
+cudaError_t allow_smem(const void *kernel, size_t bytes);
+template <typename... KArgs>
+inline cudaError_t allow_smem(void (*kern)(KArgs...), size_t bytes)
+{
+    return allow_smem(reinterpret_cast<const void *>(kern), bytes);
+}
+
 constexpr int MAX_PUSH_SHAPES = 8;
 
 struct LaunchCfg {
@@ -128,6 +138,7 @@ cudaError_t launch_load(bool fp64, const WsPtrs &W, const void *pools, const lon
                         const double *d_vt, int max_n, cudaStream_t s);
 // charge of every live slot of a discharge (-1: of all), added to cleared
 // accumulators; max_slots: the most slots a discharge can hold
+cudaError_t deposit_configure(bool fp64, const LaunchCfg &L);
 cudaError_t launch_deposit_all(bool fp64, const WsPtrs &W, const void *pools, int disc, long long max_slots,
                                const LaunchCfg &L, cudaStream_t s);
 // state arrays in SI doubles (see the kernels)

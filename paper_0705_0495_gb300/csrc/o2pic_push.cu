@@ -1786,9 +1786,9 @@ static cudaError_t push_shape_setup(LaunchCfg &L, int k)
 {
     const size_t sm = push_smem_bytes<Real>(L.maxN, 0, 0, SH::nw, SH::qcap, true);
     const size_t smd = push_smem_bytes<Real>(L.maxN, L.eedf_max, L.fm_max, SH::nw, SH::qcap, sizeof(Real) == 8);
-    cudaError_t e = cudaFuncSetAttribute(k_push<Real, false, SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_smem(k_push<Real, false, SH>, sm);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_push<Real, true, SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smd);
+    e = allow_smem(k_push<Real, true, SH>, smd);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_push<Real, false, SH>, SH::threads, sm);

@@ -579,10 +579,8 @@ template <typename Real>
 cudaError_t static_setup()
 {
     constexpr int most = (int)sizeof(unsigned) * (Sums<Real>::WORDS + 1) * STATIC_NODES;
-    cudaError_t e = cudaFuncSetAttribute(k_static_deposit<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_static_small<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * most);
-    return e;
+    const cudaError_t e = o2::allow_smem(k_static_deposit<Real>, most);
+    return e != cudaSuccess ? e : o2::allow_smem(k_static_small<Real>, 3 * most);
 }
 
 template <typename Real>
@@ -620,18 +618,26 @@ cudaError_t static_run(void *acc, const int *const *cell, const void *const *off
 
 namespace {
 template <typename Real>
+size_t deposit_smem(int maxN)
+{
+    return sizeof(unsigned) * (Sums<Real>::WORDS + 1) * (maxN + 1);
+}
+template <typename Real>
 cudaError_t deposit_discs(const o2::WsPtrs &W, const o2::Pools<Real> &P, int disc, int maxN, long long max_slots,
                           int num_sms, cudaStream_t st)
 {
-    const size_t sm = sizeof(unsigned) * (Sums<Real>::WORDS + 1) * (maxN + 1);
-    const cudaError_t e =
-        cudaFuncSetAttribute(k_deposit_disc<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
+    const size_t sm = deposit_smem<Real>(maxN);
     const int blocks = (int)std::min<long long>(max_slots / UNIT + 3, 2ll * num_sms);
     k_deposit_disc<Real><<<dim3(blocks, disc >= 0 ? 1 : W.D), UNIT_THREADS, sm, st>>>(W, P, disc);
     return cudaGetLastError();
 }
 } // namespace
+
+cudaError_t o2::deposit_configure(bool fp64, const LaunchCfg &L)
+{
+    return fp64 ? allow_smem(k_deposit_disc<double>, deposit_smem<double>(L.maxN))
+                : allow_smem(k_deposit_disc<float>, deposit_smem<float>(L.maxN));
+}
 
 cudaError_t o2::launch_deposit_all(bool fp64, const WsPtrs &W, const void *pools, int disc, long long max_slots,
                                    const LaunchCfg &L, cudaStream_t st)
