@@ -39,6 +39,9 @@
  * (allocated by the first pic_get_state()); pic_destroy() frees both.  All
  * work is issued on the CUDA stream given to pic_init().
  *
+ * Device: a handle lives on the device that is current in pic_init().  Later
+ * calls may be made with any device current and leave it current.
+ *
  * Errors: every call returns a pic_status; nothing is thrown across the ABI.
  * After an error the handle stays valid and may be destroyed; pic_last_error()
  * returns a text.

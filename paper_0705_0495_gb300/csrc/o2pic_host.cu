@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "../../include/o2pic.h"
+#include "o2pic_device.h"
 #include "o2pic_launch.h"
 
 using namespace o2;
@@ -396,6 +397,7 @@ constexpr size_t STATE_CHUNK = 65536;  // slots pic_get_state converts at a time
 
 struct pic_handle {
     int D = 0;
+    int dev = 0;  // the device that was current in pic_init
     bool fp64 = false;
     std::vector<pic_config> cfg;
     std::vector<HostTable> tabs;
@@ -511,6 +513,18 @@ size_t gather_bytes(const pic_config *c, int D)
         cudaError_t e_ = (call);                                   \
         if (e_ != cudaSuccess) return cuda_fail(h, e_, #call);     \
     } while (0)
+
+namespace {
+struct CudaDevice {
+    static int get(int *d) { return (int)cudaGetDevice(d); }
+    static int set(int d) { return (int)cudaSetDevice(d); }
+};
+} // namespace
+
+// the handle's device is the current one until the call returns
+#define ON_DEVICE(h)                        \
+    o2::OnDevice<CudaDevice> on_(h->dev);   \
+    if (on_.error()) return cuda_fail(h, (cudaError_t)on_.error(), "the handle's device")
 
 extern "C" size_t pic_workspace_size(const pic_config *cfgs, int n_discharges, const pic_xs_table *xs, int n_xs)
 {
@@ -951,6 +965,7 @@ extern "C" pic_status pic_init(const pic_config *cfgs, int n_discharges, const p
 
     int dev = 0, nsm = 0;
     CK(cudaGetDevice(&dev));
+    h->dev = dev;
     CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     h->L.maxN = L.maxN;
     h->L.eedf_max = L.eedf_max;
@@ -1203,6 +1218,7 @@ extern "C" pic_status pic_step(pic_handle *h, long long n_steps)
 {
     if (!h) return fail(nullptr, PIC_EINVAL, "NULL handle");
     if (n_steps < 0) return fail(h, PIC_EINVAL, "n_steps < 0");
+    ON_DEVICE(h);
     const pic_config &q = h->cfg[0];
     if (h->period == 0) {
         long long P = 2;
@@ -1284,6 +1300,7 @@ extern "C" pic_status pic_set_numeric_budget(pic_handle *h, double max_fraction)
 extern "C" pic_status pic_set_step(pic_handle *h, long long step)
 {
     if (!h || step < 0) return fail(h, PIC_EINVAL, "bad handle or step");
+    ON_DEVICE(h);
     unsigned long long v = (unsigned long long)step;
     CK(cudaMemcpyAsync(&h->W.ctl->step[step & 1], &v, 8, cudaMemcpyHostToDevice, h->stream));
     CK(cudaStreamSynchronize(h->stream));
@@ -1296,6 +1313,7 @@ extern "C" pic_status pic_diagnostics(pic_handle *h, int d, double *dens_sum, do
                                       int reset)
 {
     if (!h || d < 0 || d >= h->D) return fail(h, PIC_EINVAL, "bad handle or discharge");
+    ON_DEVICE(h);
     const pic_config &q = h->cfg[d];
     const Disc &D = h->disc[d];
     const int N = q.n_cells, tn = h->W.total_nodes;
@@ -1368,6 +1386,7 @@ extern "C" pic_status pic_get_state(pic_handle *h, int d, int s, double *x, doub
                                     int *alive, long long capacity_n, long long *n)
 {
     if (!h || d < 0 || d >= h->D || s < 0 || s > 2) return fail(h, PIC_EINVAL, "bad handle, discharge or species");
+    ON_DEVICE(h);
     Gather G(h);
     const size_t o_cn = G.add(h->W.cnt + 3 * d + s, sizeof(Counts)), o_cur = G.add(&h->W.ctl->cur, 4);
     CK(G.run());
@@ -1414,6 +1433,7 @@ extern "C" pic_status pic_set_state(pic_handle *h, int d, int s, long long n, co
     if (!h || d < 0 || d >= h->D || s < 0 || s > 2) return fail(h, PIC_EINVAL, "bad handle, discharge or species");
     if (n < 0 || n > h->cfg[d].capacity[s]) return fail(h, PIC_ECAPACITY, "n exceeds the species capacity");
     if (n > 0 && (!x || !vx || !vy || !vz)) return fail(h, PIC_EINVAL, "NULL state array");
+    ON_DEVICE(h);
     const Disc &D = h->disc[d];
     const int N = D.N;
     int cur = 0;
@@ -1468,6 +1488,7 @@ extern "C" pic_status pic_set_state(pic_handle *h, int d, int s, long long n, co
 extern "C" pic_status pic_fields(pic_handle *h, int d, double *rho, double *phi, double *E)
 {
     if (!h || d < 0 || d >= h->D) return fail(h, PIC_EINVAL, "bad handle or discharge");
+    ON_DEVICE(h);
     CK(launch_field(h->fp64, false, 1, h->W, (int)(h->step & 1), h->L, h->stream));
     const Disc &D = h->disc[d];
     const int N = D.N;
@@ -1492,6 +1513,7 @@ extern "C" double pic_numax(const pic_handle *h, int d, int s)
 extern "C" pic_status pic_set_timing(pic_handle *h, int on)
 {
     if (!h) return fail(nullptr, PIC_EINVAL, "NULL handle");
+    ON_DEVICE(h);
     if (on && h->ev.empty()) {
         h->ev.resize(4096);
         h->ev_kind.assign(2048, 0);
@@ -1505,6 +1527,7 @@ extern "C" pic_status pic_timing(pic_handle *h, double *push_ms, long long *push
                                  double *push_bytes, int reset)
 {
     if (!h) return fail(nullptr, PIC_EINVAL, "NULL handle");
+    ON_DEVICE(h);
     std::vector<unsigned long long> c((size_t)h->D * C_NCOUNT);
     CK(cudaMemcpyAsync(c.data(), h->W.counters, 8 * c.size(), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
@@ -1554,6 +1577,7 @@ extern "C" pic_status pic_set_launch(pic_handle *h, int kernel, int blocks_per_s
     if (blocks_per_sm < 1 || blocks_per_sm > h->L.push_max_per_sm)
         return fail(h, PIC_EINVAL, "blocks per SM out of 1 .. " + std::to_string(h->L.push_max_per_sm));
     if (blocks_per_sm == h->L.push_per_sm) return PIC_OK;
+    ON_DEVICE(h);
     // the captured period holds the old grid: wait for it, then drop it
     CK(cudaStreamSynchronize(h->stream));
     if (h->gexec) {
@@ -1608,6 +1632,7 @@ extern "C" pic_status pic_set_launch_shape(pic_handle *h, int kernel, int shape,
     if (blocks_per_sm < 1 || blocks_per_sm > mx)
         return fail(h, PIC_EINVAL, "blocks per SM out of 1 .. " + std::to_string(mx));
     if (shape == h->L.push_shape && blocks_per_sm == h->L.push_per_sm) return PIC_OK;
+    ON_DEVICE(h);
     // the captured graph holds the old grid: wait for it, then drop it
     CK(cudaStreamSynchronize(h->stream));
     if (h->gexec) {
@@ -1631,6 +1656,7 @@ extern "C" pic_status pic_kernel_timing(pic_handle *h, int kernel, double *ms, l
                                         double *bytes, int reset)
 {
     if (!h) return fail(nullptr, PIC_EINVAL, "NULL handle");
+    ON_DEVICE(h);
     if (kernel == PIC_KERNEL_PUSH || kernel == PIC_KERNEL_PUSH_DIAG) {
         // the push launches of one kind; the algorithmic bytes are shared out
         // by launches (every launch of a step moves the same particle data)
