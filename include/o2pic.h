@@ -345,9 +345,10 @@ pic_status pic_kernel_timing(pic_handle *h, int kernel, double *ms, long long *l
  * step 1 and the null-collision test of step 5) is a persistent grid of
  * blocks_per_sm blocks on every SM (of the current shape's threads, see
  * pic_launch_shapes below), each block taking tickets of tiles until none
- * are left.  pic_init sets the largest count that fits on
+ * are left.  FP32 mixed: pic_init sets the largest count that fits on
  * an SM (registers and shared memory); pic_set_launch may lower it to any
- * count in 1 .. that maximum.  Results do not depend on it: the charge sums
+ * count in 1 .. that maximum.  FP64: pic_init sets 1; pic_set_launch takes 1 or
+ * 2 (one block is resident, the second follows it).  Results do not depend on it: the charge sums
  * are exact integers and births are appended in parent order (FP32 mixed
  * state is bit for bit the same; the FP64 path adds each block's charge to
  * double accumulators, whose rounding can differ in the last bits).  The

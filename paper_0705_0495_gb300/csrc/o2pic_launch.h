@@ -65,7 +65,7 @@ constexpr int MAX_PUSH_SHAPES = 8;
 struct LaunchCfg {
     int push_blocks;      // persistent grid of the push
     int push_per_sm;      // its blocks per SM
-    int push_max_per_sm;  // the most that fit on an SM (current shape)
+    int push_max_per_sm;  // the most accepted (current shape)
     int push_shape;       // index of the push's launch shape
     int push_nshapes;     // shapes compiled for this precision
     int shape_threads[MAX_PUSH_SHAPES], shape_spt[MAX_PUSH_SHAPES], shape_max_per_sm[MAX_PUSH_SHAPES];

@@ -34,6 +34,7 @@
 // field's steps from a table, floors and energy bins off the FP64 units and one
 // block per SM to 578 us (835 with diagnostics, 1350 before; 9.2 us): about
 // five FP64 instructions a particle, 340 us for its bytes.
+#include <algorithm>
 #include <cstdio>
 
 #include "o2pic_launch.h"
@@ -1780,6 +1781,9 @@ using PushF4 = PushShape<256, 8, 2>;
 // (FP64: one block of 16 warps per SM, so that its field and sums are held once:
 // 32 bytes per cell, with room for the histograms)
 using PushD0 = PushShape<512, 4, 1>;
+// Blocks per SM that callers may set in FP64.  One is resident and the default;
+// of two the second follows the first (no block waits for another).
+constexpr int PUSH_D_BLOCKS = 2;
 
 template <typename Real, typename SH>
 static cudaError_t push_shape_setup(LaunchCfg &L, int k)
@@ -1807,6 +1811,7 @@ cudaError_t push_configure(bool fp64, LaunchCfg &L, int num_sms)
     if (fp64) {
         L.push_nshapes = 1;
         if ((e = push_shape_setup<double, PushD0>(L, 0))) return e;
+        L.shape_max_per_sm[0] = std::max(L.shape_max_per_sm[0], PUSH_D_BLOCKS);
     } else {
         L.push_nshapes = 5;
         if ((e = push_shape_setup<float, PushF0>(L, 0))) return e;
@@ -1818,7 +1823,7 @@ cudaError_t push_configure(bool fp64, LaunchCfg &L, int num_sms)
     L.num_sms = num_sms;
     L.push_shape = 0;
     L.push_max_per_sm = L.shape_max_per_sm[0];
-    L.push_per_sm = L.push_max_per_sm;
+    L.push_per_sm = fp64 ? 1 : L.push_max_per_sm;
     L.push_blocks = num_sms * L.push_per_sm;
     L.push_smem = L.shape_smem[0];
     L.push_smem_diag = L.shape_smem_diag[0];
