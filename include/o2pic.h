@@ -412,13 +412,14 @@ pic_status pic_set_launch_shape(pic_handle *h, int kernel, int shape, int blocks
  * fixed array of 3 x 4097 x 8 bytes in device memory, which every GPU that
  * loads this library reserves until the process exits.  The first call on a
  * device looks up that array's device address with the device current, and
- * under CUDA's default lazy module loading that first call also loads this
- * library's kernels and the array onto the device (a driver-side
- * allocation): make one warm-up call per device before any region that must
- * not allocate and before any stream capture, or run with
- * CUDA_MODULE_LOADING=EAGER.  All calls on a
- * device share the array and clear it first: calls that can run at the same
- * time on the GPU (unordered streams) race and corrupt each other's output.
+ * under CUDA's default lazy module loading that first call also loads the
+ * kernels of every size and precision and the array onto the device (a
+ * driver-side allocation): make one warm-up call per device, of any size and
+ * precision, before any region that must not allocate and before any stream
+ * capture, or run with CUDA_MODULE_LOADING=EAGER.  Calls of more than 128000
+ * slots (n[0] + n[1] + n[2]) share the array and clear it first: two of them
+ * that can run at the same time on the GPU (unordered streams) race and
+ * corrupt each other's output.  Smaller calls use shared memory only.
  */
 pic_status pic_field_solve_static(const pic_config *cfg, long long step,
                                   const int *const *d_cell,

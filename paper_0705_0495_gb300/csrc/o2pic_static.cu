@@ -575,12 +575,16 @@ pic_status static_fail(pic_status s, const std::string &m)
     return s;
 }
 
+// Reaches every kernel that a call may launch, whatever the first call's size
+// and precision: asking for a kernel's attributes loads it.
 template <typename Real>
 cudaError_t static_setup()
 {
     constexpr int most = (int)sizeof(unsigned) * (Sums<Real>::WORDS + 1) * STATIC_NODES;
-    const cudaError_t e = o2::allow_smem(k_static_deposit<Real>, most);
-    return e != cudaSuccess ? e : o2::allow_smem(k_static_small<Real>, 3 * most);
+    cudaError_t e = o2::allow_smem(k_static_deposit<Real>, most);
+    if (e == cudaSuccess) e = o2::allow_smem(k_static_small<Real>, 3 * most);
+    if (e == cudaSuccess) e = o2::allow_smem(k_static_solve<Real>, 0);
+    return e;
 }
 
 template <typename Real>
