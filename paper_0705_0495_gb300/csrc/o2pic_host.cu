@@ -413,6 +413,7 @@ struct pic_handle {
     std::vector<Disc> disc;
     std::vector<NuBin> nubin;   // [D * NUBIN_MAX]
     std::vector<double> numax;  // [D*3]
+    std::vector<int> slots;     // [D*3] slots in use at the last look
     std::string err;
     // largest accepted fraction of nu_max violations among null-collision
     // candidates and of Eq. 1 P > 1 clamps among Eq. 1 evaluations
@@ -497,7 +498,7 @@ struct Gather {
 };
 size_t gather_bytes(const pic_config *c, int D)
 {
-    size_t most = 8ull * C_NCOUNT * D + 64;
+    size_t most = (8ull * C_NCOUNT + sizeof(Counts) * 3) * D + 64;
     for (int d = 0; d < D; ++d) {
         const size_t nodes = c[d].n_cells + 1, fm = c[d].fm_bins > 0 ? (size_t)c[d].fm_xbins * c[d].fm_bins : 0;
         const size_t diag = 8 * 3 * nodes + 16 * nodes + 4 * (size_t)c[d].eedf_bins + 8 * (size_t)c[d].iedf_bins + 4 * fm +
@@ -921,6 +922,7 @@ extern "C" pic_status pic_init(const pic_config *cfgs, int n_discharges, const p
     h->disc.resize(n_discharges);
     h->nubin.assign((size_t)n_discharges * NUBIN_MAX, NuBin{});
     h->numax.assign(3 * n_discharges, 0.0);
+    h->slots.resize(3 * n_discharges);
     for (int d = 0; d < n_discharges; ++d) build_disc(h, d, gas, gcount, pair_tab);
     // node-major gas tables: row k of (d, s) holds n_j dx sigma_j(E_k), j < nch
     std::vector<double> gt(std::max(1LL, L.gtab_n), 0.0);
@@ -1003,6 +1005,7 @@ extern "C" pic_status pic_init(const pic_config *cfgs, int n_discharges, const p
     for (int d = 0; d < n_discharges; ++d)
         for (int s = 0; s < 3; ++s) {
             ninit[3 * d + s] = h->cfg[d].n_init[s];
+            h->slots[3 * d + s] = (int)h->cfg[d].n_init[s];
             vt[3 * d + s] = std::sqrt(h->cfg[d].T0_eV[s] * QE / MASS[s]);
             cnt[3 * d + s] = Counts{(int)h->cfg[d].n_init[s], 0, 0, 0};
             max_n = std::max(max_n, (int)h->cfg[d].n_init[s]);
@@ -1108,7 +1111,7 @@ static cudaError_t enqueue_step(pic_handle *h, long long n, int &nk, bool timed,
     }
     if (coul) {
         if ((e = time_open(h, timed, st))) return e;
-        e = launch_coulomb(h->fp64, h->W, h->pools(), par, st);
+        e = launch_coulomb(h->fp64, h->W, h->pools(), par, h->L, st);
         if (e) return e;
         ++nk;
         if (q.coulomb_inter) {
@@ -1159,9 +1162,11 @@ static pic_status harvest_events(pic_handle *h)
 static pic_status check_status(pic_handle *h)
 {
     Gather G(h);
-    const size_t o_st = G.add(&h->W.ctl->status, 4), o_c = G.add(h->W.counters, 8ull * h->D * C_NCOUNT);
+    const size_t o_st = G.add(&h->W.ctl->status, 4), o_c = G.add(h->W.counters, 8ull * h->D * C_NCOUNT),
+                 o_n = G.add(h->W.cnt, sizeof(Counts) * 3 * h->D);
     CK(G.run());
     const char *pin = reinterpret_cast<const char *>(h->pin);
+    for (int k = 0; k < 3 * h->D; ++k) h->slots[k] = reinterpret_cast<const Counts *>(pin + o_n)[k].n;
     const unsigned status = *reinterpret_cast<const unsigned *>(pin + o_st);
     const unsigned long long *c = reinterpret_cast<const unsigned long long *>(pin + o_c);
     if (status & ST_TIMEOUT) return fail(h, PIC_ETIMEOUT, "a bounded device wait (sort column scan) gave up");
@@ -1211,6 +1216,39 @@ static bool capture_steps(pic_handle *h, long long nsteps, cudaGraphExec_t *out,
     return ok;
 }
 
+// The captured graphs hold the launches as they were: waits for them, drops them.
+static cudaError_t drop_graphs(pic_handle *h)
+{
+    cudaError_t e = cudaStreamSynchronize(h->stream);
+    for (cudaGraphExec_t *g : {&h->gexec, &h->gexec_cycle})
+        if (e == cudaSuccess && *g) {
+            e = cudaGraphExecDestroy(*g);
+            if (e == cudaSuccess) *g = nullptr;
+        }
+    return e;
+}
+
+// Does the Coulomb pass take its cells in groups, a warp each?  By the mean
+// particles per cell of every species at the last look (the cost follows the
+// particles, which grow many times over in a run, not the capacity).  Groups win
+// until a species' cells pass COUL_WARP, which a group then works off one after
+// the other; a block each for all cells wins when they are resident in a few
+// turns anyway.  Groups / a block each: 2688 cells of 78 electrons or O- and 156
+// O2+ 15 / 55 us, four times that 54 / 56, ten times 104 / 66; 1536 cells of 2000
+// to 4000 131 / 58; 48 cells of 600 to 1250 76 / 12.  (The gap between the two
+// lines keeps a run near them from recording its graphs again and again.)
+static bool coulomb_groups(const pic_handle *h)
+{
+    const double line = COUL_WARP * (h->L.coul_groups ? 0.9 : 0.8);
+    long long cells = 0;
+    for (int d = 0; d < h->D; ++d)
+        for (int s = 0; s < 3; ++s) {
+            cells += h->cfg[d].n_cells;
+            if (h->slots[3 * d + s] > line * h->cfg[d].n_cells) return false;
+        }
+    return cells > 4LL * h->L.num_sms;
+}
+
 // the longest stretch captured as one graph
 constexpr long long MAX_GRAPH_STEPS = 8192;
 
@@ -1236,6 +1274,10 @@ extern "C" pic_status pic_step(pic_handle *h, long long n_steps)
         h->cycle_steps = 0;
         if (c >= P && std::fabs(spc - (double)c) <= 1e-6 * spc && c % P == 0 && c <= MAX_GRAPH_STEPS)
             h->cycle_steps = c;
+    }
+    if (q.n2 > 0 && coulomb_groups(h) != h->L.coul_groups) {
+        CK(drop_graphs(h));
+        h->L.coul_groups = !h->L.coul_groups;
     }
     long long left = n_steps;
     while (left > 0) {
@@ -1473,6 +1515,7 @@ extern "C" pic_status pic_set_state(pic_handle *h, int d, int s, long long n, co
                                h->stream));
         }
     }
+    h->slots[3 * d + s] = (int)n;
     Counts cn{(int)n, 0, 0, 0};
     CK(cudaMemcpyAsync(h->W.cnt + 3 * d + s, &cn, sizeof cn, cudaMemcpyHostToDevice, h->stream));
     const int tn = h->W.total_nodes;
@@ -1578,16 +1621,7 @@ extern "C" pic_status pic_set_launch(pic_handle *h, int kernel, int blocks_per_s
         return fail(h, PIC_EINVAL, "blocks per SM out of 1 .. " + std::to_string(h->L.push_max_per_sm));
     if (blocks_per_sm == h->L.push_per_sm) return PIC_OK;
     ON_DEVICE(h);
-    // the captured period holds the old grid: wait for it, then drop it
-    CK(cudaStreamSynchronize(h->stream));
-    if (h->gexec) {
-        CK(cudaGraphExecDestroy(h->gexec));
-        h->gexec = nullptr;
-    }
-    if (h->gexec_cycle) {
-        CK(cudaGraphExecDestroy(h->gexec_cycle));
-        h->gexec_cycle = nullptr;
-    }
+    CK(drop_graphs(h));
     h->L.push_per_sm = blocks_per_sm;
     h->L.push_blocks = h->L.num_sms * blocks_per_sm;
     return PIC_OK;
@@ -1633,16 +1667,7 @@ extern "C" pic_status pic_set_launch_shape(pic_handle *h, int kernel, int shape,
         return fail(h, PIC_EINVAL, "blocks per SM out of 1 .. " + std::to_string(mx));
     if (shape == h->L.push_shape && blocks_per_sm == h->L.push_per_sm) return PIC_OK;
     ON_DEVICE(h);
-    // the captured graph holds the old grid: wait for it, then drop it
-    CK(cudaStreamSynchronize(h->stream));
-    if (h->gexec) {
-        CK(cudaGraphExecDestroy(h->gexec));
-        h->gexec = nullptr;
-    }
-    if (h->gexec_cycle) {
-        CK(cudaGraphExecDestroy(h->gexec_cycle));
-        h->gexec_cycle = nullptr;
-    }
+    CK(drop_graphs(h));
     h->L.push_shape = shape;
     h->L.push_max_per_sm = mx;
     h->L.push_smem = h->L.shape_smem[shape];

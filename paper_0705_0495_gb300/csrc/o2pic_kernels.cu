@@ -1590,11 +1590,10 @@ __device__ __forceinline__ void coulomb_cell(const WsPtrs &W, const Pools<Real> 
 // permutation's greatest common divisor, the copies, a few collisions per
 // thread): 2688 cells of about 150 particles took 56 us with a block each, in
 // nine waves, and 11.7 us so (cells of 2000 to 4000 particles
-// took 54 us with a block each and 5% of the whole run more in groups).  Both forms handle every size; the host
-// picks the groups when the capacity is at most COUL_GROUP_CAP slots per cell
-// (larger cells fill a block's warps, and a block per cell balances better).
+// took 58 us with a block each and 131 us in groups).  Both forms handle every
+// size and give the same bits; the host picks one by the particles that the
+// cells hold (coulomb_groups).
 constexpr int COUL_GROUP = COUL_THREADS / 32;
-constexpr int COUL_WARP = COUL_STAGE / COUL_GROUP;  // staged particles per warp
 template <typename Real, bool GROUP>
 __global__ void __launch_bounds__(COUL_THREADS, sizeof(Real) == 4 ? 2 : 1)
 k_coulomb(WsPtrs W, Pools<Real> P, int par)
@@ -2308,22 +2307,22 @@ cudaError_t launch_sort(bool fp64, const WsPtrs &W, const void *pools, const int
 size_t coulomb_smem_bytes(bool fp64) { return (size_t)COUL_STAGE * 3 * (fp64 ? 8 : 4); }
 
 template <typename Real>
-static void launch_coulomb_real(const WsPtrs &W, const Pools<Real> &P, int par, size_t smem, cudaStream_t st)
+static void launch_coulomb_real(const WsPtrs &W, const Pools<Real> &P, int par, bool groups, size_t smem, cudaStream_t st)
 {
     const int cells = W.total_cells * NSP;
-    if ((long long)P.stride <= (long long)COUL_GROUP_CAP * cells)
+    if (groups)
         launch_k(k_coulomb<Real, true>, (cells + COUL_GROUP - 1) / COUL_GROUP, COUL_THREADS, smem, st, W, P, par);
     else
         launch_k(k_coulomb<Real, false>, cells, COUL_THREADS, smem, st, W, P, par);
 }
 
-cudaError_t launch_coulomb(bool fp64, const WsPtrs &W, const void *pools, int par, cudaStream_t st)
+cudaError_t launch_coulomb(bool fp64, const WsPtrs &W, const void *pools, int par, const LaunchCfg &L, cudaStream_t st)
 {
     const size_t smem = coulomb_smem_bytes(fp64);
     if (fp64)
-        launch_coulomb_real<double>(W, *static_cast<const Pools<double> *>(pools), par, smem, st);
+        launch_coulomb_real<double>(W, *static_cast<const Pools<double> *>(pools), par, L.coul_groups, smem, st);
     else
-        launch_coulomb_real<float>(W, *static_cast<const Pools<float> *>(pools), par, smem, st);
+        launch_coulomb_real<float>(W, *static_cast<const Pools<float> *>(pools), par, L.coul_groups, smem, st);
     return cudaGetLastError();
 }
 

@@ -79,6 +79,7 @@ struct LaunchCfg {
     size_t scatter_smem;  // scatter kernel
     int sort_col_warps;   // warps of the column scan (sum over (d, s) of bucket groups x row segments)
     const int *sort_warp_base;  // device [D*3+1]: first column-scan warp per (d, s)
+    bool coul_groups;     // Coulomb pass: a block per group of cells
     int maxN;             // largest cell count over discharges
     int eedf_max, fm_max; // largest histogram sizes (shared-memory copies in the push)
 };
@@ -107,9 +108,9 @@ cudaError_t launch_field(bool fp64, bool diag, int mode, const WsPtrs &W, int pa
 
 cudaError_t launch_sort(bool fp64, const WsPtrs &W, const void *pools,
                         const int *sort_block_ds, const LaunchCfg &L, cudaStream_t s);
-// Coulomb pass: blocks of COUL_THREADS threads, one per (cell, species) or, up to
-// COUL_GROUP_CAP slots per cell, one per group of cells; cells of at most
-// COUL_STAGE particles are staged in shared memory
+// Coulomb pass: blocks of COUL_THREADS threads, one per (cell, species) or one
+// per group of cells; cells of at most COUL_STAGE particles are staged in shared
+// memory, in a group those of at most COUL_WARP by one warp each
 #ifndef O2_COUL_THREADS
 #define O2_COUL_THREADS 384
 #endif
@@ -118,12 +119,9 @@ cudaError_t launch_sort(bool fp64, const WsPtrs &W, const void *pools,
 #endif
 constexpr int COUL_THREADS = O2_COUL_THREADS;
 constexpr int COUL_STAGE = O2_COUL_STAGE;
-#ifndef O2_COUL_GROUP_CAP
-#define O2_COUL_GROUP_CAP 4096
-#endif
-constexpr int COUL_GROUP_CAP = O2_COUL_GROUP_CAP;
+constexpr int COUL_WARP = COUL_STAGE / (COUL_THREADS / 32);
 size_t coulomb_smem_bytes(bool fp64);
-cudaError_t launch_coulomb(bool fp64, const WsPtrs &W, const void *pools, int par, cudaStream_t st);
+cudaError_t launch_coulomb(bool fp64, const WsPtrs &W, const void *pools, int par, const LaunchCfg &L, cudaStream_t st);
 // inter-species Coulomb collisions (e-O-, e-O2+, O- - O2+ in turn)
 cudaError_t launch_coulomb_inter(bool fp64, const WsPtrs &W, const void *pools, int par, cudaStream_t st);
 cudaError_t launch_pair(bool fp64, const WsPtrs &W, const void *pools, int par,
