@@ -231,12 +231,12 @@ struct Ctl {
     unsigned int ticket;          // dynamic chunk counter of the push
     int total_chunks;             // chunks in the current push
     int D;                        // discharges
-    unsigned int cand_n;          // collision candidates listed by the push this step
+    unsigned int cand_n[2];       // collision candidates listed by the push, by step parity
     unsigned int colscan_ticket;  // warp order of the sort's column scan
     unsigned int sort_epoch;      // sorts so far (tags the column scan's words)
     unsigned int scatter_done;    // scatter blocks that have finished
     int tab_total[2];             // tiles of the tables in WsPtrs::tab
-    int over[2];                  // by step parity: a species has more births than room
+    int room[2];                  // by step parity: fewest free slots of a species at its start
 };
 
 // Per (discharge, species) dynamic counts.
@@ -266,7 +266,6 @@ struct WsPtrs {
     int birth_cap;            // records per sub-tile
     unsigned long long *colscan_agg;  // column totals of the sort's row segments, tagged with the sort
     int *birth_blk;           // [2][max_chunks / TILE_ALIGN + 1][3] births per append block and product species, by step parity
-    int *birth_room;          // [2][D * 3] by step parity: free slots less the births staged so far
     Counts *tab;              // [2][D * 3] the tile table of a step by its parity, for its births
     unsigned long long *acc_fix;  // [3 * total_nodes] fixed-point density accumulators
     double *acc_dbl;          // [3 * total_nodes] FP64 accumulators

@@ -83,7 +83,7 @@ struct Bump {
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 struct Layout {
-    size_t colscan_agg, sort_whist, ctl, disc, cnt, phi_s2_sum, phi0_sum, D0_sum, gtab, gtabf, gpm, gpmf, tile_cnt, births, birth_blk, birth_room, tab, sort_tot, warp_base, vmax2, nubin, cand, acc, Efield, Ereal, phi, rho, dens, dens_sum, phi_sum, nsamp,
+    size_t colscan_agg, sort_whist, ctl, disc, cnt, phi_s2_sum, phi0_sum, D0_sum, gtab, gtabf, gpm, gpmf, tile_cnt, births, birth_blk, tab, sort_tot, warp_base, vmax2, nubin, cand, acc, Efield, Ereal, phi, rho, dens, dens_sum, phi_sum, nsamp,
         counters, eedf, iedf, fm, tables, lutE, lutS, lutEf, lutSf, sort_counts, cell_start,
         sort_live, pair_bcount, cell_disc, pair_births, sort_tab, ninit, vt;
     size_t cell[2], off[2], vx[2], vy[2], vz[2];
@@ -330,7 +330,6 @@ Layout make_layout(const pic_config *c, int D, const pic_xs_table *xs, int n_xs,
     L.birth_cap = c[0].gas_scheme == 1 ? BIRTH_CAP_SEQ : BIRTH_CAP_W;
     L.births = B.take((size_t)mc * SUBTILES * L.birth_cap * (fp64 ? 40 : 24));
     L.birth_blk = B.take(2 * 4ull * 3 * (mc / TILE_ALIGN + 1));
-    L.birth_room = B.take(2 * 4ull * 3 * D);
     L.tab = B.take(2 * sizeof(Counts) * 3 * D);
     L.acc = B.take(8ull * 3 * tn);
     L.Efield = B.take(8ull * tn);
@@ -828,7 +827,6 @@ extern "C" pic_status pic_init(const pic_config *cfgs, int n_discharges, const p
     W.births = b + L.births;
     W.birth_cap = L.birth_cap;
     W.birth_blk = reinterpret_cast<int *>(b + L.birth_blk);
-    W.birth_room = reinterpret_cast<int *>(b + L.birth_room);
     W.tab = reinterpret_cast<Counts *>(b + L.tab);
     W.colscan_agg = reinterpret_cast<unsigned long long *>(b + L.colscan_agg);
     W.acc_fix = reinterpret_cast<unsigned long long *>(b + L.acc);

@@ -2,6 +2,7 @@
 // deposit kernels of libo2pic (GB300, sm_103a).
 #include <cooperative_groups.h>
 
+#include <climits>
 #include <mutex>
 
 #include "o2pic_launch.h"
@@ -366,11 +367,36 @@ __device__ __forceinline__ void field_block(const WsPtrs &W, int par, int diag, 
     }
 }
 
+// Births staged in the step of parity par, per (discharge, product species), for
+// a whole block (in shared memory).
+__device__ __forceinline__ const int *staged_births(const WsPtrs &W, int par)
+{
+    __shared__ int s_add[MAX_DISCHARGES * NSP];
+    const Counts *tab = W.tab + (par ? W.D * NSP : 0);
+    const int *words = birth_words(W, par);
+    const int n = (W.ctl->tab_total[par] * SUBTILES + BIRTHS_TILES - 1) / BIRTHS_TILES * NSP;
+    for (int k = threadIdx.x; k < W.D * NSP; k += blockDim.x) s_add[k] = 0;
+    __syncthreads();
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+        const int v = words[k];
+        if (v == 0) continue;
+        const int tile = k / NSP * TILE_ALIGN;
+        int lo = 0, hi = W.D;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (tab[mid * NSP].chunk0 <= tile) lo = mid; else hi = mid;
+        }
+        atomicAdd(&s_add[lo * NSP + k % NSP], v);
+    }
+    __syncthreads();
+    return s_add;
+}
+
 // Tile table for the step of parity par: tiles of each discharge start at a
 // multiple of TILE_ALIGN, so that the birth-append blocks never span two, and
 // those of each species at a multiple of TILES_PER_TICKET, so that a push
-// ticket never spans two; the step's birth counts are cleared and its room for
-// births is set.  With `advance`
+// ticket never spans two; the step's birth counts are cleared and the smallest
+// room of a species is noted.  With `advance`
 // the next step's counter is set and the candidate list emptied.  The counts
 // are the current ones, or (after_births) those that the births of the step
 // before will leave: its table's counts plus what staging has counted.
@@ -378,32 +404,14 @@ __device__ __forceinline__ void field_block(const WsPtrs &W, int par, int diag, 
 // list took 0.25 us per entry: 50 us of every step of 64 discharges).
 __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bool advance, bool after_births)
 {
-    __shared__ int s_warp[32];
-    __shared__ int s_add[MAX_DISCHARGES * NSP];
+    __shared__ int s_warp[32], s_room;
     Ctl *ctl = W.ctl;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NT = blockDim.x;
     constexpr int A = TILE_ALIGN, B = TILES_PER_TICKET;
     const Counts *old = W.tab + (par ? 0 : W.D * NSP);  // the table of the other parity
     Counts *keep = W.tab + (par ? W.D * NSP : 0);
-    int *room = W.birth_room + (par ? W.D * NSP : 0);
-    if (after_births) {
-        for (int k = tid; k < W.D * NSP; k += NT) s_add[k] = 0;
-        __syncthreads();
-        const int *words = birth_words(W, par ^ 1);
-        const int n = (ctl->tab_total[par ^ 1] * SUBTILES + BIRTHS_TILES - 1) / BIRTHS_TILES * NSP;
-        for (int k = tid; k < n; k += NT) {
-            const int v = words[k];
-            if (v == 0) continue;
-            const int tile = k / NSP * TILE_ALIGN;
-            int lo = 0, hi = W.D;
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (old[mid * NSP].chunk0 <= tile) lo = mid; else hi = mid;
-            }
-            atomicAdd(&s_add[lo * NSP + k % NSP], v);
-        }
-        __syncthreads();
-    }
+    const int *add = after_births ? staged_births(W, par ^ 1) : nullptr;
+    if (tid == 0) s_room = INT_MAX;
     int first = 0;  // tiles of the discharges before this pass
     for (int d0 = 0; d0 < W.D; d0 += NT) {
         const int d = d0 + tid;
@@ -411,7 +419,7 @@ __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bo
         if (d < W.D) {
 #pragma unroll
             for (int s = 0; s < NSP; ++s)
-                n[s] = after_births ? min(old[d * NSP + s].n_snap + s_add[d * NSP + s], W.disc[d].cap[s])
+                n[s] = after_births ? min(old[d * NSP + s].n_snap + add[d * NSP + s], W.disc[d].cap[s])
                                     : W.cnt[d * NSP + s].n;
         }
 #pragma unroll
@@ -428,6 +436,12 @@ __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bo
         }
         __syncthreads();  // s_warp of the pass before has been read
         if (lane == 31) s_warp[warp] = v;
+        int room = INT_MAX;
+        if (d < W.D)
+#pragma unroll
+            for (int s = 0; s < NSP; ++s) room = min(room, W.disc[d].cap[s] - n[s]);
+        room = __reduce_min_sync(0xffffffffu, room);
+        if (lane == 0) atomicMin(&s_room, room);
         __syncthreads();
         int start = first + v - size;
         for (int w = 0; w < warp; ++w) start += s_warp[w];
@@ -438,7 +452,6 @@ __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bo
                 const Counts c{n[s], n[s], start + at[s], (n[s] + CHUNK - 1) / CHUNK};
                 W.cnt[d * NSP + s] = c;
                 keep[d * NSP + s] = c;
-                room[d * NSP + s] = W.disc[d].cap[s] - n[s];
             }
             if (d == W.D - 1) {
                 int chunk = start + end;
@@ -449,9 +462,9 @@ __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bo
                 ctl->total_chunks = chunk;
                 ctl->tab_total[par] = chunk;
                 ctl->ticket = 0u;
-                ctl->over[par] = 0;
+                ctl->room[par] = s_room;
                 if (advance) {
-                    ctl->cand_n = 0u;
+                    ctl->cand_n[par] = 0u;
                     ctl->step[par ^ 1] = step + 1ull;
                 }
             }
@@ -635,30 +648,50 @@ k_births(WsPtrs W, Pools<Real> P, int par)
 // When a species has more births than room (an error that the call reports),
 // the field has to wait for the append, which drops some and takes their charge
 // back: the first cluster then does one after the other, for all discharges.
+__device__ __noinline__ bool births_overflow(const WsPtrs &W, int par)
+{
+    const int *add = staged_births(W, par);
+    const Counts *tab = W.tab + (par ? W.D * NSP : 0);
+    bool over = false;
+    for (int k = threadIdx.x; k < W.D * NSP; k += blockDim.x)
+        over |= (long long)tab[k].n_snap + add[k] > W.disc[k / NSP].cap[k % NSP];
+    return __syncthreads_or(over);
+}
+template <typename Real>
+__device__ __noinline__ void births_then_field(const WsPtrs &W, const Pools<Real> &P, int par, int diag, int csize, int rank)
+{
+    for (int blk = rank; blk <= W.max_chunks / TILE_ALIGN; blk += csize) {
+        births_block<Real>(W, P, par, blk, true);
+        __syncthreads();
+    }
+    __threadfence();
+    cooperative_groups::this_cluster().sync();
+    for (int d = 0; d < W.D; ++d) {
+        field_block<Real>(W, par ^ 1, diag, 0, csize, d, rank);
+        __syncthreads();
+    }
+    if (rank == 0) tile_table(W, par ^ 1, W.ctl->step[par ^ 1], true, false);
+}
 template <typename Real>
 __global__ void __launch_bounds__(FIELD_THREADS)
-k_births_field(WsPtrs W, Pools<Real> P, int par, int diag, int csize)
+k_births_field(const __grid_constant__ WsPtrs W, const __grid_constant__ Pools<Real> P, int par, int diag, int csize)
 {
     pdl_wait();
     const int d = blockIdx.x / csize, rank = blockIdx.x % csize;
-    const bool over = W.ctl->over[par] != 0;
-    if (over && d != 0) return;
-    int blk = over ? rank : (int)blockIdx.x - (W.D + 1) * csize;
-    const int bend = over ? W.max_chunks / TILE_ALIGN + 1 : min(blk + 1, W.max_chunks / TILE_ALIGN + 1);
-    if (blk >= 0)
-        for (; blk < bend; blk += csize) {
-            births_block<Real>(W, P, par, blk, over);
-            if (over) __syncthreads();
-        }
-    if (over) {
-        __threadfence();
-        cooperative_groups::this_cluster().sync();
+    // a candidate has at most two products of a species, so fewer than that many
+    // free slots make it worth counting
+    if (W.ctl->room[par] < 2ll * W.ctl->cand_n[par] && births_overflow(W, par)) {
+        if (d == 0) births_then_field<Real>(W, P, par, diag, csize, rank);
+        return;
     }
-    for (int k = over ? 0 : d; k < (over ? W.D : min(d + 1, W.D)); ++k) {
-        field_block<Real>(W, par ^ 1, diag, 0, csize, k, rank);
-        if (over) __syncthreads();
+    if (d < W.D) {
+        field_block<Real>(W, par ^ 1, diag, 0, csize, d, rank);
+    } else if (d == W.D) {
+        if (rank == 0) tile_table(W, par ^ 1, W.ctl->step[par ^ 1], true, true);
+    } else {
+        const int blk = blockIdx.x - (W.D + 1) * csize;
+        if (blk <= W.max_chunks / TILE_ALIGN) births_block<Real>(W, P, par, blk, false);
     }
-    if ((over || d == W.D) && rank == 0) tile_table(W, par ^ 1, W.ctl->step[par ^ 1], true, !over);
 }
 
 // ------------------------------------------------------------- sort

@@ -242,16 +242,13 @@ template <> __device__ __forceinline__ double *acc_global<double>(const WsPtrs &
 
 // Births of one candidate go straight to its sub-tile's records, in any
 // order; the tag restores parent order when they are appended.  Their charge
-// is deposited here, so that the next field does not wait for the append; a
-// birth that finds no room is noted (`over`), and the append takes its charge
-// back before that field.
+// is deposited here, so that the next field does not wait for the append (which
+// takes it back from a birth that finds no room).
 template <typename Real>
 struct BirthSink {
     BirthRec<Real> *rec;  // the sub-tile's birth_cap records
     int *n;               // the sub-tile's record count
     int *blk;             // births per product species of the sub-tile's birth-append block
-    int *room;            // the discharge's free slots per species, less the births so far
-    int *over;            // set when a species has more births than room
     typename AccT<Real>::T *acc;  // the discharge's charge accumulators, first species
     int acc_ld;           // from one species' accumulators to the next
     Ctl *ctl;
@@ -259,12 +256,11 @@ struct BirthSink {
 };
 
 template <typename Real>
-__device__ __forceinline__ BirthSink<Real> birth_sink(const WsPtrs &W, const Disc &Dd, int d, int par, int sub)
+__device__ __forceinline__ BirthSink<Real> birth_sink(const WsPtrs &W, const Disc &Dd, int par, int sub)
 {
     return BirthSink<Real>{reinterpret_cast<BirthRec<Real> *>(W.births) + (size_t)sub * W.birth_cap, W.tile_cnt + sub,
-                           birth_words(W, par) + (size_t)(sub / BIRTHS_TILES) * NSP,
-                           W.birth_room + (size_t)((par ? W.D : 0) + d) * NSP, W.ctl->over + par,
-                           acc_global<Real>(W) + Dd.gbase, W.total_nodes, W.ctl, W.birth_cap};
+                           birth_words(W, par) + (size_t)(sub / BIRTHS_TILES) * NSP, acc_global<Real>(W) + Dd.gbase,
+                           W.total_nodes, W.ctl, W.birth_cap};
 }
 
 // ask the L2 cache to fetch [p, p + bytes) (16-byte aligned, a multiple of
@@ -278,11 +274,7 @@ template <typename Real>
 __device__ __forceinline__ void stage_birth(const BirthSink<Real> &B, int tag, int sp, int c, Real off,
                                             const Real v[3])
 {
-    // (both counts asked for at once: one wait; a record that finds its sub-tile
-    // full only makes `over` show early)
-    const int left = atomicAdd(B.room + sp, -1);
     const int pos = atomicAdd(B.n, 1);
-    if (left <= 0) *B.over = 1;
     if (pos >= B.cap) {
         set_status(B.ctl, ST_BIRTHBUF);
         return;
@@ -1011,7 +1003,7 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
     auto list_out = [&]() {
         int base = 0;
         if (lane == 0) {
-            base = (int)atomicAdd(&ctl->cand_n, (unsigned)qn);
+            base = (int)atomicAdd(&ctl->cand_n[par], (unsigned)qn);
             atomicAdd(&s_cnt[C_CANDS], (unsigned)qn);
             if (Dd_binned(W, ds)) atomicAdd(&s_cnt[C_BCANDS], (unsigned)qn);
             if ((long long)base + qn > W.cand_cap) set_status(ctl, ST_BIRTHBUF);
@@ -1412,7 +1404,7 @@ k_collide(WsPtrs W, Pools<Real> P, int par)
     int q = (blockIdx.x + gridDim.x * warp) * 32 + lane;
     int2 e = q < W.cand_cap ? W.cand[q] : make_int2(0, 0);
     const int yblk = W.cand[min(blockIdx.x * 32u, (unsigned)W.cand_cap - 1u)].y;
-    const int n = (int)min((long long)ctl->cand_n, (long long)W.cand_cap);
+    const int n = (int)min((long long)ctl->cand_n[par], (long long)W.cand_cap);
     const unsigned long long step = ctl->step[par];
     const unsigned b0 = ctl->cur ? P.stride : 0u;
     if ((int)blockIdx.x * 32 >= n) return;
@@ -1440,7 +1432,7 @@ k_collide(WsPtrs W, Pools<Real> P, int par)
             const NuBin &nb = W.nubin[(size_t)d * NUBIN_MAX + (s == 0 ? bin : 0)];
             const Real nbin = pick<Real>(nb.numax_n, nb.numax_n_f);
             const Real nun = S.nbins > 0 ? nbin : pick<Real>(S.numax_n, S.numax_n_f);
-            const BirthSink<Real> B = birth_sink<Real>(W, Dd, d, par, sub);
+            const BirthSink<Real> B = birth_sink<Real>(W, Dd, par, sub);
             const Outcome o = gas_collide<Real>(W, Dd, s, (unsigned)rel, step, nun, vx, vy, vz, P.cell[0] + ib,
                                                 P.off[0] + ib, c, off, slot << 1, B);
             // a null event leaves the particle as it was: nothing to write
@@ -1693,7 +1685,7 @@ k_dsmc(WsPtrs W, Pools<Real> P, int par, int part)
                         if (pr.n > 0) {
                             const int i = pb + rel;
                             const int sub = chunk * SUBTILES + local / SUBTILE;
-                            const BirthSink<Real> B = birth_sink<Real>(W, Dd, d, par, sub);
+                            const BirthSink<Real> B = birth_sink<Real>(W, Dd, par, sub);
                             for (int q = 0; q < pr.n; ++q)
                                 stage_birth<Real>(B, ((local % SUBTILE) << 1) | pr.prod[q], pr.sp[q], cellA[i], offA[i],
                                                   pr.v[q]);
@@ -1746,7 +1738,7 @@ k_dsmc(WsPtrs W, Pools<Real> P, int par, int part)
             cellA[i] = -1;
             deposit_global(acc_global<Real>(W) + (size_t)s * W.total_nodes + Dd.gbase, c, off, -1);
             const int sub = chunk * SUBTILES + local / SUBTILE;
-            const BirthSink<Real> B = birth_sink<Real>(W, Dd, d, par, sub);
+            const BirthSink<Real> B = birth_sink<Real>(W, Dd, par, sub);
             stage_birth<Real>(B, ((local % SUBTILE) << 1) | 1, ssp[local], c, off, v);
         }
     }
