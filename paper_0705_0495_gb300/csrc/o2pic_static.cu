@@ -54,14 +54,18 @@ struct Particles {
 // then count_i - W_i + W_(i-1): the integer that adding both weights of every
 // particle gives.  (64-bit shared atomics are several times slower than
 // 32-bit ones on this part, and double ones slower still.)
-//   FP32: w1 = rn(offset 2^24), words of 12 and 13 bits, 2^19 particles.
-//   FP64: w1 = rn(offset 2^52), words of 18, 17 and 18 bits, 2^14 particles;
-//         the weights are rounded at 2^-53 of a particle, finer than the
-//         rounding of one addition to a double sum above 1.
+//   FP32: w1 = rn(offset 2^24), words of 12 and 13 bits, 2^18 particles.
+//   FP64: w1 = rn(offset 2^63), four words of 16 bits, 2^14 particles: exact for
+//         offsets from 2^-11 on, rounded at 2^-64 of a particle below.  (With
+//         2^-52 and three words, a node that held one small weight was further
+//         from 64 bits than a double sum: 2000 particles in 4096 cells, rho off
+//         by 1.4e-15 of a node's value against 7e-16; 1.3e-16 so.)
+// The sums of all species may go into the same words, electrons and O- negative
+// (modulo 2^32).
 template <typename Real> struct Sums;
 template <> struct Sums<float> {
     static constexpr int WORDS = 2, BITS = o2::FIX_BITS, SPLIT = 12;
-    static constexpr long long MOST = 1ll << 19;  // slots between two flushes
+    static constexpr long long MOST = 1ll << 18;  // slots between two flushes
     static constexpr bool RANGE = false;          // a flush is rare: it looks at every cell
     using Acc = unsigned long long;
     static __device__ __forceinline__ void weigh(float off, unsigned w[WORDS])
@@ -74,50 +78,54 @@ template <> struct Sums<float> {
     }
     static __device__ __forceinline__ long long value(const unsigned w[WORDS])
     {
-        return ((long long)w[1] << SPLIT) + w[0];
+        return (long long)(int)w[1] * (1 << SPLIT) + (int)w[0];
     }
     // a node's sum, from the words of its cell and of the cell before it
-    static __device__ __forceinline__ i128 node(unsigned cnt, const unsigned w[WORDS], const unsigned p[WORDS])
+    static __device__ __forceinline__ i128 node(int cnt, const unsigned w[WORDS], const unsigned p[WORDS])
     {
-        return ((i128)cnt << BITS) - value(w) + value(p);
+        return (i128)((long long)cnt * (1 << BITS) - value(w) + value(p));
     }
     static __device__ __forceinline__ void flush(Acc *a, i128 v) { atomicAdd(a, (Acc)(long long)v); }
     static __device__ __forceinline__ i128 read(Acc v) { return (i128)(long long)v; }
 };
 template <> struct Sums<double> {
-    static constexpr int WORDS = 3, BITS = 52;
+    static constexpr int WORDS = 4, BITS = 63;
     static constexpr long long MOST = 1ll << 14;
     static constexpr bool RANGE = true;  // a flush is frequent: it looks at the cells between the lowest and highest
     using Acc = double;
     static __device__ __forceinline__ void weigh(double off, unsigned w[WORDS])
     {
-        // outside [0, 1): clamped as in the FP32 path (on the integer units:
-        // FP64 has two units per SM here)
+        // outside [0, 1): clamped as in the FP32 path; the weight's bits come from
+        // the offset's (integer units throughout: FP64 has two units per SM here)
         if ((unsigned)__double2hiint(off) >= 0x3FF00000u) off = fmin(fmax(off, 0.0), 1.0);
-        // offset + 1 has its last bit at 2^-52
+        const unsigned long long b = (unsigned long long)__double_as_longlong(off) & 0x7FFFFFFFFFFFFFFFull;
+        const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+        const int sh = (int)(b >> 52) - 1012;  // off = m 2^(sh - 63)
         const unsigned long long v =
-            (unsigned long long)(__double_as_longlong(off + 1.0) - __double_as_longlong(1.0));
-        w[0] = (unsigned)(v & 0x3FFFFull);
-        w[1] = (unsigned)((v >> 18) & 0x1FFFFull);
-        w[2] = (unsigned)(v >> 35);
+            sh >= 0 ? m << sh : (sh >= -53 ? (m + (1ull << (-sh - 1))) >> -sh : 0ull);
+#pragma unroll
+        for (int j = 0; j < WORDS; ++j) w[j] = (unsigned)(v >> (16 * j)) & 0xFFFFu;
     }
     static __device__ __forceinline__ i128 value(const unsigned w[WORDS])
     {
-        return ((i128)w[2] << 35) + ((i128)w[1] << 18) + (i128)w[0];
+        i128 v = (int)w[WORDS - 1];
+#pragma unroll
+        for (int j = WORDS - 2; j >= 0; --j) v = v * 65536 + (int)w[j];
+        return v;
     }
-    static __device__ __forceinline__ i128 node(unsigned cnt, const unsigned w[WORDS], const unsigned p[WORDS])
+    static __device__ __forceinline__ i128 node(int cnt, const unsigned w[WORDS], const unsigned p[WORDS])
     {
-        return ((i128)cnt << BITS) - value(w) + value(p);
+        return (i128)cnt * ((i128)1 << BITS) - value(w) + value(p);
     }
     static __device__ __forceinline__ void flush(Acc *a, i128 v)
     {
-        atomicAdd(a, (double)v * (1.0 / 4503599627370496.0));
+        atomicAdd(a, (double)v * (1.0 / 9223372036854775808.0));
     }
-    // a sum of multiples of 2^-52 (any rounding of the atomics is coarser)
+    // a sum of multiples of 2^-63 (any rounding of the atomics is coarser)
     static __device__ __forceinline__ i128 read(Acc v)
     {
         const double hi = floor(v);
-        return ((i128)(long long)hi << BITS) + (i128)(long long)((v - hi) * 4503599627370496.0);
+        return (i128)(long long)hi * ((i128)1 << BITS) + (i128)(long long)((v - hi) * 9223372036854775808.0);
     }
 };
 
@@ -129,11 +137,12 @@ constexpr int STATIC_CLUSTER = 8;
 // words, each an array of `stride` cells).  As in the push: lanes whose four
 // slots sit in the first lane's cell (ordered particles) sum over the warp and
 // one lane adds for all; a lane whose four share a cell adds them once.
-// Every lane of the warp calls it; cells are -1 for nothing.
+// Every lane of the warp calls it; cells are -1 for nothing.  neg: subtracted.
 template <typename Real>
-__device__ __forceinline__ void add4(unsigned *cnt, int stride, const int c[4], const Real off[4])
+__device__ __forceinline__ void add4(unsigned *cnt, int stride, const int c[4], const Real off[4], bool neg)
 {
     using S = Sums<Real>;
+    auto add = [neg](unsigned *p, unsigned v) { atomicAdd(p, neg ? 0u - v : v); };
     unsigned w[4][S::WORDS], sum[S::WORDS];
 #pragma unroll
     for (int k = 0; k < 4; ++k) S::weigh(off[k], w[k]);
@@ -148,24 +157,24 @@ __device__ __forceinline__ void add4(unsigned *cnt, int stride, const int c[4], 
 #pragma unroll
         for (int j = 0; j < S::WORDS; ++j) all[j] = __reduce_add_sync(0xffffffffu, in ? sum[j] : 0u);
         if ((threadIdx.x & 31) == 0) {
-            atomicAdd(&cnt[c0], 4u * (unsigned)__popc(m));
+            add(&cnt[c0], 4u * (unsigned)__popc(m));
 #pragma unroll
-            for (int j = 0; j < S::WORDS; ++j) atomicAdd(&cnt[(j + 1) * stride + c0], all[j]);
+            for (int j = 0; j < S::WORDS; ++j) add(&cnt[(j + 1) * stride + c0], all[j]);
         }
         if (in) return;
     }
     if (same) {
-        atomicAdd(&cnt[c[0]], 4u);
+        add(&cnt[c[0]], 4u);
 #pragma unroll
-        for (int j = 0; j < S::WORDS; ++j) atomicAdd(&cnt[(j + 1) * stride + c[0]], sum[j]);
+        for (int j = 0; j < S::WORDS; ++j) add(&cnt[(j + 1) * stride + c[0]], sum[j]);
         return;
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         if (c[k] < 0) continue;
-        atomicAdd(&cnt[c[k]], 1u);
+        add(&cnt[c[k]], 1u);
 #pragma unroll
-        for (int j = 0; j < S::WORDS; ++j) atomicAdd(&cnt[(j + 1) * stride + c[k]], w[k][j]);
+        for (int j = 0; j < S::WORDS; ++j) add(&cnt[(j + 1) * stride + c[k]], w[k][j]);
     }
 }
 
@@ -215,7 +224,7 @@ __device__ __forceinline__ i128 node_of(const unsigned *cnt, int stride, int i)
         w[j] = cnt[(j + 1) * stride + i];
         p[j] = i > 0 ? cnt[(j + 1) * stride + i - 1] : 0u;
     }
-    return S::node(cnt[i], w, p);
+    return S::node((int)cnt[i], w, p);
 }
 
 // Charge deposit of many particles.  What bounds it: the particles' bytes
@@ -260,7 +269,7 @@ __device__ __forceinline__ void deposit_share(typename Sums<Real>::Acc *acc, siz
             fetch4<Real>(P, s, (a - u0) * UNIT + 4 * tid, N, c, off);
             for (long long q = a; q < b; ++q) {
                 if (q + 1 < b) fetch4<Real>(P, s, (q + 1 - u0) * UNIT + 4 * tid, N, cx, ox);
-                add4<Real>(ssum, stride, c, off);
+                add4<Real>(ssum, stride, c, off, false);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     if (S::RANGE) {
@@ -501,11 +510,13 @@ k_static_solve(const typename Sums<Real>::Acc *acc, SolveC C, int csize)
 }
 
 // Deposit and solve of few particles in one launch: a cluster of 8 blocks,
-// each with the sums of all three species of its share of the particles in
+// each with the net sums of its share of the particles (all three species) in
 // its own shared memory; block r then collects its nodes from all eight and
 // solves them.  What bounds it: the latency of its stages (4e4 FP64 particles
-// in 128 cells: 12.7 us; the five launches it replaces with one thread's sums
-// 53 us).  Divisions stay off the threads: FP64 runs on few units here.
+// in 128 cells: 12.4 us; the five launches it replaces with one thread's sums
+// 53 us).  Divisions stay off the threads: FP64 runs on few units here.  Sums per
+// species, three times the words to clear and to collect: the same time in up to
+// 256 cells, 2000 FP64 particles in 4096 cells 46 us, 25 so.
 constexpr int SMALL_PER = 2;  // nodes per thread: (4097 / 8) / 512
 constexpr long long SMALL_MOST = 1ll << 17;  // slots: 2^14 per block (the FP64 sums' limit) and species units
 static_assert(SMALL_MOST / STATIC_CLUSTER <= Sums<double>::MOST && SMALL_MOST / STATIC_CLUSTER <= Sums<float>::MOST, "");
@@ -518,8 +529,7 @@ k_static_small(Particles<Real> P, SolveC C)
     o2::pdl_wait();
     cg::cluster_group cl = cg::this_cluster();
     const int rank = blockIdx.x, tid = threadIdx.x, N = C.N, stride = N + 1;
-    const int per_species = (S::WORDS + 1) * stride;
-    for (int k = tid; k < 3 * per_species; k += UNIT_THREADS) ssum[k] = 0u;
+    for (int k = tid; k < (S::WORDS + 1) * stride; k += UNIT_THREADS) ssum[k] = 0u;
     __syncthreads();
     // warps of 128 slots, dealt out block by block, so that the blocks' shares differ by one at most
     int u[4] = {0, 0, 0, 0};
@@ -530,7 +540,7 @@ k_static_small(Particles<Real> P, SolveC C)
         int c[4];
         Real off[4];
         fetch4<Real>(P, s, (long long)(q - (s == 0 ? 0 : (s == 1 ? u[1] : u[2]))) * 128 + 4 * (tid & 31), N, c, off);
-        add4<Real>(ssum + s * per_species, stride, c, off);
+        add4<Real>(ssum, stride, c, off, s != 2);
     }
     cl.sync();
     const int NC = (N + STATIC_CLUSTER) / STATIC_CLUSTER;
@@ -545,13 +555,7 @@ k_static_small(Particles<Real> P, SolveC C)
         const unsigned *o = cl.map_shared_rank(ssum, tid % STATIC_CLUSTER);
         for (int j0 = 0; j0 < count; j0 += UNIT_THREADS / STATIC_CLUSTER) {
             const int j = j0 + tid / STATIC_CLUSTER, i = first + j;
-            i128 v = 0;
-            if (j < count) {
-                i128 n[3];
-#pragma unroll
-                for (int s = 0; s < 3; ++s) n[s] = node_of<Real>(o + s * per_species, stride, i);
-                v = n[2] - n[0] - n[1];
-            }
+            i128 v = j < count ? node_of<Real>(o, stride, i) : (i128)0;
 #pragma unroll
             for (int b = 1; b < STATIC_CLUSTER; b <<= 1) {
                 const unsigned long long lo64 = __shfl_xor_sync(0xffffffffu, (unsigned long long)v, b);
@@ -582,7 +586,7 @@ cudaError_t static_setup()
 {
     constexpr int most = (int)sizeof(unsigned) * (Sums<Real>::WORDS + 1) * STATIC_NODES;
     cudaError_t e = o2::allow_smem(k_static_deposit<Real>, most);
-    if (e == cudaSuccess) e = o2::allow_smem(k_static_small<Real>, 3 * most);
+    if (e == cudaSuccess) e = o2::allow_smem(k_static_small<Real>, most);
     if (e == cudaSuccess) e = o2::allow_smem(k_static_solve<Real>, 0);
     return e;
 }
@@ -603,7 +607,7 @@ cudaError_t static_run(void *acc, const int *const *cell, const void *const *off
     }
     const size_t sm = sizeof(unsigned) * (S::WORDS + 1) * (C.N + 1);
     if (all <= SMALL_MOST - 3 * 128 * STATIC_CLUSTER)  // a block's 128-slot shares stay within SMALL_MOST / 8
-        return o2::launch_cluster(k_static_small<Real>, STATIC_CLUSTER, UNIT_THREADS, STATIC_CLUSTER, st, 3 * sm, P, C);
+        return o2::launch_cluster(k_static_small<Real>, STATIC_CLUSTER, UNIT_THREADS, STATIC_CLUSTER, st, sm, P, C);
     // the array keeps the previous call's sums: clear it first
     cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * 3 * STATIC_NODES, st);
     if (e != cudaSuccess) return e;
@@ -704,7 +708,7 @@ extern "C" pic_status pic_field_solve_static(const pic_config *cfg, long long st
     C.N = N;
     C.dx = cfg->L_m / N;
     C.phi0 = cfg->U_rf_V * sin(2.0 * PI_S * cfg->f_rf_Hz * t + cfg->rf_phase);
-    const double unit = fp64 ? 1.0 / 4503599627370496.0 : 1.0 / (double)(1 << o2::FIX_BITS);
+    const double unit = fp64 ? 1.0 / 9223372036854775808.0 : 1.0 / (double)(1 << o2::FIX_BITS);
     C.c = QE_S * cfg->weight_m2 * unit * C.dx / EPS0_S;
     C.h = C.c / (2.0 * C.dx);
     C.rs = QE_S * cfg->weight_m2 * unit / C.dx;
