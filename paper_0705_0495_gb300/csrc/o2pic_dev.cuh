@@ -194,11 +194,9 @@ struct Disc {
     int cs_base;             // first entry of cell_start arrays (3*(N+2) per discharge)
     double dx, dt, L, weight;
     double U_rf, omega, phase;
-    double vol_fix;          // density per accumulated unit (interior node)
     double dens_fix, dens_fix_wall;  // weight / (node volume * 2^FIX_BITS), inside / at walls
     double Kfix;             // e weight 2^-FIX_BITS / eps0
     double Kone;             // e weight / eps0
-    double kE;               // dt^2/dx
     double f15, mu2_15;      // reaction (15) product speed factor
     double f16;              // (16): v_e = |v_Om| * f16
     double f17;              // (17): w = sqrt(E_cm * f17)
@@ -260,7 +258,6 @@ struct WsPtrs {
     Ctl *ctl;
     Disc *disc;
     Counts *cnt;              // [D*3]
-    int *chunk_ds;            // [D*3 + 1] first chunk per (d,s) (prefix), device copy
     int *tile_cnt;            // [max_chunks * SUBTILES] birth records per sub-tile (zero outside a step)
     void *births;             // [max_chunks * SUBTILES * birth_cap] staged birth records
     int birth_cap;            // records per sub-tile

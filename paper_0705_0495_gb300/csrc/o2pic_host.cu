@@ -561,7 +561,6 @@ static void build_disc(pic_handle *h, int d, const std::vector<int> &gas_tabs_by
     D.omega = 2.0 * PI * q.f_rf_Hz;
     D.phase = q.rf_phase;
     const double tdx = q.dt_s / D.dx, xdt = D.dx / q.dt_s;
-    D.kE = q.dt_s * q.dt_s / D.dx;
     D.dens_fix = q.weight_m2 / (D.dx * (double)(1 << FIX_BITS));
     D.dens_fix_wall = q.weight_m2 / (0.5 * D.dx * (double)(1 << FIX_BITS));
     D.Kfix = QE * q.weight_m2 / (double)(1 << FIX_BITS) / 8.8541878128e-12;
@@ -822,7 +821,6 @@ extern "C" pic_status pic_init(const pic_config *cfgs, int n_discharges, const p
     W.ctl = reinterpret_cast<Ctl *>(b + L.ctl);
     W.disc = reinterpret_cast<Disc *>(b + L.disc);
     W.cnt = reinterpret_cast<Counts *>(b + L.cnt);
-    W.chunk_ds = nullptr;
     W.tile_cnt = reinterpret_cast<int *>(b + L.tile_cnt);
     W.births = b + L.births;
     W.birth_cap = L.birth_cap;

@@ -10,7 +10,6 @@
 namespace o2 {
 
 constexpr double QE_ = 1.602176634e-19;
-constexpr double EPS0_ = 8.8541878128e-12;
 
 // ------------------------------------------------------------ helpers
 
@@ -102,6 +101,11 @@ __device__ int block_scan_exclusive_int(int *a, int M, int *wsum)
 // Kernel time with one block and full sums always -> this: 4096 cells FP32
 // 18.3 -> 8.3 us, FP64 62 -> 10.4 us; 128 cells FP64 13.5 -> 6.6 us; seven
 // discharges FP32 12.6 -> 5.6 us, 64 discharges 55 -> 7.3 us.
+// Why the line lies at 1024 cells (a whole time step, one block / a cluster, one
+// discharge, FP32 and FP64): 256 cells 15.9 / 16.5 and 28.6 / 29.9 us, 512 cells
+// 16.8 / 17.1 and 29.5 / 30.2, 1024 cells 17.8 / 17.3 and 31.5 / 30.4; seven
+// discharges of 1024 cells 18.9 / 18.8 and 37.1 / 36.1, 64 of them 25.0 / 32.4 and
+// 50.7 / 60.8.
 constexpr int FIELD_THREADS = 256;
 constexpr int FIELD_CLUSTER = 8;
 constexpr int FIELD_ONE = 1024;  // nodes up to which one block per discharge is used
@@ -1666,61 +1670,21 @@ k_coulomb(WsPtrs W, Pools<Real> P, int par)
     }
 }
 
-// One Coulomb collision between particles a (velocity va) and b (vb) of
-// unlike species: as coulomb_pair, with the pair's kn, a taking fa of the
-// change of g = va - vb and b minus fb of it.
-template <typename Real>
-__device__ __forceinline__ void coulomb_pair_ab(Real va[3], Real vb[3], Real kn, Real fa, Real fb, Real xi,
-                                                unsigned wphi)
-{
-    using M = CoulMath<Real>;
-    const Real g0 = va[0] - vb[0], g1 = va[1] - vb[1], g2 = va[2] - vb[2];
-    const Real u2 = g0 * g0 + g1 * g1 + g2 * g2;
-    if (!(u2 > Real(0))) return;
-    const Real u = M::sqrt_(u2);
-    const Real d = M::sqrt_(kn * M::inv_u32(Real(0), u2, u)) * xi;
-    Real sn, om;
-    if (fabs(d) <= Real(1)) {
-        const Real r = M::rcp(Real(1) + d * d);
-        sn = Real(2) * d * r;
-        om = Real(2) * d * d * r;
-    } else {
-        const Real e = M::rcp(d);
-        const Real r = M::rcp(Real(1) + e * e);
-        sn = Real(2) * e * r;
-        om = Real(2) * r;
-    }
-    Real sp, cp;
-    M::sincos2pi(unif<Real>(wphi), &sp, &cp);
-    const Real up2 = g0 * g0 + g1 * g1;
-    Real dg[3];
-    if (up2 > Real(0)) {
-        const Real up = M::sqrt_(up2), rp = M::rcp(up);
-        const Real ex = g0 * rp, ey = g1 * rp;
-        const Real a = g2 * sn * cp, b = u * sn * sp;
-        dg[0] = ex * a - ey * b - g0 * om;
-        dg[1] = ey * a + ex * b - g1 * om;
-        dg[2] = -up * sn * cp - g2 * om;
-    } else {
-        dg[0] = u * sn * cp;
-        dg[1] = u * sn * sp;
-        dg[2] = -g2 * om;
-    }
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        va[q] += fa * dg[q];
-        vb[q] -= fb * dg[q];
-    }
-}
-
 #ifndef O2_INTER_CHAINS
 #define O2_INTER_CHAINS 128
 #endif
-constexpr int INTER_CHAINS = O2_INTER_CHAINS;  // most chains (B particles) run on prepared random numbers
+// Most chains (B particles) run on prepared random numbers.  256 cells of 2000 and
+// 4000 ions, all three pairs, FP32 / FP64: 33 electrons a cell 143 / 2057 us with
+// them, 180 / 3002 without, 64 129 / 1563 and 149 / 1959, 120 125 / 1344 and 131 /
+// 1482, 200 123 / 1339 and 129 / 1467, 300 121 / 1323 and 123 / 1430.  The line
+// could lie anywhere up to a block's 384 threads: 128 and 384 take the same time
+// in a whole run (cfg2: 30.3 and 30.5 ms per 200 steps).
+constexpr int INTER_CHAINS = O2_INTER_CHAINS;
 constexpr int INTER_TILE = 1024;               // collisions prepared at a time
 
-// The change of g of one collision, from its random numbers (xi, and sp, cp =
-// sin, cos of the azimuth): coulomb_pair_ab's arithmetic.
+// The change of g = va - vb in one Coulomb collision of unlike particles (as
+// coulomb_pair, with the pair's kn), from its random numbers: xi, and sp, cp =
+// sin, cos of the azimuth.
 template <typename Real>
 __device__ __forceinline__ void coulomb_change(Real g0, Real g1, Real g2, Real kn, Real xi, Real sp, Real cp, Real dg[3])
 {
@@ -1753,6 +1717,20 @@ __device__ __forceinline__ void coulomb_change(Real g0, Real g1, Real g2, Real k
         dg[0] = u * sn * cp;
         dg[1] = u * sn * sp;
         dg[2] = -g2 * om;
+    }
+}
+// The whole collision: a takes fa of the change and b minus fb of it.
+template <typename Real>
+__device__ __forceinline__ void coulomb_pair_ab(Real va[3], Real vb[3], Real kn, Real fa, Real fb, Real xi,
+                                                unsigned wphi)
+{
+    Real sp, cp, dg[3];
+    CoulMath<Real>::sincos2pi(unif<Real>(wphi), &sp, &cp);
+    coulomb_change<Real>(va[0] - vb[0], va[1] - vb[1], va[2] - vb[2], kn, xi, sp, cp, dg);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        va[q] += fa * dg[q];
+        vb[q] -= fb * dg[q];
     }
 }
 __device__ __noinline__ float3 coulomb_change_any(float g0, float g1, float g2, float kn, float xi, float sp, float cp)

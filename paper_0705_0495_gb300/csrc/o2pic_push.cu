@@ -2,20 +2,18 @@
 //
 // One launch advances every live superparticle of every discharge by one time
 // step (paper Sec. II (i) and Sec. III):
-//   phase A, four consecutive slots per thread: gather E at x^n (linear
+//   four consecutive slots per thread: gather E at x^n (linear
 //   interpolation from a shared-memory copy of the node field) -> leapfrog
 //   v^{n+1/2}, x^{n+1} -> absorption at x < 0 or x >= L -> null-collision
 //   test against nu_max (one Philox4x32-10 block serves the four slots) ->
-//   linear charge assignment of x^{n+1} into a per-block shared-memory grid
-//   (warp aggregated, exact fixed point in the FP32 path) -> candidates
-//   queued in shared memory;
-//   phase B, one queued candidate per thread (no divergence across the
-//   collision code): a gas molecule from the Maxwellian at T, the channel
-//   walk over sum_j n_j sigma_j(E) u and the kinematics of the chosen
-//   reaction; a particle that dies leaves the shared grid again; births are
-//   staged per 1024-slot tile and appended in parent order by k_births.
-//   The shared grid is flushed to the global accumulators with one atomic
-//   per touched node.
+//   linear charge assignment of x^{n+1} into per-block shared-memory sums
+//   (warp aggregated, exact integers), flushed to the global accumulators with
+//   one atomic per touched node -> candidates listed for k_collide.
+// k_collide, one candidate per thread: a gas molecule from the Maxwellian at T,
+// the channel walk over sum_j n_j sigma_j(E) u and the kinematics of the chosen
+// reaction; a particle that dies leaves the global charge again; births are
+// staged per 128-slot sub-tile and appended in parent order by k_births.
+// k_dsmc: the sequential gas scheme's channels in its place.
 //
 // Particles are SoA with the position as (int32 cell, offset in [0,1)) and
 // velocities in cells per step.  Slots are processed in tiles of 1024
@@ -29,7 +27,7 @@
 // A warp whose 128 slots are live and stay on the grid (nearly all) takes a
 // path without masks and selects, with its floors from packed adds (FP32) or
 // off the FP64 units where a slot stays in its cell: FP32 push 293 -> 251 us,
-// FP64 1968 -> 960 us, results bit for bit the same.  The FP64 sums in 32-bit
+// FP64 1968 -> 1000 us, results bit for bit the same.  The FP64 sums in 32-bit
 // words per cell took it to 733 us (4e4 superparticles: 17 -> 10.6 us), the
 // field's steps from a table, floors and energy bins off the FP64 units and one
 // block per SM to 578 us (835 with diagnostics, 1350 before; 9.2 us): about
@@ -41,8 +39,6 @@
 
 namespace o2 {
 
-// three 256-thread blocks per SM in the FP32 path (the rare collision path
-// may spill a little), two in the FP64 path
 // tiles ahead of the current one whose particle data a push block asks the
 // L2 cache to fetch (a bulk prefetch issued by one thread; 0 = none)
 #ifndef O2_PUSH_L2_AHEAD
@@ -127,11 +123,6 @@ __device__ __forceinline__ void st4(double *p, const double v[4])
     reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
     reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
 }
-
-// the largest value below 1 (an offset that rounded up to 1 is held there)
-template <typename Real> __device__ __forceinline__ Real below_one();
-template <> __device__ __forceinline__ float below_one<float>() { return 0x1.fffffep-1f; }
-template <> __device__ __forceinline__ double below_one<double>() { return 0x1.fffffffffffffp-1; }
 
 // a < b for values that are not negative: FP64 compares as integers (their
 // bit patterns have the same order), off the few FP64 units

@@ -485,9 +485,11 @@ __device__ void static_solve(const SolveC &C, int csize, int rank, int lo, int h
     }
 }
 
-// The solve from the global accumulators: one block up to 1024 cells, a
-// cluster of 8 beyond.
-constexpr int SOLVE_THREADS = 256, SOLVE_PER = 5, SOLVE_ONE = 1024;
+// The solve from the global accumulators: one block up to SOLVE_ONE cells, a
+// cluster of 8 beyond.  Whole call for 1.8e5 slots, one block / a cluster, FP32
+// and FP64: 128 cells 7.7 / 8.5 and 10.3 / 10.9 us, 256 cells 8.3 / 8.5 and 11.4 /
+// 11.1, 512 cells 9.2 / 8.7 and 13.8 / 11.6, 1024 cells 10.9 / 9.3 and 17.8 / 12.6.
+constexpr int SOLVE_THREADS = 256, SOLVE_PER = 5, SOLVE_ONE = 256;
 template <typename Real>
 __global__ void __launch_bounds__(SOLVE_THREADS)
 k_static_solve(const typename Sums<Real>::Acc *acc, SolveC C, int csize)
