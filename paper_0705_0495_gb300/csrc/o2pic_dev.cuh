@@ -229,12 +229,12 @@ struct Ctl {
     unsigned int ticket;          // dynamic chunk counter of the push
     int total_chunks;             // chunks in the current push
     int D;                        // discharges
-    unsigned int cand_n[2];       // collision candidates listed by the push, by step parity
+    unsigned int cand_n;          // collision candidates listed by the push this step
     unsigned int colscan_ticket;  // warp order of the sort's column scan
     unsigned int sort_epoch;      // sorts so far (tags the column scan's words)
     unsigned int scatter_done;    // scatter blocks that have finished
     int tab_total[2];             // tiles of the tables in WsPtrs::tab
-    int room[2];                  // by step parity: fewest free slots of a species at its start
+    int room[2], births[2];       // by step parity: fewest free slots of a species at its start, births staged
 };
 
 // Per (discharge, species) dynamic counts.

@@ -467,8 +467,9 @@ __device__ void tile_table(const WsPtrs &W, int par, unsigned long long step, bo
                 ctl->tab_total[par] = chunk;
                 ctl->ticket = 0u;
                 ctl->room[par] = s_room;
+                ctl->births[par] = 0;
                 if (advance) {
-                    ctl->cand_n[par] = 0u;
+                    ctl->cand_n = 0u;
                     ctl->step[par ^ 1] = step + 1ull;
                 }
             }
@@ -682,9 +683,8 @@ k_births_field(const __grid_constant__ WsPtrs W, const __grid_constant__ Pools<R
 {
     pdl_wait();
     const int d = blockIdx.x / csize, rank = blockIdx.x % csize;
-    // a candidate has at most two products of a species, so fewer than that many
-    // free slots make it worth counting
-    if (W.ctl->room[par] < 2ll * W.ctl->cand_n[par] && births_overflow(W, par)) {
+    // counted per species only when all births together could be too many for one
+    if (W.ctl->room[par] < W.ctl->births[par] && births_overflow(W, par)) {
         if (d == 0) births_then_field<Real>(W, P, par, diag, csize, rank);
         return;
     }

@@ -240,6 +240,7 @@ struct BirthSink {
     BirthRec<Real> *rec;  // the sub-tile's birth_cap records
     int *n;               // the sub-tile's record count
     int *blk;             // births per product species of the sub-tile's birth-append block
+    int *all;             // births of the step
     typename AccT<Real>::T *acc;  // the discharge's charge accumulators, first species
     int acc_ld;           // from one species' accumulators to the next
     Ctl *ctl;
@@ -250,8 +251,8 @@ template <typename Real>
 __device__ __forceinline__ BirthSink<Real> birth_sink(const WsPtrs &W, const Disc &Dd, int par, int sub)
 {
     return BirthSink<Real>{reinterpret_cast<BirthRec<Real> *>(W.births) + (size_t)sub * W.birth_cap, W.tile_cnt + sub,
-                           birth_words(W, par) + (size_t)(sub / BIRTHS_TILES) * NSP, acc_global<Real>(W) + Dd.gbase,
-                           W.total_nodes, W.ctl, W.birth_cap};
+                           birth_words(W, par) + (size_t)(sub / BIRTHS_TILES) * NSP, W.ctl->births + par,
+                           acc_global<Real>(W) + Dd.gbase, W.total_nodes, W.ctl, W.birth_cap};
 }
 
 // ask the L2 cache to fetch [p, p + bytes) (16-byte aligned, a multiple of
@@ -271,6 +272,7 @@ __device__ __forceinline__ void stage_birth(const BirthSink<Real> &B, int tag, i
         return;
     }
     atomicAdd(B.blk + sp, 1);
+    atomicAdd(B.all, 1);
     deposit_global(B.acc + (size_t)sp * B.acc_ld, c, off, 1);
     BirthRec<Real> &r = B.rec[pos];
     r.c = c;
@@ -994,7 +996,7 @@ k_push(WsPtrs W, Pools<Real> P, int par, int Nmax, int eedf_max, int fm_max)
     auto list_out = [&]() {
         int base = 0;
         if (lane == 0) {
-            base = (int)atomicAdd(&ctl->cand_n[par], (unsigned)qn);
+            base = (int)atomicAdd(&ctl->cand_n, (unsigned)qn);
             atomicAdd(&s_cnt[C_CANDS], (unsigned)qn);
             if (Dd_binned(W, ds)) atomicAdd(&s_cnt[C_BCANDS], (unsigned)qn);
             if ((long long)base + qn > W.cand_cap) set_status(ctl, ST_BIRTHBUF);
@@ -1395,7 +1397,7 @@ k_collide(WsPtrs W, Pools<Real> P, int par)
     int q = (blockIdx.x + gridDim.x * warp) * 32 + lane;
     int2 e = q < W.cand_cap ? W.cand[q] : make_int2(0, 0);
     const int yblk = W.cand[min(blockIdx.x * 32u, (unsigned)W.cand_cap - 1u)].y;
-    const int n = (int)min((long long)ctl->cand_n[par], (long long)W.cand_cap);
+    const int n = (int)min((long long)ctl->cand_n, (long long)W.cand_cap);
     const unsigned long long step = ctl->step[par];
     const unsigned b0 = ctl->cur ? P.stride : 0u;
     if ((int)blockIdx.x * 32 >= n) return;

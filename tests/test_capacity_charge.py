@@ -30,12 +30,12 @@ def _built():
     __graft_entry__.build()
 
 
-def _sim(sizes, fp64, **kw):
+def _sim(sizes, fp64, numeric_budget=None, **kw):
     from paper_0705_0495_gb300 import o2pic
     base = dict(fp64=fp64, U_rf=300.0, T0_eV=(8.0, inputs.T_ION_EV, inputs.T_ION_EV), capacity_factor=1.0,
                 capacity_extra=0, **kw)
     ds = [inputs.cfg1(**dict(base, seed=3 + k, **q)) for k, q in enumerate(sizes)]
-    return o2pic.Simulation(ds, inputs.xs_tables()), ds
+    return o2pic.Simulation(ds, inputs.xs_tables(), numeric_budget=numeric_budget), ds
 
 
 def _step(sim, n):
@@ -61,8 +61,9 @@ def _live(sim, k):
 
 @pytest.mark.parametrize("fp64", [False, True])
 @pytest.mark.parametrize("sizes", list(SIZES))
-def test_fields_after_an_overflow_hold_the_particles_only(sizes, fp64):
-    sim, ds = _sim(SIZES[sizes], fp64)
+@pytest.mark.parametrize("scheme", [0, 1])
+def test_fields_after_an_overflow_hold_the_particles_only(sizes, fp64, scheme):
+    sim, ds = _sim(SIZES[sizes], fp64, numeric_budget=1.0, gas_scheme=scheme)
     over = False
     for _ in range(STEPS):
         over |= _step(sim, 1)
