@@ -40,7 +40,9 @@
  * work is issued on the CUDA stream given to pic_init().
  *
  * Device: a handle lives on the device that is current in pic_init().  Later
- * calls may be made with any device current and leave it current.
+ * calls may be made with any device current and leave it current.  Calls wait
+ * for the stream, which CUDA does not allow while a stream capture in the
+ * global mode is open in any thread.
  *
  * Errors: every call returns a pic_status; nothing is thrown across the ABI.
  * After an error the handle stays valid and may be destroyed; pic_last_error()

@@ -648,8 +648,8 @@ k_births(WsPtrs W, Pools<Real> P, int par)
 // the next step's field and tile table in the same launch: the field needs the
 // births' charge (deposited when they were staged) and the table their numbers
 // (counted then), not the append itself.  Both are chains of latencies: 5.5 and
-// 5.6 us one after the other for seven small discharges, 6.0 us together; 9.7 and
-// 8.3 us for one of 5e7 superparticles, 10.0 together.
+// 5.6 us one after the other for seven small discharges, 6.2 us together; 9.7 and
+// 8.3 us for one of 5e7 superparticles, 9.2 together.
 // When a species has more births than room (an error that the call reports),
 // the field has to wait for the append, which drops some and takes their charge
 // back: the first cluster then does one after the other, for all discharges.
